@@ -357,11 +357,20 @@ TSD_API tsd_status tsd_decoder_set_joint_kernel(tsd_decoder* dec, int32_t kind);
 TSD_API tsd_status tsd_decoder_check(tsd_decoder* dec);
 
 /* Tuning knobs, by name (drops captured graphs):
+ *   "one_launch" 1 (default) / 0: greedy decoding with at most one LM runs a
+ *              whole chunk in one launch where W_out fits a thread-block
+ *              cluster's shared memory and the call's rows fit one wave of
+ *              clusters (about 112 rows at V = 1024, H = 1024); 0, other
+ *              calls, and calls with set_timing(1), joint kernel 1, a chosen
+ *              joint_bn or fusion_path 1 run a row pass and a joint kernel per
+ *              label step.  Both take the same decisions; their fp32 sums
+ *              differ in order;
  *   "pdl"      1 (default) / 0: programmatic dependent launch between the
  *              row pass and the joint kernel, so each kernel's set-up
  *              overlaps the tail of the one before;
  *   "joint_bn" 64, 128 or 256: labels per tensor-core CTA tile (default:
- *              chosen at create from the row count and the SM count);
+ *              chosen at create from the row count and the SM count); turns
+ *              one_launch off (set it again to return to it);
  *   "fusion_path" 0 or 1, greedy decoding with at most one LM (default 0;
  *              1 keeps the V-wide logits out of memory):
  *              1 applies Eq. 1's level-0 LM term (a dense row per unigram

@@ -1,0 +1,1020 @@
+// The whole label loop of one decode_chunk call in one launch (greedy
+// decoding, at most one n-gram LM, the streaming form of Eq. 1): a cluster of
+// CS CTAs decodes R rows from the chunk's first frame to its last with W_out
+// resident in its shared memory.
+//
+// What bounds the two-kernel label step (joint_greedy.cu, row_stream.cu) at
+// few rows is not work but the chain of launches and round trips to L2: 9.4 us
+// a step for one stream (V = 1024, H = 640), 10.4 us for 64, against well
+// under 1 us of arithmetic.  Here a step has no launch, no grid-wide
+// dependency and no logits in memory (13 frames of one stream: 619 -> 212 us,
+// of 64 streams: 674 -> 302 us; 16 streams x 1 frame, H = 1024: 71 -> 36 us):
+//   * CTA c of the cluster keeps labels [c nl, (c+1) nl) of W_out in shared
+//     memory for the whole chunk (read once per chunk, not once per step);
+//   * warps 0-7 (GEMM) compute the slice's logits of all R rows: bf16
+//     mma.sync 16 x 8 x 16 with labels as the 16-row operand and rows as the
+//     8-column one, so one row costs one eighth of what a 128-row tcgen05 tile
+//     does and the eight warps split H; their partials are summed in a fixed
+//     order and sent to the row's owner CTA by st.async;
+//   * row i is owned by CTA i mod CS, group i / CS: 128 threads that keep the
+//     row's state in shared memory, take the argmax, publish the label to
+//     every CTA (8 bytes each by st.async), and only then advance the LM and
+//     trie chains and build the next state's deltas, while the GEMM warps
+//     already load the embedding rows and multiply;
+//   * a cluster stops when its rows have finished their frames.
+// Clusters never wait for one another.  Messages inside a cluster complete
+// bytes on the receiver's mbarriers: `ybar` (every CTA: the R rows' labels of
+// a step) and `lbar` (per owned row: its logits), one phase per step each.
+// Every wait is bounded (DecView::wait_ns); after an expired one the CTA
+// records a code, leaves the loop, lets messages in flight land and meets the
+// others at the cluster barrier that ends the kernel.
+//
+// The arithmetic is the streaming form's: fused + lse = (logit + D) + (c_r +
+// lambda * delta), see row_stream.cu.  Level 0 of the LM chain comes from the
+// unigram state's dense row (copied by cp.async while the label is searched),
+// the levels above overwrite their labels' deltas.  The order of every sum
+// depends on V and H only, so a row's result does not depend on the other
+// rows, on R or on CS.
+#include <algorithm>
+
+#include "row_common.cuh"
+#include "chunk_cluster.h"
+#include "tc_common.cuh"
+
+namespace tsd {
+
+namespace {
+
+using row::best_merge;
+using row::checked;
+using row::kNegInf;
+using row::lse_merge;
+
+constexpr int kGemm = 256;     // GEMM threads (8 warps, each an eighth of H)
+constexpr int kGroup = 128;    // threads of a row group
+constexpr int kWarpsG = kGroup / 32;
+static_assert(kWarpsG == 4, "a row group's four warps");
+constexpr int kTiles = 5;      // 16-label tiles per accumulator block
+constexpr int kMB = 16 * kTiles;
+constexpr int kPS = kMB + 4;   // row stride of the partials: lanes (n = 2c, m = g) fall in different banks
+constexpr int kUnits = 4;      // 32-wide pieces of H per warp: H <= 1024
+constexpr int kTrHeld = 3;     // trie chain nodes whose first children a thread requests together
+constexpr int kWPad = 64;      // bytes after a W_out row: neighbouring rows start 16 banks apart
+
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+
+// Remote stores that complete their bytes on a barrier of the receiving CTA.
+__device__ __forceinline__ void send16(uint32_t dst, float4 v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(dst),
+               "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar)
+               : "memory");
+}
+__device__ __forceinline__ void send8(uint32_t dst, int a, int b, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.s32 [%0], {%1, %2}, [%3];" ::"r"(dst), "r"(a),
+               "r"(b), "r"(bar)
+               : "memory");
+}
+
+// The phase of the given parity has completed (a look, without the wait that
+// try_wait may spend in the hardware).
+__device__ __forceinline__ bool test_cluster(uint64_t* b, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(tc::smem_u32(b)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
+__device__ __forceinline__ bool try_cluster(uint64_t* b, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(tc::smem_u32(b)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
+// Waits for the phase of the given parity; false once limit_ns has passed or
+// another warp of the CTA has given up.
+__device__ __forceinline__ bool wait_cluster(uint64_t* b, uint32_t parity, unsigned long long limit_ns,
+                                             volatile int* fail) {
+  if (test_cluster(b, parity)) return true;
+  if (limit_ns == 0) return false;  // no waiting allowed
+  const unsigned long long t0 = tc::global_ns();
+  while (!try_cluster(b, parity)) {
+    if (*fail || tc::global_ns() - t0 > limit_ns) return false;
+  }
+  return true;
+}
+
+__device__ __forceinline__ void group_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+  __syncwarp();
+}
+
+// The same barrier with a vote: true if every thread's ok is (so that all of
+// them leave a loop together, and none is left waiting at a later barrier).
+__device__ __forceinline__ bool group_all(int id, int threads, bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.and.pred q, %2, %3, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(ok ? 1u : 0u), "r"(id), "r"(threads)
+      : "memory");
+  __syncwarp();
+  return r != 0;
+}
+
+__device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                         uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "
+               "{%0, %1, %2, %3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// A float as an integer of the same order (and back); -0 counts as below +0, so
+// a value that may be -0 has 0 added first.
+__device__ __forceinline__ int order_key(float v) {
+  const int i = __float_as_int(v);
+  return i ^ ((i >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float key_value(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7fffffff)); }
+
+// bf16(ReLU(x + z)) of eight elements.  The bf16 add rounds the exact sum
+// once; rounding it to fp32 first, as the row passes do, gives the same: the
+// fp32 sum of two bf16 values is inexact only where the smaller one is below
+// 2^-16 of the larger, far from the middle between two bf16 values.
+__device__ __forceinline__ uint4 joint8(uint4 x, uint4 z) {
+  uint4 o;
+  const __nv_bfloat162* xa = reinterpret_cast<const __nv_bfloat162*>(&x);
+  const __nv_bfloat162* za = reinterpret_cast<const __nv_bfloat162*>(&z);
+  __nv_bfloat162* oa = reinterpret_cast<__nv_bfloat162*>(&o);
+  const __nv_bfloat162 zero = __floats2bfloat162_rn(0.f, 0.f);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) oa[q] = __hmax2(__hadd2(xa[q], za[q]), zero);
+  return o;
+}
+
+// A row's state and search results.
+struct RowSm {
+  int4 lmr[kLmChain + 1], trr[kTrChain];       // chain records, as in row_stream.cu
+  int4 lm_hit[kLmChain + 1], tr_hit[kTrChain]; // records found for the emitted label
+  int4 uni_hit, root_hit;
+  int lm[kLmChain + 1], tr[kTrChain];
+  int4 best[2][kWarpsG];                       // the warps' bests (value, label, wait succeeded), by step parity
+  int nl, nt;
+};
+
+// Shared-memory layout of a CTA (bytes from the 128-byte-aligned base).
+struct Layout {
+  int w, part, dflt, root, y, bars, rows, row_bytes, logits, lse, dlm, lev, dep, total;
+};
+__host__ __device__ inline Layout layout(int H, int V4, int nl, int CS, int NB, int RG) {
+  Layout L;
+  auto up = [](int x) { return (x + 127) & ~127; };
+  int o = 0;
+  L.bars = o, o += 128;                      // ybar, wbar, lbar[RG], sbar[RG], fail flag
+  L.y = o, o = up(o + 8 * CS * RG);          // (previous label, frame or -1) of every row of the cluster
+  L.w = o, o = up(o + nl * (2 * H + kWPad));
+  L.part = o, o = up(o + 8 * (8 * NB) * kPS * 4);
+  L.dflt = o, o = up(o + 4 * V4);            // the call's defaults D
+  L.root = o, o = up(o + (V4 + 31) / 32 * 4);
+  L.rows = o;
+  int r = (int)((sizeof(RowSm) + 127) & ~size_t(127));
+  L.logits = r, r = up(r + 2 * 4 * CS * nl);  // two steps' logits
+  L.lse = r, r = up(r + 2 * 8 * CS * ((nl + kMB - 1) / kMB));  // and softmax partials
+  L.dlm = r, r = up(r + 4 * V4);
+  L.lev = r, r = up(r + 2 * V4);
+  L.dep = r, r = up(r + V4);
+  L.row_bytes = r;
+  L.total = o + RG * r + 128;                // and the alignment of the base
+  return L;
+}
+
+// Aligned groups of four arcs a chain level's arcs [b, b + c) span.
+__device__ __forceinline__ int level_groups(int b, int c) { return c > 0 ? (b + c - (b & ~3) + 3) >> 2 : 0; }
+
+// Position of y in the sorted arr[0, n), or -1, by one warp (row_stream.cu
+// describes the search).  pre: this lane's probe of the whole range (n > 124)
+// or its four entries (n <= 124), loaded before y was known.
+__device__ __forceinline__ int find_from(const int32_t* __restrict__ arr, int n, int y, int lane, int4 pre) {
+  row::reconverge();
+  int lo = 0, hi = n;
+  bool whole = n <= 124;
+  if (!whole) {
+    int v = pre.x;
+    for (;;) {
+      const int step = (hi - lo + 31) >> 5;
+      const unsigned m = __ballot_sync(0xffffffffu, v <= y);
+      if (m == 0) return -1;
+      lo = lo + (31 - __clz((int)m)) * step;
+      hi = min(hi, lo + step);
+      if (hi - lo <= 124) break;
+      const int idx = lo + lane * ((hi - lo + 31) >> 5);
+      v = (idx < hi) ? __ldg(arr + idx) : INT_MAX;
+    }
+  }
+  const uintptr_t at = reinterpret_cast<uintptr_t>(arr + lo);
+  const int first = 4 * lane - (int)((at & 15u) >> 2);
+  int pos = -1;
+  if (first < hi - lo) {
+    const int4 t = whole ? pre : __ldg(reinterpret_cast<const int4*>(at & ~uintptr_t(15)) + lane);
+    const int tv[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+    for (int j = 3; j >= 0; --j)
+      if (first + j >= 0 && first + j < hi - lo && tv[j] == y) pos = lo + first + j;
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, pos >= 0);
+  return m ? __shfl_sync(0xffffffffu, pos, __ffs((int)m) - 1) : -1;
+}
+
+// What find_from wants in `pre` for the range arr[0, n).
+__device__ __forceinline__ int4 first_probe(const int32_t* __restrict__ arr, int n, int lane) {
+  int4 pre = make_int4(INT_MAX, INT_MAX, INT_MAX, INT_MAX);
+  if (n > 124) {
+    const int at = lane * ((n + 31) >> 5);
+    if (at < n) pre.x = __ldg(arr + at);
+  } else {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(arr);
+    if (4 * lane - (int)((a & 15u) >> 2) < n) pre = __ldg(reinterpret_cast<const int4*>(a & ~uintptr_t(15)) + lane);
+  }
+  return pre;
+}
+
+struct Ctx {
+  unsigned char* sm;
+  Layout L;
+  uint64_t *ybar, *wbar, *lbar, *sbar;
+  volatile int* fail;
+  int2* y;
+  int CS, rank, nl, R, row0;
+};
+
+// ---------------------------------------------------------------- GEMM warps
+
+// A lane's piece of a row's joint input operands: elements 32 un + 8 k4 ..
+// of its encoder frame and of its previous label's embedding.
+struct Piece {
+  uint4 x[kUnits], z[kUnits];
+};
+
+// One block of HT half tiles of 8 labels from label m0 of the slice: this
+// warp's part of H for 8 NB rows, written to the partials [warp][row][label].
+// Labels past the slice read its last row again, and the upper half of an odd
+// last tile its lower half: their sums are never sent.
+template <int HT, int NB>
+__device__ __forceinline__ void tile_block(const unsigned char* W, int wstride, int nl, int m0, int U, int warp, int g, int k4,
+                                           const uint4 (&b)[kUnits][NB], float* part) {
+  constexpr int MT = (HT + 1) / 2;
+  float acc[MT][NB][4];
+  int off[HT];
+#pragma unroll
+  for (int t = 0; t < HT; ++t) off[t] = min(m0 + 8 * t + g, nl - 1) * wstride + k4 * 16;
+#pragma unroll
+  for (int t = 0; t < MT; ++t)
+#pragma unroll
+    for (int j = 0; j < NB; ++j)
+#pragma unroll
+      for (int x = 0; x < 4; ++x) acc[t][j][x] = 0.f;
+#pragma unroll
+  for (int u = 0; u < kUnits; ++u) {
+    const int un = warp + 8 * u;
+    if (un < U) {
+      uint4 a[HT];
+#pragma unroll
+      for (int t = 0; t < HT; ++t) a[t] = *reinterpret_cast<const uint4*>(W + off[t] + un * 64);
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int t = 0; t < MT; ++t)
+#pragma unroll
+          for (int j = 0; j < NB; ++j) {
+            const uint4 lo = a[2 * t], hi = a[2 * t + 1 < HT ? 2 * t + 1 : 2 * t];
+            if (h == 0) mma16816(acc[t][j], lo.x, hi.x, lo.y, hi.y, b[u][j].x, b[u][j].y);
+            else mma16816(acc[t][j], lo.z, hi.z, lo.w, hi.w, b[u][j].z, b[u][j].w);
+          }
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < MT; ++t)
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+      float* o = part + (warp * 8 * NB + 8 * j + 2 * k4) * kPS + 16 * t + g;
+      o[0] = acc[t][j][0];
+      o[kPS] = acc[t][j][1];
+      if (2 * t + 1 < HT) {
+        o[8] = acc[t][j][2];
+        o[kPS + 8] = acc[t][j][3];
+      }
+    }
+}
+
+template <int NB>
+__device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = lane >> 2, k4 = lane & 3;
+  const int U = d.H / 32, H = d.H;
+  const int wstride = 2 * H + kWPad;
+  const unsigned char* W = c.sm + c.L.w;
+  float* part = reinterpret_cast<float*>(c.sm + c.L.part);
+  const uint32_t sm0 = tc::smem_u32(c.sm);
+  // this warp's operands of row i (zero for a finished row or none)
+  auto load = [&](int i, Piece& q) {
+    const int2 st = i < c.R ? c.y[i] : make_int2(0, -1);
+    const uint4* e = reinterpret_cast<const uint4*>(P.enc + ((size_t)(c.row0 + i) * P.T + max(st.y, 0)) * H) + k4;
+    const uint4* m = reinterpret_cast<const uint4*>(d.E + (size_t)st.x * H) + k4;
+#pragma unroll
+    for (int u = 0; u < kUnits; ++u) {
+      const int un = warp + 8 * u;
+      q.x[u] = q.z[u] = make_uint4(0u, 0u, 0u, 0u);
+      if (un < U && st.y >= 0) {
+        q.x[u] = __ldg(e + 4 * un);
+        q.z[u] = __ldg(m + 4 * un);
+      }
+    }
+  };
+  for (int step = 0;; ++step) {
+    // the rows' labels (at first, W_out's slice as well)
+    bool ok = wait_cluster(c.ybar, step & 1, d.wait_ns, c.fail);
+    if (step == 0) ok = ok && wait_cluster(c.wbar, 0, d.wait_ns, c.fail);
+    if (!group_all(1, kGemm, ok)) {
+      if (tid == 0) atomicOr(d.err, 1);
+      *c.fail = 1;
+      return;
+    }
+    Piece q[NB];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) load(8 * j + g, q[j]);
+    int active = 0;  // rows still decoding: the next step's publishers
+    for (int i = lane; i < c.R; i += 32) active += c.y[i].y >= 0 ? 1 : 0;
+    active = __reduce_add_sync(0xffffffffu, active);
+    if (active == 0) return;
+    if (tid == 0) tc::mbar_expect_tx(c.ybar, 8u * (uint32_t)active);
+    // the joint inputs, bf16(ReLU(enc + E)); a lane's eight consecutive
+    // elements feed two 16-deep MMAs (the same order of H in both operands)
+    uint4 b[kUnits][NB];
+#pragma unroll
+    for (int u = 0; u < kUnits; ++u)
+#pragma unroll
+      for (int j = 0; j < NB; ++j) b[u][j] = joint8(q[j].x[u], q[j].z[u]);
+    __syncwarp();
+    for (int m0 = 0; m0 < c.nl; m0 += kMB) {
+      const int left = c.nl - m0;
+      if (left > 72) tile_block<10, NB>(W, wstride, c.nl, m0, U, warp, g, k4, b, part);
+      else if (left > 64) tile_block<9, NB>(W, wstride, c.nl, m0, U, warp, g, k4, b, part);
+      else if (left > 48) tile_block<8, NB>(W, wstride, c.nl, m0, U, warp, g, k4, b, part);
+      else if (left > 32) tile_block<6, NB>(W, wstride, c.nl, m0, U, warp, g, k4, b, part);
+      else if (left > 16) tile_block<4, NB>(W, wstride, c.nl, m0, U, warp, g, k4, b, part);
+      else tile_block<2, NB>(W, wstride, c.nl, m0, U, warp, g, k4, b, part);
+      // the warps' partials summed in a fixed order and sent to the rows' owners
+      group_sync(1, kGemm);
+      const int nq = min(kMB, c.nl - m0) / 4;
+#pragma unroll
+      for (int j = 0; j < NB; ++j) {
+        const int i = 8 * j + warp;
+        if (i >= c.R || c.y[i].y < 0) continue;  // the same for the warp's lanes
+        const int grp = i / c.CS, owner = i - grp * c.CS;
+        const uint32_t row = sm0 + c.L.rows + grp * c.L.row_bytes;
+        float4 s[8];
+        if (lane < nq) {
+#pragma unroll
+          for (int w = 0; w < 8; ++w)
+            s[w] = *reinterpret_cast<const float4*>(part + (w * 8 * NB + i) * kPS + 4 * lane);
+#pragma unroll
+          for (int h = 1; h < 8; h *= 2)
+#pragma unroll
+            for (int w = 0; w < 8; w += 2 * h) {
+              s[w].x += s[w + h].x;
+              s[w].y += s[w + h].y;
+              s[w].z += s[w + h].z;
+              s[w].w += s[w + h].w;
+            }
+          const uint32_t dst = row + c.L.logits + 4 * ((step & 1) * c.CS * c.nl + c.rank * c.nl + m0 + 4 * lane);
+          send16(map_rank(dst, owner), s[0], map_rank(tc::smem_u32(c.lbar + grp), owner));
+        }
+        // the block's softmax partial (max, sum of exp) follows: an emitted
+        // label's score needs it, one step later
+        const int v0 = c.rank * c.nl + m0 + 4 * lane;
+        const float l[4] = {lane < nq && v0 < d.N ? s[0].x : kNegInf, lane < nq && v0 + 1 < d.N ? s[0].y : kNegInf,
+                            lane < nq && v0 + 2 < d.N ? s[0].z : kNegInf, lane < nq && v0 + 3 < d.N ? s[0].w : kNegInf};
+        __syncwarp();
+        const float m = key_value(__reduce_max_sync(0xffffffffu, order_key(fmaxf(fmaxf(l[0], l[1]), fmaxf(l[2], l[3])))));
+        const float m2 = m * tc::kLog2e;
+        float z = 0.f;
+        if (m != kNegInf)
+          z = (tc::ex2_approx(fmaf(l[0], tc::kLog2e, -m2)) + tc::ex2_approx(fmaf(l[1], tc::kLog2e, -m2))) +
+              (tc::ex2_approx(fmaf(l[2], tc::kLog2e, -m2)) + tc::ex2_approx(fmaf(l[3], tc::kLog2e, -m2)));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+        if (lane == 0) {
+          const int nb = (c.nl + kMB - 1) / kMB;
+          const uint32_t dst = row + c.L.lse + 8 * ((step & 1) * c.CS * nb + c.rank * nb + m0 / kMB);
+          send8(map_rank(dst, owner), __float_as_int(m), __float_as_int(z), map_rank(tc::smem_u32(c.sbar + grp), owner));
+        }
+      }
+      __syncwarp();
+      group_sync(1, kGemm);
+    }
+  }
+}
+
+// ---------------------------------------------------------------- row groups
+
+__device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int grp) {
+  const int tid = ((int)threadIdx.x - kGemm) % kGroup, lane = tid & 31, warp = tid >> 5;
+  const int i = grp * c.CS + c.rank;  // the row's place in the cluster
+  const int r = c.row0 + i;
+  const int bar = 2 + grp;
+  const int V = d.V, T = P.T;
+  unsigned char* rs = c.sm + c.L.rows + grp * c.L.row_bytes;
+  RowSm& s = *reinterpret_cast<RowSm*>(rs);
+  const float* logits = reinterpret_cast<const float*>(rs + c.L.logits);
+  float* dlm = reinterpret_cast<float*>(rs + c.L.dlm);        // every label's c_r + delta (while built: its LM delta / lambda)
+  uint16_t* lev = reinterpret_cast<uint16_t*>(rs + c.L.lev);  // LM chain levels above 0 with an arc for it (bit l)
+  uint8_t* dep = rs + c.L.dep;                                // trie goto depth (0: none)
+  const float* dflt = reinterpret_cast<const float*>(c.sm + c.L.dflt);
+  const uint32_t* root = reinterpret_cast<const uint32_t*>(c.sm + c.L.root);
+  const bool lm2 = d.has_lm && d.lm.order >= 2;
+  const float lam = P.lambda;
+  const float bscale = P.beta * (d.has_tr ? d.tr.bonus : 0.f);
+  const uint32_t y_addr = tc::smem_u32(c.y + i), y_bar = tc::smem_u32(c.ybar);
+
+  // the row's label and frame (-1: finished) to every CTA of the cluster
+  auto publish = [&](int last, int t) {
+    if (tid < c.CS) send8(map_rank(y_addr, tid), last, t < T ? t : -1, map_rank(y_bar, tid));
+  };
+
+  // state of the stream
+  const int slot = P.slots[r];
+  int last = __ldcg(d.s_last + slot);
+  if (!checked(slot >= 0 && slot < d.lm_stride && last >= 0 && last <= V, d.err, 1)) last = V;
+  publish(last, 0);
+  if (tid == 0) {
+    s.nl = d.has_lm ? __ldcg(d.s_lm_len + slot) : 0;
+    s.nt = d.has_tr ? __ldcg(d.s_tr_len + slot) : 0;
+  } else if (tid >= 32 && tid < 32 + kLmChain) {
+    const int l = tid - 32;
+    if (d.has_lm) {
+      s.lm[l] = __ldcg(d.s_lm_chain + (size_t)slot * kLmChain + l);
+      s.lmr[l] = __ldcg(d.s_lm_rec + (size_t)slot * kLmChain + l);
+    }
+  } else if (tid >= 64 && tid < 64 + kTrChain) {
+    const int k = tid - 64;
+    if (d.has_tr) {
+      s.tr[k] = __ldcg(d.s_tr_chain + (size_t)slot * kTrChain + k);
+      s.trr[k] = __ldcg(d.s_tr_rec + (size_t)slot * kTrChain + k);
+    }
+  }
+  group_sync(bar, kGroup);
+#ifdef TSD_CHECKS
+  if (tid == 0) {
+    bool ok = checked(s.nl >= 0 && s.nl <= kLmChain && s.nt >= 0 && s.nt <= kTrChain, d.err, 2);
+    for (int l = 0; ok && l < s.nl; ++l) {
+      const int4 q = s.lmr[l];
+      ok = checked(s.lm[l] >= 0 && s.lm[l] < d.lm.n_states, d.err, 4) &&
+           checked(q.x >= 0 && q.y >= 0 && (int64_t)q.x + q.y <= d.lm.n_arcs, d.err, 5) &&
+           checked(l > 0 || (q.w >= 0 && q.w < d.lm.n_dense), d.err, 6);
+    }
+    for (int k = 0; ok && k < s.nt; ++k) {
+      const int4 q = s.trr[k];
+      ok = checked(s.tr[k] > 0 && s.tr[k] < d.tr.n_nodes, d.err, 7) &&
+           checked(q.x >= 0 && q.y >= 0 && q.x + q.y <= d.tr.n_children && q.z >= 1 && q.z <= 63, d.err, 8);
+    }
+    if (!ok) s.nl = s.nt = 0;  // the row goes on from the empty context; the status word says so
+  }
+  group_sync(bar, kGroup);
+#endif
+
+  const int4* t4 = reinterpret_cast<const int4*>(d.lm.arc_tok);
+  const float4* p4 = reinterpret_cast<const float4*>(d.lm.arc_logp);
+  // level 0 of the deltas: label u's dense row by asynchronous copies (u < 0:
+  // no LM state, every delta 0), and the level and depth scratch cleared
+  auto begin_deltas = [&](int u) {
+    if (u >= 0) {
+      const float* R = d.lm.dense0 + (size_t)u * d.lm.V4;
+      for (int q = tid; q < d.V4 / 4; q += kGroup)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dlm + 4 * q)), "l"(R + 4 * q) : "memory");
+    } else {
+      for (int q = tid; q < d.V4 / 4; q += kGroup) reinterpret_cast<float4*>(dlm)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    for (int q = tid; q < d.V4 / 4; q += kGroup) {
+      reinterpret_cast<uint2*>(lev)[q] = make_uint2(0u, 0u);
+      reinterpret_cast<uint32_t*>(dep)[q] = 0u;
+    }
+  };
+  // the levels above 0 and the trie chain: every arc sets its level's bit,
+  // then the deepest level's arc overwrites its label's delta
+  // (row_stream.cu); then every label's term c_r + lambda * delta + trie
+  auto finish_deltas = [&]() {
+    const int nl = s.nl, nt = s.nt;
+    // a thread's first group of four arcs, and of four children of the trie
+    // chain's first nodes, are requested together
+    int hl = -1, hi = 0;
+    int4 ht;
+    float4 hp;
+    {
+      int g = tid;
+      for (int l = 1; l < nl; ++l) {
+        const int4 q = s.lmr[l];
+        const int n = level_groups(q.x, q.y);
+        if (g < n) {
+          hl = l, hi = (q.x & ~3) + 4 * g;
+          break;
+        }
+        g -= n;
+      }
+    }
+    if (hl >= 0) {
+      ht = __ldg(t4 + (hi >> 2));
+      hp = __ldg(p4 + (hi >> 2));
+    }
+    int4 ct[kTrHeld];
+#pragma unroll
+    for (int k = 0; k < kTrHeld; ++k)
+      if (k < nt) {
+        const int4 q = s.trr[k];
+        if (tid < level_groups(q.x, q.y)) ct[k] = __ldg(reinterpret_cast<const int4*>(d.tr.ch_tok) + (q.x >> 2) + tid);
+      }
+    auto children = [&](int k, int4 tk, int g) {  // node k's children of group g
+      const int4 q = s.trr[k];
+      const int i0 = (q.x & ~3) + 4 * g;
+      const int tv[4] = {tk.x, tk.y, tk.z, tk.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (i0 + j >= q.x && i0 + j < q.x + q.y) dep[tv[j]] = (uint8_t)q.z;
+    };
+    auto scatter = [&](int k) {
+      const int4 q = s.trr[k];
+      const int n = level_groups(q.x, q.y);
+#pragma unroll
+      for (int h = 0; h < kTrHeld; ++h)
+        if (h == k && tid < n) children(k, ct[h], tid);
+      for (int g = tid + (k < kTrHeld ? kGroup : 0); g < n; g += kGroup)
+        children(k, __ldg(reinterpret_cast<const int4*>(d.tr.ch_tok) + (q.x >> 2) + g), g);
+    };
+    uint32_t* lev2 = reinterpret_cast<uint32_t*>(lev);
+    auto offer = [&](int l, int i0, int4 tk) {
+      const int b = s.lmr[l].x, n = s.lmr[l].y;
+      const int tv[4] = {tk.x, tk.y, tk.z, tk.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (i0 + j >= b && i0 + j < b + n && checked(tv[j] >= 0 && tv[j] < V, d.err, 9))
+          atomicOr(lev2 + (tv[j] >> 1), 1u << (l + 16 * (tv[j] & 1)));
+    };
+    auto settle = [&](int l, int i0, int4 tk, float4 lq, const float (&up)[4]) {
+      const int b = s.lmr[l].x, n = s.lmr[l].y;
+      const float cum = __int_as_float(s.lmr[l].z);
+      const int tv[4] = {tk.x, tk.y, tk.z, tk.w};
+      const float pv[4] = {lq.x, lq.y, lq.z, lq.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (i0 + j >= b && i0 + j < b + n && checked(tv[j] >= 0 && tv[j] < V, d.err, 9) && 31 - __clz((int)lev[tv[j]]) == l)
+          dlm[tv[j]] = (pv[j] - cum) - up[j];
+    };
+    // log p(v) of a group's labels (groups past a level's ends hold other levels' labels: all are in range)
+    auto unigrams = [&](int4 tk, float (&up)[4]) {
+      const int tv[4] = {tk.x, tk.y, tk.z, tk.w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) up[j] = (unsigned)tv[j] < (unsigned)V ? __ldg(d.lm.uni_logp + tv[j]) : 0.f;
+    };
+    // the arcs past what a thread holds (rare: more than 512 arcs above level 0)
+    auto rest = [&](auto f) {
+      int G = 0;
+      for (int l = 1; l < nl; ++l) G += level_groups(s.lmr[l].x, s.lmr[l].y);
+      for (int g0 = tid + kGroup; g0 < G; g0 += kGroup) {
+        int l = 1, g = g0;
+        for (;; ++l) {
+          const int n = level_groups(s.lmr[l].x, s.lmr[l].y);
+          if (g < n) break;
+          g -= n;
+        }
+        f(l, (s.lmr[l].x & ~3) + 4 * g);
+      }
+    };
+    float hu[4] = {0.f, 0.f, 0.f, 0.f};
+    if (hl >= 0) {
+      unigrams(ht, hu);
+      offer(hl, hi, ht);
+    }
+    rest([&](int l, int i0) { offer(l, i0, __ldg(t4 + (i0 >> 2))); });
+    if (nt > 0) scatter(nt - 1);  // the trie chain nodes, shallowest first (the deepest overwrites)
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    group_sync(bar, kGroup);
+    if (hl >= 0) settle(hl, hi, ht, hp, hu);
+    rest([&](int l, int i0) {
+      const int4 tk = __ldg(t4 + (i0 >> 2));
+      float up[4];
+      unigrams(tk, up);
+      settle(l, i0, tk, __ldg(p4 + (i0 >> 2)), up);
+    });
+    for (int k = nt - 2; k >= 0; --k) {
+      scatter(k);
+      group_sync(bar, kGroup);
+    }
+    if (nt < 2) group_sync(bar, kGroup);
+    const float cr = lam * (nl ? __int_as_float(s.lmr[nl - 1].z) : 0.f) - bscale * (float)(nt ? s.trr[0].z - 1 : 0);
+    for (int q = tid; q < d.V4 / 4; q += kGroup) {
+      const float4 kq = reinterpret_cast<const float4*>(dlm)[q];
+      float o[4] = {lam * kq.x, lam * kq.y, lam * kq.z, lam * kq.w};
+      const uint32_t eq = reinterpret_cast<const uint32_t*>(dep)[q];
+      if (eq) {
+        const uint32_t rb = root[q >> 3] >> ((4 * q) & 31);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t e = (eq >> (8 * j)) & 0xffu;
+          if (e) o[j] += bscale * (float)e - (((rb >> j) & 1u) ? bscale : 0.f);
+        }
+      }
+      reinterpret_cast<float4*>(dlm)[q] = make_float4(cr + o[0], cr + o[1], cr + o[2], cr + o[3]);
+    }
+    // (a thread reads back only what it wrote here: no barrier)
+  };
+  // A warp's first label search of the next step, as far as it does not
+  // depend on the label: the range's 32 probes, or its entries where at most
+  // 124 are in it.
+  int4 pre = make_int4(-1, -1, -1, -1);
+  auto presearch = [&]() {
+    const int nl = s.nl, nt = s.nt;
+    if (warp >= nl + nt) return;
+    const int4 q = warp < nl ? s.lmr[warp] : s.trr[warp - nl];
+    pre = first_probe((warp < nl ? d.lm.arc_tok : d.tr.ch_tok) + q.x, q.y, lane);
+  };
+  begin_deltas(s.nl > 0 ? s.lmr[0].w : -1);
+  group_sync(bar, kGroup);  // the scratch is cleared before anyone's offers
+  finish_deltas();
+  presearch();
+
+  int t = 0, sym = 0, cnt = 0, step = 0;
+  const int nb = (c.nl + kMB - 1) / kMB;  // softmax partials per CTA
+  const uint32_t row_bytes = 4u * (uint32_t)(c.CS * c.nl), lse_bytes = 8u * (uint32_t)(c.CS * nb);
+  bool ok = true;
+  // The group's last warp consumes each step's softmax partials one step
+  // later, and writes the score of the label emitted there, if one was (e_at:
+  // its place in the row's outputs).
+  int e_at = -1;
+  float e_best = 0.f;
+  auto score_of = [&](int st) {
+    if (!__all_sync(0xffffffffu, wait_cluster(c.sbar + grp, st & 1, d.wait_ns, c.fail))) return false;
+    if (e_at >= 0) {
+      const float2* ps = reinterpret_cast<const float2*>(rs + c.L.lse) + (st & 1) * c.CS * nb;
+      float m = kNegInf, z = 0.f;
+      for (int q = lane; q < c.CS * nb; q += 32) lse_merge(m, z, ps[q].x, ps[q].y);
+      __syncwarp();
+      const float top = key_value(__reduce_max_sync(0xffffffffu, order_key(m)));
+      z = z > 0.f ? z * expf(m - top) : 0.f;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+      if (lane == 0) P.out_score[(size_t)r * (T * d.max_sym) + e_at] = e_best - (top + logf(z));
+      e_at = -1;
+    }
+    return true;
+  };
+  while (t < T) {
+    if (tid == 0) tc::mbar_expect_tx(c.lbar + grp, row_bytes);
+    if (warp == kWarpsG - 1) {
+      ok = step == 0 || score_of(step - 1);
+      if (lane == 0 && ok) tc::mbar_expect_tx(c.sbar + grp, lse_bytes);
+    }
+    if (d.cap_rows && step < d.cap_steps && tid == 0) {
+      int* q = d.cap_rows + ((size_t)step * P.n + r) * 4;
+      q[0] = t;
+      q[1] = last;
+      q[2] = s.nl ? s.lm[s.nl - 1] : 0;
+      q[3] = s.nt ? s.tr[0] : 0;
+    }
+    // the argmax of (logit + D) + (c_r + delta) over the labels (blank: its logit alone)
+    const float* lg = logits + (step & 1) * c.CS * c.nl;
+    ok = __all_sync(0xffffffffu, wait_cluster(c.lbar + grp, step & 1, d.wait_ns, c.fail)) && ok;
+    float bv = kNegInf;
+    int bi = INT_MAX;
+    if (ok) {
+      const int nq = (V + 3) >> 2;
+      for (int q = tid; q < nq; q += kGroup) {
+        const float4 lq = reinterpret_cast<const float4*>(lg)[q];
+        const float4 uq = reinterpret_cast<const float4*>(dflt)[q];
+        const float4 kq = reinterpret_cast<const float4*>(dlm)[q];
+        const float fv[4] = {(lq.x + uq.x) + kq.x, (lq.y + uq.y) + kq.y, (lq.z + uq.z) + kq.z, (lq.w + uq.w) + kq.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (fv[j] > bv && 4 * q + j < V) { bv = fv[j]; bi = 4 * q + j; }
+      }
+      if (tid == 0) {
+        const float fb = lg[V];
+        if (fb > bv) { bv = fb; bi = V; }
+      }
+    }
+    __syncwarp();
+    {
+      const int key = order_key(bv + 0.f), top = __reduce_max_sync(0xffffffffu, key);
+      bi = __reduce_min_sync(0xffffffffu, key == top ? bi : INT_MAX);
+      bv = key_value(top);
+    }
+    if (lane == 0) s.best[step & 1][warp] = make_int4(__float_as_int(bv), bi, ok ? 1 : 0, 0);
+    group_sync(bar, kGroup);
+    float best = kNegInf;
+    int bix = INT_MAX;
+#pragma unroll
+    for (int w = 0; w < kWarpsG; ++w) {
+      const int4 q = s.best[step & 1][w];
+      best_merge(best, bix, __int_as_float(q.x), q.y);
+      ok = ok && q.z;
+    }
+    if (!ok) {  // the group's threads leave together
+      if (tid == 0) atomicOr(d.err, 4);
+      *c.fail = 1;
+      break;
+    }
+    const int y = (bix >= 0 && bix <= V) ? bix : V;
+    // the row's next position, to every CTA before anything else
+    const int t_now = t;
+    if (y != V) {
+      last = y;
+      sym += 1;
+      if (sym >= d.max_sym) { t += 1; sym = 0; }
+    } else {
+      t += 1;
+      sym = 0;
+    }
+    publish(last, t);
+    if (d.cap_logits && step < d.cap_steps) {
+      float* cl = d.cap_logits + ((size_t)step * P.n + r) * d.N;
+      for (int v = tid; v < d.N; v += kGroup) cl[v] = lg[v];
+    }
+    if (y != V) {
+      // the label's searches in every chain element (row_stream.cu), level 0
+      // of the next deltas copied meanwhile
+      if (t < T) begin_deltas(lm2 ? y : -1);
+      const int nl = s.nl, nt = s.nt;
+      if (tid == kGroup - 1) s.root_hit = d.has_tr ? __ldg(d.tr.root_rec + y) : make_int4(0, 0, 0, 0);
+      else if (tid == kGroup - 2) s.uni_hit = lm2 ? __ldg(d.lm.uni_rec + y) : make_int4(-1, 0, 0, 0);
+      for (int task = warp; task < nl + nt; task += kWarpsG) {
+        const bool is_lm = task < nl;
+        const int4 q = is_lm ? s.lmr[task] : s.trr[task - nl];
+        const int32_t* arr = (is_lm ? d.lm.arc_tok : d.tr.ch_tok) + q.x;
+        const int at = find_from(arr, q.y, y, lane, task == warp ? pre : first_probe(arr, q.y, lane));
+        if (lane == 0) {
+          if (is_lm) s.lm_hit[task] = at >= 0 ? __ldg(d.lm.arc_rec + q.x + at) : make_int4(-2, 0, 0, 0);
+          else s.tr_hit[task - nl] = at >= 0 ? __ldg(d.tr.ch_rec + q.x + at) : make_int4(-1, 0, 0, 0);
+        }
+      }
+      group_sync(bar, kGroup);
+      // the new chains, in place: warp 0 the LM chain (y's unigram state, then
+      // the targets of y's arcs up to the first level without one), warp 1
+      // the trie chain (y's children of the old nodes, deepest first, then
+      // the root's; completing a phrase resets it)
+      if (warp == 0) {
+        int ln = 0;
+        if (lm2) {
+          const int4 h = lane < nl ? s.lm_hit[lane] : make_int4(-2, 0, 0, 0);
+          const bool cont = h.x >= 0 && checked(h.x < d.lm.n_states && h.y >= 0 && h.z >= 0 &&
+                                                    (int64_t)h.y + h.z <= d.lm.n_arcs, d.err, 10);
+          const unsigned miss = __ballot_sync(0xffffffffu, !cont);
+          ln = 1 + min(miss ? __ffs((int)miss) - 1 : 32, kLmChain - 1);
+          const int4 u = s.uni_hit;
+          const int px = __shfl_up_sync(0xffffffffu, h.x, 1), py = __shfl_up_sync(0xffffffffu, h.y, 1);
+          const int pz = __shfl_up_sync(0xffffffffu, h.z, 1), pw = __shfl_up_sync(0xffffffffu, h.w, 1);
+          __syncwarp();
+          if (lane < ln) {
+            s.lm[lane] = lane == 0 ? 1 + y : px;
+            s.lmr[lane] = lane == 0 ? make_int4(u.y, u.z, u.w, u.x) : make_int4(py, pz, pw, 0);
+          }
+        }
+        if (lane == 0) s.nl = ln;
+      } else if (warp == 1) {
+        const int4 h = lane < nt ? s.tr_hit[lane] : make_int4(-1, 0, 0, 0);
+        const int dd = lane < nt ? s.trr[lane].z + 1 : 0;
+        const bool hit = h.x >= 0 && checked(h.x > 0 && h.x < d.tr.n_nodes && h.w >= 0 && h.z + h.w <= d.tr.n_children,
+                                             d.err, 11);
+        const unsigned vm = __ballot_sync(0xffffffffu, hit);
+        const int nv = __popc(vm);
+        const int4 rh = s.root_hit;
+        const bool rt = rh.x != 0;
+        const int f = __ffs((int)vm) - 1;
+        const int fy = __shfl_sync(0xffffffffu, h.y, f < 0 ? 0 : f);
+        const bool reset = nv > 0 ? fy == 0 : (rt && rh.y == 0);
+        const int tn = reset ? 0 : min(nv + (rt ? 1 : 0), kTrChain);
+        __syncwarp();
+        const int pos = __popc(vm & ((1u << lane) - 1u));
+        if (hit && pos < tn) {
+          s.tr[pos] = h.x;
+          s.trr[pos] = make_int4(h.z, h.w, dd, 0);
+        }
+        if (lane == 0 && rt && nv < tn) {
+          s.tr[nv] = rh.x;
+          s.trr[nv] = make_int4(rh.z, rh.w, 2, 0);
+        }
+        if (lane == 0) s.nt = tn;
+      }
+      group_sync(bar, kGroup);
+      if (t < T) {
+        finish_deltas();
+        presearch();
+      }
+      if (warp == kWarpsG - 1) {
+        if (lane == 0) {
+          const size_t o = (size_t)r * (T * d.max_sym) + cnt;
+          P.out_tok[o] = y;
+          P.out_frame[o] = t_now;
+        }
+        e_at = cnt, e_best = best;
+      }
+      cnt += 1;
+    }
+    ++step;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  if (ok && warp == kWarpsG - 1 && !score_of(step - 1)) {
+    if (lane == 0) atomicOr(d.err, 8);
+    *c.fail = 1;
+  }
+  if (!ok) return;
+  // the stream's state, once per chunk (and the row's copy of it, which the
+  // two-kernel step and its timing replays read)
+  if (tid == 0) {
+    P.out_count[r] = cnt;
+    d.s_last[slot] = last;
+    d.m_last[r] = last;
+    d.r_t[r] = T;
+    d.r_sym[r] = 0;
+    d.r_cnt[r] = cnt;
+    if (d.has_lm) d.s_lm_len[slot] = s.nl;
+    if (d.has_tr) d.s_tr_len[slot] = s.nt;
+    d.m_lm_len[r] = s.nl;
+    d.m_tr_len[r] = s.nt;
+  } else if (tid >= 32 && tid < 32 + kLmChain && tid - 32 < s.nl) {
+    const int l = tid - 32;
+    d.s_lm_chain[(size_t)slot * kLmChain + l] = s.lm[l];
+    d.s_lm_rec[(size_t)slot * kLmChain + l] = s.lmr[l];
+    d.m_lm[(size_t)r * kLmChain + l] = s.lm[l];
+    d.m_lmr[(size_t)r * kLmChain + l] = s.lmr[l];
+  } else if (tid >= 64 && tid < 64 + kTrChain && tid - 64 < s.nt) {
+    const int k = tid - 64;
+    d.s_tr_chain[(size_t)slot * kTrChain + k] = s.tr[k];
+    d.s_tr_rec[(size_t)slot * kTrChain + k] = s.trr[k];
+    d.m_tr[(size_t)r * kTrChain + k] = s.tr[k];
+    d.m_trr[(size_t)r * kTrChain + k] = s.trr[k];
+  }
+  if (d.cap_rows)  // steps after the row's last evaluation
+    for (int q = step + tid; q < min(d.cap_steps, T * d.max_sym); q += kGroup)
+      reinterpret_cast<int4*>(d.cap_rows)[(size_t)q * P.n + r] = make_int4(-1, -1, -1, -1);
+}
+
+template <int NB, int RG>
+__global__ void __launch_bounds__(kGemm + RG * kGroup, 1)
+    k_chunk(const __grid_constant__ DecView d, const __grid_constant__ ChunkArgs P) {
+  extern __shared__ __align__(128) unsigned char raw[];
+  Ctx c;
+  c.sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(raw) + 127) & ~uintptr_t(127));
+  c.CS = P.CS;
+  c.nl = P.nl;
+  c.L = layout(d.H, d.V4, c.nl, c.CS, NB, RG);
+  c.rank = (int)(blockIdx.x % (unsigned)c.CS);
+  c.row0 = (int)(blockIdx.x / (unsigned)c.CS) * P.R;
+  c.R = min(P.R, P.n - c.row0);
+  c.ybar = reinterpret_cast<uint64_t*>(c.sm + c.L.bars);
+  c.wbar = c.ybar + 1;
+  c.lbar = c.ybar + 2;
+  c.sbar = c.lbar + RG;
+  int* fail = reinterpret_cast<int*>(c.sbar + RG);
+  c.fail = fail;
+  c.y = reinterpret_cast<int2*>(c.sm + c.L.y);
+  const int tid = threadIdx.x;
+  if (tid == 0) {
+    tc::mbar_init(c.ybar, 1);
+    tc::mbar_init(c.wbar, 1);
+    for (int g = 0; g < 2 * RG; ++g) tc::mbar_init(c.lbar + g, 1);  // lbar, then sbar
+    *fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    tc::mbar_expect_tx(c.ybar, 8u * (uint32_t)c.R);  // the rows' first labels
+    // this CTA's labels of W_out, row by row
+    tc::mbar_expect_tx(c.wbar, (uint32_t)(c.nl * 2 * d.H));
+    for (int j = 0; j < c.nl; ++j)
+      tc::bulk_g2s(c.sm + c.L.w + j * (2 * d.H + kWPad), d.Wt + (size_t)(c.rank * c.nl + j) * d.H, 2u * (uint32_t)d.H, c.wbar);
+  }
+  // the call's shared rows: the defaults D, and the labels that start a phrase
+  float* dflt = reinterpret_cast<float*>(c.sm + c.L.dflt);
+  uint32_t* root = reinterpret_cast<uint32_t*>(c.sm + c.L.root);
+  for (int v = tid; v < (d.V4 + 31) / 32 * 32; v += blockDim.x) {
+    const bool rc = d.has_tr && v < d.V && __ldg(d.tr.root_child + v) != 0;
+    float x = 0.f;
+    if (d.has_lm && v < d.V) x = P.lambda * __ldg(d.lm.uni_logp + v);
+    if (rc) x += P.beta * d.tr.bonus;
+    if (v < d.V4) dflt[v] = x;
+    const unsigned m = __ballot_sync(0xffffffffu, rc);  // whole warps: the bound is a multiple of 32
+    if ((tid & 31) == 0) root[v / 32] = m;
+  }
+  __syncthreads();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (tid < kGemm) {
+    gemm_loop<NB>(d, P, c);
+  } else {
+    const int grp = (tid - kGemm) / kGroup;
+    if (grp * c.CS + c.rank < c.R) row_loop(d, P, c, grp);
+  }
+  __syncwarp();
+  if (*c.fail) {
+    // messages and copies in flight land before the CTA's shared memory goes
+    tc::mbar_wait(c.wbar, 0);
+    const unsigned long long t0 = tc::global_ns();
+    while (tc::global_ns() - t0 < 200000ull) __nanosleep(1000);
+  }
+  __syncthreads();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+typedef void (*ChunkFn)(DecView, ChunkArgs);
+ChunkFn kernel_of(int NB, int RG) {
+  if (NB == 1) return RG == 1 ? k_chunk<1, 1> : k_chunk<1, 2>;
+  return RG == 1 ? k_chunk<2, 1> : k_chunk<2, 2>;
+}
+
+cudaLaunchConfig_t config(const ChunkShape& s, int clusters, cudaLaunchAttribute* a, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(clusters * s.CS));
+  cfg.blockDim = dim3((unsigned)(kGemm + s.RG * kGroup));
+  cfg.dynamicSmemBytes = (size_t)s.smem;
+  cfg.stream = st;
+  a[0].id = cudaLaunchAttributeClusterDimension;
+  a[0].val.clusterDim.x = (unsigned)s.CS;
+  a[0].val.clusterDim.y = 1;
+  a[0].val.clusterDim.z = 1;
+  cfg.attrs = a;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+}  // namespace
+
+cudaError_t chunk_cluster_shapes(const DecView& d, std::vector<ChunkShape>& out) {
+  out.clear();
+  if (d.H > 32 * 8 * kUnits) return cudaSuccess;
+  int dev = 0, lim = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  for (int NB = 1; NB <= 2; ++NB)
+    for (int RG = 1; RG <= 2; ++RG) {
+      const void* f = (const void*)kernel_of(NB, RG);
+      if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
+      if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess) return e;
+      for (int CS = 8; CS <= 16; CS *= 2) {
+        ChunkShape s;
+        s.CS = CS, s.RG = RG, s.NB = NB;
+        s.nl = ((d.N + CS - 1) / CS + 3) / 4 * 4;
+        const Layout L = layout(d.H, d.V4, s.nl, CS, NB, RG);
+        if (L.total > lim) continue;
+        s.smem = L.total;
+        cudaLaunchAttribute a[1];
+        cudaLaunchConfig_t cfg = config(s, 1, a, nullptr);
+        if ((e = cudaOccupancyMaxActiveClusters(&s.clusters, f, &cfg)) != cudaSuccess) return e;
+        if (s.clusters > 0) out.push_back(s);
+      }
+    }
+  return cudaSuccess;
+}
+
+// One pass of the product covers a cluster's rows (R <= 8 NB): a second pass
+// repeats the reads of W_out's slice that bound it, and with three passes and
+// more (256 rows in seven clusters of 16 CTAs: 37 each) the chunk took 1027 us
+// against 820 us by the two-kernel step.  Below that every shape measured is
+// faster here (64 rows, H = 640: 302 us against 674; one row 212 against 619).
+const ChunkShape* chunk_cluster_pick(const std::vector<ChunkShape>& shapes, int n, int H) {
+  const ChunkShape* best = nullptr;
+  double cost = 0;
+  if (n > kChunkMaxRows) return nullptr;
+  for (const ChunkShape& s : shapes) {
+    const int R = (n + s.clusters - 1) / s.clusters;
+    if (R > std::min(s.CS * s.RG, 8 * s.NB)) continue;
+    // bytes of W_out a CTA reads per step, a pass of eight more rows, another row group
+    const double c = (double)s.nl * H * 2 + 16384.0 * s.NB + 20000.0 * ((R + s.CS - 1) / s.CS);
+    if (!best || c < cost) best = &s, cost = c;
+  }
+  return best;
+}
+
+cudaError_t launch_chunk_cluster(const ChunkShape& s, const DecView& d, ChunkArgs& a, cudaStream_t st) {
+  a.CS = s.CS;
+  a.nl = s.nl;
+  a.R = (a.n + s.clusters - 1) / s.clusters;
+  const int clusters = (a.n + a.R - 1) / a.R;
+  cudaLaunchAttribute at[1];
+  cudaLaunchConfig_t cfg = config(s, clusters, at, st);
+  return cudaLaunchKernelEx(&cfg, kernel_of(s.NB, s.RG), d, a);
+}
+
+}  // namespace tsd

@@ -14,6 +14,7 @@
 #include <string>
 #include <type_traits>
 
+#include "chunk_cluster.h"
 #include "decoder.h"
 #include "gemm_tc.h"
 #include "joint_tc.h"
@@ -32,6 +33,16 @@ tsd_status set_device(const tsd_decoder* d) {
 }
 
 int steps_per_chunk(const tsd_decoder* d, int T) { return T * d->cfg.max_symbols; }
+
+// The launch shape of a chunk of n rows in one launch, or nullptr where the
+// two-kernel step runs: other forms than greedy streaming decoding with at
+// most one LM, more rows than one wave of clusters holds, W_out too large
+// for a cluster's shared memory, and instrumented calls (events at kernel
+// boundaries).
+const ChunkShape* one_launch_shape(const tsd_decoder* d, int n) {
+  if (!d->one_launch || !d->view.fused || d->view.fz_dense || d->joint_kind != 0 || d->timing || d->pred.D) return nullptr;
+  return chunk_cluster_pick(d->chunk_shapes, n, d->cfg.H);
+}
 
 // Events enqueue_chunk records with timing on: a mark before every row pass
 // and joint launch (and, for the stateful form, before the chunk's encoder
@@ -436,6 +447,8 @@ tsd_status create_impl(const tsd_decoder_cfg* cfg, const void* W_out_bf16, const
   v.pool_tok = ptok;
   v.pool_n = pn;
   v.pool_cap = kPoolCap;
+  if (fused && !pw && (ce = chunk_cluster_shapes(v, d->chunk_shapes)) != cudaSuccess)
+    return cleanup(cuda_fail(ce, "tsd_decoder_create: cluster launch shapes"));
   d->slot_open.assign((size_t)c.max_streams, 0);
   d->last_stream = s;
   *out = d.release();
@@ -558,6 +571,30 @@ extern "C" tsd_status tsd_decode_chunk(tsd_decoder* d, int32_t n, const int32_t*
   if (st) return st;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   d->last_stream = s;
+
+  if (const ChunkShape* shape = one_launch_shape(d, n)) {
+    ChunkArgs a;
+    a.enc = static_cast<const uint16_t*>(enc_bf16);
+    a.out_tok = out_tokens;
+    a.out_frame = out_frames;
+    a.out_score = out_scores;
+    a.out_count = out_counts;
+    a.n = n;
+    a.T = T;
+    a.lambda = lambda;
+    a.beta = beta;
+    std::memcpy(a.slots, slots, sizeof(int32_t) * (size_t)n);
+    d->last_n = n;
+    d->last_T = T;
+    d->host_params.resize(sizeof(Params) + sizeof(int32_t) * (size_t)n);
+    Params* hp = reinterpret_cast<Params*>(d->host_params.data());
+    *hp = Params{a.enc, out_tokens, out_frames, out_scores, out_counts, n, T, lambda, beta, {0}};
+    std::memcpy(hp->slots, slots, sizeof(int32_t) * (size_t)n);
+    NvtxRange nvtx_launch("chunk launch");
+    TSD_CUDA(launch_chunk_cluster(*shape, d->view, a, s));
+    return TSD_OK;
+  }
+  d->host_params.clear();
 
   // call parameters -> pinned staging -> device
   const int slot_i = d->ring_pos;
@@ -974,7 +1011,10 @@ extern "C" tsd_status tsd_decoder_launches_per_chunk(const tsd_decoder* d, int32
                                                      int64_t* launches) {
   clear_error();
   if (!d || !launches) return fail(TSD_EINVAL, "tsd_decoder_launches_per_chunk: NULL argument");
-  (void)n;
+  if (one_launch_shape(d, n)) {
+    *launches = 1;
+    return TSD_OK;
+  }
   const int64_t S = steps_per_chunk(d, T);
   *launches = d->pred.D ? 4 * S + 4 : 2 * S + 2;  // stateful form: + copy, projection, LSTM and joint input
   return TSD_OK;
@@ -1033,6 +1073,12 @@ extern "C" tsd_status tsd_decoder_set_option(tsd_decoder* d, const char* name, i
     d->view.fz_dense = (int32_t)value;
     return drop_graphs(d);
   }
+  if (n == "one_launch") {
+    // 1: a chunk that fits runs in one launch; 0: every label step is a row pass and a joint launch
+    if (value != 0 && value != 1) return fail(TSD_EINVAL, "tsd_decoder_set_option: one_launch must be 0 or 1");
+    d->one_launch = (int)value;
+    return TSD_OK;
+  }
   if (n == "joint_bn") {
     if (value != 64 && value != 128 && value != 256) return fail(TSD_EINVAL, "tsd_decoder_set_option: joint_bn must be 64, 128 or 256");
     tsd_status st = drop_graphs(d);
@@ -1044,6 +1090,7 @@ extern "C" tsd_status tsd_decoder_set_option(tsd_decoder* d, const char* name, i
       d->n_ptiles = d->N_pad / d->jtc->bn;
       d->view.n_ptiles = d->n_ptiles;
     }
+    d->one_launch = 0;  // a tile width is asked for: the kernel that has tiles runs
     return TSD_OK;
   }
   return fail(TSD_EINVAL, "tsd_decoder_set_option: unknown option '%s'", name);
@@ -1061,6 +1108,11 @@ extern "C" tsd_status tsd_decoder_replay(tsd_decoder* d, int32_t kernel, int32_t
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   const int M = d->last_n * d->cfg.beam_k;
   const int S = steps_per_chunk(d, d->last_T);
+  if (!d->host_params.empty()) {  // the last chunk took its parameters by value
+    TSD_CUDA(cudaMemcpyAsync(d->params_dev, d->host_params.data(), d->host_params.size(), cudaMemcpyHostToDevice, s));
+    d->host_params.clear();
+    launch_defaults(d->view, s);
+  }
   if (algo_bytes) TSD_CUDA(cudaMemsetAsync(d->view.ctr, 0, sizeof(unsigned long long), s));
   for (int i = 0; i < reps; ++i) {
     if (kernel == 0 && d->cfg.beam_k > 1) launch_row_beam(d->view, d->last_n, S - 1, 2, d->row_smem, s, false);

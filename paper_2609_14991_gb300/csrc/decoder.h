@@ -11,6 +11,7 @@
 
 namespace tsd {
 struct JointTc;
+struct ChunkShape;
 
 // Per-call parameters, copied to the device before each chunk so that one
 // captured graph serves every call of the same shape.
@@ -203,6 +204,12 @@ struct tsd_decoder {
   int pdl = 1;                  // programmatic dependent launch between kernels
   int sms = 0;
   int last_n = 0, last_T = 0;   // shape of the last decode_chunk (for replay)
+  // the chunk in one launch (chunk_cluster.cu): the shapes that fit (none:
+  // two-kernel steps), whether it may run, and the parameters of the last
+  // call that ran so (they are on the host only; replay needs them)
+  std::vector<tsd::ChunkShape> chunk_shapes;
+  int one_launch = 1;
+  std::vector<char> host_params;
   // per-kernel-class device time of timed chunks: 0 row pass, 1 joint,
   // 2 prediction network and projections (stateful form)
   double ms[3] = {0, 0, 0};
