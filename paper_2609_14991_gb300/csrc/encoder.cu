@@ -5,7 +5,7 @@
 //
 // Per chunk of n streams x C frames (M = n C rows, row b C + t = frame t of
 // the call's stream b), one CUDA graph runs: the subsampling GEMM into the
-// fp32 residual stream x, then per block 15 launches (layer norms, the
+// fp32 residual stream x, then per block 14 launches (layer norms, the
 // tensor-core GEMMs of encoder_gemm.cu with their fused epilogues, the
 // attention kernel, the depthwise convolution), then a kernel that advances
 // every stream's frame count.  Caches live per slot in device memory:
@@ -20,6 +20,7 @@
 #include <memory>
 
 #include "encoder.h"
+#include "tc_common.cuh"
 
 namespace tsd {
 
@@ -90,6 +91,20 @@ __device__ __forceinline__ void store_bf16(uint16_t* yr, const float4 (&v)[kMaxQ
 template <bool FINAL, int kMaxQ>  // d <= 128 kMaxQ
 __global__ void __launch_bounds__(256) k_ln(float* x, uint16_t* y, int M, int d, const float* g, const float* b,
                                             const float* g2, const float* b2) {
+  // the gains and shifts (weights) go to shared memory while the kernel
+  // before this one ends, so no load waits between the reductions
+  __shared__ __align__(16) float s_w[FINAL ? 4 : 2][128 * kMaxQ];
+  for (int i = 4 * threadIdx.x; i < d; i += 1024) {
+    *reinterpret_cast<float4*>(s_w[0] + i) = __ldg(reinterpret_cast<const float4*>(g + i));
+    *reinterpret_cast<float4*>(s_w[1] + i) = __ldg(reinterpret_cast<const float4*>(b + i));
+    if (FINAL && g2) {
+      *reinterpret_cast<float4*>(s_w[FINAL ? 2 : 0] + i) = __ldg(reinterpret_cast<const float4*>(g2 + i));
+      *reinterpret_cast<float4*>(s_w[FINAL ? 3 : 1] + i) = __ldg(reinterpret_cast<const float4*>(b2 + i));
+    }
+  }
+  __syncthreads();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = blockIdx.x * 8 + warp;
   if (r >= M) return;
@@ -99,12 +114,12 @@ __global__ void __launch_bounds__(256) k_ln(float* x, uint16_t* y, int M, int d,
 #pragma unroll
   for (int i = 0; i < kMaxQ; ++i)
     if (i < nq) v[i] = *reinterpret_cast<const float4*>(xr + 128 * i + 4 * lane);
-  ln_regs<kMaxQ>(v, nq, d, lane, g, b);
+  ln_regs<kMaxQ>(v, nq, d, lane, s_w[0], s_w[1]);
   if (FINAL) {
 #pragma unroll
     for (int i = 0; i < kMaxQ; ++i)
       if (i < nq) *reinterpret_cast<float4*>(xr + 128 * i + 4 * lane) = v[i];
-    if (g2) ln_regs<kMaxQ>(v, nq, d, lane, g2, b2);
+    if (g2) ln_regs<kMaxQ>(v, nq, d, lane, s_w[FINAL ? 2 : 0], s_w[FINAL ? 3 : 1]);
   }
   if (y) store_bf16<kMaxQ>(y + (size_t)r * d, v, nq, lane);
 }
@@ -178,6 +193,8 @@ __global__ void __launch_bounds__(kAttnThreads) k_attn(AttnArgs a) {
   extern __shared__ __align__(16) unsigned char sm[];
   constexpr int RS = DH + 8;  // bf16 row stride
   constexpr int E8 = DH / 8;  // 16-byte groups per row
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int b = blockIdx.x, h = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int C = a.C, d = a.d;
   const int slot = a.slots[b];
@@ -342,14 +359,14 @@ struct ConvArgs {
 };
 
 // Causal depthwise convolution over [cached K-1 frames, chunk frames], the
-// batch-norm affine map and Swish; thread = channel.  The last K-1 frames of
-// the window become the cache.  KT > 0: the kernel width as a constant, so
-// the taps stay in registers.
-template <int KT>
+// batch-norm affine map and Swish; thread = channel, any kernel width.  The
+// last K-1 frames of the window become the cache.
 __global__ void __launch_bounds__(128) k_dwconv(ConvArgs a) {
   extern __shared__ float seq[];  // [K-1+C][128]
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int b = blockIdx.x, c = blockIdx.y * 128 + threadIdx.x, tid = threadIdx.x;
-  const int K = KT > 0 ? KT : a.K;
+  const int K = a.K;
   const int K1 = K - 1, C = a.C, d = a.d;
   const int slot = a.slots[b];
   uint16_t* cc = a.cache + ((size_t)slot * a.layers + a.layer) * (size_t)K1 * d;
@@ -359,23 +376,90 @@ __global__ void __launch_bounds__(128) k_dwconv(ConvArgs a) {
   for (int t = 0; t < C; ++t) seq[(K1 + t) * 128 + tid] = bf2f(a.glu[(size_t)(b * C + t) * d + c]);
   const float* w = a.w + (size_t)c * K;
   const float bias = a.bias[c], sc = a.sc[c], sh = a.sh[c];
-  float wk[KT > 0 ? KT : 1];
-  if (KT > 0) {
-#pragma unroll
-    for (int k = 0; k < KT; ++k) wk[k] = w[k];
-  }
   for (int t = 0; t < C; ++t) {
     float acc = 0.f;
-    if (KT > 0) {
-#pragma unroll
-      for (int k = 0; k < KT; ++k) acc = fmaf(wk[k], seq[(t + k) * 128 + tid], acc);
-    } else {
-      for (int k = 0; k < K; ++k) acc = fmaf(w[k], seq[(t + k) * 128 + tid], acc);
-    }
+    for (int k = 0; k < K; ++k) acc = fmaf(w[k], seq[(t + k) * 128 + tid], acc);
     const float yv = (acc + bias) * sc + sh;
     a.z[(size_t)(b * C + t) * d + c] = f2bf(yv / (1.f + expf(-yv)));
   }
   for (int t = 0; t < K1; ++t) cc[(size_t)t * d + c] = f2bf(seq[(C + t) * 128 + tid]);
+}
+
+// The same for K = 9, four channels per thread and no shared memory: a
+// thread's window slides through registers, every load is 8 bytes and the
+// cached frames, taps and affine map load before the wait for the GLU outputs.
+// With a channel per thread and 2-byte loads the 0.6B shape's 256 streams took
+// 18 us (its 22 MB need 4); with four 10.3, of which the launch is two.
+constexpr int kConvThreads = 64;
+__global__ void __launch_bounds__(kConvThreads) k_dwconv9(ConvArgs a) {
+  constexpr int K = 9, K1 = K - 1;
+  const int b = blockIdx.x, c = 4 * (blockIdx.y * kConvThreads + threadIdx.x), C = a.C, d = a.d;
+  float wk[K][4];
+  float4 bias, sc, sh;
+  float win[K][4];  // the last K frames, win[K1] the newest
+  const bool in = c < d;
+  uint2* cc = nullptr;
+  auto frame = [&](uint2 v, float (&f)[4]) {
+    f[0] = __uint_as_float(v.x << 16), f[1] = __uint_as_float(v.x & 0xffff0000u);
+    f[2] = __uint_as_float(v.y << 16), f[3] = __uint_as_float(v.y & 0xffff0000u);
+  };
+  const size_t row = (size_t)d / 4;  // 8-byte groups per frame
+  if (in) {
+    cc = reinterpret_cast<uint2*>(a.cache + ((size_t)a.slots[b] * a.layers + a.layer) * (size_t)K1 * d + c);
+    uint2 v[K1];
+#pragma unroll
+    for (int t = 0; t < K1; ++t) v[t] = cc[t * row];
+    float w[4 * K];  // four channels' taps: 36 consecutive floats
+#pragma unroll
+    for (int i = 0; i < K; ++i) *reinterpret_cast<float4*>(w + 4 * i) = __ldg(reinterpret_cast<const float4*>(a.w + (size_t)c * K) + i);
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) wk[k][j] = w[j * K + k];
+    bias = __ldg(reinterpret_cast<const float4*>(a.bias + c));
+    sc = __ldg(reinterpret_cast<const float4*>(a.sc + c));
+    sh = __ldg(reinterpret_cast<const float4*>(a.sh + c));
+#pragma unroll
+    for (int t = 0; t < K1; ++t) frame(v[t], win[t + 1]);
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!in) return;
+  const uint2* gl = reinterpret_cast<const uint2*>(a.glu + (size_t)b * C * d + c);
+  uint2* z = reinterpret_cast<uint2*>(a.z + (size_t)b * C * d + c);
+  constexpr int kAhead = 16;  // frames whose loads are in flight together
+  const float bi[4] = {bias.x, bias.y, bias.z, bias.w}, s1[4] = {sc.x, sc.y, sc.z, sc.w}, s0[4] = {sh.x, sh.y, sh.z, sh.w};
+  for (int t0 = 0; t0 < C; t0 += kAhead) {
+    uint2 v[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      if (t0 + u < C) v[u] = gl[(t0 + u) * row];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      if (t0 + u < C) {
+#pragma unroll
+        for (int k = 0; k < K1; ++k)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) win[k][j] = win[k + 1][j];
+        frame(v[u], win[K1]);
+        float o[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          float acc = 0.f;
+#pragma unroll
+          for (int k = 0; k < K; ++k) acc = fmaf(wk[k][j], win[k][j], acc);
+          const float yv = (acc + bi[j]) * s1[j] + s0[j];
+          o[j] = yv * tc::sigmoid(yv);
+        }
+        z[(t0 + u) * row] = make_uint2((uint32_t)f2bf(o[0]) | ((uint32_t)f2bf(o[1]) << 16),
+                                       (uint32_t)f2bf(o[2]) | ((uint32_t)f2bf(o[3]) << 16));
+      }
+  }
+  // the window's last K-1 frames (bf16 values, exactly) are the cache
+#pragma unroll
+  for (int t = 0; t < K1; ++t)
+    cc[t * row] = make_uint2((__float_as_uint(win[t + 1][0]) >> 16) | (__float_as_uint(win[t + 1][1]) & 0xffff0000u),
+                             (__float_as_uint(win[t + 1][2]) >> 16) | (__float_as_uint(win[t + 1][3]) & 0xffff0000u));
 }
 
 // P[row][c] = bf16(sum_k W_pos[c][k] r_k(delta)), delta = row - (cmax - 1), r
@@ -422,19 +506,32 @@ tsd_status set_device(tsd_encoder* e) {
 
 int n_marks(const tsd_encoder* e) { return 2 + 14 * e->cfg.layers + 1 + 1; }
 
-void launch_attn(const tsd_encoder* e, const AttnArgs& a, int n, cudaStream_t s) {
+template <class... P, class... A>
+void launch(void (*f)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, bool pdl, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, f, static_cast<P>(args)...);
+}
+
+void launch_attn(const tsd_encoder* e, const AttnArgs& a, int n, cudaStream_t s, bool pdl) {
   const size_t sm = attn_smem(e->cfg.d / e->cfg.heads, e->cfg.left, a.C);
   dim3 grid(n, e->cfg.heads);
-  if (e->cfg.d / e->cfg.heads == 64) k_attn<64><<<grid, kAttnThreads, sm, s>>>(a);
-  else k_attn<128><<<grid, kAttnThreads, sm, s>>>(a);
+  launch(e->cfg.d / e->cfg.heads == 64 ? k_attn<64> : k_attn<128>, grid, kAttnThreads, sm, s, pdl, a);
 }
 
 template <bool FINAL>
-void ln_launch(dim3 grid, cudaStream_t s, float* x, uint16_t* y, int M, int d, const float* g, const float* b,
+void ln_launch(dim3 grid, cudaStream_t s, bool pdl, float* x, uint16_t* y, int M, int d, const float* g, const float* b,
                const float* g2 = nullptr, const float* b2 = nullptr) {
-  if (d <= 512) k_ln<FINAL, 4><<<grid, 256, 0, s>>>(x, y, M, d, g, b, g2, b2);
-  else if (d <= 1024) k_ln<FINAL, 8><<<grid, 256, 0, s>>>(x, y, M, d, g, b, g2, b2);
-  else k_ln<FINAL, 16><<<grid, 256, 0, s>>>(x, y, M, d, g, b, g2, b2);
+  launch(d <= 512 ? k_ln<FINAL, 4> : d <= 1024 ? k_ln<FINAL, 8> : k_ln<FINAL, 16>, grid, 256, 0, s, pdl, x, y, M, d, g, b, g2,
+         b2);
 }
 
 // The block sequence for streams [off, off + n) of the call (their rows
@@ -451,51 +548,59 @@ void enqueue_rows(tsd_encoder* e, int off, int n, int C, cudaStream_t s, const s
     ++mk;
   };
   const dim3 ln_grid((M + 7) / 8);
-  auto gemm = [&](int epi, const CUtensorMap& A, const CUtensorMap& B, int N, int K, const float* bias, void* out,
-                  int ld, float alpha) {
+  // programmatic dependent launch: each kernel's set-up (and a GEMM's first
+  // weight tiles) overlaps the kernel before it; every kernel waits for its
+  // predecessor before it touches anything the chunk writes, and lets the
+  // next one start after that wait (before it: three streams through the
+  // 115M shape 1015 us against 968)
+  bool pdl = false;  // the first kernel follows copies or the fork
+  auto gemm = [&](int epi, const EncMapA& A, const EncMapB& B, int N, int K, const float* bias, void* out, int ld,
+                  const EncMapO& O, float alpha) {
     mark(0);
     EGemm g{M, N, K, bias, out, ld, alpha, e->err, r0};
-    launch_egemm(epi, g, A, B, s);
+    launch_egemm(epi, g, A, B, O, s, pdl);
+    pdl = !ev;
   };
   float* x = e->x + (size_t)r0 * d;
   uint16_t* nrm = e->nrm + (size_t)r0 * d;
   const int32_t* slots = e->slots_dev + off;
-  gemm(kEInit, e->m_feat, e->m_sub, d, c.stack * c.feat, e->sub_b, e->x, d, 1.f);
+  gemm(kEInit, e->m_feat, e->m_sub, d, c.stack * c.feat, e->sub_b, e->x, d, e->o_x, 1.f);
   mark(2);
-  ln_launch<false>(ln_grid, s, x, nrm, M, d, e->L[0].ln_ff1_g, e->L[0].ln_ff1_b);
+  ln_launch<false>(ln_grid, s, pdl, x, nrm, M, d, e->L[0].ln_ff1_g, e->L[0].ln_ff1_b);
   for (int l = 0; l < c.layers; ++l) {
     EncLayerDev& L = e->L[(size_t)l];
     // the first module's norm of this block ran with the previous block's closing norm
-    gemm(kESwish, e->m_nrm, L.m_ff1_w1, c.ff, d, L.ff1_b1, e->hid, c.ff, 1.f);
-    gemm(kEResid, e->m_hid, L.m_ff1_w2, d, c.ff, L.ff1_b2, e->x, d, 0.5f);
+    gemm(kESwish, e->m_nrm, L.m_ff1_w1, c.ff, d, L.ff1_b1, e->hid, c.ff, e->o_hid, 1.f);
+    gemm(kEResid, e->m_hid, L.m_ff1_w2, d, c.ff, L.ff1_b2, e->x, d, e->o_x, 0.5f);
     mark(2);
-    ln_launch<false>(ln_grid, s, x, nrm, M, d, L.ln_att_g, L.ln_att_b);
-    gemm(kEPlain, e->m_nrm, L.m_qkv, 3 * d, d, L.qkv_b, e->qkv, 3 * d, 1.f);
+    ln_launch<false>(ln_grid, s, pdl, x, nrm, M, d, L.ln_att_g, L.ln_att_b);
+    gemm(kEPlain, e->m_nrm, L.m_qkv, 3 * d, d, L.qkv_b, e->qkv, 3 * d, e->o_qkv, 1.f);
     mark(1);
     AttnArgs aa{e->qkv + (size_t)r0 * 3 * d, e->att + (size_t)r0 * d, L.pos_tab, L.pos_u, L.pos_v, e->kc, e->vc,
                 e->seen, slots, d, c.heads, c.left, c.layers, l, C, c.max_chunk, 1.f / sqrtf((float)(d / c.heads))};
-    launch_attn(e, aa, n, s);
-    gemm(kEResid, e->m_att, L.m_out, d, d, L.out_b, e->x, d, 1.f);
+    launch_attn(e, aa, n, s, pdl);
+    gemm(kEResid, e->m_att, L.m_out, d, d, L.out_b, e->x, d, e->o_x, 1.f);
     mark(2);
-    ln_launch<false>(ln_grid, s, x, nrm, M, d, L.ln_conv_g, L.ln_conv_b);
-    gemm(kEGlu, e->m_nrm, L.m_pw1, 2 * d, d, L.pw1_b, e->glu, d, 1.f);
+    ln_launch<false>(ln_grid, s, pdl, x, nrm, M, d, L.ln_conv_g, L.ln_conv_b);
+    gemm(kEGlu, e->m_nrm, L.m_pw1, 2 * d, d, L.pw1_b, e->glu, d, e->o_glu, 1.f);
     mark(2);
     ConvArgs ca{e->glu + (size_t)r0 * d, e->convz + (size_t)r0 * d, e->cc, L.dw_w, L.dw_b, L.bn_scale, L.bn_shift,
                 slots, d, c.kernel, C, c.layers, l};
-    const size_t conv_smem = (size_t)(c.kernel - 1 + C) * 128 * sizeof(float);
-    if (c.kernel == 9) k_dwconv<9><<<dim3(n, d / 128), 128, conv_smem, s>>>(ca);
-    else k_dwconv<0><<<dim3(n, d / 128), 128, conv_smem, s>>>(ca);
-    gemm(kEResid, e->m_convz, L.m_pw2, d, d, L.pw2_b, e->x, d, 1.f);
+    if (c.kernel == 9)
+      launch(k_dwconv9, dim3(n, (d / 4 + kConvThreads - 1) / kConvThreads), kConvThreads, 0, s, pdl, ca);
+    else
+      launch(k_dwconv, dim3(n, d / 128), 128, (size_t)(c.kernel - 1 + C) * 128 * sizeof(float), s, pdl, ca);
+    gemm(kEResid, e->m_convz, L.m_pw2, d, d, L.pw2_b, e->x, d, e->o_x, 1.f);
     mark(2);
-    ln_launch<false>(ln_grid, s, x, nrm, M, d, L.ln_ff2_g, L.ln_ff2_b);
-    gemm(kESwish, e->m_nrm, L.m_ff2_w1, c.ff, d, L.ff2_b1, e->hid, c.ff, 1.f);
-    gemm(kEResid, e->m_hid, L.m_ff2_w2, d, c.ff, L.ff2_b2, e->x, d, 0.5f);
+    ln_launch<false>(ln_grid, s, pdl, x, nrm, M, d, L.ln_ff2_g, L.ln_ff2_b);
+    gemm(kESwish, e->m_nrm, L.m_ff2_w1, c.ff, d, L.ff2_b1, e->hid, c.ff, e->o_hid, 1.f);
+    gemm(kEResid, e->m_hid, L.m_ff2_w2, d, c.ff, L.ff2_b2, e->x, d, e->o_x, 0.5f);
     mark(2);
     if (l + 1 < c.layers)
-      ln_launch<true>(ln_grid, s, x, nrm, M, d, L.ln_out_g, L.ln_out_b, e->L[(size_t)l + 1].ln_ff1_g,
+      ln_launch<true>(ln_grid, s, pdl, x, nrm, M, d, L.ln_out_g, L.ln_out_b, e->L[(size_t)l + 1].ln_ff1_g,
                       e->L[(size_t)l + 1].ln_ff1_b);
     else
-      ln_launch<true>(ln_grid, s, x, e->outb + (size_t)r0 * d, M, d, L.ln_out_g, L.ln_out_b);
+      ln_launch<true>(ln_grid, s, pdl, x, e->outb + (size_t)r0 * d, M, d, L.ln_out_g, L.ln_out_b);
   }
 }
 
@@ -503,10 +608,15 @@ void enqueue_rows(tsd_encoder* e, int off, int n, int C, cudaStream_t s, const s
 // different streams never meet until the output, so one branch's attention,
 // layer norms and convolution fill the SMs while another's GEMMs run):
 // branch i takes streams at[i] .. at[i+1]-1.  Up to kEncBranches branches
-// of at least 256 rows each; a boundary moves up to a multiple of the
-// 128-row tile where one lies within its share.  Returns the branch count.
-int branch_points(int n, int C, int* at) {
-  int P = std::min(kEncBranches, n * C / 256);
+// of at least 256 rows each, while the widest GEMM of the whole call has at
+// most `wide` tiles of 128 x 128 (half of the SMs): past that a GEMM fills
+// the SMs by itself, and fewer, larger GEMMs round up to fewer tiles (four
+// blocks, one branch against two: d 256, 72 tiles 238 / 235 us; d 512, 80 tiles
+// 295 / 308; d 1024, 160 tiles 499 / 553, 832 tiles 993 / 1122); a
+// boundary moves up to a multiple of the 128-row tile where one lies within
+// its share.  Returns the branch count.
+int branch_points(int n, int C, int ff, int wide, int* at) {
+  int P = (n * C + 127) / 128 * ((ff + 127) / 128) <= wide ? std::min(kEncBranches, n * C / 256) : 1;
   P = std::min(P, n);
   at[0] = 0;
   if (P < 2) {
@@ -530,7 +640,7 @@ void enqueue(tsd_encoder* e, int n, int C, cudaStream_t s, const std::vector<cud
              std::vector<int8_t>* cls) {
   int mk = 0;
   int at[kEncBranches + 1];
-  const int P = ev ? 1 : branch_points(n, C, at);
+  const int P = ev ? 1 : branch_points(n, C, e->cfg.ff, e->sms / 2, at);
   if (P == 1) {
     enqueue_rows(e, 0, n, C, s, ev, cls, mk);
   } else {
@@ -630,6 +740,7 @@ extern "C" tsd_status tsd_encoder_create(const tsd_encoder_cfg* cfg, const void*
   TSD_CUDA(cudaGetDevice(&e->device));
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   e->last_stream = s;
+  TSD_CUDA(cudaDeviceGetAttribute(&e->sms, cudaDevAttrMultiProcessorCount, e->device));
   TSD_CUDA(egemm_prepare());
   const int d = c.d, ff = c.ff, K1 = c.kernel - 1, dh = d / c.heads;
   const size_t asm_ = attn_smem(dh, c.left, c.max_chunk);
@@ -698,7 +809,9 @@ extern "C" tsd_status tsd_encoder_create(const tsd_encoder_cfg* cfg, const void*
   TSD_CUDA(cudaMemsetAsync(e->convz, 0, Mp * d * 2, s));
   if (!egemm_map_a(&e->m_feat, e->feat, e->M_pad, (int)SF) || !egemm_map_a(&e->m_nrm, e->nrm, e->M_pad, d) ||
       !egemm_map_a(&e->m_hid, e->hid, e->M_pad, ff) || !egemm_map_a(&e->m_att, e->att, e->M_pad, d) ||
-      !egemm_map_a(&e->m_convz, e->convz, e->M_pad, d) || !egemm_map_b(&e->m_sub, e->sub_w, d, (int)SF))
+      !egemm_map_a(&e->m_convz, e->convz, e->M_pad, d) || !egemm_map_b(&e->m_sub, e->sub_w, d, (int)SF) ||
+      !egemm_map_out(&e->o_x, true, e->x, e->M_pad, d) || !egemm_map_out(&e->o_hid, false, e->hid, e->M_pad, ff) ||
+      !egemm_map_out(&e->o_qkv, false, e->qkv, e->M_pad, 3 * d) || !egemm_map_out(&e->o_glu, false, e->glu, e->M_pad, d))
     return fail(TSD_ECUDA, "tsd_encoder_create: tensor map encoding failed");
   TSD_CUDA(cudaMallocHost(&e->slots_host, sizeof(int32_t) * (size_t)c.max_streams));
   TSD_CUDA(cudaEventCreateWithFlags(&e->slots_ev, cudaEventDisableTiming));
@@ -868,7 +981,7 @@ extern "C" tsd_status tsd_encoder_launches_per_chunk(const tsd_encoder* e, int32
   if (n < 1 || n > e->cfg.max_streams || C < 1 || C > e->cfg.max_chunk)
     return fail(TSD_EINVAL, "tsd_encoder_launches_per_chunk: n=%d C=%d out of range", n, C);
   int at[kEncBranches + 1];
-  const int P = branch_points(n, C, at);
+  const int P = branch_points(n, C, e->cfg.ff, e->sms / 2, at);
   *launches = (int64_t)P * (2 + 14 * e->cfg.layers) + 1;
   return TSD_OK;
 }

@@ -33,13 +33,25 @@ struct EGemm {
                       // may read further rows of A, but write nothing there)
 };
 
-constexpr int kEgBN = 128;  // output-tile width (B rows per tile)
+// TMA maps of a GEMM's operands, one per box height: 128 and 64 rows of A;
+// 128, 64 and 32 rows of B.
+struct EncMapA {
+  CUtensorMap m[2];
+};
+struct EncMapB {
+  CUtensorMap m[3];
+};
+// ... and of its output: whole 128-byte boxes, and half as wide (bf16).
+struct EncMapO {
+  CUtensorMap m[2];
+};
 constexpr int kEncBranches = 2;  // most parallel branches of the encoder's chunk graph
 
-bool egemm_map_a(CUtensorMap* m, const uint16_t* A, int rows, int K);
-bool egemm_map_b(CUtensorMap* m, const uint16_t* B, int rows, int K);
+bool egemm_map_a(EncMapA* m, const uint16_t* A, int rows, int K);
+bool egemm_map_b(EncMapB* m, const uint16_t* B, int rows, int K);
+bool egemm_map_out(EncMapO* m, bool fp32, void* out, int rows, int ld);
 cudaError_t egemm_prepare();
-void launch_egemm(int epi, const EGemm& g, const CUtensorMap& a, const CUtensorMap& b, cudaStream_t s);
+void launch_egemm(int epi, const EGemm& g, const EncMapA& a, const EncMapB& b, const EncMapO& o, cudaStream_t s, bool pdl);
 
 // Device pointers of one block's weights (B operands repacked where noted).
 struct EncLayerDev {
@@ -49,7 +61,7 @@ struct EncLayerDev {
   float *ff1_b1, *ff1_b2, *qkv_b, *pos_u, *pos_v, *out_b, *pw1_b /*interleaved*/, *dw_w, *dw_b, *bn_scale,
       *bn_shift, *pw2_b, *ff2_b1, *ff2_b2;
   uint16_t* pos_tab;  // [n_off][d] bf16: W_pos r(delta) for delta = -(max_chunk-1) .. left+max_chunk-1
-  CUtensorMap m_ff1_w1, m_ff1_w2, m_qkv, m_out, m_pw1, m_pw2, m_ff2_w1, m_ff2_w2;
+  EncMapB m_ff1_w1, m_ff1_w2, m_qkv, m_out, m_pw1, m_pw2, m_ff2_w1, m_ff2_w2;
 };
 
 }  // namespace tsd
@@ -57,18 +69,20 @@ struct EncLayerDev {
 struct tsd_encoder {
   tsd_encoder_cfg cfg{};
   int device = 0;
+  int sms = 0;
   tsd::DevArena arena;
   int n_off = 0;  // rows of each position table
   int M_pad = 0;  // work-buffer rows (max_streams * max_chunk, padded to 128)
   uint16_t* sub_w = nullptr;
   float* sub_b = nullptr;
-  CUtensorMap m_sub{};
+  tsd::EncMapB m_sub{};
   std::vector<tsd::EncLayerDev> L;
   // work buffers
   uint16_t *feat = nullptr, *nrm = nullptr, *hid = nullptr, *qkv = nullptr, *att = nullptr, *glu = nullptr,
            *convz = nullptr, *outb = nullptr;
   float* x = nullptr;
-  CUtensorMap m_feat{}, m_nrm{}, m_hid{}, m_att{}, m_convz{};
+  tsd::EncMapA m_feat{}, m_nrm{}, m_hid{}, m_att{}, m_convz{};
+  tsd::EncMapO o_x{}, o_hid{}, o_qkv{}, o_glu{};  // GEMM outputs
   // per-slot state
   uint16_t *kc = nullptr, *vc = nullptr, *cc = nullptr;  // [slot][layer][head][left][dh] x2, [slot][layer][K-1][d]
   int32_t* seen = nullptr;

@@ -1,20 +1,43 @@
 // Tensor-core GEMM of the cache-aware encoder: out = A . B^T with A [M][K]
 // and B [N][K] bf16 K-major (B = a weight stored [out][in]), fp32 accumulate
-// in TMEM, 128 x 128 output tiles.  Persistent: one CTA per SM walks the
-// tile list (tiles of one weight column block are adjacent, so concurrent
-// CTAs share B in L2).  Warp 0 streams A and B k-blocks by TMA into a
-// 6-stage ring of 128-byte-swizzled stages that continues across tiles;
-// warp 1 allocates two 128-column TMEM accumulators and issues the MMAs of
-// tile i into accumulator i mod 2; warps 2-9 run the epilogue of tile i
-// (thread = output row; warp w reads TMEM lanes 32 (w mod 4) .., the two
-// warps of a lane quadrant alternate 32-column chunks) while the MMAs of
-// tile i+1 run, then hand the accumulator back.  The epilogue
-// applies the bias and one of: the residual update of the fp32 stream
-// (x = acc + b, or x += alpha (acc + b)), Swish to bf16, plain bf16, or GLU
-// to bf16.  Every mbarrier wait is bounded in time; on expiry the kernel
-// records an error bit and the other roles run out their own bounded waits.
+// in TMEM.  Persistent: one CTA (or CTA pair) per SM (pair) walks the tile
+// list (tiles of one weight column block are adjacent, so concurrent CTAs
+// share B in L2).  Warp 0 streams A and B k-blocks by TMA into a ring of
+// 128-byte-swizzled stages that continues across tiles; warp 1 issues the
+// MMAs of tile i into accumulator i mod 2; warps 2-17 run the epilogue of tile
+// i (thread = output row; warp w reads TMEM lanes 32 (w mod 4) .., the four
+// warps of a lane quadrant take different columns) while the MMAs of tile
+// i+1 run, then hand the accumulator back.  The epilogue applies the bias and
+// one of: the fp32 stream's start (x = acc + b), its residual update (x +=
+// alpha (acc + b)), Swish to bf16, plain bf16 (q/k/v), GLU to bf16.
+//
+// Tile shapes, all with the same order of the sum over K (a row's result does
+// not depend on the batch):
+//   256 x 256 over two CTAs (cta_group::2): each CTA stages its 128 rows of A
+//          and half of B, 32 KB per 64-deep k-block for twice the product of
+//          a 128 x 128 tile.  A 128 x 128 tile needs 126 bytes per clock and SM
+//          from L2 at the tensor rate, twice what arrives (measured: 50-62,
+//          15-19 TB/s over the chip); the pair needs 64;
+//   128 x 128, 128 x 64, 128 x 32 on one CTA, for fewer rows or narrow
+//          outputs: narrower tiles put more SMs on the weights; calls of at
+//          most 64 rows stage 64 rows of A.
+// What bounds them (0.6B shape, 3328 x 4096 x 1024 with Swish, 20.5 us in the
+// kernel): 1.5 us to the first operands, 5.2 us per tile and pair of which the
+// MMAs are 4.2 (the operands' way from L2 is the rest), 2.4 us of epilogue
+// after the last tile.  With 128 x 128 tiles for everything, libm's expf and an
+// IEEE division and row-per-thread stores the same rows took two launches of
+// 26.7 us, 18.5 us of each without the epilogue.  Swish and GLU use the
+// hardware's 2^x and reciprocal (tc::sigmoid, relative error below 4e-7,
+// rounded to bf16 after) on pairs of values, and blocks of 32 rows leave through
+// shared memory by TMA: bf16 stores, and for the residual update an fp32
+// add in L2 (one writer per element), so x is not read at all.
+//
+// Every mbarrier wait is bounded in time; on expiry the kernel records an
+// error bit and the other roles run out their own bounded waits.
 #include <cuda.h>
 #include <cuda_bf16.h>
+
+#include <algorithm>
 
 #include "encoder.h"
 #include "tc_common.cuh"
@@ -25,42 +48,182 @@ namespace {
 
 using namespace tc;
 
-constexpr int kBN = kEgBN;
-constexpr int kStages = 6;
-constexpr int kThreads = 320;  // warp 0 TMA, warp 1 MMA, warps 2-9 epilogue
-constexpr int kEpiWarps = 8;
-constexpr int kABytes = kBM * kBK * 2;
-constexpr int kBBytes = kBN * kBK * 2;
-constexpr int kStageBytes = kABytes + kBBytes;
-constexpr int kBarBytes = 256;
-constexpr int kSmem = kStages * kStageBytes + 1024 /*align*/ + kBarBytes + kEpiWarps * 2 * kBN * 4 /*bias: per warp, per accumulator*/;
-static_assert((2 * kStages + 4) * 8 + 4 <= kBarBytes, "barrier area");
+constexpr int kEpiWarps = 16;
+constexpr int kThreads = 64 + 32 * kEpiWarps;  // warp 0 TMA, warp 1 MMA, warps 2-17 epilogue
 int g_sms = 148;
 
-__device__ __forceinline__ float sigm(float x) { return 1.f / (1.f + expf(-x)); }
+// One tile shape: BN output columns, PAIR: two CTAs (each with BN / 2 rows of
+// B), AR rows of A staged per CTA (64: a call of at most 64 rows; the rest of
+// the MMA's 128 rows are whatever shared memory holds, and never stored).
+template <int BN, bool PAIR, int AR>
+struct Shape {
+  static constexpr int kABytes = AR * kBK * 2;
+  static constexpr int kBRows = PAIR ? BN / 2 : BN;
+  static constexpr int kStageBytes = kABytes + kBRows * kBK * 2;
+  static constexpr int kBlk = BN == 256 ? 64 : 32;                 // columns an epilogue warp takes at a time
+  static constexpr int kParts = BN / kBlk < 4 ? BN / kBlk : 4;     // warps of a lane quadrant with work
+  static constexpr int kStgBytes = 4 * kParts * 4096;              // staging: a 4 KB block for each of them
+  // as many stages as fit (at most 16; the MMA reads 128 rows of A from the last one)
+  static constexpr int kFit = (227 * 1024 - 1024 - 512 - kStgBytes - (kBM - AR) * kBK * 2) / kStageBytes;
+  static constexpr int kStages = kFit < 16 ? kFit : 16;
+  static constexpr int kStgOff = kStages * kStageBytes + (kBM - AR) * kBK * 2;
+  static constexpr int kBarOff = kStgOff + kStgBytes;
+  static constexpr int kSmem = kBarOff + 512 + 1024 /*align*/;
+  static_assert((2 * kStages + 4) * 8 + 4 <= 512, "barrier area");
+  static_assert(kSmem <= 227 * 1024 && kStages >= 4, "shared memory per CTA");
+};
 
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  const __nv_bfloat16 x = __float2bfloat16_rn(a), y = __float2bfloat16_rn(b);
-  return (uint32_t)(*reinterpret_cast<const uint16_t*>(&x)) | ((uint32_t)(*reinterpret_cast<const uint16_t*>(&y)) << 16);
+// Pairs of fp32 values in one instruction (each rounded as the scalar ones).
+__device__ __forceinline__ uint64_t pair_of(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpair(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
 }
 
-template <int EPI>
+// tc::sigmoid of two values
+__device__ __forceinline__ uint64_t sigmoid2(uint64_t x) {
+  const uint64_t c = pair_of(-kLog2e, -kLog2e);
+  const uint64_t hi = mul2(x, c);
+  float h0, h1;
+  unpair(hi, h0, h1);
+  const uint64_t lo = fma2(x, c, pair_of(-h0, -h1));
+  const uint64_t e = pair_of(ex2_approx(h0), ex2_approx(h1));
+  const uint64_t e1 = add2(fma2(e, mul2(lo, pair_of(0.6931471805599453f, 0.6931471805599453f)), e), pair_of(1.f, 1.f));
+  float a, b;
+  unpair(e1, a, b);
+  asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(a));
+  asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(b));
+  return pair_of(a, b);
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(uint64_t x) {
+  float a, b;
+  unpair(x, a, b);
+  const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+
+// TMA load whose bytes complete on a barrier of this CTA or its pair's leader.
+template <bool PAIR>
+__device__ __forceinline__ void load_2d(void* dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
+  if constexpr (PAIR)
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, %3}], [%4];" ::"r"(
+            smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+  else
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+            smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
+
+template <bool PAIR>
+__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  if constexpr (PAIR)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(acc)
+        : "memory");
+  else
+    mma_bf16(d, a, b, idesc, acc);
+}
+
+// The MMAs issued so far, on completion, arrive on the barrier (of both CTAs of a pair).
+template <bool PAIR>
+__device__ __forceinline__ void commit(uint64_t* bar) {
+  if constexpr (PAIR)
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_u32(bar)),
+        "h"((uint16_t)3)
+        : "memory");
+  else
+    mma_commit(bar);
+}
+
+// fp32 add of a staged box to global memory.
+__device__ __forceinline__ void tma_add_2d(const CUtensorMap* map, const void* src, int x, int y) {
+  asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(smem_u32(src)), "r"(x), "r"(y)
+               : "memory");
+}
+
+// fp32 adds of four values to global memory (no value comes back to wait for).
+__device__ __forceinline__ void add4(float4* p, float4 v) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+               : "memory");
+}
+
+__device__ __forceinline__ bool elect() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
+// 32 accumulator columns from `taddr` with their bias (the same addresses for every lane), as pairs
+__device__ __forceinline__ void load_cols(uint32_t taddr, const float* bias, uint64_t (&v)[16]) {
+  float f[32];
+  tmem_ld32(taddr, f);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(bias) + i);
+    v[2 * i] = add2(pair_of(f[4 * i], f[4 * i + 1]), pair_of(q.x, q.y));
+    v[2 * i + 1] = add2(pair_of(f[4 * i + 2], f[4 * i + 3]), pair_of(q.z, q.w));
+  }
+}
+
+template <int EPI, int BN, bool PAIR, int AR>
 __global__ void __launch_bounds__(kThreads, 1)
-    k_egemm(EGemm g, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB) {
+    k_egemm(EGemm g, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+            const __grid_constant__ CUtensorMap tmO) {
+  using S = Shape<BN, PAIR, AR>;
+  constexpr int kStages = S::kStages, kABytes = S::kABytes;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::kBarOff);
   uint64_t* empty = full + kStages;
   uint64_t* accf = empty + kStages;  // [2] accumulator holds a finished tile
-  uint64_t* acce = accf + 2;         // [2] accumulator read out by the epilogue
+  uint64_t* acce = accf + 2;         // [2] accumulator read out by the epilogue (of both CTAs)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + 2);
-  float* s_bias = reinterpret_cast<float*>(smem + kStages * kStageBytes + kBarBytes);  // [8 warps][2][kBN]
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const int rank = PAIR ? (int)(blockIdx.x & 1) : 0;
+  const int first = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, stride = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
   const int KB = g.K / kBK;
-  const int Mt = (g.M + kBM - 1) / kBM, Nt = (g.N + kBN - 1) / kBN;
+  constexpr int kTM = PAIR ? 2 * kBM : kBM;  // rows per tile
+  const int Mt = (g.M + kTM - 1) / kTM, Nt = (g.N + BN - 1) / BN;
   const int tiles = Mt * Nt;
 
+  // the kernel after this one may start its own set-up (it waits for this
+  // grid's end before it touches anything the chunk writes)
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(full + s, 1);
@@ -68,223 +231,355 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(accf + b, 1);
-      mbar_init(acce + b, kEpiWarps);  // one arrival per epilogue warp
+      mbar_init(acce + b, kEpiWarps * (PAIR ? 2 : 1));  // one arrival per epilogue warp
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(2 * kBN)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (PAIR) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(2 * BN)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(2 * BN)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   fence_before();
+  if constexpr (PAIR)  // the pair's barriers and accumulators exist before either CTA uses them
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   __syncthreads();
   fence_after();
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect()) {
       int it = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-        const int m0 = g.m0 + (t % Mt) * kBM, n0 = (t / Mt) * kBN;
+      auto bar = [&](int st) { return PAIR ? map_rank(smem_u32(full + st), 0) : smem_u32(full + st); };
+      auto load_b = [&](int st, int t, int kb) {
+        if (rank == 0) mbar_expect_tx(full + st, (PAIR ? 2 : 1) * S::kStageBytes);
+        load_2d<PAIR>(smem + st * S::kStageBytes + kABytes, &tmB, bar(st), kb * kBK, (t / Mt) * BN + rank * S::kBRows);
+      };
+      // B is a weight, A the previous kernel's output: the first stages'
+      // tiles of B are requested before the wait
+      const int pre = first < tiles ? min(KB, kStages) : 0;
+      for (int kb = 0; kb < pre; ++kb) load_b(kb, first, kb);
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+      for (int t = first; t < tiles && ok; t += stride) {
+        const int m0 = g.m0 + (t % Mt) * kTM + rank * kBM;
         for (int kb = 0; kb < KB; ++kb, ++it) {
           const int s = it % kStages;
           const uint32_t ph = (uint32_t)(it / kStages) & 1u;
           if (it >= kStages && !mbar_wait(empty + s, ph ^ 1u)) { ok = false; break; }
-          unsigned char* sa = smem + s * kStageBytes;
-          mbar_expect_tx(full + s, kStageBytes);
-          tma_load_2d(sa, &tmA, full + s, kb * kBK, m0);
-          tma_load_2d(sa + kABytes, &tmB, full + s, kb * kBK, n0);
+          if (it >= pre) load_b(s, t, kb);
+          load_2d<PAIR>(smem + s * S::kStageBytes, &tmA, bar(s), kb * kBK, m0);
         }
       }
       if (!ok) {
-        // drain this CTA's copies still in flight
-        for (int j = max(0, it - kStages); j < it; ++j) mbar_wait(full + j % kStages, (uint32_t)(j / kStages) & 1u);
+        // drain the copies still in flight (the leader's barriers count the pair's)
+        if (rank == 0)
+          for (int j = max(0, it - kStages); j < it; ++j) mbar_wait(full + j % kStages, (uint32_t)(j / kStages) & 1u);
         atomicOr(g.err, 1u);
       }
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = idesc_bf16(kBM, kBN);
+    if (rank == 0 && elect()) {
+      const uint32_t idesc = idesc_bf16(kTM, BN);
       int it = 0, tl = 0;
       bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
+      for (int t = first; t < tiles && ok; t += stride, ++tl) {
         const int buf = tl & 1, use = tl >> 1;
         if (tl >= 2 && !mbar_wait(acce + buf, (uint32_t)(use - 1) & 1u)) { ok = false; break; }
         fence_after();
-        const uint32_t acc = tmem + (uint32_t)(buf * kBN);
+        const uint32_t acc = tmem + (uint32_t)(buf * BN);
         for (int kb = 0; kb < KB; ++kb, ++it) {
           const int s = it % kStages;
           const uint32_t ph = (uint32_t)(it / kStages) & 1u;
           if (!mbar_wait(full + s, ph)) { ok = false; break; }
           fence_after();
-          const uint32_t sa = smem_u32(smem + s * kStageBytes);
+          const uint32_t sa = smem_u32(smem + s * S::kStageBytes);
           const uint64_t ad = sw128_desc(sa), bd = sw128_desc(sa + kABytes);
 #pragma unroll
           for (int k = 0; k < kBK / 16; ++k)
-            mma_bf16(acc, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (kb | k) ? 1u : 0u);
-          mma_commit(empty + s);
+            mma<PAIR>(acc, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (kb | k) ? 1u : 0u);
+          commit<PAIR>(empty + s);
         }
-        mma_commit(accf + buf);  // also after a timeout: nothing is left in flight
+        commit<PAIR>(accf + buf);  // also after a timeout: nothing is left in flight
       }
       if (!ok) atomicOr(g.err, 2u);
     }
     __syncwarp();
   } else {
+    // x (the residual update) and the buffers written here belong to kernels before this one
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int q = warp & 3;             // TMEM lane quadrant this warp may access
-    const int half = (warp - 2) >> 2;   // the quadrant's two warps take alternate chunks
+    const int part = (warp - 2) >> 2;   // this warp among the quadrant's
+    unsigned char* stg = smem + S::kStgOff + (warp - 2) * 4096;
     int tl = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tl) {
+    // the staged block may be written again once its store has read it
+    auto stage = [&]() {
+      if (lane == 0) tma_store_wait_read<0>();
+      __syncwarp();
+      return stg;
+    };
+    auto ship = [&](const unsigned char* src, int x, int y, bool add) {
+      fence_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        if (add) tma_add_2d(&tmO, src, x, y);
+        else tma_store_2d(&tmO, src, x, y);
+        tma_store_commit();
+      }
+    };
+    for (int t = first; t < tiles && ok; t += stride, ++tl) {
       const int buf = tl & 1, use = tl >> 1;
-      const int m0 = g.m0 + (t % Mt) * kBM, n0 = (t / Mt) * kBN;
-      const int gr = m0 + q * 32 + lane;
-      const bool live = gr < g.m0 + g.M;
-      // each epilogue warp keeps its own copy of the tile's bias (no
-      // cross-warp barrier: a warp that gives up cannot stall the others)
-      float* bias = s_bias + ((warp - 2) * 2 + buf) * kBN;
-      {
-        const int c = 4 * lane;
-        const float4 bv = n0 + c < g.N ? *reinterpret_cast<const float4*>(g.bias + n0 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-        *reinterpret_cast<float4*>(bias + c) = bv;
-      }
-      // this warp's chunks of the residual row segment are read while the MMAs run
-      float4 xr[EPI == kEResid ? kBN / 8 : 1];
-      if (EPI == kEResid && live) {
-        const float4* xp = reinterpret_cast<const float4*>(static_cast<float*>(g.out) + (size_t)gr * g.ld + n0);
-#pragma unroll
-        for (int c2 = 0; c2 < kBN / 64; ++c2) {
-          const int c = 2 * c2 + half;
-#pragma unroll
-          for (int i = 0; i < 8; ++i)
-            if (n0 + 32 * c + 4 * i < g.N) xr[c2 * 8 + i] = xp[c * 8 + i];
-        }
-      }
-      __syncwarp();  // the warp's bias copy is in place
+      const int m0 = g.m0 + (t % Mt) * kTM + rank * kBM, n0 = (t / Mt) * BN;
+      const int r0 = m0 + q * 32, gr = r0 + lane;
+      const int end = g.m0 + g.M;
+      const bool live = gr < end;
+      const bool whole = r0 + 32 <= end;  // all 32 rows of the warp are this call's (branch's): boxes by TMA
       ok = __all_sync(0xffffffffu, mbar_wait(accf + buf, (uint32_t)use & 1u));
       if (!ok) {
         if (lane == 0) atomicOr(g.err, 4u);
         break;
       }
       fence_after();
-      const uint32_t tbase = tmem + (uint32_t)(buf * kBN) + ((uint32_t)(q * 32) << 16);
-      if (EPI == kEGlu) {
-        // tile columns [64 p, 64 p + 32) are values, [64 p + 32, 64 p + 64) their gates;
-        // group p = half of this warp
+      const uint32_t tbase = tmem + (uint32_t)(buf * BN) + ((uint32_t)(q * 32) << 16);
+      constexpr int kBlk = EPI == kEGlu ? 64 : S::kBlk;
+      if (r0 < end) {
+        // blocks of kBlk columns in turn
+#pragma unroll 1
+        for (int p = part; p < BN / kBlk; p += kEpiWarps / 4) {
+          const int c0 = n0 + kBlk * p;
+          if (c0 >= g.N) break;
+          const uint32_t tc0 = tbase + (uint32_t)(kBlk * p);
+          unsigned char* st = nullptr;
+          if constexpr (EPI == kEGlu) {
+            // columns [64 p, 64 p + 32) are values, [64 p + 32, 64 p + 64) their gates
+            __syncwarp();
+            uint64_t a[16], b[16];
+            load_cols(tc0 + 32, g.bias + c0 + 32, b);
 #pragma unroll
-        for (int p = half; p < kBN / 64; p += 2) {
-          __syncwarp();
-          float a[32], b[32];
-          tmem_ld32(tbase + (uint32_t)(64 * p), a);
-          tmem_ld32(tbase + (uint32_t)(64 * p + 32), b);
-          if (!live || n0 + 64 * p >= g.N) continue;
-          const float* ba = bias + 64 * p;
-          const float* bg = ba + 32;
-          uint4* o = reinterpret_cast<uint4*>(static_cast<uint16_t*>(g.out) + (size_t)gr * g.ld + (n0 + 64 * p) / 2);
+            for (int i = 0; i < 16; ++i) b[i] = sigmoid2(b[i]);
+            load_cols(tc0, g.bias + c0, a);
+            uint32_t w[16];
 #pragma unroll
-          for (int i = 0; i < 32; i += 8) {
-            uint4 w;
-            w.x = pack_bf16((a[i] + ba[i]) * sigm(b[i] + bg[i]), (a[i + 1] + ba[i + 1]) * sigm(b[i + 1] + bg[i + 1]));
-            w.y = pack_bf16((a[i + 2] + ba[i + 2]) * sigm(b[i + 2] + bg[i + 2]),
-                            (a[i + 3] + ba[i + 3]) * sigm(b[i + 3] + bg[i + 3]));
-            w.z = pack_bf16((a[i + 4] + ba[i + 4]) * sigm(b[i + 4] + bg[i + 4]),
-                            (a[i + 5] + ba[i + 5]) * sigm(b[i + 5] + bg[i + 5]));
-            w.w = pack_bf16((a[i + 6] + ba[i + 6]) * sigm(b[i + 6] + bg[i + 6]),
-                            (a[i + 7] + ba[i + 7]) * sigm(b[i + 7] + bg[i + 7]));
-            o[i / 8] = w;
-          }
-        }
-      } else {
+            for (int i = 0; i < 16; ++i) w[i] = pack_bf16(mul2(a[i], b[i]));
+            if (whole) st = stage();
+            uint16_t* o = static_cast<uint16_t*>(g.out) + (size_t)gr * g.ld + c0 / 2;
 #pragma unroll
-        for (int c2 = 0; c2 < kBN / 64; ++c2) {
-          const int c = 2 * c2 + half;
-          __syncwarp();
-          float v[32];
-          tmem_ld32(tbase + (uint32_t)(c * 32), v);
-          const int c0 = n0 + c * 32;
-          if (!live || c0 >= g.N) continue;
-          const float* bb = bias + c * 32;
-#pragma unroll
-          for (int i = 0; i < 32; ++i) v[i] += bb[i];
-          if (EPI == kEInit || EPI == kEResid) {
-            float4* xp = reinterpret_cast<float4*>(static_cast<float*>(g.out) + (size_t)gr * g.ld + c0);
-#pragma unroll
-            for (int i = 0; i < 32; i += 4) {
-              float4 r = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-              if (EPI == kEResid) {
-                const float4 o = xr[c2 * 8 + i / 4];
-                r = make_float4(o.x + g.alpha * r.x, o.y + g.alpha * r.y, o.z + g.alpha * r.z, o.w + g.alpha * r.w);
-              }
-              xp[i / 4] = r;
+            for (int e = 0; e < 4; ++e) {
+              const uint4 x = make_uint4(w[4 * e], w[4 * e + 1], w[4 * e + 2], w[4 * e + 3]);
+              if (whole) *reinterpret_cast<uint4*>(st + lane * 64 + ((e ^ ((lane >> 1) & 3)) << 4)) = x;
+              else if (live) reinterpret_cast<uint4*>(o)[e] = x;
             }
+            if (whole) ship(st, c0 / 2, r0, false);
           } else {
-            if (EPI == kESwish) {
 #pragma unroll
-              for (int i = 0; i < 32; ++i) v[i] = v[i] * sigm(v[i]);
+            for (int h = 0; h < kBlk / 32; ++h) {
+              __syncwarp();
+              uint64_t v[16];
+              load_cols(tc0 + (uint32_t)(32 * h), g.bias + c0 + 32 * h, v);
+              if constexpr (EPI == kEInit || EPI == kEResid) {
+                if (EPI == kEResid) {
+#pragma unroll
+                  for (int i = 0; i < 16; ++i) v[i] = mul2(v[i], pair_of(g.alpha, g.alpha));
+                }
+                if (whole) st = stage();
+                float4* xp = reinterpret_cast<float4*>(static_cast<float*>(g.out) + (size_t)gr * g.ld + c0 + 32 * h);
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                  float4 x;
+                  unpair(v[2 * e], x.x, x.y);
+                  unpair(v[2 * e + 1], x.z, x.w);
+                  if (whole) {
+                    *reinterpret_cast<float4*>(st + lane * 128 + ((e ^ (lane & 7)) << 4)) = x;
+                  } else if (live) {
+                    if (EPI == kEResid) add4(xp + e, x);
+                    else xp[e] = x;
+                  }
+                }
+                if (whole) ship(st, c0 + 32 * h, r0, EPI == kEResid);
+              } else {
+                if (EPI == kESwish) {
+#pragma unroll
+                  for (int i = 0; i < 16; ++i) v[i] = mul2(v[i], sigmoid2(v[i]));
+                }
+                uint32_t w[16];
+#pragma unroll
+                for (int i = 0; i < 16; ++i) w[i] = pack_bf16(v[i]);
+                if (whole && h == 0) st = stage();
+                uint16_t* o = static_cast<uint16_t*>(g.out) + (size_t)gr * g.ld + c0 + 32 * h;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                  const uint4 x = make_uint4(w[4 * e], w[4 * e + 1], w[4 * e + 2], w[4 * e + 3]);
+                  if (whole)
+                    *reinterpret_cast<uint4*>(st + (kBlk == 64 ? lane * 128 + (((4 * h + e) ^ (lane & 7)) << 4)
+                                                               : lane * 64 + ((e ^ ((lane >> 1) & 3)) << 4))) = x;
+                  else if (live)
+                    reinterpret_cast<uint4*>(o)[e] = x;
+                }
+                if (whole && h == kBlk / 32 - 1) ship(st, c0, r0, false);
+              }
             }
-            uint4* o = reinterpret_cast<uint4*>(static_cast<uint16_t*>(g.out) + (size_t)gr * g.ld + c0);
-#pragma unroll
-            for (int i = 0; i < 32; i += 8)
-              o[i / 8] = make_uint4(pack_bf16(v[i], v[i + 1]), pack_bf16(v[i + 2], v[i + 3]),
-                                    pack_bf16(v[i + 4], v[i + 5]), pack_bf16(v[i + 6], v[i + 7]));
           }
         }
       }
       // this warp's reads of the accumulator are done: hand it back
       fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(acce + buf);
+      if (lane == 0) {
+        if (rank == 0) mbar_arrive(acce + buf);
+        else
+          asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(map_rank(smem_u32(acce + buf), 0))
+                       : "memory");
+      }
     }
+    // the staged blocks must have been read before the CTA's shared memory
+    // goes; the stores' writes complete with the grid
+    if (lane == 0) tma_store_wait_read<0>();
+    __syncwarp();
   }
   fence_before();
   __syncthreads();
+  if constexpr (PAIR)  // neither CTA leaves while the other may still signal it or read its operands
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (warp == 1) {
     fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kBN) : "memory");
+    if constexpr (PAIR)
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
+    else
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
   }
 }
 
+// Clocks of a GEMM on a tile shape: rounds of tiles over the SMs, each
+// k-block the larger of its MMAs (measured per 16-deep MMA: 129 clocks at 256
+// columns over a pair, 65 at 128, 49 at 64, 41 at 32) and its operands at 64
+// bytes per clock and SM, and a launch's fill and last epilogue.
+double cost(int M, int N, int K, int BN, bool pair, int a_rows) {
+  const int tm = pair ? 2 * kBM : kBM;
+  const int tiles = ((M + tm - 1) / tm) * ((N + BN - 1) / BN);
+  const int slots = pair ? g_sms / 2 : g_sms;
+  const double mma = 4.0 * (pair ? 129 : BN == 128 ? 65 : BN == 64 ? 49 : 41);
+  const double load = ((pair ? kBM : a_rows) + (pair ? BN / 2 : BN)) * 128.0 / 64.0;
+  const int rounds = (tiles + slots - 1) / slots;
+  return rounds * (K / kBK) * std::max(mma, load) + 1000.0 + 12.0 * BN;
+}
+
+template <int EPI, int BN, bool PAIR, int AR>
+cudaError_t launch_shape(const EGemm& g, const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& o, cudaStream_t s,
+                         bool pdl) {
+  constexpr int tm = PAIR ? 2 * kBM : kBM;
+  const int tiles = ((g.M + tm - 1) / tm) * ((g.N + BN - 1) / BN);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(PAIR ? 2 * std::min(tiles, g_sms / 2) : std::min(tiles, g_sms)));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = Shape<BN, PAIR, AR>::kSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (PAIR) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = 2;
+    at[n].val.clusterDim.y = 1;
+    at[n++].val.clusterDim.z = 1;
+  }
+  if (pdl) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = (unsigned)n;
+  return cudaLaunchKernelEx(&cfg, k_egemm<EPI, BN, PAIR, AR>, g, a, b, o);
+}
+
 template <int EPI>
-void launch_one(const EGemm& g, const CUtensorMap& a, const CUtensorMap& b, cudaStream_t s) {
-  const int tiles = ((g.M + kBM - 1) / kBM) * ((g.N + kBN - 1) / kBN);
-  k_egemm<EPI><<<tiles < g_sms ? tiles : g_sms, kThreads, kSmem, s>>>(g, a, b);
+void launch_one(const EGemm& g, const EncMapA& A, const EncMapB& B, const EncMapO& O, cudaStream_t s, bool pdl) {
+  // a call of at most 64 rows stages 64 rows of A
+  const bool few = g.m0 == 0 && g.M <= 64;
+  const int ar = few ? 64 : kBM;
+  double best = few ? 1e30 : cost(g.M, g.N, g.K, 256, true, kBM);
+  int pick = 0;
+  const int bns[3] = {128, 64, 32};
+  for (int i = few ? 1 : 0; i < (EPI == kEGlu ? 2 : 3); ++i) {  // GLU pairs need 64 columns
+    const double c = cost(g.M, g.N, g.K, bns[i], false, ar);
+    if (c < best) best = c, pick = 1 + i;
+  }
+  const CUtensorMap& o = (EPI == kESwish || EPI == kEPlain) ? O.m[pick == 0 ? 0 : 1] : O.m[EPI == kEGlu ? 1 : 0];
+  if (pick == 0) launch_shape<EPI, 256, true, 128>(g, A.m[0], B.m[0], o, s, pdl);
+  else if (pick == 1) launch_shape<EPI, 128, false, 128>(g, A.m[0], B.m[0], o, s, pdl);
+  else if (pick == 2 && few) launch_shape<EPI, 64, false, 64>(g, A.m[1], B.m[1], o, s, pdl);
+  else if (pick == 2) launch_shape<EPI, 64, false, 128>(g, A.m[0], B.m[1], o, s, pdl);
+  else if constexpr (EPI != kEGlu) {
+    if (few) launch_shape<EPI, 32, false, 64>(g, A.m[1], B.m[2], o, s, pdl);
+    else launch_shape<EPI, 32, false, 128>(g, A.m[0], B.m[2], o, s, pdl);
+  }
+}
+
+template <int EPI, int BN, bool PAIR, int AR>
+void prepare_shape(cudaError_t& e) {
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_egemm<EPI, BN, PAIR, AR>, cudaFuncAttributeMaxDynamicSharedMemorySize, Shape<BN, PAIR, AR>::kSmem);
+}
+
+template <int EPI>
+void prepare_one(cudaError_t& e) {
+  prepare_shape<EPI, 256, true, 128>(e);
+  prepare_shape<EPI, 128, false, 128>(e);
+  prepare_shape<EPI, 64, false, 128>(e);
+  prepare_shape<EPI, 64, false, 64>(e);
+  if constexpr (EPI != kEGlu) {
+    prepare_shape<EPI, 32, false, 128>(e);
+    prepare_shape<EPI, 32, false, 64>(e);
+  }
 }
 
 }  // namespace
 
-bool egemm_map_a(CUtensorMap* m, const uint16_t* A, int rows, int K) {
-  return tc::make_map(m, A, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, rows, tc::kBK, tc::kBM);
+bool egemm_map_a(EncMapA* m, const uint16_t* A, int rows, int K) {
+  for (int i = 0; i < 2; ++i)
+    if (!tc::make_map(&m->m[i], A, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, rows, tc::kBK, tc::kBM >> i)) return false;
+  return true;
 }
 
-bool egemm_map_b(CUtensorMap* m, const uint16_t* B, int rows, int K) {
-  return tc::make_map(m, B, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, rows, tc::kBK, kBN);
+bool egemm_map_b(EncMapB* m, const uint16_t* B, int rows, int K) {
+  for (int i = 0; i < 3; ++i)
+    if (!tc::make_map(&m->m[i], B, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, K, rows, tc::kBK, 128 >> i)) return false;
+  return true;
+}
+
+bool egemm_map_out(EncMapO* m, bool fp32, void* out, int rows, int ld) {
+  // boxes of 32 rows: 32 fp32 columns; 64 bf16 columns, or 32 (the narrow tiles, GLU)
+  if (fp32) return tc::make_map(&m->m[0], out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, ld, rows, 32, 32);
+  return tc::make_map(&m->m[0], out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ld, rows, 64, 32) &&
+         tc::make_map(&m->m[1], out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ld, rows, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
 cudaError_t egemm_prepare() {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&g_sms, cudaDevAttrMultiProcessorCount, dev);
-  auto set = [&](const void* f) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
-  };
-  set((const void*)k_egemm<kEInit>);
-  set((const void*)k_egemm<kEResid>);
-  set((const void*)k_egemm<kESwish>);
-  set((const void*)k_egemm<kEPlain>);
-  set((const void*)k_egemm<kEGlu>);
+  prepare_one<kEInit>(e);
+  prepare_one<kEResid>(e);
+  prepare_one<kESwish>(e);
+  prepare_one<kEPlain>(e);
+  prepare_one<kEGlu>(e);
   return e;
 }
 
-void launch_egemm(int epi, const EGemm& g, const CUtensorMap& a, const CUtensorMap& b, cudaStream_t s) {
+void launch_egemm(int epi, const EGemm& g, const EncMapA& a, const EncMapB& b, const EncMapO& o, cudaStream_t s, bool pdl) {
   switch (epi) {
-    case kEInit: launch_one<kEInit>(g, a, b, s); break;
-    case kEResid: launch_one<kEResid>(g, a, b, s); break;
-    case kESwish: launch_one<kESwish>(g, a, b, s); break;
-    case kEPlain: launch_one<kEPlain>(g, a, b, s); break;
-    default: launch_one<kEGlu>(g, a, b, s); break;
+    case kEInit: launch_one<kEInit>(g, a, b, o, s, pdl); break;
+    case kEResid: launch_one<kEResid>(g, a, b, o, s, pdl); break;
+    case kESwish: launch_one<kESwish>(g, a, b, o, s, pdl); break;
+    case kEPlain: launch_one<kEPlain>(g, a, b, o, s, pdl); break;
+    default: launch_one<kEGlu>(g, a, b, o, s, pdl); break;
   }
 }
 

@@ -20,6 +20,17 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
+// 1 / (1 + e^-x): the exponent's product with log2 e in two parts, so that
+// the approximations of 2^x and 1/x (relative errors of 2^-22 and 2^-23) are
+// what remains at any x.
+__device__ __forceinline__ float sigmoid(float x) {
+  const float hi = x * -kLog2e, lo = fmaf(x, -kLog2e, -hi);
+  const float e = ex2_approx(hi);
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + fmaf(e, lo * 0.6931471805599453f, e)));
+  return r;
+}
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
@@ -201,10 +212,10 @@ inline EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// 2-D row-major map with the 128-byte swizzle: `inner` elements per row,
-// boxes of box_inner x box_rows.
+// 2-D row-major map (by default with the 128-byte swizzle): `inner` elements
+// per row, boxes of box_inner x box_rows.
 inline bool make_map(CUtensorMap* m, const void* base, CUtensorMapDataType dtype, int elem_bytes, int inner, int rows,
-              int box_inner, int box_rows) {
+              int box_inner, int box_rows, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   cuuint64_t dims[2] = {(cuuint64_t)inner, (cuuint64_t)rows};
@@ -212,7 +223,7 @@ inline bool make_map(CUtensorMap* m, const void* base, CUtensorMapDataType dtype
   cuuint32_t box[2] = {(cuuint32_t)box_inner, (cuuint32_t)box_rows};
   cuuint32_t es[2] = {1, 1};
   return fn(m, dtype, 2, const_cast<void*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+            swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
          CUDA_SUCCESS;
 }
 
