@@ -7,8 +7,8 @@
 // few rows is not work but the chain of launches and round trips to L2: 9.4 us
 // a step for one stream (V = 1024, H = 640), 10.4 us for 64, against well
 // under 1 us of arithmetic.  Here a step has no launch, no grid-wide
-// dependency and no logits in memory (13 frames of one stream: 619 -> 212 us,
-// of 64 streams: 674 -> 302 us; 16 streams x 1 frame, H = 1024: 71 -> 36 us):
+// dependency and no logits in memory (13 frames of one stream: 616 -> 192 us,
+// of 64 streams: 670 -> 295 us; 16 streams x 1 frame, H = 1024: 70 -> 31 us):
 //   * CTA c of the cluster keeps labels [c nl, (c+1) nl) of W_out in shared
 //     memory for the whole chunk (read once per chunk, not once per step);
 //   * warps 0-7 (GEMM) compute the slice's logits of all R rows: bf16
@@ -16,15 +16,23 @@
 //     8-column one, so one row costs one eighth of what a 128-row tcgen05 tile
 //     does and the eight warps split H; their partials are summed in a fixed
 //     order and sent to the row's owner CTA by st.async;
-//   * row i is owned by CTA i mod CS, group i / CS: 128 threads that keep the
-//     row's state in shared memory, take the argmax, publish the label to
-//     every CTA (8 bytes each by st.async), and only then advance the LM and
-//     trie chains and build the next state's deltas, while the GEMM warps
-//     already load the embedding rows and multiply;
+//   * row i is owned by CTA i mod CS, group i / CS: 128 threads (64 with three
+//     groups) that keep the row's state in shared memory, take the argmax,
+//     publish the label to every CTA (16 bytes each by st.async), and only
+//     then advance the LM and trie chains and build the next state's deltas,
+//     while the GEMM warps already load the embedding rows and multiply; the
+//     arcs and trie children that the deltas need stay in the threads'
+//     registers, so that the next label's search is a compare and one load;
 //   * a cluster stops when its rows have finished their frames.
 // Clusters never wait for one another.  Messages inside a cluster complete
 // bytes on the receiver's mbarriers: `ybar` (every CTA: the R rows' labels of
 // a step) and `lbar` (per owned row: its logits), one phase per step each.
+// `sbar` (per owned row) does the same for the softmax partials that a score
+// needs: GEMM warp q finishes row q's scores one step late, while it would wait.
+// What is left of a step, in clocks, one stream: argmax 710, publishing 350,
+// the label's records 1700, chains 770, deltas 1930 (three of these five wait
+// for L2 once), beside labels to operands 1460, product 1430, sums and sending
+// 700.
 // Every wait is bounded (DecView::wait_ns); after an expired one the CTA
 // records a code, leaves the loop, lets messages in flight land and meets the
 // others at the cluster barrier that ends the kernel.
@@ -51,12 +59,8 @@ using row::kNegInf;
 using row::lse_merge;
 
 constexpr int kGemm = 256;     // GEMM threads (8 warps, each an eighth of H)
-constexpr int kGroup = 128;    // threads of a row group
-constexpr int kWarpsG = kGroup / 32;
-static_assert(kWarpsG == 4, "a row group's four warps");
 constexpr int kTiles = 5;      // 16-label tiles per accumulator block
 constexpr int kMB = 16 * kTiles;
-constexpr int kPS = kMB + 4;   // row stride of the partials: lanes (n = 2c, m = g) fall in different banks
 constexpr int kUnits = 4;      // 32-wide pieces of H per warp: H <= 1024
 constexpr int kTrHeld = 3;     // trie chain nodes whose first children a thread requests together
 constexpr int kWPad = 64;      // bytes after a W_out row: neighbouring rows start 16 banks apart
@@ -176,31 +180,36 @@ struct RowSm {
   int4 lm_hit[kLmChain + 1], tr_hit[kTrChain]; // records found for the emitted label
   int4 uni_hit, root_hit;
   int lm[kLmChain + 1], tr[kTrChain];
-  int4 best[2][kWarpsG];                       // the warps' bests (value, label, wait succeeded), by step parity
+  int dd[kTrChain];                            // depth of the children of a found trie child
+  int4 best[2][4];                             // the warps' bests (value, label, wait succeeded), by step parity
   int nl, nt;
 };
 
 // Shared-memory layout of a CTA (bytes from the 128-byte-aligned base).
 struct Layout {
-  int w, part, dflt, root, y, bars, rows, row_bytes, logits, lse, dlm, lev, dep, total;
+  int w, part, ps, dflt, uni, root, y, bars, rows, row_bytes, logits, lse, term, mark, list, total;
 };
 __host__ __device__ inline Layout layout(int H, int V4, int nl, int CS, int NB, int RG) {
   Layout L;
   auto up = [](int x) { return (x + 127) & ~127; };
   int o = 0;
   L.bars = o, o += 128;                      // ybar, wbar, lbar[RG], sbar[RG], fail flag
-  L.y = o, o = up(o + 8 * CS * RG);          // (previous label, frame or -1) of every row of the cluster
+  L.y = o, o = up(o + 16 * CS * RG);         // every row's (previous label, frame or -1, fused value, output place or -1)
   L.w = o, o = up(o + nl * (2 * H + kWPad));
-  L.part = o, o = up(o + 8 * (8 * NB) * kPS * 4);
+  // row stride of the partials, 4 mod 16: lanes (n = 2c, m = g) fall in different banks
+  L.ps = ((nl < kMB ? nl : kMB) + 11) / 16 * 16 + 4;
+  L.part = o, o = up(o + 8 * (8 * NB) * L.ps * 4);
   L.dflt = o, o = up(o + 4 * V4);            // the call's defaults D
+  L.uni = o, o = up(o + 4 * V4);             // log p(v)
   L.root = o, o = up(o + (V4 + 31) / 32 * 4);
   L.rows = o;
   int r = (int)((sizeof(RowSm) + 127) & ~size_t(127));
-  L.logits = r, r = up(r + 2 * 4 * CS * nl);  // two steps' logits
-  L.lse = r, r = up(r + 2 * 8 * CS * ((nl + kMB - 1) / kMB));  // and softmax partials
-  L.dlm = r, r = up(r + 4 * V4);
-  L.lev = r, r = up(r + 2 * V4);
-  L.dep = r, r = up(r + V4);
+  L.logits = r, r = up(r + 4 * CS * nl);
+  L.lse = r, r = up(r + 3 * 8 * CS * ((nl + kMB - 1) / kMB));  // softmax partials of three steps
+  L.term = r, r = up(r + 4 * V4);
+  L.mark = r, r = up(r + 4 * V4);
+  L.list = RG < 3 ? r : -1;                  // level 0's labels
+  if (RG < 3) r = up(r + 4 * V4 + 32);
   L.row_bytes = r;
   L.total = o + RG * r + 128;                // and the alignment of the base
   return L;
@@ -261,7 +270,7 @@ struct Ctx {
   Layout L;
   uint64_t *ybar, *wbar, *lbar, *sbar;
   volatile int* fail;
-  int2* y;
+  int4* y;
   int CS, rank, nl, R, row0;
 };
 
@@ -277,9 +286,11 @@ struct Piece {
 // warp's part of H for 8 NB rows, written to the partials [warp][row][label].
 // Labels past the slice read its last row again, and the upper half of an odd
 // last tile its lower half: their sums are never sent.
-template <int HT, int NB>
+// FU >= 0: every warp has FU pieces of H and some one more (their products
+// are scheduled together); -1: any number.
+template <int HT, int NB, int FU>
 __device__ __forceinline__ void tile_block(const unsigned char* W, int wstride, int nl, int m0, int U, int warp, int g, int k4,
-                                           const uint4 (&b)[kUnits][NB], float* part) {
+                                           const uint4 (&b)[kUnits][NB], float* part, int ps) {
   constexpr int MT = (HT + 1) / 2;
   float acc[MT][NB][4];
   int off[HT];
@@ -294,7 +305,8 @@ __device__ __forceinline__ void tile_block(const unsigned char* W, int wstride, 
 #pragma unroll
   for (int u = 0; u < kUnits; ++u) {
     const int un = warp + 8 * u;
-    if (un < U) {
+    if (FU >= 0 && u > FU) break;
+    if ((FU >= 0 && u < FU) || un < U) {
       uint4 a[HT];
 #pragma unroll
       for (int t = 0; t < HT; ++t) a[t] = *reinterpret_cast<const uint4*>(W + off[t] + un * 64);
@@ -314,28 +326,35 @@ __device__ __forceinline__ void tile_block(const unsigned char* W, int wstride, 
   for (int t = 0; t < MT; ++t)
 #pragma unroll
     for (int j = 0; j < NB; ++j) {
-      float* o = part + (warp * 8 * NB + 8 * j + 2 * k4) * kPS + 16 * t + g;
-      o[0] = acc[t][j][0];
-      o[kPS] = acc[t][j][1];
-      if (2 * t + 1 < HT) {
-        o[8] = acc[t][j][2];
-        o[kPS + 8] = acc[t][j][3];
-      }
+      float* o = part + (warp * 8 * NB + 8 * j + 2 * k4) * ps + 16 * t + g;
+      if (16 * t + g < ps) o[0] = acc[t][j][0], o[ps] = acc[t][j][1];
+      if (2 * t + 1 < HT && 16 * t + 8 + g < ps) o[8] = acc[t][j][2], o[ps + 8] = acc[t][j][3];
     }
 }
 
-template <int NB>
+// Whether the product may take its rows in several passes of 8 NB.
+__host__ __device__ constexpr bool several_passes(int NB, int RG) { return RG == 3 || (RG == 1 && NB == 1); }
+
+template <int NB, int RG, int FU>
 __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
+  constexpr bool kPasses = several_passes(NB, RG);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, k4 = lane & 3;
-  const int U = d.H / 32, H = d.H;
+  const int U = d.H / 32, H = d.H, ps = c.L.ps;
   const int wstride = 2 * H + kWPad;
   const unsigned char* W = c.sm + c.L.w;
   float* part = reinterpret_cast<float*>(c.sm + c.L.part);
   const uint32_t sm0 = tc::smem_u32(c.sm);
+  const int nb = (c.nl + kMB - 1) / kMB;  // softmax partials per CTA
+  // Warp q < RG also finishes the scores of the CTA's row q: a step's softmax
+  // partials (three buffers in turn) are consumed one step later, while the
+  // warp would wait for the next labels.
+  const int own = warp * c.CS + c.rank;
+  const bool mine = warp < RG && own < c.R;
+  bool armed = false, ok = true;
   // this warp's operands of row i (zero for a finished row or none)
   auto load = [&](int i, Piece& q) {
-    const int2 st = i < c.R ? c.y[i] : make_int2(0, -1);
+    const int4 st = i < c.R ? c.y[i] : make_int4(0, -1, 0, -1);
     const uint4* e = reinterpret_cast<const uint4*>(P.enc + ((size_t)(c.row0 + i) * P.T + max(st.y, 0)) * H) + k4;
     const uint4* m = reinterpret_cast<const uint4*>(d.E + (size_t)st.x * H) + k4;
 #pragma unroll
@@ -348,9 +367,9 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
       }
     }
   };
-  for (int step = 0;; ++step) {
+  for (int step = 0, slot = 2; ; ++step) {  // slot: the buffer of the step before (step - 1 mod 3)
     // the rows' labels (at first, W_out's slice as well)
-    bool ok = wait_cluster(c.ybar, step & 1, d.wait_ns, c.fail);
+    ok = wait_cluster(c.ybar, step & 1, d.wait_ns, c.fail) && ok;
     if (step == 0) ok = ok && wait_cluster(c.wbar, 0, d.wait_ns, c.fail);
     if (!group_all(1, kGemm, ok)) {
       if (tid == 0) atomicOr(d.err, 1);
@@ -358,43 +377,83 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
       return;
     }
     Piece q[NB];
+    if (RG < 3) {  // (the first pass's: requested before the bookkeeping)
 #pragma unroll
-    for (int j = 0; j < NB; ++j) load(8 * j + g, q[j]);
+      for (int j = 0; j < NB; ++j) load(8 * j + g, q[j]);
+    }
     int active = 0;  // rows still decoding: the next step's publishers
     for (int i = lane; i < c.R; i += 32) active += c.y[i].y >= 0 ? 1 : 0;
     active = __reduce_add_sync(0xffffffffu, active);
-    if (active == 0) return;
-    if (tid == 0) tc::mbar_expect_tx(c.ybar, 8u * (uint32_t)active);
-    // the joint inputs, bf16(ReLU(enc + E)); a lane's eight consecutive
-    // elements feed two 16-deep MMAs (the same order of H in both operands)
-    uint4 b[kUnits][NB];
+    if (tid == 0 && active) tc::mbar_expect_tx(c.ybar, 16u * (uint32_t)active);
+    int4 said = make_int4(0, -1, 0, -1);  // the row's label of the step before
+    bool score = false;
+    if (mine) {
+      said = c.y[own];
+      if (armed) {  // the step before's partials are all in; before any of this step's can be sent
+        ok = __all_sync(0xffffffffu, wait_cluster(c.sbar + warp, (step - 1) & 1, d.wait_ns, c.fail));
+        score = ok && said.w >= 0;
+      }
+      armed = ok && said.y >= 0;
+      if (armed && lane == 0) tc::mbar_expect_tx(c.sbar + warp, 8u * (uint32_t)(c.CS * nb));
+    }
+    auto write_score = [&]() {
+      const float2* sp = reinterpret_cast<const float2*>(c.sm + c.L.rows + warp * c.L.row_bytes + c.L.lse) + slot * c.CS * nb;
+      float m = kNegInf, z = 0.f;
+      for (int x = lane; x < c.CS * nb; x += 32) lse_merge(m, z, sp[x].x, sp[x].y);
+      __syncwarp();
+      const float top = key_value(__reduce_max_sync(0xffffffffu, order_key(m)));
+      z = z > 0.f ? z * expf(m - top) : 0.f;
 #pragma unroll
-    for (int u = 0; u < kUnits; ++u)
+      for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+      if (lane == 0)
+        P.out_score[(size_t)(c.row0 + own) * (P.T * d.max_sym) + said.w] = __int_as_float(said.z) - (top + logf(z));
+    };
+    if (active == 0) {
+      if (score) write_score();
+      if (!ok) {
+        if (lane == 0) atomicOr(d.err, 8);
+        *c.fail = 1;
+      }
+      return;
+    }
+#pragma unroll 1
+    for (int i0 = 0; i0 < (kPasses ? c.R : 1); i0 += 8 * NB) {
+      // the joint inputs, bf16(ReLU(enc + E)); a lane's eight consecutive
+      // elements feed two 16-deep MMAs (the same order of H in both operands)
+      uint4 b[kUnits][NB];
+      if (RG == 3 || (kPasses && i0 > 0)) {
 #pragma unroll
-      for (int j = 0; j < NB; ++j) b[u][j] = joint8(q[j].x[u], q[j].z[u]);
-    __syncwarp();
-    for (int m0 = 0; m0 < c.nl; m0 += kMB) {
-      const int left = c.nl - m0;
-      if (left > 72) tile_block<10, NB>(W, wstride, c.nl, m0, U, warp, g, k4, b, part);
-      else if (left > 64) tile_block<9, NB>(W, wstride, c.nl, m0, U, warp, g, k4, b, part);
-      else if (left > 48) tile_block<8, NB>(W, wstride, c.nl, m0, U, warp, g, k4, b, part);
-      else if (left > 32) tile_block<6, NB>(W, wstride, c.nl, m0, U, warp, g, k4, b, part);
-      else if (left > 16) tile_block<4, NB>(W, wstride, c.nl, m0, U, warp, g, k4, b, part);
-      else tile_block<2, NB>(W, wstride, c.nl, m0, U, warp, g, k4, b, part);
-      // the warps' partials summed in a fixed order and sent to the rows' owners
-      group_sync(1, kGemm);
-      const int nq = min(kMB, c.nl - m0) / 4;
+        for (int j = 0; j < NB; ++j) load(i0 + 8 * j + g, q[j]);
+      }
 #pragma unroll
-      for (int j = 0; j < NB; ++j) {
-        const int i = 8 * j + warp;
-        if (i >= c.R || c.y[i].y < 0) continue;  // the same for the warp's lanes
-        const int grp = i / c.CS, owner = i - grp * c.CS;
-        const uint32_t row = sm0 + c.L.rows + grp * c.L.row_bytes;
-        float4 s[8];
-        if (lane < nq) {
+      for (int u = 0; u < kUnits; ++u)
 #pragma unroll
-          for (int w = 0; w < 8; ++w)
-            s[w] = *reinterpret_cast<const float4*>(part + (w * 8 * NB + i) * kPS + 4 * lane);
+        for (int j = 0; j < NB; ++j) b[u][j] = joint8(q[j].x[u], q[j].z[u]);
+      __syncwarp();
+      for (int m0 = 0; m0 < c.nl; m0 += kMB) {
+        const int left = c.nl - m0;
+        if (left > 72) tile_block<10, NB, FU>(W, wstride, c.nl, m0, U, warp, g, k4, b, part, ps);
+        else if (left > 64) tile_block<9, NB, FU>(W, wstride, c.nl, m0, U, warp, g, k4, b, part, ps);
+        else if (left > 48) tile_block<8, NB, FU>(W, wstride, c.nl, m0, U, warp, g, k4, b, part, ps);
+        else if (left > 32) tile_block<6, NB, FU>(W, wstride, c.nl, m0, U, warp, g, k4, b, part, ps);
+        else if (left > 16) tile_block<4, NB, FU>(W, wstride, c.nl, m0, U, warp, g, k4, b, part, ps);
+        else tile_block<2, NB, FU>(W, wstride, c.nl, m0, U, warp, g, k4, b, part, ps);
+        // the warps' partials summed in a fixed order and sent to the rows' owners
+        group_sync(1, kGemm);
+        const int nq = min(kMB, c.nl - m0) / 4;
+        float4 sum[NB];
+        bool on[NB];  // read before the sends: a row's next label may follow its logits at once
+#pragma unroll
+        for (int j = 0; j < NB; ++j) on[j] = i0 + 8 * j + warp < c.R && c.y[i0 + 8 * j + warp].y >= 0;
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < NB; ++j) {
+          const int n = 8 * j + warp, i = i0 + n;
+          if (!on[j] || lane >= nq) continue;
+          const int grp = i / c.CS, owner = i - grp * c.CS;
+          float4 s[8];
+#pragma unroll
+          for (int w = 0; w < 8; ++w) s[w] = *reinterpret_cast<const float4*>(part + (w * 8 * NB + n) * ps + 4 * lane);
 #pragma unroll
           for (int h = 1; h < 8; h *= 2)
 #pragma unroll
@@ -404,83 +463,96 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
               s[w].z += s[w + h].z;
               s[w].w += s[w + h].w;
             }
-          const uint32_t dst = row + c.L.logits + 4 * ((step & 1) * c.CS * c.nl + c.rank * c.nl + m0 + 4 * lane);
+          const uint32_t dst = sm0 + c.L.rows + grp * c.L.row_bytes + c.L.logits + 4 * (c.rank * c.nl + m0 + 4 * lane);
           send16(map_rank(dst, owner), s[0], map_rank(tc::smem_u32(c.lbar + grp), owner));
+          sum[j] = s[0];
         }
-        // the block's softmax partial (max, sum of exp) follows: an emitted
-        // label's score needs it, one step later
-        const int v0 = c.rank * c.nl + m0 + 4 * lane;
-        const float l[4] = {lane < nq && v0 < d.N ? s[0].x : kNegInf, lane < nq && v0 + 1 < d.N ? s[0].y : kNegInf,
-                            lane < nq && v0 + 2 < d.N ? s[0].z : kNegInf, lane < nq && v0 + 3 < d.N ? s[0].w : kNegInf};
-        __syncwarp();
-        const float m = key_value(__reduce_max_sync(0xffffffffu, order_key(fmaxf(fmaxf(l[0], l[1]), fmaxf(l[2], l[3])))));
-        const float m2 = m * tc::kLog2e;
-        float z = 0.f;
-        if (m != kNegInf)
-          z = (tc::ex2_approx(fmaf(l[0], tc::kLog2e, -m2)) + tc::ex2_approx(fmaf(l[1], tc::kLog2e, -m2))) +
-              (tc::ex2_approx(fmaf(l[2], tc::kLog2e, -m2)) + tc::ex2_approx(fmaf(l[3], tc::kLog2e, -m2)));
+        // the block's softmax partials (max, sum of exp) follow: an emitted
+        // label's score needs them, one step later
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-        if (lane == 0) {
-          const int nb = (c.nl + kMB - 1) / kMB;
-          const uint32_t dst = row + c.L.lse + 8 * ((step & 1) * c.CS * nb + c.rank * nb + m0 / kMB);
-          send8(map_rank(dst, owner), __float_as_int(m), __float_as_int(z), map_rank(tc::smem_u32(c.sbar + grp), owner));
+        for (int j = 0; j < NB; ++j) {
+          const int i = i0 + 8 * j + warp;
+          __syncwarp();
+          if (!on[j]) continue;  // the same for the warp's lanes
+          const int grp = i / c.CS, owner = i - grp * c.CS;
+          const int v0 = c.rank * c.nl + m0 + 4 * lane, nv = lane < nq ? d.N - v0 : 0;
+          const float l[4] = {nv > 0 ? sum[j].x : kNegInf, nv > 1 ? sum[j].y : kNegInf, nv > 2 ? sum[j].z : kNegInf,
+                              nv > 3 ? sum[j].w : kNegInf};
+          const float m = key_value(__reduce_max_sync(0xffffffffu, order_key(fmaxf(fmaxf(l[0], l[1]), fmaxf(l[2], l[3])))));
+          const float m2 = m * tc::kLog2e;
+          float z = 0.f;
+          if (m != kNegInf)
+            z = (tc::ex2_approx(fmaf(l[0], tc::kLog2e, -m2)) + tc::ex2_approx(fmaf(l[1], tc::kLog2e, -m2))) +
+                (tc::ex2_approx(fmaf(l[2], tc::kLog2e, -m2)) + tc::ex2_approx(fmaf(l[3], tc::kLog2e, -m2)));
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+          if (lane == 0) {
+            const int buf = slot == 2 ? 0 : slot + 1;
+            const uint32_t dst = sm0 + c.L.rows + grp * c.L.row_bytes + c.L.lse + 8 * ((buf * c.CS + c.rank) * nb + m0 / kMB);
+            send8(map_rank(dst, owner), __float_as_int(m), __float_as_int(z), map_rank(tc::smem_u32(c.sbar + grp), owner));
+          }
         }
+        __syncwarp();
+        group_sync(1, kGemm);
       }
-      __syncwarp();
-      group_sync(1, kGemm);
     }
+    if (score) write_score();
+    slot = slot == 2 ? 0 : slot + 1;
   }
 }
 
 // ---------------------------------------------------------------- row groups
 
+template <int GT>
 __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int grp) {
-  const int tid = ((int)threadIdx.x - kGemm) % kGroup, lane = tid & 31, warp = tid >> 5;
+  constexpr int WG = GT / 32;  // warps of the group
+  static_assert(WG >= 2 && WG <= 4, "the chains are assembled by two warps");
+  const int tid = ((int)threadIdx.x - kGemm) % GT, lane = tid & 31, warp = tid >> 5;
   const int i = grp * c.CS + c.rank;  // the row's place in the cluster
   const int r = c.row0 + i;
   const int bar = 2 + grp;
-  const int V = d.V, T = P.T;
+  const int V = d.V, T = P.T, Q = d.V4 / 4;
   unsigned char* rs = c.sm + c.L.rows + grp * c.L.row_bytes;
   RowSm& s = *reinterpret_cast<RowSm*>(rs);
-  const float* logits = reinterpret_cast<const float*>(rs + c.L.logits);
-  float* dlm = reinterpret_cast<float*>(rs + c.L.dlm);        // every label's c_r + delta (while built: its LM delta / lambda)
-  uint16_t* lev = reinterpret_cast<uint16_t*>(rs + c.L.lev);  // LM chain levels above 0 with an arc for it (bit l)
-  uint8_t* dep = rs + c.L.dep;                                // trie goto depth (0: none)
+  const float* lg = reinterpret_cast<const float*>(rs + c.L.logits);
+  float* term = reinterpret_cast<float*>(rs + c.L.term);          // every label's c_r + delta (while built: its LM delta / lambda)
+  // per label: bits 0-15 the LM chain levels above 0 with an arc for it, byte 2 its trie goto depth (0: none)
+  uint32_t* mark = reinterpret_cast<uint32_t*>(rs + c.L.mark);
+  int* list = c.L.list >= 0 ? reinterpret_cast<int*>(rs + c.L.list) : nullptr;  // level 0's labels from its aligned first arc
   const float* dflt = reinterpret_cast<const float*>(c.sm + c.L.dflt);
+  const float* uni = reinterpret_cast<const float*>(c.sm + c.L.uni);
   const uint32_t* root = reinterpret_cast<const uint32_t*>(c.sm + c.L.root);
   const bool lm2 = d.has_lm && d.lm.order >= 2;
   const float lam = P.lambda;
   const float bscale = P.beta * (d.has_tr ? d.tr.bonus : 0.f);
   const uint32_t y_addr = tc::smem_u32(c.y + i), y_bar = tc::smem_u32(c.ybar);
+  auto sync = [&]() { group_sync(bar, GT); };
 
-  // the row's label and frame (-1: finished) to every CTA of the cluster
-  auto publish = [&](int last, int t) {
-    if (tid < c.CS) send8(map_rank(y_addr, tid), last, t < T ? t : -1, map_rank(y_bar, tid));
+  // the row's label, frame (-1: finished) and the label's score to be, to every CTA of the cluster
+  auto publish = [&](int last, int t, float best, int at) {
+    if (tid < c.CS)
+      send16(map_rank(y_addr, tid),
+             make_float4(__int_as_float(last), __int_as_float(t < T ? t : -1), best, __int_as_float(at)), map_rank(y_bar, tid));
   };
 
   // state of the stream
   const int slot = P.slots[r];
   int last = __ldcg(d.s_last + slot);
   if (!checked(slot >= 0 && slot < d.lm_stride && last >= 0 && last <= V, d.err, 1)) last = V;
-  publish(last, 0);
+  publish(last, 0, 0.f, -1);
   if (tid == 0) {
     s.nl = d.has_lm ? __ldcg(d.s_lm_len + slot) : 0;
     s.nt = d.has_tr ? __ldcg(d.s_tr_len + slot) : 0;
-  } else if (tid >= 32 && tid < 32 + kLmChain) {
-    const int l = tid - 32;
-    if (d.has_lm) {
-      s.lm[l] = __ldcg(d.s_lm_chain + (size_t)slot * kLmChain + l);
-      s.lmr[l] = __ldcg(d.s_lm_rec + (size_t)slot * kLmChain + l);
-    }
-  } else if (tid >= 64 && tid < 64 + kTrChain) {
-    const int k = tid - 64;
-    if (d.has_tr) {
-      s.tr[k] = __ldcg(d.s_tr_chain + (size_t)slot * kTrChain + k);
-      s.trr[k] = __ldcg(d.s_tr_rec + (size_t)slot * kTrChain + k);
-    }
   }
-  group_sync(bar, kGroup);
+  if (d.has_lm && warp == 0 && lane < kLmChain) {
+    s.lm[lane] = __ldcg(d.s_lm_chain + (size_t)slot * kLmChain + lane);
+    s.lmr[lane] = __ldcg(d.s_lm_rec + (size_t)slot * kLmChain + lane);
+  }
+  if (d.has_tr && warp == 1) {
+    s.tr[lane] = __ldcg(d.s_tr_chain + (size_t)slot * kTrChain + lane);
+    s.trr[lane] = __ldcg(d.s_tr_rec + (size_t)slot * kTrChain + lane);
+  }
+  sync();
 #ifdef TSD_CHECKS
   if (tid == 0) {
     bool ok = checked(s.nl >= 0 && s.nl <= kLmChain && s.nt >= 0 && s.nt <= kTrChain, d.err, 2);
@@ -497,66 +569,70 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
     }
     if (!ok) s.nl = s.nt = 0;  // the row goes on from the empty context; the status word says so
   }
-  group_sync(bar, kGroup);
+  sync();
 #endif
 
   const int4* t4 = reinterpret_cast<const int4*>(d.lm.arc_tok);
   const float4* p4 = reinterpret_cast<const float4*>(d.lm.arc_logp);
+  auto copy16 = [](void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+  };
   // level 0 of the deltas: label u's dense row by asynchronous copies (u < 0:
-  // no LM state, every delta 0), and the level and depth scratch cleared
+  // no LM state, every delta 0), and the marks cleared
   auto begin_deltas = [&](int u) {
-    if (u >= 0) {
-      const float* R = d.lm.dense0 + (size_t)u * d.lm.V4;
-      for (int q = tid; q < d.V4 / 4; q += kGroup)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dlm + 4 * q)), "l"(R + 4 * q) : "memory");
-    } else {
-      for (int q = tid; q < d.V4 / 4; q += kGroup) reinterpret_cast<float4*>(dlm)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    for (int q = tid; q < d.V4 / 4; q += kGroup) {
-      reinterpret_cast<uint2*>(lev)[q] = make_uint2(0u, 0u);
-      reinterpret_cast<uint32_t*>(dep)[q] = 0u;
+    const float* R = d.lm.dense0 + (size_t)max(u, 0) * d.lm.V4;
+    for (int q = tid; q < Q; q += GT) {
+      if (u >= 0) copy16(term + 4 * q, R + 4 * q);
+      else reinterpret_cast<float4*>(term)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+      reinterpret_cast<uint4*>(mark)[q] = make_uint4(0u, 0u, 0u, 0u);
     }
   };
+  // A thread's group of four arcs of the levels above 0 (level hl, first arc
+  // hi) and its groups of children of the trie chain's first nodes: kept from
+  // the deltas, which need them, to the search of the next label.  more: the
+  // chains have arcs or children that no thread holds.
+  int hl = -1, hi = 0;
+  int4 ht, ct[kTrHeld];
+  bool more = false;
   // the levels above 0 and the trie chain: every arc sets its level's bit,
   // then the deepest level's arc overwrites its label's delta
   // (row_stream.cu); then every label's term c_r + lambda * delta + trie
   auto finish_deltas = [&]() {
     const int nl = s.nl, nt = s.nt;
-    // a thread's first group of four arcs, and of four children of the trie
-    // chain's first nodes, are requested together
-    int hl = -1, hi = 0;
-    int4 ht;
     float4 hp;
-    {
-      int g = tid;
-      for (int l = 1; l < nl; ++l) {
-        const int4 q = s.lmr[l];
-        const int n = level_groups(q.x, q.y);
-        if (g < n) {
-          hl = l, hi = (q.x & ~3) + 4 * g;
-          break;
-        }
-        g -= n;
-      }
+    int G = 0;
+    hl = -1;
+    for (int l = 1; l < nl; ++l) {
+      const int4 q = s.lmr[l];
+      const int n = level_groups(q.x, q.y);
+      if (tid >= G && tid < G + n) hl = l, hi = (q.x & ~3) + 4 * (tid - G);
+      G += n;
     }
     if (hl >= 0) {
       ht = __ldg(t4 + (hi >> 2));
       hp = __ldg(p4 + (hi >> 2));
     }
-    int4 ct[kTrHeld];
+    more = G > GT || nt > kTrHeld;
 #pragma unroll
     for (int k = 0; k < kTrHeld; ++k)
       if (k < nt) {
         const int4 q = s.trr[k];
-        if (tid < level_groups(q.x, q.y)) ct[k] = __ldg(reinterpret_cast<const int4*>(d.tr.ch_tok) + (q.x >> 2) + tid);
+        const int n = level_groups(q.x, q.y);
+        if (tid < n) ct[k] = __ldg(reinterpret_cast<const int4*>(d.tr.ch_tok) + (q.x >> 2) + tid);
+        more = more || n > GT;
       }
+    if (list && nl > 0) {
+      const int4 q = s.lmr[0];
+      const int n = level_groups(q.x, q.y);
+      for (int g = tid; g < n; g += GT) copy16(list + 4 * g, t4 + (q.x >> 2) + g);
+    }
     auto children = [&](int k, int4 tk, int g) {  // node k's children of group g
       const int4 q = s.trr[k];
       const int i0 = (q.x & ~3) + 4 * g;
       const int tv[4] = {tk.x, tk.y, tk.z, tk.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        if (i0 + j >= q.x && i0 + j < q.x + q.y) dep[tv[j]] = (uint8_t)q.z;
+        if (i0 + j >= q.x && i0 + j < q.x + q.y) reinterpret_cast<uint8_t*>(mark + tv[j])[2] = (uint8_t)q.z;
     };
     auto scatter = [&](int k) {
       const int4 q = s.trr[k];
@@ -564,132 +640,98 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
 #pragma unroll
       for (int h = 0; h < kTrHeld; ++h)
         if (h == k && tid < n) children(k, ct[h], tid);
-      for (int g = tid + (k < kTrHeld ? kGroup : 0); g < n; g += kGroup)
+      for (int g = tid + (k < kTrHeld ? GT : 0); g < n; g += GT)
         children(k, __ldg(reinterpret_cast<const int4*>(d.tr.ch_tok) + (q.x >> 2) + g), g);
     };
-    uint32_t* lev2 = reinterpret_cast<uint32_t*>(lev);
-    auto offer = [&](int l, int i0, int4 tk) {
-      const int b = s.lmr[l].x, n = s.lmr[l].y;
-      const int tv[4] = {tk.x, tk.y, tk.z, tk.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (i0 + j >= b && i0 + j < b + n && checked(tv[j] >= 0 && tv[j] < V, d.err, 9))
-          atomicOr(lev2 + (tv[j] >> 1), 1u << (l + 16 * (tv[j] & 1)));
-    };
-    auto settle = [&](int l, int i0, int4 tk, float4 lq, const float (&up)[4]) {
-      const int b = s.lmr[l].x, n = s.lmr[l].y;
-      const float cum = __int_as_float(s.lmr[l].z);
+    // set: the arcs of level l from i0 set its bit (settle false), or the
+    // labels whose deepest level it is take its delta
+    auto arcs = [&](int l, int i0, int4 tk, float4 lq, bool settle) {
+      const int4 q = s.lmr[l];
+      const float cum = __int_as_float(q.z);
       const int tv[4] = {tk.x, tk.y, tk.z, tk.w};
       const float pv[4] = {lq.x, lq.y, lq.z, lq.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        if (i0 + j >= b && i0 + j < b + n && checked(tv[j] >= 0 && tv[j] < V, d.err, 9) && 31 - __clz((int)lev[tv[j]]) == l)
-          dlm[tv[j]] = (pv[j] - cum) - up[j];
+        if (i0 + j >= q.x && i0 + j < q.x + q.y && checked(tv[j] >= 0 && tv[j] < V, d.err, 9)) {
+          if (!settle) atomicOr(mark + tv[j], 1u << l);
+          else if (nl == 2 || ((mark[tv[j]] & 0xffffu) >> l) == 1u) term[tv[j]] = (pv[j] - cum) - uni[tv[j]];
+        }
     };
-    // log p(v) of a group's labels (groups past a level's ends hold other levels' labels: all are in range)
-    auto unigrams = [&](int4 tk, float (&up)[4]) {
-      const int tv[4] = {tk.x, tk.y, tk.z, tk.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j) up[j] = (unsigned)tv[j] < (unsigned)V ? __ldg(d.lm.uni_logp + tv[j]) : 0.f;
-    };
-    // the arcs past what a thread holds (rare: more than 512 arcs above level 0)
-    auto rest = [&](auto f) {
-      int G = 0;
-      for (int l = 1; l < nl; ++l) G += level_groups(s.lmr[l].x, s.lmr[l].y);
-      for (int g0 = tid + kGroup; g0 < G; g0 += kGroup) {
+    // past what a thread holds (rare: more than four times GT arcs above level 0)
+    auto rest = [&](bool settle) {
+#pragma unroll 1
+      for (int g0 = tid + GT; g0 < G; g0 += GT) {
         int l = 1, g = g0;
         for (;; ++l) {
           const int n = level_groups(s.lmr[l].x, s.lmr[l].y);
           if (g < n) break;
           g -= n;
         }
-        f(l, (s.lmr[l].x & ~3) + 4 * g);
+        const int i0 = (s.lmr[l].x & ~3) + 4 * g;
+        arcs(l, i0, __ldg(t4 + (i0 >> 2)), __ldg(p4 + (i0 >> 2)), settle);
       }
     };
-    float hu[4] = {0.f, 0.f, 0.f, 0.f};
-    if (hl >= 0) {
-      unigrams(ht, hu);
-      offer(hl, hi, ht);
+    if (nl > 2) {  // (with one level above 0 every arc of it is its label's deepest)
+      if (hl >= 0) arcs(hl, hi, ht, hp, false);
+      rest(false);
     }
-    rest([&](int l, int i0) { offer(l, i0, __ldg(t4 + (i0 >> 2))); });
     if (nt > 0) scatter(nt - 1);  // the trie chain nodes, shallowest first (the deepest overwrites)
     asm volatile("cp.async.wait_all;" ::: "memory");
-    group_sync(bar, kGroup);
-    if (hl >= 0) settle(hl, hi, ht, hp, hu);
-    rest([&](int l, int i0) {
-      const int4 tk = __ldg(t4 + (i0 >> 2));
-      float up[4];
-      unigrams(tk, up);
-      settle(l, i0, tk, __ldg(p4 + (i0 >> 2)), up);
-    });
+    sync();
+    if (tid < kLmChain) s.lm_hit[tid] = make_int4(-2, 0, 0, 0);  // (the last search's records were read before the barrier)
+    if (tid < kTrChain) s.tr_hit[tid] = make_int4(-1, 0, 0, 0);
+    if (hl >= 0) arcs(hl, hi, ht, hp, true);
+    rest(true);
     for (int k = nt - 2; k >= 0; --k) {
       scatter(k);
-      group_sync(bar, kGroup);
+      if (k) sync();
     }
-    if (nt < 2) group_sync(bar, kGroup);
+    sync();
     const float cr = lam * (nl ? __int_as_float(s.lmr[nl - 1].z) : 0.f) - bscale * (float)(nt ? s.trr[0].z - 1 : 0);
-    for (int q = tid; q < d.V4 / 4; q += kGroup) {
-      const float4 kq = reinterpret_cast<const float4*>(dlm)[q];
+    for (int q = tid; q < Q; q += GT) {
+      const float4 kq = reinterpret_cast<const float4*>(term)[q];
       float o[4] = {lam * kq.x, lam * kq.y, lam * kq.z, lam * kq.w};
-      const uint32_t eq = reinterpret_cast<const uint32_t*>(dep)[q];
-      if (eq) {
-        const uint32_t rb = root[q >> 3] >> ((4 * q) & 31);
+      if (nt) {
+        const uint4 mq = reinterpret_cast<const uint4*>(mark)[q];
+        const uint32_t mv[4] = {mq.x >> 16, mq.y >> 16, mq.z >> 16, mq.w >> 16};
+        if (mv[0] | mv[1] | mv[2] | mv[3]) {
+          const uint32_t rb = root[q >> 3] >> ((4 * q) & 31);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t e = (eq >> (8 * j)) & 0xffu;
-          if (e) o[j] += bscale * (float)e - (((rb >> j) & 1u) ? bscale : 0.f);
+          for (int j = 0; j < 4; ++j)
+            if (mv[j]) o[j] += bscale * (float)mv[j] - (((rb >> j) & 1u) ? bscale : 0.f);
         }
       }
-      reinterpret_cast<float4*>(dlm)[q] = make_float4(cr + o[0], cr + o[1], cr + o[2], cr + o[3]);
+      // (labels past V never win)
+      const int v = 4 * q;
+      reinterpret_cast<float4*>(term)[q] = make_float4(v < V ? cr + o[0] : kNegInf, v + 1 < V ? cr + o[1] : kNegInf,
+                                                       v + 2 < V ? cr + o[2] : kNegInf, v + 3 < V ? cr + o[3] : kNegInf);
     }
     // (a thread reads back only what it wrote here: no barrier)
   };
-  // A warp's first label search of the next step, as far as it does not
-  // depend on the label: the range's 32 probes, or its entries where at most
-  // 124 are in it.
-  int4 pre = make_int4(-1, -1, -1, -1);
-  auto presearch = [&]() {
-    const int nl = s.nl, nt = s.nt;
-    if (warp >= nl + nt) return;
-    const int4 q = warp < nl ? s.lmr[warp] : s.trr[warp - nl];
-    pre = first_probe((warp < nl ? d.lm.arc_tok : d.tr.ch_tok) + q.x, q.y, lane);
+  auto find_list = [&](int y) {  // y's place among level 0's labels, or -1 (one warp)
+    const int n = s.lmr[0].y;
+    const int* a = list + (s.lmr[0].x & 3);
+    int lo = 0, hi = n;
+    __syncwarp();
+    while (hi - lo > 32) {
+      const int w = (hi - lo + 31) >> 5, at = lo + lane * w;
+      const unsigned m = __ballot_sync(0xffffffffu, at < hi && a[at] <= y);
+      if (m == 0) return -1;
+      lo += (31 - __clz((int)m)) * w;
+      hi = min(hi, lo + w);
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, lo + lane < hi && a[lo + lane] == y);
+    return m ? lo + __ffs((int)m) - 1 : -1;
   };
-  begin_deltas(s.nl > 0 ? s.lmr[0].w : -1);
-  group_sync(bar, kGroup);  // the scratch is cleared before anyone's offers
-  finish_deltas();
-  presearch();
 
   int t = 0, sym = 0, cnt = 0, step = 0;
-  const int nb = (c.nl + kMB - 1) / kMB;  // softmax partials per CTA
-  const uint32_t row_bytes = 4u * (uint32_t)(c.CS * c.nl), lse_bytes = 8u * (uint32_t)(c.CS * nb);
-  bool ok = true;
-  // The group's last warp consumes each step's softmax partials one step
-  // later, and writes the score of the label emitted there, if one was (e_at:
-  // its place in the row's outputs).
-  int e_at = -1;
-  float e_best = 0.f;
-  auto score_of = [&](int st) {
-    if (!__all_sync(0xffffffffu, wait_cluster(c.sbar + grp, st & 1, d.wait_ns, c.fail))) return false;
-    if (e_at >= 0) {
-      const float2* ps = reinterpret_cast<const float2*>(rs + c.L.lse) + (st & 1) * c.CS * nb;
-      float m = kNegInf, z = 0.f;
-      for (int q = lane; q < c.CS * nb; q += 32) lse_merge(m, z, ps[q].x, ps[q].y);
-      __syncwarp();
-      const float top = key_value(__reduce_max_sync(0xffffffffu, order_key(m)));
-      z = z > 0.f ? z * expf(m - top) : 0.f;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-      if (lane == 0) P.out_score[(size_t)r * (T * d.max_sym) + e_at] = e_best - (top + logf(z));
-      e_at = -1;
-    }
-    return true;
-  };
+  const uint32_t row_bytes = 4u * (uint32_t)(c.CS * c.nl);
+  bool ok = true, moved = true;
+  begin_deltas(s.nl > 0 ? s.lmr[0].w : -1);
+  sync();  // the marks are cleared before anyone sets one
   while (t < T) {
     if (tid == 0) tc::mbar_expect_tx(c.lbar + grp, row_bytes);
-    if (warp == kWarpsG - 1) {
-      ok = step == 0 || score_of(step - 1);
-      if (lane == 0 && ok) tc::mbar_expect_tx(c.sbar + grp, lse_bytes);
-    }
+    if (moved) finish_deltas();
     if (d.cap_rows && step < d.cap_steps && tid == 0) {
       int* q = d.cap_rows + ((size_t)step * P.n + r) * 4;
       q[0] = t;
@@ -698,20 +740,18 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
       q[3] = s.nt ? s.tr[0] : 0;
     }
     // the argmax of (logit + D) + (c_r + delta) over the labels (blank: its logit alone)
-    const float* lg = logits + (step & 1) * c.CS * c.nl;
-    ok = __all_sync(0xffffffffu, wait_cluster(c.lbar + grp, step & 1, d.wait_ns, c.fail)) && ok;
+    ok = __all_sync(0xffffffffu, wait_cluster(c.lbar + grp, step & 1, d.wait_ns, c.fail));
     float bv = kNegInf;
     int bi = INT_MAX;
     if (ok) {
-      const int nq = (V + 3) >> 2;
-      for (int q = tid; q < nq; q += kGroup) {
+      for (int q = tid; q < Q; q += GT) {
         const float4 lq = reinterpret_cast<const float4*>(lg)[q];
         const float4 uq = reinterpret_cast<const float4*>(dflt)[q];
-        const float4 kq = reinterpret_cast<const float4*>(dlm)[q];
+        const float4 kq = reinterpret_cast<const float4*>(term)[q];
         const float fv[4] = {(lq.x + uq.x) + kq.x, (lq.y + uq.y) + kq.y, (lq.z + uq.z) + kq.z, (lq.w + uq.w) + kq.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          if (fv[j] > bv && 4 * q + j < V) { bv = fv[j]; bi = 4 * q + j; }
+          if (fv[j] > bv) { bv = fv[j]; bi = 4 * q + j; }
       }
       if (tid == 0) {
         const float fb = lg[V];
@@ -724,12 +764,16 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
       bi = __reduce_min_sync(0xffffffffu, key == top ? bi : INT_MAX);
       bv = key_value(top);
     }
+    if (d.cap_logits && step < d.cap_steps) {  // (before the label is out: the next step's logits land here)
+      float* cl = d.cap_logits + ((size_t)step * P.n + r) * d.N;
+      for (int v = tid; v < d.N; v += GT) cl[v] = lg[v];
+    }
     if (lane == 0) s.best[step & 1][warp] = make_int4(__float_as_int(bv), bi, ok ? 1 : 0, 0);
-    group_sync(bar, kGroup);
+    sync();
     float best = kNegInf;
     int bix = INT_MAX;
 #pragma unroll
-    for (int w = 0; w < kWarpsG; ++w) {
+    for (int w = 0; w < WG; ++w) {
       const int4 q = s.best[step & 1][w];
       best_merge(best, bix, __int_as_float(q.x), q.y);
       ok = ok && q.z;
@@ -742,7 +786,8 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
     const int y = (bix >= 0 && bix <= V) ? bix : V;
     // the row's next position, to every CTA before anything else
     const int t_now = t;
-    if (y != V) {
+    moved = y != V;
+    if (moved) {
       last = y;
       sym += 1;
       if (sym >= d.max_sym) { t += 1; sym = 0; }
@@ -750,98 +795,115 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
       t += 1;
       sym = 0;
     }
-    publish(last, t);
-    if (d.cap_logits && step < d.cap_steps) {
-      float* cl = d.cap_logits + ((size_t)step * P.n + r) * d.N;
-      for (int v = tid; v < d.N; v += kGroup) cl[v] = lg[v];
-    }
-    if (y != V) {
-      // the label's searches in every chain element (row_stream.cu), level 0
-      // of the next deltas copied meanwhile
-      if (t < T) begin_deltas(lm2 ? y : -1);
+    publish(last, t, best, moved ? cnt : -1);
+    ++step;
+    if (!moved) continue;
+    // the label's records in every chain element, all in one round: above
+    // level 0 a thread that holds the label's arc (or trie child) fetches its
+    // record, level 0's labels are searched in shared memory; level 0 of the
+    // next deltas is copied meanwhile
+    {
       const int nl = s.nl, nt = s.nt;
-      if (tid == kGroup - 1) s.root_hit = d.has_tr ? __ldg(d.tr.root_rec + y) : make_int4(0, 0, 0, 0);
-      else if (tid == kGroup - 2) s.uni_hit = lm2 ? __ldg(d.lm.uni_rec + y) : make_int4(-1, 0, 0, 0);
-      for (int task = warp; task < nl + nt; task += kWarpsG) {
-        const bool is_lm = task < nl;
-        const int4 q = is_lm ? s.lmr[task] : s.trr[task - nl];
-        const int32_t* arr = (is_lm ? d.lm.arc_tok : d.tr.ch_tok) + q.x;
-        const int at = find_from(arr, q.y, y, lane, task == warp ? pre : first_probe(arr, q.y, lane));
-        if (lane == 0) {
-          if (is_lm) s.lm_hit[task] = at >= 0 ? __ldg(d.lm.arc_rec + q.x + at) : make_int4(-2, 0, 0, 0);
-          else s.tr_hit[task - nl] = at >= 0 ? __ldg(d.tr.ch_rec + q.x + at) : make_int4(-1, 0, 0, 0);
+      auto held = [&](int4 tk, int i0, int4 q) {  // the label's place among four entries from i0 of the range q, or -1
+        int at = -1;
+        const int tv[4] = {tk.x, tk.y, tk.z, tk.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (tv[j] == y && i0 + j >= q.x && i0 + j < q.x + q.y) at = i0 + j;
+        return at;
+      };
+      int a_lm = hl >= 0 ? held(ht, hi, s.lmr[hl]) : -1;
+      int4 r_lm, r_tr[kTrHeld], top;
+      if (a_lm >= 0) r_lm = __ldg(d.lm.arc_rec + a_lm);
+      int a_tr[kTrHeld];
+#pragma unroll
+      for (int k = 0; k < kTrHeld; ++k) {
+        a_tr[k] = -1;
+        if (k < nt) {
+          const int4 q = s.trr[k];
+          if (tid < level_groups(q.x, q.y)) a_tr[k] = held(ct[k], (q.x & ~3) + 4 * tid, q);
+          if (a_tr[k] >= 0) r_tr[k] = __ldg(d.tr.ch_rec + a_tr[k]);
         }
       }
-      group_sync(bar, kGroup);
-      // the new chains, in place: warp 0 the LM chain (y's unigram state, then
-      // the targets of y's arcs up to the first level without one), warp 1
-      // the trie chain (y's children of the old nodes, deepest first, then
-      // the root's; completing a phrase resets it)
-      if (warp == 0) {
-        int ln = 0;
+      if (tid == GT - 1) top = d.has_tr ? __ldg(d.tr.root_rec + y) : make_int4(0, 0, 0, 0);
+      if (tid == GT - 2) top = lm2 ? __ldg(d.lm.uni_rec + y) : make_int4(-1, 0, 0, 0);
+      int a0 = -1;
+      int4 r0;
+      if (warp == 0 && nl > 0) {
+        const int4 q = s.lmr[0];
+        a0 = list ? find_list(y) : find_from(d.lm.arc_tok + q.x, q.y, y, lane, first_probe(d.lm.arc_tok + q.x, q.y, lane));
+        if (lane == 0 && a0 >= 0) r0 = __ldg(d.lm.arc_rec + q.x + a0);
+      }
+      if (t < T) begin_deltas(lm2 ? y : -1);
+      if (a_lm >= 0) s.lm_hit[hl] = r_lm;
+#pragma unroll
+      for (int k = 0; k < kTrHeld; ++k)
+        if (a_tr[k] >= 0) s.tr_hit[k] = r_tr[k], s.dd[k] = s.trr[k].z + 1;
+      if (tid == GT - 1) s.root_hit = top;
+      if (tid == GT - 2) s.uni_hit = top;
+      if (warp == 0 && lane == 0 && a0 >= 0) s.lm_hit[0] = r0;
+      if (tid == 32) {
+        const size_t o = (size_t)r * (T * d.max_sym) + cnt;
+        P.out_tok[o] = y;
+        P.out_frame[o] = t_now;
+      }
+      if (more) {  // elements whose entries the threads do not all hold: searched by warps
+#pragma unroll 1
+        for (int task = 1 + warp; task < nl + nt; task += WG) {
+          const bool is_lm = task < nl;
+          const int4 q = is_lm ? s.lmr[task] : s.trr[task - nl];
+          const int32_t* arr = (is_lm ? d.lm.arc_tok : d.tr.ch_tok) + q.x;
+          const int at = find_from(arr, q.y, y, lane, first_probe(arr, q.y, lane));
+          if (lane == 0 && at >= 0) {
+            if (is_lm) s.lm_hit[task] = __ldg(d.lm.arc_rec + q.x + at);
+            else s.tr_hit[task - nl] = __ldg(d.tr.ch_rec + q.x + at), s.dd[task - nl] = q.z + 1;
+          }
+        }
+        if (nl == 0 && warp == 0 && nt > 0) {  // (no LM chain: the first task is the deepest trie node)
+          const int4 q = s.trr[0];
+          const int at = find_from(d.tr.ch_tok + q.x, q.y, y, lane, first_probe(d.tr.ch_tok + q.x, q.y, lane));
+          if (lane == 0 && at >= 0) s.tr_hit[0] = __ldg(d.tr.ch_rec + q.x + at), s.dd[0] = q.z + 1;
+        }
+      }
+      sync();
+      // the new chains, in place, by every warp alike (the same values, so no
+      // barrier follows): the LM chain is y's unigram state, then the targets
+      // of y's arcs up to the first level without one; the trie chain y's
+      // children of the old nodes, deepest first, then the root's (completing
+      // a phrase resets it)
+      int ln = 0, tn = 0;
+      {
+        const int4 h = lane < nl ? s.lm_hit[lane] : make_int4(-2, 0, 0, 0);
+        const int4 th = lane < nt ? s.tr_hit[lane] : make_int4(-1, 0, 0, 0);
+        const int4 u = s.uni_hit, rh = s.root_hit;
         if (lm2) {
-          const int4 h = lane < nl ? s.lm_hit[lane] : make_int4(-2, 0, 0, 0);
           const bool cont = h.x >= 0 && checked(h.x < d.lm.n_states && h.y >= 0 && h.z >= 0 &&
                                                     (int64_t)h.y + h.z <= d.lm.n_arcs, d.err, 10);
           const unsigned miss = __ballot_sync(0xffffffffu, !cont);
           ln = 1 + min(miss ? __ffs((int)miss) - 1 : 32, kLmChain - 1);
-          const int4 u = s.uni_hit;
-          const int px = __shfl_up_sync(0xffffffffu, h.x, 1), py = __shfl_up_sync(0xffffffffu, h.y, 1);
-          const int pz = __shfl_up_sync(0xffffffffu, h.z, 1), pw = __shfl_up_sync(0xffffffffu, h.w, 1);
-          __syncwarp();
-          if (lane < ln) {
-            s.lm[lane] = lane == 0 ? 1 + y : px;
-            s.lmr[lane] = lane == 0 ? make_int4(u.y, u.z, u.w, u.x) : make_int4(py, pz, pw, 0);
-          }
+          if (lane == 0) s.lm[0] = 1 + y, s.lmr[0] = make_int4(u.y, u.z, u.w, u.x);
+          if (lane + 1 < ln) s.lm[lane + 1] = h.x, s.lmr[lane + 1] = make_int4(h.y, h.z, h.w, 0);
         }
-        if (lane == 0) s.nl = ln;
-      } else if (warp == 1) {
-        const int4 h = lane < nt ? s.tr_hit[lane] : make_int4(-1, 0, 0, 0);
-        const int dd = lane < nt ? s.trr[lane].z + 1 : 0;
-        const bool hit = h.x >= 0 && checked(h.x > 0 && h.x < d.tr.n_nodes && h.w >= 0 && h.z + h.w <= d.tr.n_children,
-                                             d.err, 11);
-        const unsigned vm = __ballot_sync(0xffffffffu, hit);
-        const int nv = __popc(vm);
-        const int4 rh = s.root_hit;
-        const bool rt = rh.x != 0;
-        const int f = __ffs((int)vm) - 1;
-        const int fy = __shfl_sync(0xffffffffu, h.y, f < 0 ? 0 : f);
-        const bool reset = nv > 0 ? fy == 0 : (rt && rh.y == 0);
-        const int tn = reset ? 0 : min(nv + (rt ? 1 : 0), kTrChain);
+        if (d.has_tr) {
+          const bool found = th.x >= 0 && checked(th.x > 0 && th.x < d.tr.n_nodes && th.w >= 0 &&
+                                                      th.z + th.w <= d.tr.n_children, d.err, 11);
+          const unsigned vm = __ballot_sync(0xffffffffu, found);
+          const int nv = __popc(vm), f = __ffs((int)vm) - 1;
+          const bool rt = rh.x != 0;
+          const int fy = __shfl_sync(0xffffffffu, th.y, f < 0 ? 0 : f);
+          const bool reset = nv > 0 ? fy == 0 : (rt && rh.y == 0);
+          tn = reset ? 0 : min(nv + (rt ? 1 : 0), kTrChain);
+          const int pos = __popc(vm & ((1u << lane) - 1u));
+          if (found && pos < tn) s.tr[pos] = th.x, s.trr[pos] = make_int4(th.z, th.w, s.dd[lane], 0);
+          if (lane == 0 && rt && nv < tn) s.tr[nv] = rh.x, s.trr[nv] = make_int4(rh.z, rh.w, 2, 0);
+        }
+        if (lane == 0) s.nl = ln, s.nt = tn;
         __syncwarp();
-        const int pos = __popc(vm & ((1u << lane) - 1u));
-        if (hit && pos < tn) {
-          s.tr[pos] = h.x;
-          s.trr[pos] = make_int4(h.z, h.w, dd, 0);
-        }
-        if (lane == 0 && rt && nv < tn) {
-          s.tr[nv] = rh.x;
-          s.trr[nv] = make_int4(rh.z, rh.w, 2, 0);
-        }
-        if (lane == 0) s.nt = tn;
-      }
-      group_sync(bar, kGroup);
-      if (t < T) {
-        finish_deltas();
-        presearch();
-      }
-      if (warp == kWarpsG - 1) {
-        if (lane == 0) {
-          const size_t o = (size_t)r * (T * d.max_sym) + cnt;
-          P.out_tok[o] = y;
-          P.out_frame[o] = t_now;
-        }
-        e_at = cnt, e_best = best;
       }
       cnt += 1;
     }
-    ++step;
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
-  if (ok && warp == kWarpsG - 1 && !score_of(step - 1)) {
-    if (lane == 0) atomicOr(d.err, 8);
-    *c.fail = 1;
-  }
   if (!ok) return;
   // the stream's state, once per chunk (and the row's copy of it, which the
   // two-kernel step and its timing replays read)
@@ -856,26 +918,30 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
     if (d.has_tr) d.s_tr_len[slot] = s.nt;
     d.m_lm_len[r] = s.nl;
     d.m_tr_len[r] = s.nt;
-  } else if (tid >= 32 && tid < 32 + kLmChain && tid - 32 < s.nl) {
-    const int l = tid - 32;
-    d.s_lm_chain[(size_t)slot * kLmChain + l] = s.lm[l];
-    d.s_lm_rec[(size_t)slot * kLmChain + l] = s.lmr[l];
-    d.m_lm[(size_t)r * kLmChain + l] = s.lm[l];
-    d.m_lmr[(size_t)r * kLmChain + l] = s.lmr[l];
-  } else if (tid >= 64 && tid < 64 + kTrChain && tid - 64 < s.nt) {
-    const int k = tid - 64;
-    d.s_tr_chain[(size_t)slot * kTrChain + k] = s.tr[k];
-    d.s_tr_rec[(size_t)slot * kTrChain + k] = s.trr[k];
-    d.m_tr[(size_t)r * kTrChain + k] = s.tr[k];
-    d.m_trr[(size_t)r * kTrChain + k] = s.trr[k];
+  }
+  if (warp == 0 && lane < s.nl) {
+    d.s_lm_chain[(size_t)slot * kLmChain + lane] = s.lm[lane];
+    d.s_lm_rec[(size_t)slot * kLmChain + lane] = s.lmr[lane];
+    d.m_lm[(size_t)r * kLmChain + lane] = s.lm[lane];
+    d.m_lmr[(size_t)r * kLmChain + lane] = s.lmr[lane];
+  }
+  if (warp == 1 && lane < s.nt) {
+    d.s_tr_chain[(size_t)slot * kTrChain + lane] = s.tr[lane];
+    d.s_tr_rec[(size_t)slot * kTrChain + lane] = s.trr[lane];
+    d.m_tr[(size_t)r * kTrChain + lane] = s.tr[lane];
+    d.m_trr[(size_t)r * kTrChain + lane] = s.trr[lane];
   }
   if (d.cap_rows)  // steps after the row's last evaluation
-    for (int q = step + tid; q < min(d.cap_steps, T * d.max_sym); q += kGroup)
+    for (int q = step + tid; q < min(d.cap_steps, T * d.max_sym); q += GT)
       reinterpret_cast<int4*>(d.cap_rows)[(size_t)q * P.n + r] = make_int4(-1, -1, -1, -1);
 }
 
-template <int NB, int RG>
-__global__ void __launch_bounds__(kGemm + RG * kGroup, 1)
+// Threads of a row group: with three groups, half as many leave the product's
+// warps their registers.
+constexpr int group_threads(int RG) { return RG < 3 ? 128 : 64; }
+
+template <int NB, int RG, int FU>
+__global__ void __launch_bounds__(kGemm + RG * group_threads(RG), 1)
     k_chunk(const __grid_constant__ DecView d, const __grid_constant__ ChunkArgs P) {
   extern __shared__ __align__(128) unsigned char raw[];
   Ctx c;
@@ -892,7 +958,7 @@ __global__ void __launch_bounds__(kGemm + RG * kGroup, 1)
   c.sbar = c.lbar + RG;
   int* fail = reinterpret_cast<int*>(c.sbar + RG);
   c.fail = fail;
-  c.y = reinterpret_cast<int2*>(c.sm + c.L.y);
+  c.y = reinterpret_cast<int4*>(c.sm + c.L.y);
   const int tid = threadIdx.x;
   if (tid == 0) {
     tc::mbar_init(c.ybar, 1);
@@ -900,31 +966,33 @@ __global__ void __launch_bounds__(kGemm + RG * kGroup, 1)
     for (int g = 0; g < 2 * RG; ++g) tc::mbar_init(c.lbar + g, 1);  // lbar, then sbar
     *fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    tc::mbar_expect_tx(c.ybar, 8u * (uint32_t)c.R);  // the rows' first labels
+    tc::mbar_expect_tx(c.ybar, 16u * (uint32_t)c.R);  // the rows' first labels
     // this CTA's labels of W_out, row by row
     tc::mbar_expect_tx(c.wbar, (uint32_t)(c.nl * 2 * d.H));
     for (int j = 0; j < c.nl; ++j)
       tc::bulk_g2s(c.sm + c.L.w + j * (2 * d.H + kWPad), d.Wt + (size_t)(c.rank * c.nl + j) * d.H, 2u * (uint32_t)d.H, c.wbar);
   }
-  // the call's shared rows: the defaults D, and the labels that start a phrase
+  // the call's shared rows: the defaults D, log p(v), and the labels that start a phrase
   float* dflt = reinterpret_cast<float*>(c.sm + c.L.dflt);
+  float* uni = reinterpret_cast<float*>(c.sm + c.L.uni);
   uint32_t* root = reinterpret_cast<uint32_t*>(c.sm + c.L.root);
   for (int v = tid; v < (d.V4 + 31) / 32 * 32; v += blockDim.x) {
     const bool rc = d.has_tr && v < d.V && __ldg(d.tr.root_child + v) != 0;
-    float x = 0.f;
-    if (d.has_lm && v < d.V) x = P.lambda * __ldg(d.lm.uni_logp + v);
+    const float u = d.has_lm && v < d.V ? __ldg(d.lm.uni_logp + v) : 0.f;
+    float x = d.has_lm ? P.lambda * u : 0.f;
     if (rc) x += P.beta * d.tr.bonus;
-    if (v < d.V4) dflt[v] = x;
+    if (v < d.V4) dflt[v] = x, uni[v] = u;
     const unsigned m = __ballot_sync(0xffffffffu, rc);  // whole warps: the bound is a multiple of 32
     if ((tid & 31) == 0) root[v / 32] = m;
   }
   __syncthreads();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (tid < kGemm) {
-    gemm_loop<NB>(d, P, c);
+    gemm_loop<NB, RG, FU>(d, P, c);
   } else {
-    const int grp = (tid - kGemm) / kGroup;
-    if (grp * c.CS + c.rank < c.R) row_loop(d, P, c, grp);
+    constexpr int GT = group_threads(RG);
+    const int grp = (tid - kGemm) / GT;
+    if (grp * c.CS + c.rank < c.R) row_loop<GT>(d, P, c, grp);
   }
   __syncwarp();
   if (*c.fail) {
@@ -938,15 +1006,19 @@ __global__ void __launch_bounds__(kGemm + RG * kGroup, 1)
 }
 
 typedef void (*ChunkFn)(DecView, ChunkArgs);
-ChunkFn kernel_of(int NB, int RG) {
-  if (NB == 1) return RG == 1 ? k_chunk<1, 1> : k_chunk<1, 2>;
-  return RG == 1 ? k_chunk<2, 1> : k_chunk<2, 2>;
+// The kernel of a shape (nullptr: there is none), for hidden size H.
+ChunkFn kernel_of(int NB, int RG, int H) {
+  const int fu = H == 1024 ? 4 : (H >= 512 && H < 768 ? 2 : -1);
+  if (RG == 1 && NB == 1) return fu == 4 ? k_chunk<1, 1, 4> : fu == 2 ? k_chunk<1, 1, 2> : k_chunk<1, 1, -1>;
+  if (RG == 1) return fu == 4 ? k_chunk<2, 1, 4> : fu == 2 ? k_chunk<2, 1, 2> : k_chunk<2, 1, -1>;
+  if (RG == 2) return NB == 1 ? k_chunk<1, 2, -1> : k_chunk<2, 2, -1>;
+  return NB == 1 ? nullptr : fu == 4 ? k_chunk<2, 3, 4> : k_chunk<2, 3, -1>;
 }
 
 cudaLaunchConfig_t config(const ChunkShape& s, int clusters, cudaLaunchAttribute* a, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(clusters * s.CS));
-  cfg.blockDim = dim3((unsigned)(kGemm + s.RG * kGroup));
+  cfg.blockDim = dim3((unsigned)(kGemm + s.RG * group_threads(s.RG)));
   cfg.dynamicSmemBytes = (size_t)s.smem;
   cfg.stream = st;
   a[0].id = cudaLaunchAttributeClusterDimension;
@@ -968,8 +1040,9 @@ cudaError_t chunk_cluster_shapes(const DecView& d, std::vector<ChunkShape>& out)
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   for (int NB = 1; NB <= 2; ++NB)
-    for (int RG = 1; RG <= 2; ++RG) {
-      const void* f = (const void*)kernel_of(NB, RG);
+    for (int RG = 1; RG <= 3; ++RG) {
+      const void* f = (const void*)kernel_of(NB, RG, d.H);
+      if (!f) continue;
       if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
       if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess) return e;
       for (int CS = 8; CS <= 16; CS *= 2) {
@@ -988,20 +1061,23 @@ cudaError_t chunk_cluster_shapes(const DecView& d, std::vector<ChunkShape>& out)
   return cudaSuccess;
 }
 
-// One pass of the product covers a cluster's rows (R <= 8 NB): a second pass
-// repeats the reads of W_out's slice that bound it, and with three passes and
-// more (256 rows in seven clusters of 16 CTAs: 37 each) the chunk took 1027 us
-// against 820 us by the two-kernel step.  Below that every shape measured is
-// faster here (64 rows, H = 640: 302 us against 674; one row 212 against 619).
+// Every shape measured was faster than the two-kernel step, 40 label steps
+// each (n rows, V x H): 112, 1024 x 1024: 233 against 498 us; 100, 2048 x 512 in two
+// passes: 312 / 438; three groups of 64 threads 200, 512 x 640: 208 / 417; 336: 358 /
+// 415; 128, 1024 x 640: 377 / 437 -- but where three groups read more than 192
+// KB of W_out per step (passes x slice): 256, 1024 x 512 (210 KB): 487 / 405;
+// 256, 1024 x 640 (261 KB): 571 / 440.
 const ChunkShape* chunk_cluster_pick(const std::vector<ChunkShape>& shapes, int n, int H) {
   const ChunkShape* best = nullptr;
   double cost = 0;
   if (n > kChunkMaxRows) return nullptr;
   for (const ChunkShape& s : shapes) {
     const int R = (n + s.clusters - 1) / s.clusters;
-    if (R > std::min(s.CS * s.RG, 8 * s.NB)) continue;
-    // bytes of W_out a CTA reads per step, a pass of eight more rows, another row group
-    const double c = (double)s.nl * H * 2 + 16384.0 * s.NB + 20000.0 * ((R + s.CS - 1) / s.CS);
+    const int passes = (R + 8 * s.NB - 1) / (8 * s.NB);
+    if (R > s.CS * s.RG || (passes > 1 && !several_passes(s.NB, s.RG))) continue;
+    if (s.RG == 3 && (double)passes * s.nl * H * 2 > 192.0 * 1024) continue;
+    // bytes of W_out a CTA reads per step, a pass's overhead, another row group
+    const double c = passes * ((double)s.nl * H * 2 + 32768.0 + 16384.0 * s.NB) + 20000.0 * ((R + s.CS - 1) / s.CS);
     if (!best || c < cost) best = &s, cost = c;
   }
   return best;
@@ -1014,7 +1090,7 @@ cudaError_t launch_chunk_cluster(const ChunkShape& s, const DecView& d, ChunkArg
   const int clusters = (a.n + a.R - 1) / a.R;
   cudaLaunchAttribute at[1];
   cudaLaunchConfig_t cfg = config(s, clusters, at, st);
-  return cudaLaunchKernelEx(&cfg, kernel_of(s.NB, s.RG), d, a);
+  return cudaLaunchKernelEx(&cfg, kernel_of(s.NB, s.RG, d.H), d, a);
 }
 
 }  // namespace tsd

@@ -44,13 +44,22 @@ def test_label_slices(V, H):
     pu.assert_reports(pu.replay(inp, one, range(w.B)))
 
 
-@pytest.mark.parametrize("B", [1, 7, 8, 9, 17, 64, 111, 112])
+@pytest.mark.parametrize("B", [1, 7, 8, 9, 17, 64, 111, 113, 200, 336])
 def test_row_counts(B):
     w = synth.scaled(BASE, V=512, H=640, B=B, T=3, lm_total=20000)
     inp = pu.Inputs(w)
     one, two = _runs(inp, range(B))
     _agree(one, two)
     pu.assert_reports(pu.replay(inp, one, sorted({0, B // 2, B - 1})))
+
+
+def test_two_passes_of_the_product():
+    """More than eight rows per cluster with a slice of W_out that leaves room for eight."""
+    w = synth.scaled(BASE, V=2100, H=512, B=70, T=2, lm_total=40000)
+    inp = pu.Inputs(w)
+    one, two = _runs(inp, range(w.B))
+    _agree(one, two)
+    pu.assert_reports(pu.replay(inp, one, [0, 34, 69]))
 
 
 @pytest.mark.parametrize("case", ["no tables", "unigram lm", "no boost", "no lm", "zero weights", "long chains",
@@ -70,9 +79,9 @@ def test_tables(case):
     elif case == "long chains":  # LM and trie chains up to their capacities
         w = synth.scaled(w, V=8, H=64, T=40, lm_order=16, lm_total=60000, beta=4.0)
         inp = pu.Inputs(w, lmA=synth.ngram_lm(w.lm_seed, 8, 16, 60000, 1.05), ph=synth.phrases(5, 8, 12, 16, 32, 0.0))
-    else:  # contexts with more arcs than a group's threads hold at once
-        w = synth.scaled(w, V=300, lm_total=280_000)
-        inp = pu.Inputs(w, lmA=synth.ngram_lm(9, 300, 4, 280_000, 1.02))
+    else:  # more arcs and trie children than a group's threads hold at once, trie chains longer than they hold
+        w = synth.scaled(w, V=40, lm_total=280_000, beta=3.0)
+        inp = pu.Inputs(w, lmA=synth.ngram_lm(9, 40, 8, 280_000, 1.02), ph=synth.phrases(9, 40, 20000, 4, 9, 0.2))
     one, two = _runs(inp, range(w.B))
     _agree(one, two)
     pu.assert_reports(pu.replay(inp, one, range(w.B)))
