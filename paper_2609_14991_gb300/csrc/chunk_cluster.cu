@@ -55,8 +55,10 @@ namespace {
 
 using row::best_merge;
 using row::checked;
+using row::key_value;
 using row::kNegInf;
 using row::lse_merge;
+using row::order_key;
 
 constexpr int kGemm = 256;     // GEMM threads (8 warps, each an eighth of H)
 constexpr int kTiles = 5;      // 16-label tiles per accumulator block
@@ -150,14 +152,6 @@ __device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1
                : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-
-// A float as an integer of the same order (and back); -0 counts as below +0, so
-// a value that may be -0 has 0 added first.
-__device__ __forceinline__ int order_key(float v) {
-  const int i = __float_as_int(v);
-  return i ^ ((i >> 31) & 0x7fffffff);
-}
-__device__ __forceinline__ float key_value(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7fffffff)); }
 
 // bf16(ReLU(x + z)) of eight elements.  The bf16 add rounds the exact sum
 // once; rounding it to fp32 first, as the row passes do, gives the same: the

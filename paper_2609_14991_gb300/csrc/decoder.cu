@@ -259,7 +259,7 @@ tsd_status create_impl(const tsd_decoder_cfg* cfg, const void* W_out_bf16, const
   }
   if (c.beam_k > 1) {
     const size_t pool = (size_t)c.max_streams * kPoolCap;
-    if ((st = A.alloc(&bpart, (size_t)d->M_pad * (d->N_pad / 64) * (1 + c.beam_k))) || (st = A.alloc(&hscore, SK)) ||
+    if ((st = A.alloc(&v.logits, (size_t)d->M_pad * d->N_pad)) || (st = A.alloc(&v.dvec, (size_t)d->N_pad)) || (st = A.alloc(&hscore, SK)) ||
         (st = A.alloc(&hlive, SK)) || (st = A.alloc(&hnode, SK)) || (st = A.alloc(&hlen, SK)) ||
         (st = A.alloc(&hhash, SK)) || (st = A.alloc(&ppar, pool)) || (st = A.alloc(&ptok, pool)) ||
         (st = A.alloc(&pn, (size_t)c.max_streams)) || (st = A.alloc(&v.f_score, SK)) ||
@@ -271,10 +271,13 @@ tsd_status create_impl(const tsd_decoder_cfg* cfg, const void* W_out_bf16, const
       A.release();
       return st;
     }
+    // the joint kernel adds no defaults to a beam's logits: the bias row holds all of Eq. 1's terms
+    TSD_CUDA(cudaMemsetAsync(v.dvec, 0, sizeof(float) * (size_t)d->N_pad, s));
+    TSD_CUDA(cudaMemsetAsync(v.logits, 0, sizeof(float) * (size_t)d->M_pad * d->N_pad, s));
     TSD_CUDA(cudaMemsetAsync(v.f_live, 0, SK * sizeof(int32_t), s));
     TSD_CUDA(cudaMemsetAsync(v.b_frame, 0, (size_t)c.max_streams * sizeof(int32_t), s));
     TSD_CUDA(cudaMemsetAsync(v.b_exp, 0, (size_t)c.max_streams * sizeof(int32_t), s));
-    if (!bpart || !hscore || !hlive || !hnode || !hlen || !hhash || !ppar || !ptok || !pn) {
+    if (!hscore || !hlive || !hnode || !hlen || !hhash || !ppar || !ptok || !pn) {
       A.release();
       return fail(TSD_ENOMEM, "tsd_decoder_create: beam state not allocated");
     }

@@ -66,7 +66,7 @@ struct DecView {
   int32_t* cap_rows;
   int32_t cap_steps;
   // beam search (K > 1), per slot x K hypotheses
-  float2* bpart;        // [M_pad][n_ptiles][1 + K]: (max, sum exp), then top-K (value, label)
+  float2* bpart;        // pruned fusion: [M_pad][n_ptiles][1 + topk]: (max, sum exp), then the top (logit, label)s
   double* h_score;      // hypothesis score
   int32_t* h_live;      // 1 if the hypothesis slot holds a live hypothesis
   int32_t* h_node;      // label-sequence node (-1 = empty sequence)
@@ -86,7 +86,7 @@ struct DecView {
   unsigned long long* f_hash;
   int32_t* b_frame;     // [slots] frame of the chunk the beam is in (T: done)
   int32_t* b_exp;       // [slots] expansions taken in that frame
-  int32_t topk;       // entries per row and tile in bpart: beam width, or prune_k
+  int32_t topk;       // candidates per row: beam width, or prune_k
   int32_t prune;      // prune_k (0: fusion over every label)
   int32_t n_lm;       // n-gram LMs fused (0: none; several: greedy only)
   int32_t sms;        // SMs of the device (launch shapes)
@@ -109,7 +109,7 @@ struct DecView {
   // adds the row's LM and trie terms before it takes the argmax.
   int32_t fused;
   int32_t fz_dense;     // 1: the dense epilogue with the correction list; 0: streaming
-  float* logits;        // [M_pad][N_pad] fp32: the listed labels' raw logits (dense) or every label's logit + dvec
+  float* logits;        // [M_pad][N_pad] fp32: the listed labels' raw logits (dense) or every label's logit + dvec (also beam search)
   float* dvec;          // [N_pad] per call: lambda*log p(v) + beta*bonus*[the root has a child v]; 0 from V on
   int32_t* c_lab;       // [M_pad][V4] the row's listed labels
   float* c_add;         // [M_pad][V4] their term: F[v] = logit[v] + c_add

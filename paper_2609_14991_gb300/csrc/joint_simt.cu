@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(256) k_joint_simt(DecView d, int step) {
     const uint32_t* mrow = nullptr;
     const float lam = d.params->lambda;
     const bool dense = d.fused && d.fz_dense;
+    const bool stream = (d.fused && !dense) || d.K > 1;
     if (dense) {
       const int u = __ldcg(&d.c_info[gr].x);
       if (u >= 0 && u < d.lm.n_dense) urow = d.lm.dense0 + (size_t)u * d.V4;
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(256) k_joint_simt(DecView d, int step) {
       if (gc < N) {
         mx = fmaxf(mx, l[q]);
         float f;
-        if (d.fused && !dense) {
+        if (stream) {
           f = l[q];  // the streaming form: the row pass takes the argmax
         } else if (dense) {
           if ((__ldcg(mrow + (gc >> 5)) >> (gc & 31)) & 1u) {  // listed: the row pass evaluates it
@@ -147,7 +148,7 @@ __global__ void __launch_bounds__(256) k_joint_simt(DecView d, int step) {
     for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
     if (lane == 0)
       d.part[(size_t)gr * d.n_ptiles + blockIdx.x] = make_float4(mx, se, bv, __int_as_float(bi));
-    if (d.fused && !dense) {  // the streaming form: logit + D of every label
+    if (stream) {  // the streaming form: logit + D of every label
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int gc = n0 + lane * 4 + q;

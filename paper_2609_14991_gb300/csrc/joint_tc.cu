@@ -10,8 +10,8 @@
 // 32-column chunks) and reduce it on chip to the row's selection partial for
 // this tile: softmax max and sum over the real labels, and the best fused
 // value logit + bias (the dense fusion bias row of several LMs), ties to the
-// lowest label, or (BEAM) the tile's top K.  Greedy decoding with at most one
-// LM runs joint_greedy.cu instead.  Logits never leave the SM.
+// lowest label, or (pruned fusion) the tile's top K.  Greedy decoding with at
+// most one LM and beam search run joint_greedy.cu instead.  Logits never leave the SM.
 //
 // Warp roles (320 threads): warp 0 TMA producer, warp 1 TMEM allocator and
 // MMA issuer, warps 2-9 epilogue.  Every wait on an mbarrier is bounded in
@@ -61,11 +61,10 @@ __device__ __forceinline__ float sum_exp2_32(const float* l, float s2) {
   return (a[0] + a[1]) + (a[2] + a[3]);
 }
 
-// BEAM: instead of the single best fused label, each row keeps the top-K
-// (K = d.topk <= 8: the beam width, or the pruned-fusion candidate count)
-// values of the tile, ties to the lower label.  With pruned fusion (d.prune)
-// the values are the plain logits: no bias tile is loaded.
-template <int BN, bool BEAM>
+// TOPK (pruned fusion): instead of the single best fused label, each row
+// keeps the top K (K = d.topk <= 8, the candidate count) logits of the tile,
+// ties to the lower label; no bias tile is loaded.
+template <int BN, bool TOPK>
 __global__ void __launch_bounds__(kThreads, 1)
     k_joint_tc(DecView d, int step, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmBias) {
@@ -81,7 +80,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n0 = blockIdx.x * BN, m0 = blockIdx.y * kBM;
-  const bool use_bias = !(BEAM && d.prune);
+  constexpr bool use_bias = !TOPK;
   const int M = d.params->n * d.K;
   const int KB = d.H / kBK;
 
@@ -254,7 +253,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int i = 0; i < w; ++i) { t[i] = fmaxf(t[i], t[i + w]); u[i] = fmaxf(u[i], u[i + w]); }
         const float cm = t[0], fm = u[0];
-        if (!BEAM) {
+        if (!TOPK) {
           // the first label of the chunk holding the chunk's best fused value
           if (fm > bv) {
             int j = 31;
@@ -336,7 +335,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (ok) {
         xch[0] = mx;
         xch[1] = se;
-        if (!BEAM) {
+        if (!TOPK) {
           xch[2] = bv;
           xch[3] = __int_as_float(bi);
         } else {
@@ -357,7 +356,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           mx = m2;
         }
       }
-      if (!BEAM) {
+      if (!TOPK) {
         const float v1 = xch[2];
         const int i1 = __float_as_int(xch[3]);
         if (v1 > bv || (v1 == bv && i1 < bi)) { bv = v1; bi = i1; }
@@ -440,15 +439,14 @@ cudaError_t joint_tc_prepare(JointTc* jt, const uint16_t* A, int M_pad, const ui
 namespace {
 template <int BN>
 void launch_bn(cudaLaunchConfig_t& cfg, const JointTc& jt, const DecView& d, int step) {
-  const bool beam = d.topk > 1 || d.prune > 0;  // the top-K epilogue
   cfg.dynamicSmemBytes = Smem<BN>::kBytes;
-  if (beam) cudaLaunchKernelEx(&cfg, k_joint_tc<BN, true>, d, step, jt.mapA, jt.mapB, jt.mapBias);
+  if (d.prune > 0) cudaLaunchKernelEx(&cfg, k_joint_tc<BN, true>, d, step, jt.mapA, jt.mapB, jt.mapBias);
   else cudaLaunchKernelEx(&cfg, k_joint_tc<BN, false>, d, step, jt.mapA, jt.mapB, jt.mapBias);
 }
 }  // namespace
 
 void launch_joint_tc(const JointTc& jt, const DecView& d, int M, int step, cudaStream_t s, bool pdl) {
-  if (d.fused) {
+  if (d.fused || d.K > 1) {
     launch_joint_greedy(jt, d, M, step, s, pdl);
     return;
   }

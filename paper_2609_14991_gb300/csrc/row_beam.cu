@@ -1,15 +1,16 @@
 // Beam-search row pass: one cluster of K CTAs per stream, K hypotheses per
-// stream.  The cluster's first CTA does steps 1-5; then every CTA k of the
-// cluster builds step 6 for beam member k, reading its chains from the
-// first CTA's shared memory.
+// stream.  CTA k of the cluster does step 1 for hypothesis k and leaves its
+// candidates in the first CTA's shared memory; the first CTA does steps 2-5;
+// then every CTA k builds step 6 for beam member k, reading its chains from
+// the first CTA's shared memory.
 //
 // The search is frame-synchronous with at most S = max_symbols labels per
 // frame: each label step is one expansion of the hypotheses still in their
-// frame (set A).  At a step the first CTA
-//   1. turns the joint kernel's per-tile partials into each hypothesis of A's
-//      log-sum-exp and its K best extensions (blank keeps the labels, label v
-//      appends v), scored hypothesis score + fused value - log-sum-exp (Eq. 1
-//      summed along the hypothesis);
+// frame (set A).  A step
+//   1. turns the joint kernel's logits and per-tile softmax partials into each
+//      hypothesis of A's log-sum-exp and its K best extensions (blank keeps
+//      the labels, label v appends v), scored hypothesis score + fused value -
+//      log-sum-exp (Eq. 1 summed along the hypothesis);
 //   2. keeps the top K of those candidates by (score desc, hypothesis asc,
 //      label asc) and sends each, in that order, to the frame-exit set F
 //      (the blank, or a label at the frame's S-th expansion) or to the next A,
@@ -39,7 +40,6 @@ using row::lse_merge;
 using row::warp_find;
 
 constexpr int kMaxK = 8;
-constexpr int kCandPerLane = 16;  // per-hypothesis candidates: n_tiles * K <= 512
 
 __device__ __forceinline__ unsigned long long hash_push(unsigned long long h, int v) {
   return h * 0x100000001B3ull + (unsigned long long)(v + 1);
@@ -70,7 +70,7 @@ __device__ bool seq_equal(const int32_t* par, const int32_t* tok, int a, int ea,
 
 __device__ __forceinline__ double log_add(double a, double b) {
   const double m = fmax(a, b);
-  return m + log(exp(a - m) + exp(b - m));
+  return m + log(1.0 + exp(fmin(a, b) - m));  // (the larger one's exponential is 1)
 }
 
 // candidate order: score desc, hypothesis asc, label asc
@@ -107,7 +107,6 @@ __global__ void __launch_bounds__(kRowThreads) k_row_beam(DecView d, int step, i
   __shared__ double n_score[kMaxK];
   __shared__ unsigned long long n_hash[kMaxK];
   __shared__ int n_lm[kMaxK][kLmChain], n_tr[kMaxK][kTrChain];
-  __shared__ double c_score[kMaxK * kMaxK];
   __shared__ float c_inc[kMaxK * kMaxK];
   __shared__ int c_tok[kMaxK * kMaxK];
   __shared__ int s_sel[kMaxK], s_into[kMaxK];
@@ -132,10 +131,15 @@ __global__ void __launch_bounds__(kRowThreads) k_row_beam(DecView d, int step, i
   __shared__ int f_cnt, f_src[kMaxK];  // F after this step: entry (>= 0 new record j, <= -2 loaded entry -2-j)
   __shared__ int q_src[2 * kMaxK];     // F before pruning, in insertion order
   __shared__ double q_score[2 * kMaxK];
-  __shared__ int s_bt, s_be, s_done;
+  __shared__ int s_bt, s_be, s_done, s_pool;
+  __shared__ float2 s_top[kRowThreads / 32 * kMaxK];  // the warps' bests (value, label)
+  __shared__ int s_rank[kMaxK * kMaxK];               // candidates that come before one
+  __shared__ float s_lse;
 
   __shared__ int m_cnt, m_lml, m_trl, m_last, m_frame;  // member crank, copied from the first CTA
   __shared__ int m_lm[kLmChain], m_tr[kTrChain];
+  // (the first CTA runs before the others write to its shared memory)
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   if (crank == 0) {
   // previous state of this stream's hypotheses (written by the previous row
   // pass; L2-only loads, see the greedy pass)
@@ -160,12 +164,14 @@ __global__ void __launch_bounds__(kRowThreads) k_row_beam(DecView d, int step, i
     o_lml[tid] = d.has_lm ? __ldcg(d.s_lm_len + h) : 0;
     o_trl[tid] = d.has_tr ? __ldcg(d.s_tr_len + h) : 0;
   }
+  if (tid < kMaxK * kMaxK) s_rank[tid] = 0;
   if (tid == K) {
     // frame and expansion of this stream (reset at the chunk's first step;
     // a replay redoes one expansion of the final beam)
     s_bt = (step == 0 || mode == 2) ? 0 : __ldcg(d.b_frame + slot);
     s_be = (step == 0 || mode == 2) ? 0 : __ldcg(d.b_exp + slot);
     s_done = (step > 0 && mode != 2 && s_bt >= T) ? 1 : 0;
+    s_pool = __ldcg(d.pool_n + slot);
     e_cnt = 0;
   }
   row::block_sync();
@@ -205,171 +211,215 @@ __global__ void __launch_bounds__(kRowThreads) k_row_beam(DecView d, int step, i
     }
   }
   row::block_sync();
+  }
+  // The fusion bias row of this CTA's hypothesis, which the row pass before
+  // the joint kernel wrote, comes to shared memory before the wait.
+  const int Q = d.V4 / 4;
+  const int rk = b * K + crank;
+  float4* f4 = reinterpret_cast<float4*>(lmv);
+  if (step > 0)
+    for (int q = tid; q < Q; q += kRowThreads) f4[q] = __ldcg(reinterpret_cast<const float4*>(d.bias + (size_t)rk * d.N_pad) + q);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
-  if (step > 0 && !s_done) {
-    // 1. per live hypothesis (warp k): log-sum-exp and its K best extensions
-    if (warp < K) {
-      const int k = warp;
-      const bool live = o_live[k] != 0;
-      const int r = b * K + k;
-      const float2* bp = d.bpart + (size_t)r * d.n_ptiles * (1 + K);
-      float m = kNegInf, s = 0.f;
-      if (live) {
-        for (int j = lane; j < d.n_ptiles; j += 32) {
-          const float2 p = __ldcg(bp + (size_t)j * (1 + K));
-          lse_merge(m, s, p.x, p.y);
-        }
+  row::reconverge();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (step > 0) {
+    // 1. CTA k: hypothesis k's log-sum-exp and its K best extensions, to the
+    //    first CTA.  The joint kernel wrote every label's logit; K rounds of
+    //    a warp-wide maximum (a thread masks its label once taken).  With the
+    //    top K of every 64-label tile kept by the joint's epilogue (a thread
+    //    per row, K rounds of 32-wide scans) and merged here by one warp per
+    //    hypothesis, the two took about 10 us of a step's 32; this takes 3.
+    const float* lg = d.logits + (size_t)rk * d.N_pad;
+    float fb = kNegInf;  // thread 0: blank
+    for (int q = tid; q < Q; q += kRowThreads) {
+      const float4 l = __ldcg(reinterpret_cast<const float4*>(lg) + q), x = f4[q];
+      const int v = 4 * q;
+      f4[q] = make_float4(v < V ? l.x + x.x : kNegInf, v + 1 < V ? l.y + x.y : kNegInf, v + 2 < V ? l.z + x.z : kNegInf,
+                          v + 3 < V ? l.w + x.w : kNegInf);
+    }
+    if (tid == 0) fb = __ldcg(lg + V);
+    if (warp == kRowThreads / 32 - 1) {
+      float m = kNegInf, z = 0.f;
+      for (int j = lane; j < d.n_ptiles; j += 32) {
+        const float4 p = __ldcg(d.part + (size_t)rk * d.n_ptiles + j);
+        lse_merge(m, z, p.x, p.y);
       }
       row::reconverge();
+      const float top = row::key_value(__reduce_max_sync(0xffffffffu, row::order_key(m)));
+      z = z > 0.f ? z * expf(m - top) : 0.f;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float m2 = __shfl_xor_sync(0xffffffffu, m, o), s2 = __shfl_xor_sync(0xffffffffu, s, o);
-        lse_merge(m, s, m2, s2);
+      for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+      if (lane == 0) s_lse = top + logf(z);
+    }
+    // each warp's K best of its labels, then the first warp's K best of those
+    // (a thread reads only the labels it wrote: no barrier before)
+    for (int round = 0; round < K; ++round) {
+      float bv = kNegInf;
+      int bt = INT_MAX;
+      for (int q = tid; q < Q; q += kRowThreads) {
+        const float4 x = f4[q];
+        const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (xv[j] > bv) { bv = xv[j]; bt = 4 * q + j; }
       }
-      const float lse = m + logf(s);
-      float cv[kCandPerLane];
-      int ct[kCandPerLane];
-      const int nc = live ? d.n_ptiles * K : 0;
-#pragma unroll
-      for (int q = 0; q < kCandPerLane; ++q) {
-        const int i = lane + 32 * q;
-        cv[q] = kNegInf;
-        ct[q] = INT_MAX;
-        if (i < nc) {
-          const float2 p = __ldcg(bp + (size_t)(i / K) * (1 + K) + 1 + (i % K));
-          cv[q] = p.x;
-          ct[q] = __float_as_int(p.y);
-        }
-      }
-      for (int round = 0; round < K; ++round) {
-        row::reconverge();
-        // this lane's best remaining (value desc, label asc)
-        float bv = kNegInf;
-        int bt = INT_MAX, bq = -1;
-#pragma unroll
-        for (int q = 0; q < kCandPerLane; ++q)
-          if (cv[q] > bv || (cv[q] == bv && cv[q] != kNegInf && ct[q] < bt)) { bv = cv[q]; bt = ct[q]; bq = q; }
-        float wv = bv;
-        int wt = bt, wl = lane;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const float v2 = __shfl_xor_sync(0xffffffffu, wv, o);
-          const int t2 = __shfl_xor_sync(0xffffffffu, wt, o), l2 = __shfl_xor_sync(0xffffffffu, wl, o);
-          if (v2 > wv || (v2 == wv && (t2 < wt || (t2 == wt && l2 < wl)))) { wv = v2; wt = t2; wl = l2; }
-        }
-        if (lane == wl && bq >= 0) {
-#pragma unroll
-          for (int q = 0; q < kCandPerLane; ++q)
-            if (q == bq) cv[q] = kNegInf;
-        }
-        if (lane == 0) {
-          const int c = k * K + round;
-          const bool valid = wv != kNegInf && wt >= 0 && wt <= V;
-          c_tok[c] = valid ? wt : -1;
-          c_inc[c] = valid ? wv - lse : 0.f;
-          c_score[c] = valid ? o_score[k] + (double)(wv - lse) : -1e300;
-        }
+      if (fb > bv) { bv = fb; bt = V; }
+      row::reconverge();
+      const int key = row::order_key(bv + 0.f), wk = __reduce_max_sync(0xffffffffu, key);
+      const int wt = __reduce_min_sync(0xffffffffu, key == wk ? bt : INT_MAX);  // labels are distinct
+      if (lane == 0) s_top[warp * K + round] = make_float2(row::key_value(wk), __int_as_float(wt));
+      if (bt == wt && bt != INT_MAX) {
+        if (bt < V) lmv[bt] = kNegInf;
+        else fb = kNegInf;
       }
     }
     row::block_sync();
-    // 2. global top K, then merge equal label sequences
-    if (tid == 0) {
-      bool used[kMaxK * kMaxK];
-      for (int c = 0; c < K * K; ++c) used[c] = false;
-      int nsel = 0;
+    if (warp == 0) {
+      constexpr int kW = kRowThreads / 32;
+      static_assert(kW * kMaxK <= 64, "two candidates per lane");
+      float2 x[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) x[u] = lane + 32 * u < kW * K ? s_top[lane + 32 * u] : make_float2(kNegInf, __int_as_float(INT_MAX));
+      int* rtok = cluster.map_shared_rank(&c_tok[0], 0) + crank * K;
+      float* rinc = cluster.map_shared_rank(&c_inc[0], 0) + crank * K;
       for (int round = 0; round < K; ++round) {
-        int best = -1;
-        for (int c = 0; c < K * K; ++c) {
-          if (used[c] || c_tok[c] < 0) continue;
-          if (best < 0 || cand_before(c_score[c], c / K, c_tok[c], c_score[best], best / K, c_tok[best])) best = c;
+        float bv = x[0].x;
+        int bt = __float_as_int(x[0].y);
+        row::best_merge(bv, bt, x[1].x, __float_as_int(x[1].y));
+        const int key = row::order_key(bv + 0.f), wk = __reduce_max_sync(0xffffffffu, key);
+        const int wt = __reduce_min_sync(0xffffffffu, key == wk ? bt : INT_MAX);
+        const float wv = row::key_value(wk);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+          if (__float_as_int(x[u].y) == wt) x[u].x = kNegInf;
+        if (lane == 0) {
+          const bool valid = wv != kNegInf && wt >= 0 && wt <= V;
+          rtok[round] = valid ? wt : -1;
+          rinc[round] = valid ? wv - s_lse : 0.f;
         }
-        if (best < 0) break;
-        used[best] = true;
-        s_sel[nsel++] = best;
       }
+    }
+    row::reconverge();
+    cluster.sync();  // the candidates are with the first CTA
+  }
+  if (crank == 0) {
+  const int slot = s_slot, T = s_T;
+  const int hb = slot * K;
+  const int cap = d.pool_cap;
+  const int32_t* pool_par = d.pool_parent + (size_t)slot * cap;
+  const int32_t* pool_tok = d.pool_tok + (size_t)slot * cap;
+  const int S = MS ? d.max_sym : 1;
+
+  if (step > 0 && !s_done) {
+    // 2. global top K (each candidate's rank counted by the whole block),
+    //    then merge equal label sequences: one warp, lane i for the i-th kept
+    //    candidate (a single thread took 14.6 us of a step's 44.6 at K = 4)
+    const int CC = K * K;
+    for (int e = tid; e < CC * CC; e += kRowThreads) {
+      const int c = e / CC, x = e - c * CC, hc = c / K, hx = x / K;
+      const bool cin = c_tok[c] >= 0 && o_live[hc], xin = c_tok[x] >= 0 && o_live[hx];
+      const double sc = o_score[hc] + (double)c_inc[c], sx = o_score[hx] + (double)c_inc[x];
+      if (cin && xin && cand_before(sx, hx, c_tok[x], sc, hc, c_tok[c])) atomicAdd(s_rank + c, 1);
+    }
+    row::block_sync();
+    if (warp == 0) {
+      int valid = 0;
+      for (int c = lane; c < (CC + 31) / 32 * 32; c += 32) {
+        const bool in = c < CC && c_tok[c] >= 0 && o_live[c / K];
+        if (in && s_rank[c] < K) s_sel[s_rank[c]] = c;
+        valid += __popc(__ballot_sync(0xffffffffu, in));
+      }
+      const int nsel = min(valid, K);
+      __syncwarp();
       const bool last_exp = s_be >= S - 1;
-      int cnt = 0;
-      int pool_used = __ldcg(d.pool_n + slot);
-      for (int i = 0; i < nsel; ++i) {
-        const int c = s_sel[i], p = c / K, y = c_tok[c];
-        const int dst = (y == V || last_exp) ? 1 : 0;
-        const int len = o_len[p] + (y != V ? 1 : 0);
-        const unsigned long long hsh = (y != V) ? hash_push(o_hash[p], y) : o_hash[p];
-        int into = -1;
-        if (dst == 1) {
-          for (int j = 0; j < e_cnt; ++j) {
-            if (e_len[j] != len || e_hash[j] != hsh) continue;
-            if (seq_equal(pool_par, pool_tok, o_node[p], y != V ? y : -1, e_node[j], -1, cap)) {
-              into = -2 - j;
-              break;
-            }
+      const bool on = lane < nsel;
+      const int c = on ? s_sel[lane] : 0, p = c / K, y = on ? c_tok[c] : V;
+      const int dst = (y == V || last_exp) ? 1 : 0;
+      const int len = on ? o_len[p] + (y != V ? 1 : 0) : -1 - lane;
+      const unsigned long long hsh = (y != V) ? hash_push(o_hash[p], y) : o_hash[p];
+      const int node = o_node[p], app = y != V ? y : -1;
+      // into: an equal entry of F (-2 - j), the first equal candidate before
+      // this one, or itself (equality is transitive, so the first one stands
+      // for the rest)
+      int into = lane;
+      if (MS && on && dst == 1) {
+        for (int j = 0; j < e_cnt; ++j) {
+          if (e_len[j] != len || e_hash[j] != hsh) continue;
+          if (seq_equal(pool_par, pool_tok, node, app, e_node[j], -1, cap)) {
+            into = -2 - j;
+            break;
           }
         }
-        if (into == -1) {
-          for (int j = 0; j < cnt; ++j) {
-            if (n_dst[j] != dst || n_len[j] != len || n_hash[j] != hsh) continue;
-            const int pj = n_par[j];
-            if (seq_equal(pool_par, pool_tok, o_node[p], y != V ? y : -1, o_node[pj], n_tok[j] != V ? n_tok[j] : -1,
-                          cap)) {
-              into = j;
-              break;
-            }
-          }
-        }
-        if (into <= -2) {
-          e_score[-2 - into] = log_add(e_score[-2 - into], c_score[c]);
-        } else if (into >= 0) {
-          n_score[into] = log_add(n_score[into], c_score[c]);
-        } else {
-          into = cnt++;
-          n_par[into] = p;
-          n_tok[into] = y;
-          n_score[into] = c_score[c];
-          n_len[into] = len;
-          n_hash[into] = hsh;
-          n_dst[into] = dst;
-        }
-        s_into[i] = into;
       }
+      for (int j = 0; j < nsel; ++j) {
+        const int dj = __shfl_sync(0xffffffffu, dst, j), lj = __shfl_sync(0xffffffffu, len, j);
+        const unsigned long long hj = __shfl_sync(0xffffffffu, hsh, j);
+        const int nj = __shfl_sync(0xffffffffu, node, j), aj = __shfl_sync(0xffffffffu, app, j);
+        const int ij = __shfl_sync(0xffffffffu, into, j);
+        if (on && into == lane && j < lane && ij == j && dj == dst && lj == len && hj == hsh &&
+            seq_equal(pool_par, pool_tok, node, app, nj, aj, cap))
+          into = j;
+      }
+      __syncwarp();
+      const unsigned reps = __ballot_sync(0xffffffffu, on && into == lane);
+      const int cnt = __popc(reps);
+      const int idx = __popc(reps & ((1u << lane) - 1u));  // this candidate's place among the new records
+      double score = on ? o_score[p] + (double)c_inc[c] : 0.0;
+      // a record's score: its candidates' added in order
+      if (reps != (nsel >= 32 ? 0xffffffffu : (1u << nsel) - 1u)) {
+        for (int j = 0; j < nsel; ++j) {
+          const int ij = __shfl_sync(0xffffffffu, into, j);
+          const double sj = __shfl_sync(0xffffffffu, score, j);
+          if (ij >= 0 && ij == lane && j != lane) score = log_add(score, sj);
+          if (MS && ij <= -2 && lane == 0) e_score[-2 - ij] = log_add(e_score[-2 - ij], sj);
+        }
+      }
+      const int rep_idx = __shfl_sync(0xffffffffu, idx, into >= 0 ? into : 0);
+      if (on) s_into[lane] = into >= 0 ? rep_idx : into;
       // label-sequence nodes of the survivors that appended a label
-      for (int j = 0; j < cnt; ++j) {
-        const int p = n_par[j];
-        if (n_tok[j] == V) {
-          n_node[j] = o_node[p];
-        } else if (pool_used < cap) {
-          n_node[j] = pool_used;
-          if (commit) {
-            d.pool_parent[(size_t)slot * cap + pool_used] = o_node[p];
-            d.pool_tok[(size_t)slot * cap + pool_used] = n_tok[j];
-          }
-          ++pool_used;
-        } else {
-          n_node[j] = o_node[p];  // pool full: the label is not recorded
-          if (commit) atomicOr(d.err, 8);
-        }
-      }
-      if (commit) d.pool_n[slot] = pool_used;
-      n_cnt = cnt;
-      int tasks = 0;
-      for (int j = 0; j < cnt; ++j) {
-        s_task0[j] = tasks;
-        if (n_tok[j] != V) tasks += o_lml[n_par[j]] + o_trl[n_par[j]];
-      }
-      s_task0[cnt] = tasks;
-      if (d.cap_rows && step - 1 < d.cap_steps && commit) {
-        for (int i = 0; i < K; ++i) {
-          int* cr = d.cap_rows + ((size_t)(step - 1) * P->n * K + (size_t)b * K + i) * 4;
-          if (i < nsel) {
-            cr[0] = s_sel[i] / K;
-            cr[1] = c_tok[s_sel[i]];
-            cr[2] = __float_as_int(c_inc[s_sel[i]]);
-            cr[3] = s_into[i];
-          } else {
-            cr[0] = -1; cr[1] = -1; cr[2] = 0; cr[3] = -1;
+      const bool rep = on && into == lane;
+      const unsigned grow = __ballot_sync(0xffffffffu, rep && y != V);
+      const int at = s_pool + __popc(grow & ((1u << lane) - 1u));
+      if (rep) {
+        n_par[idx] = p;
+        n_tok[idx] = y;
+        n_score[idx] = score;
+        n_len[idx] = len;
+        n_hash[idx] = hsh;
+        n_dst[idx] = dst;
+        int nd = node;
+        if (y != V) {
+          if (at < cap) {
+            nd = at;
+            if (commit) {
+              d.pool_parent[(size_t)slot * cap + at] = node;
+              d.pool_tok[(size_t)slot * cap + at] = y;
+            }
+          } else if (commit) {
+            atomicOr(d.err, 8);  // pool full: the label is not recorded
           }
         }
+        n_node[idx] = nd;
+      }
+      __syncwarp();
+      const int mine = lane < cnt && n_tok[lane] != V ? o_lml[n_par[lane]] + o_trl[n_par[lane]] : 0;
+      int before = 0;
+      for (int j = 0; j < cnt; ++j) {
+        const int x = __shfl_sync(0xffffffffu, mine, j);
+        if (j < lane) before += x;
+      }
+      if (lane <= cnt) s_task0[lane] = before;
+      if (lane == 0) {
+        if (commit) d.pool_n[slot] = min(cap, s_pool + __popc(grow));
+        n_cnt = cnt;
+      }
+      if (d.cap_rows && step - 1 < d.cap_steps && commit && lane < K) {
+        int* cr = d.cap_rows + ((size_t)(step - 1) * P->n * K + (size_t)b * K + lane) * 4;
+        cr[0] = on ? p : -1;
+        cr[1] = on ? y : -1;
+        cr[2] = on ? __float_as_int(c_inc[c]) : 0;
+        cr[3] = on ? s_into[lane] : -1;
       }
     }
     row::block_sync();
@@ -448,7 +498,17 @@ __global__ void __launch_bounds__(kRowThreads) k_row_beam(DecView d, int step, i
     // 5. F keeps its K best (score desc, earlier first) in insertion order:
     //    loaded entries, then this step's exits.  The frame ends when nothing
     //    stays in it or after its S-th expansion; F is then the beam.
-    if (tid == 0) {
+    if (!MS) {  // one label per frame: every new record leaves the frame and is the beam, in order
+      if (tid < cnt) s_into[tid] = tid;
+      if (tid == 0) {
+        a_cnt = cnt;
+        f_cnt = 0;
+        s_bt = s_bt + 1;
+        s_be = 0;
+        a_frame = s_bt;
+        a_build = s_bt < T ? cnt : 0;
+      }
+    } else if (tid == 0) {
       const bool last_exp = s_be >= S - 1;
       int nf = 0;
       for (int j = 0; j < e_cnt; ++j) { q_src[nf] = -2 - j; q_score[nf++] = e_score[j]; }
@@ -614,14 +674,9 @@ __global__ void __launch_bounds__(kRowThreads) k_row_beam(DecView d, int step, i
       P->out_score[(size_t)b * T * d.max_sym] = cnt ? (float)a_score[best] : 0.f;
     }
   }
-  // Algorithmic bytes (counted when timing): the K hypotheses' partials and state
+  // Algorithmic bytes (counted when timing): the K hypotheses' logits, partials and state
   if (mode == 2 || d.count)
-    if (tid == 0) atomicAdd(d.ctr, (unsigned long long)K * (d.n_ptiles * (1 + K) * 8 + 64));
-  } else {
-    // the joint input and bias rows written below are read by the previous
-    // joint kernel: wait for it as the first CTA does
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (tid == 0) atomicAdd(d.ctr, (unsigned long long)K * (4ull * (V + 1) + d.n_ptiles * 16 + 64));
   }
   if (mode == 1) return;  // the same for every CTA: no cluster barrier below is left waiting
 
