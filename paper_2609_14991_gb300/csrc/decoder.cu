@@ -391,7 +391,7 @@ tsd_status create_impl(const tsd_decoder_cfg* cfg, const void* W_out_bf16, const
   v.K = c.beam_k;
   v.topk = topk;
   v.prune = c.prune_k;
-  d->n_ptiles = d->N_pad / d->jtc->bn;
+  d->n_ptiles = (d->N + d->jtc->bn - 1) / d->jtc->bn;
   v.n_ptiles = d->n_ptiles;
   v.V4 = d->V4;
   v.params = reinterpret_cast<const Params*>(pdev);
@@ -1046,7 +1046,7 @@ extern "C" tsd_status tsd_decoder_set_joint_kernel(tsd_decoder* d, int32_t kind)
   if (kind == 1 && d->cfg.prune_k > 0)
     return fail(TSD_EINVAL, "tsd_decoder_set_joint_kernel: the CUDA-core kernel has no pruned-fusion epilogue");
   d->joint_kind = kind;
-  d->n_ptiles = kind == 0 ? d->N_pad / d->jtc->bn : d->N_pad / kPartialCols;
+  d->n_ptiles = kind == 0 ? (d->N + d->jtc->bn - 1) / d->jtc->bn : d->N_pad / kPartialCols;
   d->view.n_ptiles = d->n_ptiles;
   return drop_graphs(d);
 }
@@ -1090,7 +1090,7 @@ extern "C" tsd_status tsd_decoder_set_option(tsd_decoder* d, const char* name, i
                                       d->view.bias, d->view.logits);
     if (ce != cudaSuccess) return cuda_fail(ce, "tsd_decoder_set_option: joint_bn");
     if (d->joint_kind == 0) {
-      d->n_ptiles = d->N_pad / d->jtc->bn;
+      d->n_ptiles = (d->N + d->jtc->bn - 1) / d->jtc->bn;
       d->view.n_ptiles = d->n_ptiles;
     }
     d->one_launch = 0;  // a tile width is asked for: the kernel that has tiles runs

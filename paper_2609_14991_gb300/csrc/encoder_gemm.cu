@@ -182,12 +182,6 @@ __device__ __forceinline__ void add4(float4* p, float4 v) {
                : "memory");
 }
 
-__device__ __forceinline__ bool elect() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
-  return p != 0;
-}
-
 // 32 accumulator columns from `taddr` with their bias (the same addresses for every lane), as pairs
 __device__ __forceinline__ void load_cols(uint32_t taddr, const float* bias, uint64_t (&v)[16]) {
   float f[32];

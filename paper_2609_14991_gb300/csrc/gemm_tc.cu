@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kGThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect()) {
       const uint32_t idesc = idesc_bf16(kBM, kGN);
       for (int kb = 0; kb < KB; ++kb) {
         const int s = kb % kGStages;

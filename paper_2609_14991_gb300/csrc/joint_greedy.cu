@@ -18,10 +18,10 @@
 // stores) and the softmax partial; the row pass after it (row_stream.cu)
 // adds the row's LM and trie terms and takes the argmax.
 //
-// Warp roles (320 threads): warp 0 TMA producer (A tile 128 x 64 and W_out
-// tile BN x 64 per stage, 128-byte swizzle), warp 1 TMEM
-// allocator and MMA issuer, warps 2-9 epilogue (thread = row; the two warps
-// of a TMEM lane quadrant take alternate 32-column chunks).  Every wait on an
+// Warp roles: warp 0 TMA producer (A tile BM x 64 and W_out tile BN x 64 per
+// stage, 128-byte swizzle), warp 1 TMEM allocator and MMA issuer, the others
+// epilogue (thread = row; the two or four warps of a TMEM lane quadrant take
+// 32-column chunks in turn).  Every wait on an
 // mbarrier is bounded; on expiry the kernel records an error in the
 // decoder's status word, drains its own copies and MMAs and returns.
 #include <cuda.h>
@@ -35,9 +35,6 @@ namespace tsd {
 namespace {
 
 using namespace tc;
-constexpr int kEW = 4;                 // epilogue warps per TMEM lane quadrant
-constexpr int kDEpi = 128 * kEW;       // epilogue threads: warps 2 .. 2 + 4 kEW - 1
-constexpr int kDThreads = 64 + kDEpi;  // and the producer and MMA warps
 constexpr float kNegInf = -__builtin_huge_valf();
 
 // Shared memory: [operand stages][defaults D][barriers].  After the
@@ -46,9 +43,15 @@ constexpr float kNegInf = -__builtin_huge_valf();
 // that the 16-byte reads of eight consecutive rows fall in different bank
 // groups) or the streaming epilogue's staging buffers (two 32 x 32 fp32
 // boxes per warp).
-template <int BN>
+// BM = 64 (streaming, BN = 64): rows 16 q .. 16 q + 15 are lanes 0-15 of
+// quadrant q, and the boxes are 16 rows high.
+template <int BN, int BM>
 struct DSmem {
-  static constexpr int kABytes = kBM * kBK * 2;
+  static constexpr int kEW = BN == 64 ? 2 : 4;  // epilogue warps per TMEM lane quadrant
+  static constexpr int kEpi = 128 * kEW;        // epilogue threads: warps 2 .. 2 + 4 kEW - 1
+  static constexpr int kThreads = 64 + kEpi;    // and the producer and MMA warps
+  static constexpr int kQRows = BM / 4;         // rows per quadrant
+  static constexpr int kABytes = BM * kBK * 2;
   static constexpr int kBBytes = BN * kBK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
   static constexpr int kStages = BN == 256 ? 4 : (BN == 128 ? 5 : 8);
@@ -56,12 +59,13 @@ struct DSmem {
   static constexpr int kDenseOff = 10240;  // past the epilogue warps' exchange
   static constexpr int kCW = 32;            // columns per TMEM load in the epilogue
   static constexpr int kStageOff = 16384;   // streaming: staging buffers, two 32 x 32 boxes per warp
-  static constexpr int kStageWarp = 2 * (kCW / 32) * 4096;
+  static constexpr int kBoxBytes = kQRows * 128;
+  static constexpr int kStageWarp = 2 * (kCW / 32) * kBoxBytes;
   static constexpr int kDOff = kStages * kStageBytes;
   static constexpr int kBarOff = kDOff + BN * 4;
   static constexpr int kBytes = kBarOff + 256 + 1024 /*align*/;
-  static_assert(kBM * 4 * (kEW - 1) * 4 + 4 * 4 * kEW <= kDenseOff, "the exchange stays clear of the dense rows");
-  static_assert(kDenseOff + kBM * kRowStride <= kStages * kStageBytes, "the dense rows fit the drained stages");
+  static_assert(BM * 4 * (kEW - 1) * 4 + 4 * 4 * kEW <= kDenseOff, "the exchange stays clear of the dense rows");
+  static_assert(kDenseOff + BM * kRowStride <= kStages * kStageBytes, "the dense rows fit the drained stages");
   static_assert(kStageOff + 4 * kEW * kStageWarp <= kStages * kStageBytes, "the staging buffers fit the drained stages");
   static_assert(kBytes <= 227 * 1024, "shared memory per CTA");
 };
@@ -96,11 +100,13 @@ __device__ __forceinline__ uint32_t pick(const uint32_t (&a)[N], int k) {
   return v;
 }
 
-template <int BN, bool DENSE>
-__global__ void __launch_bounds__(kDThreads, 1)
+template <int BN, bool DENSE, int BM>
+__global__ void __launch_bounds__((DSmem<BN, BM>::kThreads), 1)
     k_joint_greedy(DecView d, int step, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmLogits) {
-  using S = DSmem<BN>;
+  using S = DSmem<BN, BM>;
+  static_assert(BM == kBM || !DENSE, "the 64-row tile is the streaming epilogue's");
+  constexpr int kEW = S::kEW, kDEpi = S::kEpi;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   float* sD = reinterpret_cast<float*>(smem + S::kDOff);
@@ -111,7 +117,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(dbar + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n0 = blockIdx.x * BN, m0 = blockIdx.y * kBM;
+  const int n0 = blockIdx.x * BN, m0 = blockIdx.y * BM;
   const int M = d.params->n * d.K;
   const int KB = d.H / kBK;
 
@@ -121,7 +127,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
       mbar_init(empty + s, 1);
     }
     mbar_init(accum, 1);
-    mbar_init(dbar, kBM);  // one arrival per row
+    mbar_init(dbar, BM);  // one arrival per row
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -174,9 +180,9 @@ __global__ void __launch_bounds__(kDThreads, 1)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect()) {
       bool ok = true;
-      const uint32_t idesc = idesc_bf16(kBM, BN);
+      const uint32_t idesc = idesc_bf16(BM, BN);
       for (int kb = 0; kb < KB; ++kb) {
         const int s = kb % S::kStages;
         const uint32_t ph = (uint32_t)(kb / S::kStages) & 1u;
@@ -204,9 +210,9 @@ __global__ void __launch_bounds__(kDThreads, 1)
     constexpr int kWB = kCW / 32;          // mask words and 32 x 32 store boxes per block
     const int q = warp & 3;  // TMEM lane quadrant this warp may access
     const int ehalf = (warp - 2) >> 2;  // this warp's turn among its quadrant's warps
-    const int row = q * 32 + lane;
+    const int row = q * S::kQRows + lane;
     const int gr = m0 + row;
-    const bool live = gr < M;
+    const bool live = lane < S::kQRows && gr < M;
     const int N = d.N, V4 = d.V4;
     float mx = kNegInf, se = 0.f, bv = kNegInf;
     int bi = INT_MAX;
@@ -304,21 +310,21 @@ __global__ void __launch_bounds__(kDThreads, 1)
             const float4 dq = dv4[j];
             l[4 * j] += dq.x; l[4 * j + 1] += dq.y; l[4 * j + 2] += dq.z; l[4 * j + 3] += dq.w;
           }
-          unsigned char* stg = smem + S::kStageOff + (warp - 2) * S::kStageWarp + (k & 1) * kWB * 4096;
+          unsigned char* stg = smem + S::kStageOff + (warp - 2) * S::kStageWarp + (k & 1) * kWB * S::kBoxBytes;
           if (lane == 0) tma_store_wait_read<kWB>();  // the stores of two blocks ago have read this set
           __syncwarp();
 #pragma unroll
           for (int j = 0; j < kWB; ++j)
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-              *reinterpret_cast<float4*>(stg + j * 4096 + lane * 128 + ((e ^ (lane & 7)) << 4)) =
+              if (lane < S::kQRows) *reinterpret_cast<float4*>(stg + j * S::kBoxBytes + lane * 128 + ((e ^ (lane & 7)) << 4)) =
                   make_float4(l[32 * j + 4 * e], l[32 * j + 4 * e + 1], l[32 * j + 4 * e + 2], l[32 * j + 4 * e + 3]);
           fence_async_smem();
           __syncwarp();
           if (lane == 0) {
 #pragma unroll
             for (int j = 0; j < kWB; ++j) {
-              tma_store_2d(&tmLogits, stg + j * 4096, c0 + 32 * j, m0 + q * 32);
+              tma_store_2d(&tmLogits, stg + j * S::kBoxBytes, c0 + 32 * j, m0 + q * S::kQRows);
               tma_store_commit();
             }
           }
@@ -382,16 +388,12 @@ __global__ void __launch_bounds__(kDThreads, 1)
       mbar_wait(accum, 0);
       if (DENSE) mbar_wait(dbar, 0);
     }
-    // the staging buffers must have been read before the CTA's shared memory
-    // goes; the stores' writes complete with the grid (the row pass reads
-    // them after its dependency wait)
-    if (!DENSE && lane == 0) tma_store_wait_read<0>();
     __syncwarp();
     // merge the quadrant's warps' partials of each row: warps 1..kEW-1 of the
     // quadrant leave theirs in the drained stages, warp 0 combines and stores
     float* xbase = reinterpret_cast<float*>(smem);
-    int* xok = reinterpret_cast<int*>(xbase + kBM * 4 * (kEW - 1));  // [quadrant][warp 1..]
-    if (ehalf > 0) {
+    int* xok = reinterpret_cast<int*>(xbase + BM * 4 * (kEW - 1));  // [quadrant][warp 1..]
+    if (ehalf > 0 && lane < S::kQRows) {
       float* xch = xbase + (row * (kEW - 1) + ehalf - 1) * 4;
       if (ok) {
         xch[0] = mx;
@@ -428,6 +430,11 @@ __global__ void __launch_bounds__(kDThreads, 1)
       }
       if (all) d.part[(size_t)gr * d.n_ptiles + blockIdx.x] = make_float4(mx, se, bv, __int_as_float(bi));
     }
+    // the staging buffers must have been read before the CTA's shared memory
+    // goes; the stores' writes complete with the grid (the row pass reads
+    // them after its dependency wait)
+    if (!DENSE && lane == 0) tma_store_wait_read<0>();
+    __syncwarp();
   }
   fence_before();
   __syncthreads();
@@ -439,44 +446,57 @@ __global__ void __launch_bounds__(kDThreads, 1)
 
 }  // namespace
 
-cudaError_t joint_greedy_prepare(int bn) {
-  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaSuccess;
-  if (bn == 256) {
-    e = cudaFuncSetAttribute(k_joint_greedy<256, true>, attr, DSmem<256>::kBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_joint_greedy<256, false>, attr, DSmem<256>::kBytes);
-  } else if (bn == 128) {
-    e = cudaFuncSetAttribute(k_joint_greedy<128, true>, attr, DSmem<128>::kBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_joint_greedy<128, false>, attr, DSmem<128>::kBytes);
-  } else {
-    e = cudaFuncSetAttribute(k_joint_greedy<64, true>, attr, DSmem<64>::kBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_joint_greedy<64, false>, attr, DSmem<64>::kBytes);
-  }
-  return e;
-}
-
 namespace {
+template <int BN, bool DENSE, int BM = kBM>
+cudaError_t prepare_one() {
+  return cudaFuncSetAttribute(k_joint_greedy<BN, DENSE, BM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              DSmem<BN, BM>::kBytes);
+}
 template <int BN>
-void launch_greedy_bn(cudaLaunchConfig_t& cfg, const JointTc& jt, const DecView& d, int step) {
-  cfg.dynamicSmemBytes = DSmem<BN>::kBytes;
-  if (d.fz_dense) cudaLaunchKernelEx(&cfg, k_joint_greedy<BN, true>, d, step, jt.mapA, jt.mapB, jt.mapLogits);
-  else cudaLaunchKernelEx(&cfg, k_joint_greedy<BN, false>, d, step, jt.mapA, jt.mapB, jt.mapLogits);
+cudaError_t prepare_bn() {
+  const cudaError_t e = prepare_one<BN, true>();
+  return e == cudaSuccess ? prepare_one<BN, false>() : e;
+}
+template <int BN, bool DENSE, int BM = kBM>
+void launch_one(cudaLaunchConfig_t& cfg, const CUtensorMap& a, const JointTc& jt, const CUtensorMap& logits,
+                const DecView& d, int M, int step) {
+  cfg.gridDim = dim3(d.n_ptiles, (M + BM - 1) / BM);
+  cfg.blockDim = dim3(DSmem<BN, BM>::kThreads);
+  cfg.dynamicSmemBytes = DSmem<BN, BM>::kBytes;
+  cudaLaunchKernelEx(&cfg, k_joint_greedy<BN, DENSE, BM>, d, step, a, jt.mapB, logits);
+}
+template <int BN>
+void launch_bn(cudaLaunchConfig_t& cfg, const JointTc& jt, const DecView& d, int M, int step) {
+  if (d.fz_dense) launch_one<BN, true>(cfg, jt.mapA, jt, jt.mapLogits, d, M, step);
+  else launch_one<BN, false>(cfg, jt.mapA, jt, jt.mapLogits, d, M, step);
 }
 }  // namespace
 
+cudaError_t joint_greedy_prepare(int bn) {
+  if (bn == 256) return prepare_bn<256>();
+  if (bn == 128) return prepare_bn<128>();
+  const cudaError_t e = prepare_bn<64>();
+  return e == cudaSuccess ? prepare_one<64, false, 64>() : e;
+}
+
 void launch_joint_greedy(const JointTc& jt, const DecView& d, int M, int step, cudaStream_t s, bool pdl) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(d.N_pad / jt.bn, (M + kBM - 1) / kBM);
-  cfg.blockDim = dim3(kDThreads);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  if (jt.bn == 256) launch_greedy_bn<256>(cfg, jt, d, step);
-  else if (jt.bn == 128) launch_greedy_bn<128>(cfg, jt, d, step);
-  else launch_greedy_bn<64>(cfg, jt, d, step);
+  if (jt.bn == 256) launch_bn<256>(cfg, jt, d, M, step);
+  else if (jt.bn == 128) launch_bn<128>(cfg, jt, d, M, step);
+  // Narrow label tiles are bound by what an SM takes in from L2 (about 60 bytes
+  // a clock): after the dependency wait a 128 x 64 tile of K = 1024 reads 327 KB,
+  // a 64 x 64 tile 196 KB.  256 rows x 1025 labels, operands to last MMA: 4.85
+  // us in 128-row tiles, 2.55 in 64-row tiles (34 and 68 CTAs).  The line is one
+  // wave: past it a second 64-row tile would follow on some SM.
+  else if (!d.fz_dense && (M + 63) / 64 * d.n_ptiles <= d.sms)
+    launch_one<64, false, 64>(cfg, jt.mapA64, jt, jt.mapLogits16, d, M, step);
+  else launch_bn<64>(cfg, jt, d, M, step);
 }
 
 }  // namespace tsd

@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();  // reconverge before the CTA barrier below (bar.sync is warp-aligned)
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect()) {
       const uint32_t idesc = idesc_bf16(kBM, BN);
       for (int kb = 0; kb < KB; ++kb) {
         const int s = kb % S::kStages;
@@ -420,6 +420,9 @@ cudaError_t joint_tc_prepare(JointTc* jt, const uint16_t* A, int M_pad, const ui
     return cudaErrorInvalidValue;
   if (!make_map(&jt->mapLogits, logits ? logits : bias, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, N_pad, M_pad, 32, 32))
     return cudaErrorInvalidValue;
+  if (!make_map(&jt->mapA64, A, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, H, M_pad, kBK, 64) ||
+      !make_map(&jt->mapLogits16, logits ? logits : bias, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, N_pad, M_pad, 32, 16))
+    return cudaErrorInvalidValue;
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e = cudaSuccess;
   if (bn == 256) {
@@ -451,7 +454,7 @@ void launch_joint_tc(const JointTc& jt, const DecView& d, int M, int step, cudaS
     return;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(d.N_pad / jt.bn, (M + kBM - 1) / kBM);
+  cfg.gridDim = dim3(d.n_ptiles, (M + kBM - 1) / kBM);
   cfg.blockDim = dim3(kThreads);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];

@@ -13,6 +13,7 @@ struct JointTc {
   CUtensorMap mapB;  // W_out label-major [N_pad][H], bn x 64 boxes
   CUtensorMap mapBias;  // fusion bias fp32 [M_pad][N_pad], 32 x 128 boxes
   CUtensorMap mapLogits;  // logits fp32 [M_pad][N_pad], 32 x 32 boxes (the streaming epilogue's stores)
+  CUtensorMap mapA64, mapLogits16;  // the 64-row tile's: 64 x 64 and 32 x 16 boxes
   int bn = 256;      // labels per CTA tile (one selection partial each)
 };
 
