@@ -130,19 +130,8 @@ __global__ void __launch_bounds__(kGThreads, 1)
     __syncwarp();
   } else if (warp == 1) {
     if (elect()) {
-      const uint32_t idesc = idesc_bf16(kBM, kGN);
-      for (int kb = 0; kb < KB; ++kb) {
-        const int s = kb % kGStages;
-        const uint32_t ph = (uint32_t)(kb / kGStages) & 1u;
-        if (!mbar_wait(full + s, ph)) { ok = false; break; }
-        fence_after();
-        const uint32_t sa = smem_u32(smem + s * kGStageBytes);
-        const uint64_t ad = sw128_desc(sa), bd = sw128_desc(sa + kGABytes);
-#pragma unroll
-        for (int k = 0; k < kBK / 16; ++k)
-          mma_bf16(tmem, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (kb | k) ? 1u : 0u);
-        mma_commit(empty + s);
-      }
+      ok = mma_tile<kGStages, kGStageBytes, kGABytes>(tmem, smem_u32(smem), full, empty, KB,
+                                                                 idesc_bf16(kBM, kGN), kWaitNs);
       mma_commit(accum);
       if (!ok) atomicOr(d.err, 128);
     }

@@ -54,7 +54,7 @@ struct DSmem {
   static constexpr int kABytes = BM * kBK * 2;
   static constexpr int kBBytes = BN * kBK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kStages = BN == 256 ? 4 : (BN == 128 ? 5 : 8);
+  static constexpr int kStages = BN == 256 ? 4 : (BN == 128 ? 5 : (BM == 64 ? 12 : 8));
   static constexpr int kRowStride = BN * 4 + 16;
   static constexpr int kDenseOff = 10240;  // past the epilogue warps' exchange
   static constexpr int kCW = 32;            // columns per TMEM load in the epilogue
@@ -181,20 +181,8 @@ __global__ void __launch_bounds__((DSmem<BN, BM>::kThreads), 1)
     __syncwarp();
   } else if (warp == 1) {
     if (elect()) {
-      bool ok = true;
-      const uint32_t idesc = idesc_bf16(BM, BN);
-      for (int kb = 0; kb < KB; ++kb) {
-        const int s = kb % S::kStages;
-        const uint32_t ph = (uint32_t)(kb / S::kStages) & 1u;
-        if (!mbar_wait(full + s, ph, d.wait_ns)) { ok = false; break; }
-        fence_after();
-        const uint32_t sa = smem_u32(smem + s * S::kStageBytes);
-        const uint64_t ad = sw128_desc(sa), bd = sw128_desc(sa + S::kABytes);
-#pragma unroll
-        for (int k = 0; k < kBK / 16; ++k)
-          mma_bf16(tmem, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (kb | k) ? 1u : 0u);
-        mma_commit(empty + s);
-      }
+      const bool ok = mma_tile<S::kStages, S::kStageBytes, S::kABytes>(tmem, smem_u32(smem), full, empty, KB,
+                                                                       idesc_bf16(BM, BN), d.wait_ns);
       // signals the epilogue once every issued MMA has completed (also after
       // a timeout, so nothing is in flight when TMEM is released)
       mma_commit(accum);
@@ -449,8 +437,9 @@ __global__ void __launch_bounds__((DSmem<BN, BM>::kThreads), 1)
 namespace {
 template <int BN, bool DENSE, int BM = kBM>
 cudaError_t prepare_one() {
-  return cudaFuncSetAttribute(k_joint_greedy<BN, DENSE, BM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              DSmem<BN, BM>::kBytes);
+  const auto f = k_joint_greedy<BN, DENSE, BM>;
+  const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, DSmem<BN, BM>::kBytes);
+  return e == cudaSuccess ? cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) : e;
 }
 template <int BN>
 cudaError_t prepare_bn() {

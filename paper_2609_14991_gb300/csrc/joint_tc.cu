@@ -154,19 +154,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();  // reconverge before the CTA barrier below (bar.sync is warp-aligned)
   } else if (warp == 1) {
     if (elect()) {
-      const uint32_t idesc = idesc_bf16(kBM, BN);
-      for (int kb = 0; kb < KB; ++kb) {
-        const int s = kb % S::kStages;
-        const uint32_t ph = (uint32_t)(kb / S::kStages) & 1u;
-        if (!mbar_wait(full + s, ph, d.wait_ns)) { ok = false; break; }
-        fence_after();
-        const uint32_t sa = smem_u32(smem + s * S::kStageBytes);
-        const uint64_t ad = sw128_desc(sa), bd = sw128_desc(sa + S::kABytes);
-#pragma unroll
-        for (int k = 0; k < kBK / 16; ++k)  // K = 16 per instruction: +32 bytes in the swizzle atom
-          mma_bf16(tmem, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (kb | k) ? 1u : 0u);
-        mma_commit(empty + s);
-      }
+      ok = mma_tile<S::kStages, S::kStageBytes, S::kABytes>(tmem, smem_u32(smem), full, empty, KB,
+                                                                       idesc_bf16(kBM, BN), d.wait_ns);
       // signals the epilogue once every issued MMA has completed (also after a
       // timeout, so nothing is in flight when TMEM is released)
       mma_commit(accum);

@@ -92,27 +92,36 @@ __device__ __forceinline__ void best_merge(float& v, int& i, float v2, int i2) {
   if (v2 > v || (v2 == v && i2 < i)) { v = v2; i = i2; }
 }
 
+// Eight values of the joint input, bf16(ReLU(x + z)).
+__device__ __forceinline__ uint4 joint_input(uint4 x, uint4 z) {
+  const __nv_bfloat162* xa = reinterpret_cast<const __nv_bfloat162*>(&x);
+  const __nv_bfloat162* za = reinterpret_cast<const __nv_bfloat162*>(&z);
+  uint4 out;
+  __nv_bfloat162* oa = reinterpret_cast<__nv_bfloat162*>(&out);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    float2 xf = __bfloat1622float2(xa[q]);
+    float2 zf = __bfloat1622float2(za[q]);
+    float lo = fmaxf(xf.x + zf.x, 0.f), hi = fmaxf(xf.y + zf.y, 0.f);
+    oa[q] = __floats2bfloat162_rn(lo, hi);
+  }
+  return out;
+}
+
+// Constant 16 bytes, the load issued where it stands.
+__device__ __forceinline__ uint4 load_now(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+
 // Joint input of one row: A[r] = bf16(ReLU(enc_row + E[last])), block-strided.
 __device__ __forceinline__ void build_joint_input(const DecView& d, const uint16_t* enc_row, int last, int r) {
   const int H = d.H;
   const uint4* e = reinterpret_cast<const uint4*>(enc_row);
   const uint4* g = reinterpret_cast<const uint4*>(d.E + (size_t)last * H);
   uint4* a = reinterpret_cast<uint4*>(d.A + (size_t)r * H);
-  for (int i = threadIdx.x; i < H / 8; i += blockDim.x) {
-    uint4 x = __ldg(e + i), z = __ldg(g + i);
-    const __nv_bfloat162* xa = reinterpret_cast<const __nv_bfloat162*>(&x);
-    const __nv_bfloat162* za = reinterpret_cast<const __nv_bfloat162*>(&z);
-    uint4 out;
-    __nv_bfloat162* oa = reinterpret_cast<__nv_bfloat162*>(&out);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      float2 xf = __bfloat1622float2(xa[q]);
-      float2 zf = __bfloat1622float2(za[q]);
-      float lo = fmaxf(xf.x + zf.x, 0.f), hi = fmaxf(xf.y + zf.y, 0.f);
-      oa[q] = __floats2bfloat162_rn(lo, hi);
-    }
-    a[i] = out;
-  }
+  for (int i = threadIdx.x; i < H / 8; i += blockDim.x) a[i] = joint_input(__ldg(e + i), __ldg(g + i));
 }
 
 // Shared-memory records of the chains a bias row is built from.

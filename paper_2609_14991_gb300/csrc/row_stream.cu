@@ -41,7 +41,15 @@
 //      emitted and advances the chains, assembled from independent searches
 //      of y in every chain element, each hit carrying the next state's table
 //      record (first arc, arcs, summed backoff) in the same 16-byte load;
-//   4. writes the joint input of step s, bf16(ReLU(enc_t + E[last])).
+//   4. writes the joint input of step s, bf16(ReLU(enc_t + E[last])): it needs
+//      the decision alone, so its loads go out before the searches'.
+//
+// Bound by dependent round trips to L2, not by bytes: after the joint kernel's
+// logits are there, one trip for them, then the embedding row beside the
+// searches (their first loads were made before the wait; a hit costs one or
+// two more).  256 rows, V 1024, H 1024, order 6: 3.3 us from the logits to the
+// last joint input, 4.9 with the joint input after the chains' assembly, 128
+// threads a row and no early loads; a step 8.2 against 10.4 us.
 #include <algorithm>
 
 #include "row_common.cuh"
@@ -55,10 +63,7 @@ using row::checked;
 using row::kNegInf;
 using row::lse_merge;
 
-constexpr int kFzThreads = 128;  // 4 warps: seven CTAs per SM at 72 registers
-constexpr int kStream = 4;       // level-0 arc groups of four per thread whose loads are issued together
-constexpr int kDense = 8;        // dense level-0 quads per thread whose loads are issued together
-constexpr int kFzWarps = kFzThreads / 32;
+constexpr int kStream = 4;  // level-0 arc groups of four per thread whose loads are issued together
 
 // Aligned groups of four arcs a chain level's arcs [b, b + c) span.
 __device__ __forceinline__ int level_groups(int b, int c) { return c > 0 ? (b + c - (b & ~3) + 3) >> 2 : 0; }
@@ -69,13 +74,19 @@ __device__ __forceinline__ int level_groups(int b, int c) { return c > 0 ? (b + 
 // reads at most three entries before and after the range, inside the table
 // (its label arrays start 16-byte aligned and are padded by four).  At most
 // two dependent loads for n <= 3968.
-__device__ __forceinline__ int warp_find_wide(const int32_t* __restrict__ arr, int n, int y, int lane) {
+// PRE: `pre` holds this lane's first load (first_load below), made before y
+// was known.
+template <bool PRE>
+__device__ __forceinline__ int warp_find_wide(const int32_t* __restrict__ arr, int n, int y, int lane, int4 pre) {
   row::reconverge();
   int lo = 0, hi = n;
+  bool held = PRE;
   while (hi - lo > 124) {
     const int step = (hi - lo + 31) >> 5;
     const int idx = lo + lane * step;
-    const int v = (idx < hi) ? __ldg(arr + idx) : INT_MAX;
+    int v = pre.x;
+    if (!held) v = (idx < hi) ? __ldg(arr + idx) : INT_MAX;
+    held = false;
     const unsigned m = __ballot_sync(0xffffffffu, v <= y);
     if (m == 0) return -1;
     lo = lo + (31 - __clz((int)m)) * step;
@@ -86,7 +97,7 @@ __device__ __forceinline__ int warp_find_wide(const int32_t* __restrict__ arr, i
   const int first = 4 * lane - (int)((at & 15u) >> 2);  // this lane's first entry, relative to lo
   int pos = -1;
   if (first < hi - lo) {
-    const int4 t = __ldg(g + lane);
+    const int4 t = held ? pre : __ldg(g + lane);
     const int tv[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
     for (int j = 3; j >= 0; --j)
@@ -96,15 +107,39 @@ __device__ __forceinline__ int warp_find_wide(const int32_t* __restrict__ arr, i
   return m ? __shfl_sync(0xffffffffu, pos, __ffs((int)m) - 1) : -1;
 }
 
+__device__ __forceinline__ int4 first_load(const int32_t* __restrict__ arr, int n, int lane) {
+  int4 t = make_int4(INT_MAX, INT_MAX, INT_MAX, INT_MAX);
+  if (n > 124) {
+    const int idx = lane * ((n + 31) >> 5);
+    if (idx < n) t.x = __ldg(arr + idx);
+  } else {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(arr);
+    if (4 * lane - (int)((at & 15u) >> 2) < n) t = __ldg(reinterpret_cast<const int4*>(at & ~uintptr_t(15)) + lane);
+  }
+  return t;
+}
+
+template <class T>
+__device__ __forceinline__ void touch(T* p) { asm volatile("" ::"l"(p)); }
+
 // mode: 0 = label step, 1 = final step (apply the last decision only),
 // 2 = replay (redo the step's work without committing any state or output;
 // used only to time the kernel in isolation).
 // VAR bit 0: the stateful form (LSTM input rows instead of the joint input);
-// bit 2: few rows (at most two CTAs per SM are needed, registers are free).
+// bit 2: few rows (at most two per SM): eight warps, so that every chain
+// element's search is one warp's and its first load precedes the wait.
+// Otherwise four warps: seven CTAs per SM at 72 registers.  72 also let two
+// rows of eight warps start beside a joint CTA (80 registers and 192 threads:
+// 629 us a chunk of 256 rows, 64 registers, which spill: 675, this: 616).
 template <int VAR>
-__global__ void __launch_bounds__(kFzThreads) __maxnreg__((VAR & 4) ? 128 : 72) k_row_fz(DecView d, int step, int mode) {
-  constexpr bool PRED = (VAR & 1) != 0;
-  constexpr int QB = 8;     // label quads per thread whose loads are issued together
+constexpr int kThreadsOf = (VAR & 4) ? 256 : 128;
+
+template <int VAR>
+__global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
+  constexpr bool PRED = (VAR & 1) != 0, FEW = (VAR & 4) != 0;
+  constexpr int kFzThreads = kThreadsOf<VAR>, kFzWarps = kFzThreads / 32;
+  constexpr int kDense = FEW ? 2 : 8;  // dense level-0 quads per thread whose loads are issued together
+  constexpr int QB = FEW ? 2 : 8;      // label quads per thread whose loads are issued together
   constexpr int kHeld = 1;  // arc groups of four of the levels above 0 a thread keeps in registers
   const Params* __restrict__ P = d.params;
   const int r = blockIdx.x;
@@ -119,20 +154,19 @@ __global__ void __launch_bounds__(kFzThreads) __maxnreg__((VAR & 4) ? 128 : 72) 
   uint16_t* lev = reinterpret_cast<uint16_t*>(dlm + d.V4);  // [V4]
   uint8_t* dep = reinterpret_cast<uint8_t*>(lev + d.V4);    // [V4]
 
-  __shared__ int s_t, s_sym, s_cnt, s_y, s_last, s_slot, s_T, s_n;
+  __shared__ int s_t, s_sym, s_cnt, s_last, s_slot, s_T, s_n;
   __shared__ int s_nl, s_nt;
   __shared__ int32_t* s_out_tok;
   __shared__ int32_t* s_out_frame;
   __shared__ float* s_out_score;
   __shared__ int32_t* s_out_count;
   __shared__ const uint16_t* s_enc;
-  __shared__ float s_lam, s_beta, s_score, s_lse;
+  __shared__ float s_lam, s_beta, s_lse;
   __shared__ int s_lm[kLmChain], s_tr[kTrChain];
   __shared__ int4 s_lmr[kLmChain];    // LM chain records: (first arc, arcs, summed backoff bits, -)
   __shared__ int4 s_trr[kTrChain];    // trie chain records: (first child, children, depth of the children, -)
   __shared__ int4 s_lm_hit[kLmChain]; // target record of y's arc at each old level (x = -2: none)
   __shared__ int4 s_tr_hit[kTrChain]; // child record of y at each old trie node (x = -1: none)
-  __shared__ int4 s_uni_hit, s_root_hit;
   __shared__ float s_bv[kFzWarps];
   __shared__ int s_bi[kFzWarps];
   __shared__ unsigned long long s_bytes;  // algorithmic bytes of the row-step (when counting)
@@ -252,6 +286,13 @@ __global__ void __launch_bounds__(kFzThreads) __maxnreg__((VAR & 4) ? 128 : 72) 
   const float lam = s_lam;
   const float bscale = s_beta * (d.has_tr ? d.tr.bonus : 0.f);
 
+  // warp w searches chain elements w, w + warps, ...: the first one's first load
+  int4 pre = make_int4(0, 0, 0, 0);
+  if (FEW && evaluated && warp < nl_old + nt_old) {
+    const bool is_lm = warp < nl_old;
+    const int4 c = is_lm ? s_lmr[warp] : s_trr[warp - nl_old];
+    pre = first_load((is_lm ? d.lm.arc_tok : d.tr.ch_tok) + c.x, c.y, lane);
+  }
   if (evaluated) {
     const int4* t4 = reinterpret_cast<const int4*>(d.lm.arc_tok);
     const float4* p4 = reinterpret_cast<const float4*>(d.lm.arc_logp);
@@ -289,6 +330,25 @@ __global__ void __launch_bounds__(kFzThreads) __maxnreg__((VAR & 4) ? 128 : 72) 
         hl[u] = l;
       }
     }
+    //     and warp w the first 128 children of trie chain node w
+    int4 ct = make_int4(0, 0, 0, 0);
+    if (warp < nt_old && lane < level_groups(s_trr[warp].x, s_trr[warp].y))
+      ct = __ldg(reinterpret_cast<const int4*>(d.tr.ch_tok) + (s_trr[warp].x >> 2) + lane);
+    // trie chain node k's children get their depth (shallower nodes first)
+    auto trie_node = [&](int k) {
+      const int b = s_trr[k].x, e = b + s_trr[k].y, a0 = b & ~3;
+      const uint8_t dd = (uint8_t)s_trr[k].z;
+      auto put = [&](int i0, int4 t) {
+        if (i0 >= b && i0 < e) dep[t.x] = dd;
+        if (i0 + 1 >= b && i0 + 1 < e) dep[t.y] = dd;
+        if (i0 + 2 >= b && i0 + 2 < e) dep[t.z] = dd;
+        if (i0 + 3 >= b && i0 + 3 < e) dep[t.w] = dd;
+      };
+      const bool held = k < kFzWarps;
+      if (held && warp == k) put(a0 + 4 * lane, ct);
+      for (int g = (held ? 32 : 0) + tid; a0 + 4 * g < e; g += kFzThreads)
+        put(a0 + 4 * g, __ldg(reinterpret_cast<const int4*>(d.tr.ch_tok + a0) + g));
+    };
     // 1b. level 0 (the previous label's continuations, up to all V labels),
     //     streamed once: every label's level-0 delta (0 for no arc), which
     //     the deepest level above overwrites below
@@ -366,9 +426,19 @@ __global__ void __launch_bounds__(kFzThreads) __maxnreg__((VAR & 4) ? 128 : 72) 
       const int i0 = locate(g, l);
       offer(l, i0, __ldg(t4 + (i0 >> 2)));
     }
-    if (nt_old > 0) {  // the trie chain nodes, shallowest first (the deepest overwrites)
-      const int k = nt_old - 1;
-      row::scatter_trie_node(d.tr.ch_tok, s_trr[k].x, s_trr[k].x + s_trr[k].y, (uint8_t)s_trr[k].z, dep);
+    if (nt_old > 0) trie_node(nt_old - 1);  // the trie chain nodes, shallowest first (the deepest overwrites)
+    float hu[kHeld][4];  // the held arcs' unigram terms, on their way over the barrier
+#pragma unroll
+    for (int u = 0; u < kHeld; ++u) {
+      if (hl[u] >= 0) {
+        const int b = s_lmr[hl[u]].x, e = b + s_lmr[hl[u]].y;
+        const int tv[4] = {ht[u].x, ht[u].y, ht[u].z, ht[u].w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          hu[u][j] = hi[u] + j >= b && hi[u] + j < e && checked(tv[j] >= 0 && tv[j] < V, d.err, 9)
+                         ? __ldg(d.lm.uni_logp + tv[j])
+                         : 0.f;
+      }
     }
     row::block_sync();
     // 1d. the arc of each label at its deepest level writes the label's delta
@@ -384,7 +454,7 @@ __global__ void __launch_bounds__(kFzThreads) __maxnreg__((VAR & 4) ? 128 : 72) 
         for (int j = 0; j < 4; ++j) {
           const int i = hi[u] + j;
           if (i >= b && i < b + c && checked(tv[j] >= 0 && tv[j] < V, d.err, 9) && deepest(tv[j]) == l)
-            dlm[tv[j]] = delta_of(l, pv[j], tv[j]);
+            dlm[tv[j]] = lam * (pv[j] - __int_as_float(s_lmr[l].z)) - lam * hu[u][j];
         }
       }
     }
@@ -401,22 +471,27 @@ __global__ void __launch_bounds__(kFzThreads) __maxnreg__((VAR & 4) ? 128 : 72) 
         if (i0 + j >= b && i0 + j < b + c && checked(tv[j] >= 0 && tv[j] < V, d.err, 9) && deepest(tv[j]) == l)
           dlm[tv[j]] = delta_of(l, pv[j], tv[j]);
     }
-    if (nt_old > 1) {
-      const int k = nt_old - 2;
-      row::scatter_trie_node(d.tr.ch_tok, s_trr[k].x, s_trr[k].x + s_trr[k].y, (uint8_t)s_trr[k].z, dep);
-    }
+    if (nt_old > 1) trie_node(nt_old - 2);
     for (int k = nt_old - 3; k >= 0; --k) {
       row::block_sync();
-      row::scatter_trie_node(d.tr.ch_tok, s_trr[k].x, s_trr[k].x + s_trr[k].y, (uint8_t)s_trr[k].z, dep);
+      trie_node(k);
     }
     row::block_sync();
   }
+  // the parameters used after the wait go through the constant cache once now
+  touch(d.logits); touch(d.part); touch(d.droot); touch(d.E); touch(d.A); touch(d.tr.root_rec); touch(d.lm.uni_rec);
+  touch(d.lm.arc_tok); touch(d.lm.arc_rec); touch(d.tr.ch_tok); touch(d.tr.ch_rec); touch(d.s_lm_chain);
+  touch(d.s_lm_rec); touch(d.m_lm); touch(d.m_lmr); touch(d.s_lm_len); touch(d.m_lm_len); touch(d.s_tr_chain);
+  touch(d.s_tr_rec); touch(d.m_tr); touch(d.m_trr); touch(d.s_tr_len); touch(d.m_tr_len); touch(d.s_last);
+  touch(d.m_last); touch(d.r_t); touch(d.r_sym); touch(d.r_cnt); touch(d.cap_rows);
   // Programmatic dependent launch: everything above reads only state the
   // previous row pass wrote (complete before the joint kernel in between let
   // this grid launch) and constant tables; the logits need the wait.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
+  int y = V;
+  float best = 0.f;
   if (evaluated) {
     // 2. the argmax of logit + D + c_r + delta over the labels (blank takes
     //    its logit alone); the log-sum-exp of the raw logits (from the tile
@@ -496,201 +571,210 @@ __global__ void __launch_bounds__(kFzThreads) __maxnreg__((VAR & 4) ? 128 : 72) 
     int bix = s_bi[0];
 #pragma unroll
     for (int w = 1; w < kFzWarps; ++w) best_merge(b, bix, s_bv[w], s_bi[w]);
-    const int y = (bix >= 0 && bix <= V) ? bix : V;
-    if (tid == 0) {
-      s_y = y;
-      s_score = b;  // the fused score less the log-sum-exp
-    }
-    if (!PRED) row::prefetch_span(d.E + (size_t)(y != V ? y : s_last) * d.H, (size_t)d.H * 2, 32);
-    if (y != V) {
-      // 3a. independent searches of y in every chain element; each hit's
-      //     record is the next chain element's
-      if (tid == kFzThreads - 1) {
-        s_root_hit = d.has_tr ? __ldg(d.tr.root_rec + y) : make_int4(0, 0, 0, 0);
-      } else if (tid == kFzThreads - 2) {
-        s_uni_hit = (d.has_lm && d.lm.order >= 2) ? __ldg(d.lm.uni_rec + y) : make_int4(-1, 0, 0, 0);
-      }
-      // the last warp's first tile partials load while it searches
-      const float4* pr = d.part + (size_t)r * d.n_ptiles;
-      float4 p0 = make_float4(kNegInf, 0.f, 0.f, 0.f);
-      if (warp == kFzWarps - 1 && lane < d.n_ptiles) p0 = __ldcg(pr + lane);  // written by the joint kernel
-      for (int task = warp; task < nl_old + nt_old; task += kFzWarps) {
-        if (task < nl_old) {
-          const int b = s_lmr[task].x, c = s_lmr[task].y;
-          const int i = warp_find_wide(d.lm.arc_tok + b, c, y, lane);
-          if (lane == 0) s_lm_hit[task] = (i >= 0) ? __ldg(d.lm.arc_rec + b + i) : make_int4(-2, 0, 0, 0);
-          if (counting && lane == 0) atomicAdd(&s_bytes, 4ull * (32 - __clz(c + 1)) + 16);
-        } else {
-          const int k = task - nl_old;
-          const int b = s_trr[k].x, c = s_trr[k].y;
-          const int i = warp_find_wide(d.tr.ch_tok + b, c, y, lane);
-          if (lane == 0) s_tr_hit[k] = (i >= 0) ? __ldg(d.tr.ch_rec + b + i) : make_int4(-1, 0, 0, 0);
-          if (counting && lane == 0) atomicAdd(&s_bytes, 4ull * (32 - __clz(c + 1)) + 16);
-        }
-      }
-      if (warp == kFzWarps - 1) {  // the log-sum-exp of the raw logits
-        float pm = kNegInf, ps = 0.f;
-        lse_merge(pm, ps, p0.x, p0.y);
-        for (int j = lane + 32; j < d.n_ptiles; j += 32) {
-          const float4 p = __ldcg(pr + j);
-          lse_merge(pm, ps, p.x, p.y);
-        }
-        row::reconverge();
-        for (int o = 16; o > 0; o >>= 1) {
-          const float m2 = __shfl_xor_sync(0xffffffffu, pm, o);
-          const float s2 = __shfl_xor_sync(0xffffffffu, ps, o);
-          lse_merge(pm, ps, m2, s2);
-        }
-        if (lane == 0) s_lse = pm + logf(ps);
-      }
-      row::block_sync();
-      // 3b. assemble the new chains in place (shared memory) and commit them
-      //     (by slot, and by row for the next step): warp 0 the LM chain
-      //     (y's unigram state, then the targets of y's arcs at the old levels
-      //     up to the first level without one), warp 1 the trie chain (y's
-      //     children of the old chain nodes, deepest first, then the root's;
-      //     completing a phrase resets it), warp 2 the outputs
-      if (warp == 0) {
-        int ln = 0;
-        if (d.has_lm && d.lm.order >= 2) {
-          const int4 h = lane < nl_old ? s_lm_hit[lane] : make_int4(-2, 0, 0, 0);
-          const bool cont =
-              h.x >= 0 && checked(h.x < d.lm.n_states && h.y >= 0 && h.z >= 0 && (int64_t)h.y + h.z <= d.lm.n_arcs,
-                                  d.err, 10);
-          const unsigned miss = __ballot_sync(0xffffffffu, !cont);
-          ln = 1 + min(miss ? __ffs((int)miss) - 1 : 32, kLmChain - 1);
-          const int4 u = s_uni_hit;  // u.x is y's dense row
-          // lane l >= 1 takes the hit of old level l - 1
-          const int px = __shfl_up_sync(0xffffffffu, h.x, 1), py = __shfl_up_sync(0xffffffffu, h.y, 1);
-          const int pz = __shfl_up_sync(0xffffffffu, h.z, 1), pw = __shfl_up_sync(0xffffffffu, h.w, 1);
-          const int nst = lane == 0 ? 1 + y : px;
-          const int4 nrec = lane == 0 ? make_int4(u.y, u.z, u.w, u.x) : make_int4(py, pz, pw, 0);
-          __syncwarp();
-          if (lane < ln) {
-            s_lm[lane] = nst;
-            s_lmr[lane] = nrec;
-            if (commit) {
-              d.s_lm_chain[(size_t)slot * kLmChain + lane] = nst;
-              d.s_lm_rec[(size_t)slot * kLmChain + lane] = nrec;
-              d.m_lm[(size_t)r * kLmChain + lane] = nst;
-              d.m_lmr[(size_t)r * kLmChain + lane] = nrec;
-            }
-          }
-        }
-        if (lane == 0) {
-          s_nl = ln;
-          if (commit) {
-            if (d.has_lm) d.s_lm_len[slot] = ln;
-            d.m_lm_len[r] = ln;
-          }
-        }
-      } else if (warp == 1) {
-        const int4 h = lane < nt_old ? s_tr_hit[lane] : make_int4(-1, 0, 0, 0);
-        const int dd = lane < nt_old ? s_trr[lane].z + 1 : 0;  // the child's children sit one deeper
-        const bool ok = h.x >= 0 && checked(h.x > 0 && h.x < d.tr.n_nodes && h.w >= 0 && h.z + h.w <= d.tr.n_children,
-                                            d.err, 11);
-        const unsigned vm = __ballot_sync(0xffffffffu, ok);
-        const int nv = __popc(vm);
-        const int4 rh = s_root_hit;
-        const bool root = rh.x != 0;
-        // the first element of the new chain ends a phrase: the chain resets
-        const int f = __ffs((int)vm) - 1;
-        const int fy = __shfl_sync(0xffffffffu, h.y, f < 0 ? 0 : f);
-        const bool reset = nv > 0 ? fy == 0 : (root && rh.y == 0);
-        const int tn = reset ? 0 : min(nv + (root ? 1 : 0), kTrChain);
-        __syncwarp();
-        const int pos = __popc(vm & ((1u << lane) - 1u));
-        if (ok && pos < tn) {
-          s_tr[pos] = h.x;
-          s_trr[pos] = make_int4(h.z, h.w, dd, 0);
-        }
-        if (lane == 0 && root && nv < tn) {
-          s_tr[nv] = rh.x;
-          s_trr[nv] = make_int4(rh.z, rh.w, 2, 0);
-        }
-        __syncwarp();
-        if (commit && lane < tn) {
-          d.s_tr_chain[slot * kTrChain + lane] = s_tr[lane];
-          d.s_tr_rec[(size_t)slot * kTrChain + lane] = s_trr[lane];
-          d.m_tr[(size_t)r * kTrChain + lane] = s_tr[lane];
-          d.m_trr[(size_t)r * kTrChain + lane] = s_trr[lane];
-        }
-        if (lane == 0) {
-          s_nt = tn;
-          if (commit) {
-            if (d.has_tr) d.s_tr_len[slot] = tn;
-            d.m_tr_len[r] = tn;
-          }
-        }
-      } else if (tid == 64) {
-        if (commit) {
-          const int cap = T * d.max_sym;
-          const int o = r * cap + s_cnt;
-          s_out_tok[o] = y;
-          s_out_frame[o] = s_t;
-          s_out_score[o] = s_score - s_lse;
-          d.s_last[slot] = y;
-          d.m_last[r] = y;
-        }
-        s_cnt += 1;
-        s_last = y;
-        s_sym += 1;
-        if (s_sym >= d.max_sym) { s_t += 1; s_sym = 0; }
-      }
-    } else if (tid == 0) {
-      s_t += 1;
-      s_sym = 0;
-    }
-    row::block_sync();
+    y = (bix >= 0 && bix <= V) ? bix : V;
+    best = b;  // the fused score less the log-sum-exp
   }
-
+  // the frame, the labels in it and the last label after the decision
+  const bool label = evaluated && y != V;
+  int t1 = s_t, sym1 = s_sym;
+  if (label) {
+    if (++sym1 >= d.max_sym) { ++t1; sym1 = 0; }
+  } else if (evaluated) {
+    ++t1;
+    sym1 = 0;
+  }
+  const int last1 = label ? y : s_last;
+  const int t = commit ? t1 : min(t1, T - 1);
+  const bool next = mode != 1 && t < T;  // another label step follows
+  // 4. the joint input of this step needs y alone: its loads go out before the
+  //    searches', and it is written while they are in flight
+  const bool joint = !PRED && next;
+  const uint4* enc_row = reinterpret_cast<const uint4*>(s_enc + ((size_t)r * T + t) * d.H);
+  const uint4* emb_row = reinterpret_cast<const uint4*>(d.E + (size_t)last1 * d.H);
+  uint4 jx, jz;
+  if (joint && tid < d.H / 8) {
+    jx = row::load_now(enc_row + tid);
+    jz = row::load_now(emb_row + tid);
+  }
+  uint4 px;
+  bool stepped = false;
+  const uint4* pred_src[2] = {nullptr, nullptr};
   if (PRED) {
     // Stateful form: the prediction network reads the label just emitted
     // (or, at a stream's first step, the start of sequence) and the row's h
     // from before this step; the LSTM kernel after this one runs the cell.
     const bool fresh = step == 0 && __ldcg(d.pred_fresh + slot) != 0;
-    const bool stepped = fresh || (evaluated && s_y != V);
+    stepped = fresh || label;
     if (tid == 0) {
       d.pflag[r] = stepped ? 1 : 0;
       if (fresh && commit) d.pred_fresh[slot] = 0;
     }
-    if (stepped) {
-      const int D = d.pred_D;
-      const int lab = fresh ? V : s_y;
-      const uint4* src_x = reinterpret_cast<const uint4*>(d.pred_emb + (size_t)lab * D);
-      const uint4* src_h = reinterpret_cast<const uint4*>(d.pred_h + (size_t)slot * D);
-      uint4* dst = reinterpret_cast<uint4*>(d.pred_x + (size_t)r * 2 * D);
-      for (int i = tid; i < D / 4; i += blockDim.x) dst[i] = (i < D / 8) ? __ldg(src_x + i) : __ldcg(src_h + i - D / 8);
+    pred_src[0] = reinterpret_cast<const uint4*>(d.pred_emb + (size_t)(fresh ? V : y) * d.pred_D);
+    pred_src[1] = reinterpret_cast<const uint4*>(d.pred_h + (size_t)slot * d.pred_D) - d.pred_D / 8;
+    if (stepped && tid < d.pred_D / 4) px = tid < d.pred_D / 8 ? __ldg(pred_src[0] + tid) : __ldcg(pred_src[1] + tid);
+  }
+  const int4 rhit = warp == 1 && label && d.has_tr ? __ldg(d.tr.root_rec + y) : make_int4(0, 0, 0, 0);
+  const int4 uhit = warp == 0 && label && d.has_lm && d.lm.order >= 2 ? __ldg(d.lm.uni_rec + y) : make_int4(-1, 0, 0, 0);
+  if (label) {
+    // 3a. independent searches of y in every chain element; each hit's
+    //     record is the next chain element's
+    // the last warp's first tile partials load while it searches
+    const float4* pr = d.part + (size_t)r * d.n_ptiles;
+    float4 p0 = make_float4(kNegInf, 0.f, 0.f, 0.f);
+    if (warp == kFzWarps - 1 && lane < d.n_ptiles) p0 = __ldcg(pr + lane);  // written by the joint kernel
+    for (int task = warp; task < nl_old + nt_old; task += kFzWarps) {
+      const bool is_lm = task < nl_old;
+      const int k = is_lm ? task : task - nl_old;
+      const int4 rec = is_lm ? s_lmr[k] : s_trr[k];
+      const int32_t* arr = (is_lm ? d.lm.arc_tok : d.tr.ch_tok) + rec.x;
+      const int i = FEW && task == warp ? warp_find_wide<true>(arr, rec.y, y, lane, pre)
+                                        : warp_find_wide<false>(arr, rec.y, y, lane, pre);
+      if (lane == 0) {
+        if (is_lm) s_lm_hit[k] = (i >= 0) ? __ldg(d.lm.arc_rec + rec.x + i) : make_int4(-2, 0, 0, 0);
+        else s_tr_hit[k] = (i >= 0) ? __ldg(d.tr.ch_rec + rec.x + i) : make_int4(-1, 0, 0, 0);
+        if (counting) atomicAdd(&s_bytes, 4ull * (32 - __clz(rec.y + 1)) + 16);
+      }
+    }
+    if (warp == kFzWarps - 1) {  // the log-sum-exp of the raw logits
+      float pm = kNegInf, ps = 0.f;
+      lse_merge(pm, ps, p0.x, p0.y);
+      for (int j = lane + 32; j < d.n_ptiles; j += 32) {
+        const float4 p = __ldcg(pr + j);
+        lse_merge(pm, ps, p.x, p.y);
+      }
+      row::reconverge();
+      for (int o = 16; o > 0; o >>= 1) {
+        const float m2 = __shfl_xor_sync(0xffffffffu, pm, o);
+        const float s2 = __shfl_xor_sync(0xffffffffu, ps, o);
+        lse_merge(pm, ps, m2, s2);
+      }
+      if (lane == 0) s_lse = pm + logf(ps);
+    }
+  }
+  if (joint) {
+    uint4* a = reinterpret_cast<uint4*>(d.A + (size_t)r * d.H);
+    if (tid < d.H / 8) a[tid] = row::joint_input(jx, jz);
+    for (int i = tid + kFzThreads; i < d.H / 8; i += kFzThreads) a[i] = row::joint_input(__ldg(enc_row + i), __ldg(emb_row + i));
+  }
+  if (PRED && stepped) {
+    uint4* dst = reinterpret_cast<uint4*>(d.pred_x + (size_t)r * 2 * d.pred_D);
+    if (tid < d.pred_D / 4) dst[tid] = px;
+    for (int i = tid + kFzThreads; i < d.pred_D / 4; i += kFzThreads)
+      dst[i] = i < d.pred_D / 8 ? __ldg(pred_src[0] + i) : __ldcg(pred_src[1] + i);
+  }
+  if (label) {
+    row::block_sync();
+    // 3b. assemble the new chains in place (shared memory) and commit them
+    //     (by slot, and by row for the next step): warp 0 the LM chain
+    //     (y's unigram state, then the targets of y's arcs at the old levels
+    //     up to the first level without one), warp 1 the trie chain (y's
+    //     children of the old chain nodes, deepest first, then the root's;
+    //     completing a phrase resets it), warp 2 the outputs
+    if (warp == 0) {
+      int ln = 0;
+      if (d.has_lm && d.lm.order >= 2) {
+        const int4 h = lane < nl_old ? s_lm_hit[lane] : make_int4(-2, 0, 0, 0);
+        const bool cont =
+            h.x >= 0 && checked(h.x < d.lm.n_states && h.y >= 0 && h.z >= 0 && (int64_t)h.y + h.z <= d.lm.n_arcs,
+                                d.err, 10);
+        const unsigned miss = __ballot_sync(0xffffffffu, !cont);
+        ln = 1 + min(miss ? __ffs((int)miss) - 1 : 32, kLmChain - 1);
+        const int4 u = uhit;  // u.x is y's dense row
+        // lane l >= 1 takes the hit of old level l - 1
+        const int px = __shfl_up_sync(0xffffffffu, h.x, 1), py = __shfl_up_sync(0xffffffffu, h.y, 1);
+        const int pz = __shfl_up_sync(0xffffffffu, h.z, 1), pw = __shfl_up_sync(0xffffffffu, h.w, 1);
+        const int nst = lane == 0 ? 1 + y : px;
+        const int4 nrec = lane == 0 ? make_int4(u.y, u.z, u.w, u.x) : make_int4(py, pz, pw, 0);
+        __syncwarp();
+        if (lane < ln) {
+          s_lm[lane] = nst;
+          s_lmr[lane] = nrec;
+          if (commit) {
+            d.s_lm_chain[(size_t)slot * kLmChain + lane] = nst;
+            d.s_lm_rec[(size_t)slot * kLmChain + lane] = nrec;
+            d.m_lm[(size_t)r * kLmChain + lane] = nst;
+            d.m_lmr[(size_t)r * kLmChain + lane] = nrec;
+          }
+        }
+      }
+      if (lane == 0) {
+        s_nl = ln;
+        if (commit) {
+          if (d.has_lm) d.s_lm_len[slot] = ln;
+          d.m_lm_len[r] = ln;
+        }
+      }
+    } else if (warp == 1) {
+      const int4 h = lane < nt_old ? s_tr_hit[lane] : make_int4(-1, 0, 0, 0);
+      const int dd = lane < nt_old ? s_trr[lane].z + 1 : 0;  // the child's children sit one deeper
+      const bool ok = h.x >= 0 && checked(h.x > 0 && h.x < d.tr.n_nodes && h.w >= 0 && h.z + h.w <= d.tr.n_children,
+                                          d.err, 11);
+      const unsigned vm = __ballot_sync(0xffffffffu, ok);
+      const int nv = __popc(vm);
+      const int4 rh = rhit;
+      const bool root = rh.x != 0;
+      // the first element of the new chain ends a phrase: the chain resets
+      const int f = __ffs((int)vm) - 1;
+      const int fy = __shfl_sync(0xffffffffu, h.y, f < 0 ? 0 : f);
+      const bool reset = nv > 0 ? fy == 0 : (root && rh.y == 0);
+      const int tn = reset ? 0 : min(nv + (root ? 1 : 0), kTrChain);
+      __syncwarp();
+      const int pos = __popc(vm & ((1u << lane) - 1u));
+      if (ok && pos < tn) {
+        s_tr[pos] = h.x;
+        s_trr[pos] = make_int4(h.z, h.w, dd, 0);
+      }
+      if (lane == 0 && root && nv < tn) {
+        s_tr[nv] = rh.x;
+        s_trr[nv] = make_int4(rh.z, rh.w, 2, 0);
+      }
+      __syncwarp();
+      if (commit && lane < tn) {
+        d.s_tr_chain[slot * kTrChain + lane] = s_tr[lane];
+        d.s_tr_rec[(size_t)slot * kTrChain + lane] = s_trr[lane];
+        d.m_tr[(size_t)r * kTrChain + lane] = s_tr[lane];
+        d.m_trr[(size_t)r * kTrChain + lane] = s_trr[lane];
+      }
+      if (lane == 0) {
+        s_nt = tn;
+        if (commit) {
+          if (d.has_tr) d.s_tr_len[slot] = tn;
+          d.m_tr_len[r] = tn;
+        }
+      }
     }
   }
   if (counting && tid == 0 && evaluated) atomicAdd(d.ctr, s_bytes);
-  if (mode == 1) {
-    if (tid == 0) s_out_count[r] = s_cnt;
-    return;
-  }
-  if (tid == 0 && commit) {
-    d.r_t[r] = s_t;
-    d.r_sym[r] = s_sym;
-    d.r_cnt[r] = s_cnt;
-  }
-  const int t = commit ? s_t : min(s_t, T - 1);
-  const int nl = s_nl, nt = s_nt;
-  if (d.cap_rows && step < d.cap_steps && tid == 0 && commit) {
-    int* c = d.cap_rows + ((size_t)step * s_n + r) * 4;
-    if (t < T) {
-      c[0] = t;
-      c[1] = s_last;
-      c[2] = nl ? s_lm[nl - 1] : 0;
-      c[3] = nt ? s_tr[0] : 0;
-    } else {
-      c[0] = -1; c[1] = -1; c[2] = -1; c[3] = -1;
+  if (tid == 64) {  // the outputs and the row's place in the chunk
+    const int cnt = s_cnt;
+    if (label && commit) {
+      const int o = r * T * d.max_sym + cnt;
+      s_out_tok[o] = y;
+      s_out_frame[o] = s_t;
+      s_out_score[o] = best - s_lse;
+      d.s_last[slot] = y;
+      d.m_last[r] = y;
+    }
+    const int cnt1 = cnt + (label ? 1 : 0);
+    if (mode == 1) {
+      s_out_count[r] = cnt1;
+    } else if (commit) {
+      d.r_t[r] = t1;
+      d.r_sym[r] = sym1;
+      d.r_cnt[r] = cnt1;
     }
   }
-  if (t >= T) return;
-
-  // 4. joint input of this step
-  if (!PRED) row::build_joint_input(d, s_enc + ((size_t)r * T + t) * d.H, s_last, r);
-  if (counting && tid == 0 && !PRED) atomicAdd(d.ctr, 6ull * d.H);  // encoder frame, embedding row, A row
+  if (counting && tid == 0 && joint) atomicAdd(d.ctr, 6ull * d.H);  // encoder frame, embedding row, A row
+  if (d.cap_rows && step < d.cap_steps && mode == 0) {
+    row::block_sync();
+    if (tid == 0) {
+      int* c = d.cap_rows + ((size_t)step * s_n + r) * 4;
+      c[0] = next ? t : -1;
+      c[1] = next ? last1 : -1;
+      c[2] = next ? (s_nl ? s_lm[s_nl - 1] : 0) : -1;
+      c[3] = next ? (s_nt ? s_tr[0] : 0) : -1;
+    }
+  }
 }
 
 }  // namespace
@@ -698,17 +782,22 @@ __global__ void __launch_bounds__(kFzThreads) __maxnreg__((VAR & 4) ? 128 : 72) 
 size_t row_stream_smem_bytes(int V4) { return (size_t)V4 * (sizeof(float) + sizeof(uint16_t) + sizeof(uint8_t)); }
 
 cudaError_t prepare_stream_kernels(size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(k_row_fz<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_row_fz<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_row_fz<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_row_fz<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  return e;
+  const void* f[] = {(const void*)k_row_fz<0>, (const void*)k_row_fz<1>, (const void*)k_row_fz<4>, (const void*)k_row_fz<5>};
+  // the joint kernel's shared-memory split: the next row pass starts on an SM
+  // whose joint CTA still runs only if neither kernel asks for another
+  for (const void* k : f) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 void launch_row_stream(const DecView& d, int M, int step, int mode, size_t smem, cudaStream_t s, bool pdl) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(M);
-  cfg.blockDim = dim3(kFzThreads);
+  const bool few = M <= 2 * d.sms;
+  cfg.blockDim = dim3(few ? kThreadsOf<4> : kThreadsOf<0>);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -716,7 +805,6 @@ void launch_row_stream(const DecView& d, int M, int step, int mode, size_t smem,
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  const bool few = M <= 2 * d.sms;
   if (d.pred_D) {
     if (few) cudaLaunchKernelEx(&cfg, k_row_fz<5>, d, step, mode);
     else cudaLaunchKernelEx(&cfg, k_row_fz<1>, d, step, mode);

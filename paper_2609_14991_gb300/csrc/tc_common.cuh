@@ -82,6 +82,19 @@ __device__ __forceinline__ bool mbar_try(uint64_t* b, uint32_t parity) {
   return ok != 0;
 }
 
+// Whether the phase has completed, without waiting.
+__device__ __forceinline__ bool mbar_test(uint64_t* b, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(b)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // Waits for the phase of the given parity; false if it did not complete
 // within limit_ns nanoseconds.
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, unsigned long long limit_ns = kWaitNs) {
@@ -154,6 +167,34 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+
+// The MMAs of one tile over KB operand stages (A, then B at A_BYTES, 64-deep,
+// 128-byte swizzle) by the calling thread; each stage is handed back to the
+// producer when its MMAs have completed.  False if a wait expired.  The next
+// stage's barrier is read while this stage's MMAs are issued: a narrow tile's
+// stage otherwise takes 315 clocks (64 x 64) with its operands long there.
+template <int STAGES, int STAGE_BYTES, int A_BYTES>
+__device__ __forceinline__ bool mma_tile(uint32_t tmem, uint32_t smem, uint64_t* full, uint64_t* empty, int KB,
+                                         uint32_t idesc, unsigned long long limit_ns) {
+  int s = 0;
+  uint32_t ph = 0;
+  bool ready = mbar_test(full, 0);
+  for (int kb = 0; kb < KB; ++kb) {
+    if (!ready && !mbar_wait(full + s, ph, limit_ns)) return false;
+    const int s1 = s + 1 == STAGES ? 0 : s + 1;
+    const uint32_t ph1 = s1 == 0 ? ph ^ 1u : ph;
+    ready = kb + 1 < KB && mbar_test(full + s1, ph1);
+    fence_after();
+    const uint64_t ad = sw128_desc(smem + s * STAGE_BYTES), bd = sw128_desc(smem + s * STAGE_BYTES + A_BYTES);
+#pragma unroll
+    for (int k = 0; k < kBK / 16; ++k)  // K = 16 per instruction: +32 bytes in the swizzle atom
+      mma_bf16(tmem, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (kb | k) ? 1u : 0u);
+    mma_commit(empty + s);
+    s = s1;
+    ph = ph1;
+  }
+  return true;
+}
 
 // 32 consecutive fp32 columns of this warp's 32 TMEM lanes (one per thread).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
