@@ -189,7 +189,7 @@ tsd_status create_impl(const tsd_decoder_cfg* cfg, const void* W_out_bf16, const
   d->V4 = round_up(c.V, 16);
   // greedy decoding with at most one LM (whose unigram states have their
   // dense rows): the joint kernel's epilogue applies Eq. 1 up to the row's
-  // correction list; several LMs and beam search keep the dense bias row
+  // correction list; several LMs and beam search build the whole bias row
   const bool fused = c.beam_k == 1 && c.prune_k == 0 && n_lms <= 1 &&
                      (n_lms == 0 || !lm_weights || lm_weights[0] == 1.f) &&
                      (!lm || lm->view.order < 2 || lm->view.n_dense == lm->view.V);
@@ -218,12 +218,12 @@ tsd_status create_impl(const tsd_decoder_cfg* cfg, const void* W_out_bf16, const
   char* pdev = nullptr;
   tsd_status st;
   if ((st = A.alloc(&Wt, (size_t)d->N_pad * c.H)) || (st = A.alloc(&E, (size_t)d->N * c.H)) ||
-      (st = A.alloc(&Abuf, (size_t)d->M_pad * c.H)) || (st = A.alloc(&bias, (size_t)d->M_pad * d->N_pad)) ||
+      (st = A.alloc(&Abuf, (size_t)d->M_pad * c.H)) ||
       (st = A.alloc(&part, (size_t)d->M_pad * (d->N_pad / 64))) || (st = A.alloc(&err, 1)) || (st = A.alloc(&ctr, 2)) || (st = A.alloc(&dflt, (size_t)d->V4)) || (st = A.alloc(&droot, (size_t)(d->V4 + 31) / 32)) || (st = A.alloc(&rt, (size_t)d->M_pad)) ||
       (st = A.alloc(&rs, (size_t)d->M_pad)) || (st = A.alloc(&rc, (size_t)d->M_pad)) ||
       (st = A.alloc(&sl, SK)) || (st = A.alloc(&sll, SK * NL)) || (st = A.alloc(&slc, SK * NL * kLmChain)) ||
       (st = A.alloc(&stl, SK)) || (st = A.alloc(&stc, SK * kTrChain)) || (st = A.alloc(&pdev, d->params_bytes)) ||
-      (st = A.alloc(&slr, SK * kLmChain)) || (st = A.alloc(&strc, SK * kTrChain))) {
+      (st = A.alloc(&slr, SK * NL * kLmChain)) || (st = A.alloc(&strc, SK * kTrChain))) {
     A.release();
     return st;
   }
@@ -257,6 +257,14 @@ tsd_status create_impl(const tsd_decoder_cfg* cfg, const void* W_out_bf16, const
       return st;
     }
   }
+  if (!fused && c.beam_k == 1 && c.prune_k == 0) {  // the bias row holds all of Eq. 1's terms: no defaults
+    if ((st = A.alloc(&v.logits, (size_t)d->M_pad * d->N_pad)) || (st = A.alloc(&v.dvec, (size_t)d->N_pad))) {
+      A.release();
+      return st;
+    }
+    TSD_CUDA(cudaMemsetAsync(v.dvec, 0, sizeof(float) * (size_t)d->N_pad, s));
+    TSD_CUDA(cudaMemsetAsync(v.logits, 0, sizeof(float) * (size_t)d->M_pad * d->N_pad, s));
+  }
   if (c.beam_k > 1) {
     const size_t pool = (size_t)c.max_streams * kPoolCap;
     if ((st = A.alloc(&v.logits, (size_t)d->M_pad * d->N_pad)) || (st = A.alloc(&v.dvec, (size_t)d->N_pad)) || (st = A.alloc(&hscore, SK)) ||
@@ -272,6 +280,10 @@ tsd_status create_impl(const tsd_decoder_cfg* cfg, const void* W_out_bf16, const
       return st;
     }
     // the joint kernel adds no defaults to a beam's logits: the bias row holds all of Eq. 1's terms
+    if ((st = A.alloc(&bias, (size_t)d->M_pad * d->N_pad))) {
+      A.release();
+      return st;
+    }
     TSD_CUDA(cudaMemsetAsync(v.dvec, 0, sizeof(float) * (size_t)d->N_pad, s));
     TSD_CUDA(cudaMemsetAsync(v.logits, 0, sizeof(float) * (size_t)d->M_pad * d->N_pad, s));
     TSD_CUDA(cudaMemsetAsync(v.f_live, 0, SK * sizeof(int32_t), s));
@@ -318,7 +330,7 @@ tsd_status create_impl(const tsd_decoder_cfg* cfg, const void* W_out_bf16, const
   };
   cudaError_t ce;
   if ((ce = cudaMemsetAsync(Abuf, 0, sizeof(uint16_t) * (size_t)d->M_pad * c.H, s)) != cudaSuccess ||
-      (ce = cudaMemsetAsync(bias, 0, sizeof(float) * (size_t)d->M_pad * d->N_pad, s)) != cudaSuccess ||
+      (bias && (ce = cudaMemsetAsync(bias, 0, sizeof(float) * (size_t)d->M_pad * d->N_pad, s)) != cudaSuccess) ||
       (ce = cudaMemsetAsync(sll, 0, sizeof(int32_t) * SK * NL, s)) != cudaSuccess ||
       (ce = cudaMemsetAsync(stl, 0, sizeof(int32_t) * SK, s)) != cudaSuccess ||
       (ce = cudaMemsetAsync(err, 0, sizeof(int32_t), s)) != cudaSuccess ||
@@ -371,7 +383,7 @@ tsd_status create_impl(const tsd_decoder_cfg* cfg, const void* W_out_bf16, const
     d->sms = sms;
     d->view.sms = sms;
     const int bn = joint_tc_pick_bn(d->M_max, d->N_pad, sms);
-    if ((ce = joint_tc_prepare(d->jtc, Abuf, d->M_pad, Wt, d->N_pad, c.H, bn, bias, v.logits)) != cudaSuccess)
+    if ((ce = joint_tc_prepare(d->jtc, Abuf, d->M_pad, Wt, d->N_pad, c.H, bn, v.logits)) != cudaSuccess)
       return cleanup(cuda_fail(ce, "tsd_decoder_create: tensor-core GEMM setup (TMA descriptors)"));
   }
   for (int i = 0; i < tsd_decoder::kRing; ++i) {
@@ -1087,7 +1099,7 @@ extern "C" tsd_status tsd_decoder_set_option(tsd_decoder* d, const char* name, i
     tsd_status st = drop_graphs(d);
     if (st) return st;
     cudaError_t ce = joint_tc_prepare(d->jtc, d->view.A, d->M_pad, d->view.Wt, d->N_pad, d->cfg.H, (int)value,
-                                      d->view.bias, d->view.logits);
+                                      d->view.logits);
     if (ce != cudaSuccess) return cuda_fail(ce, "tsd_decoder_set_option: joint_bn");
     if (d->joint_kind == 0) {
       d->n_ptiles = (d->N + d->jtc->bn - 1) / d->jtc->bn;
@@ -1135,7 +1147,7 @@ extern "C" tsd_status tsd_decoder_replay(tsd_decoder* d, int32_t kernel, int32_t
       // per launch, plus the dense unigram and root rows every launch reads once
       const int64_t shared = (int64_t)d->cfg.V * ((d->lm ? 4 : 0) + (d->boost ? 4 : 0));
       *algo_bytes = (int64_t)(b / (unsigned long long)reps) + shared;
-    } else if (d->view.fused && !d->view.fz_dense) {
+    } else if (!d->view.fz_dense && !d->cfg.prune_k) {
       // joint, streaming epilogue: the operands once (A rows, W_out), the
       // logits written and the softmax partials
       *algo_bytes = (int64_t)M * d->cfg.H * 2 + (int64_t)d->N * d->cfg.H * 2 + (int64_t)M * d->N * 4 +

@@ -33,7 +33,7 @@ struct DecView {
   const uint16_t* E;   // [N][H] bf16
   const uint16_t* Wt;  // [N_pad][H] bf16, label-major (rows >= N are zero)
   uint16_t* A;         // [M_pad][H] bf16, joint input of the current step
-  float* bias;         // [M_pad][N_pad] fp32, lambda*LM + beta*boost of the current step
+  float* bias;         // beam search: [M_pad][N_pad] fp32, lambda*LM + beta*boost of the current step
   float4* part;        // [M_pad][n_ptiles] (max logit, sum exp, best fused, best label)
   int32_t* r_t;        // [M_pad] frame
   int32_t* r_sym;      // [M_pad] labels emitted in this frame
@@ -46,7 +46,7 @@ struct DecView {
   int32_t* s_tr_chain;  // [.][kTrChain]
   // greedy: the table records of each chain element, kept with the chain so
   // the next step's searches start without fetching them:
-  int4* s_lm_rec;       // [slots][kLmChain] first LM: (first arc, arcs, cumulative backoff bits, 0)
+  int4* s_lm_rec;       // [LMs][slots][kLmChain] (first arc, arcs, cumulative backoff bits, dense row or -)
   int4* s_tr_rec;       // [slots][kTrChain] trie: (first child, children, depth of the children, 0)
   // stateful form (pred_D > 0): prediction network state and its buffers
   int32_t pred_D;       // LSTM width (0: the stateless joint input enc + E[last])
@@ -109,7 +109,7 @@ struct DecView {
   // adds the row's LM and trie terms before it takes the argmax.
   int32_t fused;
   int32_t fz_dense;     // 1: the dense epilogue with the correction list; 0: streaming
-  float* logits;        // [M_pad][N_pad] fp32: the listed labels' raw logits (dense) or every label's logit + dvec (also beam search)
+  float* logits;        // [M_pad][N_pad] fp32: the listed labels' raw logits (dense) or every label's logit + dvec (also several LMs and beam search, whose dvec is 0)
   float* dvec;          // [N_pad] per call: lambda*log p(v) + beta*bonus*[the root has a child v]; 0 from V on
   int32_t* c_lab;       // [M_pad][V4] the row's listed labels
   float* c_add;         // [M_pad][V4] their term: F[v] = logit[v] + c_add

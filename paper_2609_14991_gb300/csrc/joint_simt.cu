@@ -1,17 +1,16 @@
-// Joint GEMM with the fused selection epilogue, CUDA-core version.
+// Joint GEMM, CUDA-core version.
 //
 // logits[r][v] = sum_k A[r][k] * Wt[v][k]  (bf16 inputs, fp32 accumulation;
 // the joint network's output projection), then per row and 128-label tile:
 // the softmax partial (max logit, sum exp(logit - max)) over the V+1 real
-// labels and the best fused value logit + bias (bias = lambda*LM +
-// beta*boost, 0 for blank), ties to the lowest label.  With DecView::fused
-// the fused value is logit + D[v] + lambda*dense0[u][v] (the call's defaults
-// and the dense LM row of the row's unigram state u), and the labels on the
-// row's correction list are no candidates: their raw logits are stored for
-// the row pass.  With fusion_path 0 (DecView::fz_dense = 0) the row's logits
-// plus the call's defaults are written out instead and the row pass fuses.
+// labels; the row's logits plus the call's defaults are written out and the
+// row pass fuses.  With fusion_path 1 (DecView::fz_dense) the tile's best
+// fused value is taken instead, logit + D[v] + lambda*dense0[u][v] (the
+// call's defaults and the dense LM row of the row's unigram state u), ties to
+// the lowest label; the labels on the row's correction list are no
+// candidates: their raw logits are stored for the row pass.
 // This is the simple reference-grade kernel for small row counts; the
-// tensor-core kernel in joint_tc.cu does the same contraction with tcgen05.
+// tensor-core kernel in joint_greedy.cu does the same contraction with tcgen05.
 #include "decoder.h"
 
 namespace tsd {
@@ -96,12 +95,10 @@ __global__ void __launch_bounds__(256) k_joint_simt(DecView d, int step) {
     const int row = warp * (kJM / 8) + rr;
     const int gr = m0 + row;
     if (gr >= M) break;
-    const float* brow = d.bias + (size_t)gr * d.N_pad;
     const float* urow = nullptr;
     const uint32_t* mrow = nullptr;
     const float lam = d.params->lambda;
     const bool dense = d.fused && d.fz_dense;
-    const bool stream = (d.fused && !dense) || d.K > 1;
     if (dense) {
       const int u = __ldcg(&d.c_info[gr].x);
       if (u >= 0 && u < d.lm.n_dense) urow = d.lm.dense0 + (size_t)u * d.V4;
@@ -117,16 +114,14 @@ __global__ void __launch_bounds__(256) k_joint_simt(DecView d, int step) {
       if (gc < N) {
         mx = fmaxf(mx, l[q]);
         float f;
-        if (stream) {
+        if (!dense) {
           f = l[q];  // the streaming form: the row pass takes the argmax
-        } else if (dense) {
+        } else {
           if ((__ldcg(mrow + (gc >> 5)) >> (gc & 31)) & 1u) {  // listed: the row pass evaluates it
             d.logits[(size_t)gr * d.N_pad + gc] = l[q];
             continue;
           }
           f = l[q] + fmaf(lam, (urow && gc < V) ? __ldg(urow + gc) : 0.f, __ldcg(d.dvec + gc));
-        } else {
-          f = l[q] + (gc < V ? brow[gc] : 0.f);
         }
         if (f > bv) { bv = f; bi = gc; }
       }
@@ -148,7 +143,7 @@ __global__ void __launch_bounds__(256) k_joint_simt(DecView d, int step) {
     for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
     if (lane == 0)
       d.part[(size_t)gr * d.n_ptiles + blockIdx.x] = make_float4(mx, se, bv, __int_as_float(bi));
-    if (stream) {  // the streaming form: logit + D of every label
+    if (!dense) {  // the streaming form: logit + D of every label
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int gc = n0 + lane * 4 + q;

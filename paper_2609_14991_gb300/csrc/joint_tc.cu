@@ -1,5 +1,5 @@
-// Joint GEMM on the 5th-generation tensor cores (tcgen05) with the fused
-// selection epilogue.
+// Joint GEMM on the 5th-generation tensor cores (tcgen05) with the selection
+// epilogue of pruned fusion.
 //
 // logits[r][v] = sum_k A[r][k] * Wt[v][k]: A (joint input, bf16 [M][H]) and
 // Wt (W_out label-major, bf16 [N_pad][H]) are both K-major, loaded by TMA
@@ -8,10 +8,9 @@
 // tensor memory.  Eight epilogue warps read the accumulator back with
 // tcgen05.ld (thread = row; two warps per 32-lane quadrant take alternate
 // 32-column chunks) and reduce it on chip to the row's selection partial for
-// this tile: softmax max and sum over the real labels, and the best fused
-// value logit + bias (the dense fusion bias row of several LMs), ties to the
-// lowest label, or (pruned fusion) the tile's top K.  Greedy decoding with at
-// most one LM and beam search run joint_greedy.cu instead.  Logits never leave the SM.
+// this tile: softmax max and sum over the real labels, and the tile's top K
+// logits, ties to the lower label.  Logits never leave the SM.  (Every other
+// form stores its logits: joint_greedy.cu.)
 //
 // Warp roles (320 threads): warp 0 TMA producer, warp 1 TMEM allocator and
 // MMA issuer, warps 2-9 epilogue.  Every wait on an mbarrier is bounded in
@@ -31,25 +30,15 @@ using namespace tc;  // kBM, kBK and the tcgen05 / TMA helpers
 constexpr int kThreads = 320;
 constexpr int kEpiThreads = 256;  // warps 2-9
 constexpr float kNegInf = -__builtin_huge_valf();
-// Shared memory: [operand stages][bias boxes][barriers].  With a fusion
-// bias (several LMs), the bias of the tile (128 rows x BN fp32) arrives by
-// TMA in 128 x 32 boxes with the 128-byte swizzle while the mainloop runs;
-// at BN = 256 only the first half has its own buffer and the second half
-// lands in the drained stages.
+// Shared memory: [operand stages][barriers].
 template <int BN>
 struct Smem {
-  static constexpr int kStages = (BN == 256) ? 3 : (BN == 128 ? 4 : 8);
+  static constexpr int kStages = (BN == 256) ? 4 : (BN == 128 ? 6 : 8);
   static constexpr int kABytes = kBM * kBK * 2;
   static constexpr int kBBytes = BN * kBK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kBoxBytes = kBM * 32 * 4;
-  static constexpr int kBoxes = BN / 32;
-  static constexpr int kEarly = (BN == 256) ? 4 : kBoxes;
-  static constexpr int kBiasBytes = kEarly * kBoxBytes;
-  static constexpr int kBytes = kStages * kStageBytes + kBiasBytes + 1024 /*align*/ + 256 /*barriers*/;
-  static_assert((kBoxes - kEarly) * kBoxBytes <= kStages * kStageBytes, "late bias boxes fit the stages");
-  // the epilogue halves' exchange (per row 18 floats, 4 flags) after the late boxes
-  static_assert((kBoxes - kEarly) * kBoxBytes + kBM * 18 * 4 + 16 <= kStages * kStageBytes, "exchange fits");
+  static constexpr int kBytes = kStages * kStageBytes + 1024 /*align*/ + 256 /*barriers*/;
+  static_assert(kBM * 18 * 4 + 16 <= kStages * kStageBytes, "the epilogue halves' exchange (per row 18 floats, 4 flags) fits");
 };
 
 // Sum over a chunk of 2^(l[i] * log2 e - s2) in four independent
@@ -61,26 +50,20 @@ __device__ __forceinline__ float sum_exp2_32(const float* l, float s2) {
   return (a[0] + a[1]) + (a[2] + a[3]);
 }
 
-// TOPK (pruned fusion): instead of the single best fused label, each row
-// keeps the top K (K = d.topk <= 8, the candidate count) logits of the tile,
-// ties to the lower label; no bias tile is loaded.
-template <int BN, bool TOPK>
+// K = d.topk <= 8, the candidate count.
+template <int BN>
 __global__ void __launch_bounds__(kThreads, 1)
-    k_joint_tc(DecView d, int step, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               const __grid_constant__ CUtensorMap tmBias) {
+    k_joint_tc(DecView d, int step, const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB) {
   using S = Smem<BN>;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  unsigned char* bias_early = smem + S::kStages * S::kStageBytes;
-  uint64_t* full = reinterpret_cast<uint64_t*>(bias_early + S::kBiasBytes);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::kStages * S::kStageBytes);
   uint64_t* empty = full + S::kStages;
   uint64_t* accum = empty + S::kStages;
-  uint64_t* biasbar = accum + 1;  // [0] early boxes, [1] late boxes
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(biasbar + 2);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(accum + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n0 = blockIdx.x * BN, m0 = blockIdx.y * kBM;
-  constexpr bool use_bias = !TOPK;
   const int M = d.params->n * d.K;
   const int KB = d.H / kBK;
 
@@ -90,8 +73,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(empty + s, 1);
     }
     mbar_init(accum, 1);
-    mbar_init(biasbar, 1);
-    mbar_init(biasbar + 1, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -115,19 +96,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   }
   // Programmatic dependent launch: the set-up above overlaps the row pass;
-  // its outputs (joint input, bias) are read only after the wait.  The next
+  // its output (the joint input) is read only after the wait.  The next
   // row pass may launch once every CTA is past this point.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   if (warp == 0) {
     if (lane == 0) {
-      // the bias tile first: the epilogue needs it as soon as the MMAs end
-      if (use_bias) {
-        mbar_expect_tx(biasbar, S::kEarly * S::kBoxBytes);
-        for (int c = 0; c < S::kEarly; ++c)
-          tma_load_2d(bias_early + c * S::kBoxBytes, &tmBias, biasbar, n0 + 32 * c, m0);
-      }
       int issued = 0;
       for (int kb = 0; kb < KB; ++kb) {
         const int s = kb % S::kStages;
@@ -171,8 +146,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int gr = m0 + row;
     const bool live = gr < M;
     const int N = d.N;
-    float mx = kNegInf, se = 0.f, bv = kNegInf;
-    int bi = INT_MAX;
+    float mx = kNegInf, se = 0.f;
     const int K = d.topk;
     float tv[8];
     int ti[8];
@@ -182,84 +156,40 @@ __global__ void __launch_bounds__(kThreads, 1)
     ok = __all_sync(0xffffffffu, mbar_wait(accum, 0, d.wait_ns));  // warp-uniform: tcgen05.ld is .sync.aligned
     if (!ok && lane == 0) atomicOr(d.err, 4);
     fence_after();
-    // the second half of a 256-wide bias tile goes into the drained stages
-    // (every MMA has completed, so nothing reads them any more)
-    const bool late = ok && use_bias && S::kEarly < S::kBoxes;
-    if (late && warp == 2 && lane == 0) {
-      mbar_expect_tx(biasbar + 1, (S::kBoxes - S::kEarly) * S::kBoxBytes);
-      for (int c = S::kEarly; c < S::kBoxes; ++c)
-        tma_load_2d(smem + (c - S::kEarly) * S::kBoxBytes, &tmBias, biasbar + 1, n0 + 32 * c, m0);
-    }
-    const bool have_early = use_bias ? __all_sync(0xffffffffu, mbar_wait(biasbar, 0, d.wait_ns)) : true;
-    if (!have_early) {
-      ok = false;
-      if (lane == 0) atomicOr(d.err, 16);
-    }
-    bool late_done = !late;
     if (ok) {
       const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16);
-      const int sw = row & 7;  // 128-byte swizzle: 16-byte chunk j of a row sits at j ^ (row % 8)
 #pragma unroll 1
       for (int c = half; c < BN / 32; c += 2) {
         __syncwarp();  // the per-chunk selection branches; tcgen05.ld wants the warp whole
-        if (use_bias && c >= S::kEarly && !late_done) {
-          late_done = true;
-          if (!__all_sync(0xffffffffu, mbar_wait(biasbar + 1, 0, d.wait_ns))) {
-            if (lane == 0) atomicOr(d.err, 32);
-            break;
-          }
-        }
-        const unsigned char* box = (c < S::kEarly) ? bias_early + c * S::kBoxBytes : smem + (c - S::kEarly) * S::kBoxBytes;
-        float b[32];
-        if (use_bias) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float4 v = *reinterpret_cast<const float4*>(box + row * 128 + ((j ^ sw) << 4));
-            b[4 * j] = v.x; b[4 * j + 1] = v.y; b[4 * j + 2] = v.z; b[4 * j + 3] = v.w;
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) b[j] = 0.f;
-        }
         float l[32];
         tmem_ld32(tbase + (uint32_t)(c * 32), l);
         const int c0 = n0 + c * 32;
         // Labels at or past V+1 (padding of the last tile) take no part:
-        // their logit becomes -inf.  Blank (label V) has bias 0 in the row.
+        // their logit becomes -inf.
         if (c0 + 32 > N) {
 #pragma unroll
           for (int i = 0; i < 32; ++i)
             if (c0 + i >= N) l[i] = kNegInf;
         }
-        // fused values f = logit + bias (reuse b), chunk maxima by trees
-        float t[16], u[16];
+        // the values still to take (b), the chunk's maximum by a tree
+        float b[32], u[16];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) b[i] += l[i];
+        for (int i = 0; i < 32; ++i) b[i] = l[i];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) { t[i] = fmaxf(l[i], l[i + 16]); u[i] = fmaxf(b[i], b[i + 16]); }
+        for (int i = 0; i < 16; ++i) u[i] = fmaxf(b[i], b[i + 16]);
 #pragma unroll
         for (int w = 8; w > 0; w >>= 1)
 #pragma unroll
-          for (int i = 0; i < w; ++i) { t[i] = fmaxf(t[i], t[i + w]); u[i] = fmaxf(u[i], u[i + w]); }
-        const float cm = t[0], fm = u[0];
-        if (!TOPK) {
-          // the first label of the chunk holding the chunk's best fused value
-          if (fm > bv) {
-            int j = 31;
-#pragma unroll
-            for (int i = 31; i >= 0; --i)
-              if (b[i] == fm) j = i;
-            bv = fm;
-            bi = c0 + j;
-          }
-        } else if (fm > tmin) {
+          for (int i = 0; i < w; ++i) u[i] = fmaxf(u[i], u[i + w]);
+        const float cm = u[0];
+        if (cm > tmin) {
           // Take the chunk's values in decreasing order while they beat the
           // K-th kept value: at most K rounds, usually none after the first
           // chunks.  Each round finds the first (lowest-label) position of the
           // chunk maximum, bubbles it into the sorted list (an equal value
           // already kept stays ahead: it has the lower label), masks it out
           // and takes the next maximum.
-          float cmx = fm;
+          float cmx = cm;
 #pragma unroll 1
           for (int it = 0; it < K && cmx > tmin; ++it) {
             int jx = 31;
@@ -307,30 +237,22 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
       }
     }
-    // never leave with bias boxes still landing in shared memory or MMAs
-    // still writing the accumulator (these drains keep the long limit
+    // never leave with MMAs still writing the accumulator (the long limit
     // whatever wait_ns is)
-    if (!late_done && warp == 2 && lane == 0) mbar_wait(biasbar + 1, 0);
-    if (!have_early && warp == 2 && lane == 0) mbar_wait(biasbar, 0);
     if (warp == 2 && lane == 0) mbar_wait(accum, 0);
     __syncwarp();
     // Merge the two halves' partials of each row: the second half leaves its
-    // partial in shared memory past the late bias boxes (the stages are
-    // drained: every MMA has completed), the first half combines and stores.
-    float* xbase = reinterpret_cast<float*>(smem + (S::kBoxes - S::kEarly) * S::kBoxBytes);
-    float* xch = xbase + row * 18;  // (max, sum, then best or top-8 (value, label))
+    // partial in shared memory (the stages are drained: every MMA has
+    // completed), the first half combines and stores.
+    float* xbase = reinterpret_cast<float*>(smem);
+    float* xch = xbase + row * 18;  // (max, sum, then the top 8 (value, label))
     int* xok = reinterpret_cast<int*>(xbase + kBM * 18);  // per quadrant: the second half finished
     if (half == 1) {
       if (ok) {
         xch[0] = mx;
         xch[1] = se;
-        if (!TOPK) {
-          xch[2] = bv;
-          xch[3] = __int_as_float(bi);
-        } else {
 #pragma unroll
-          for (int j = 0; j < 8; ++j) { xch[2 + 2 * j] = tv[j]; xch[3 + 2 * j] = __int_as_float(ti[j]); }
-        }
+        for (int j = 0; j < 8; ++j) { xch[2 + 2 * j] = tv[j]; xch[3 + 2 * j] = __int_as_float(ti[j]); }
       }
       if (lane == 0) xok[q] = ok ? 1 : 0;
     }
@@ -345,36 +267,29 @@ __global__ void __launch_bounds__(kThreads, 1)
           mx = m2;
         }
       }
-      if (!TOPK) {
-        const float v1 = xch[2];
-        const int i1 = __float_as_int(xch[3]);
-        if (v1 > bv || (v1 == bv && i1 < bi)) { bv = v1; bi = i1; }
-        d.part[(size_t)gr * d.n_ptiles + blockIdx.x] = make_float4(mx, se, bv, __int_as_float(bi));
-      } else {
-        // merge two lists sorted by (value desc, label asc): an entry's
-        // place is its index plus the other list's entries ordered before it
-        // (unfilled entries (-inf, INT_MAX) of both lists land on the same
-        // trailing places with the same contents)
-        float2* bp = d.bpart + ((size_t)gr * d.n_ptiles + blockIdx.x) * (1 + K);
-        bp[0] = make_float2(mx, se);
-        float ov[8];
-        int oi[8];
+      // merge two lists sorted by (value desc, label asc): an entry's
+      // place is its index plus the other list's entries ordered before it
+      // (unfilled entries (-inf, INT_MAX) of both lists land on the same
+      // trailing places with the same contents)
+      float2* bp = d.bpart + ((size_t)gr * d.n_ptiles + blockIdx.x) * (1 + K);
+      bp[0] = make_float2(mx, se);
+      float ov[8];
+      int oi[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) { ov[j] = xch[2 + 2 * j]; oi[j] = __float_as_int(xch[3 + 2 * j]); }
+      for (int j = 0; j < 8; ++j) { ov[j] = xch[2 + 2 * j]; oi[j] = __float_as_int(xch[3 + 2 * j]); }
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          if (i < K) {
-            int pa = i, pb = i;
+      for (int i = 0; i < 8; ++i) {
+        if (i < K) {
+          int pa = i, pb = i;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              if (j < K) {
-                pa += (ov[j] > tv[i] || (ov[j] == tv[i] && oi[j] < ti[i])) ? 1 : 0;
-                pb += (tv[j] > ov[i] || (tv[j] == ov[i] && ti[j] < oi[i])) ? 1 : 0;
-              }
+          for (int j = 0; j < 8; ++j) {
+            if (j < K) {
+              pa += (ov[j] > tv[i] || (ov[j] == tv[i] && oi[j] < ti[i])) ? 1 : 0;
+              pb += (tv[j] > ov[i] || (tv[j] == ov[i] && ti[j] < oi[i])) ? 1 : 0;
             }
-            if (pa < K) bp[1 + pa] = make_float2(tv[i], __int_as_float(ti[i]));
-            if (pb < K) bp[1 + pb] = make_float2(ov[i], __int_as_float(oi[i]));
           }
+          if (pa < K) bp[1 + pa] = make_float2(tv[i], __int_as_float(ti[i]));
+          if (pb < K) bp[1 + pb] = make_float2(ov[i], __int_as_float(oi[i]));
         }
       }
     }
@@ -401,29 +316,19 @@ int joint_tc_pick_bn(int M_max, int N_pad, int sms) {
 }
 
 cudaError_t joint_tc_prepare(JointTc* jt, const uint16_t* A, int M_pad, const uint16_t* Wt, int N_pad, int H, int bn,
-                             const float* bias, const float* logits) {
+                             const float* logits) {
   jt->bn = bn;
   if (!make_map(&jt->mapA, A, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, H, M_pad, kBK, kBM)) return cudaErrorInvalidValue;
   if (!make_map(&jt->mapB, Wt, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, H, N_pad, kBK, bn)) return cudaErrorInvalidValue;
-  if (!make_map(&jt->mapBias, bias, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, N_pad, M_pad, 32, kBM))
+  // pruned fusion stores no logits
+  if (logits && (!make_map(&jt->mapLogits, logits, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, N_pad, M_pad, 32, 32) ||
+                 !make_map(&jt->mapLogits16, logits, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, N_pad, M_pad, 32, 16)))
     return cudaErrorInvalidValue;
-  if (!make_map(&jt->mapLogits, logits ? logits : bias, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, N_pad, M_pad, 32, 32))
-    return cudaErrorInvalidValue;
-  if (!make_map(&jt->mapA64, A, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, H, M_pad, kBK, 64) ||
-      !make_map(&jt->mapLogits16, logits ? logits : bias, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, N_pad, M_pad, 32, 16))
-    return cudaErrorInvalidValue;
+  if (!make_map(&jt->mapA64, A, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, H, M_pad, kBK, 64)) return cudaErrorInvalidValue;
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaSuccess;
-  if (bn == 256) {
-    e = cudaFuncSetAttribute(k_joint_tc<256, false>, attr, Smem<256>::kBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_joint_tc<256, true>, attr, Smem<256>::kBytes);
-  } else if (bn == 128) {
-    e = cudaFuncSetAttribute(k_joint_tc<128, false>, attr, Smem<128>::kBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_joint_tc<128, true>, attr, Smem<128>::kBytes);
-  } else {
-    e = cudaFuncSetAttribute(k_joint_tc<64, false>, attr, Smem<64>::kBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_joint_tc<64, true>, attr, Smem<64>::kBytes);
-  }
+  cudaError_t e = bn == 256   ? cudaFuncSetAttribute(k_joint_tc<256>, attr, Smem<256>::kBytes)
+                  : bn == 128 ? cudaFuncSetAttribute(k_joint_tc<128>, attr, Smem<128>::kBytes)
+                              : cudaFuncSetAttribute(k_joint_tc<64>, attr, Smem<64>::kBytes);
   if (e == cudaSuccess) e = joint_greedy_prepare(bn);
   return e;
 }
@@ -432,13 +337,12 @@ namespace {
 template <int BN>
 void launch_bn(cudaLaunchConfig_t& cfg, const JointTc& jt, const DecView& d, int step) {
   cfg.dynamicSmemBytes = Smem<BN>::kBytes;
-  if (d.prune > 0) cudaLaunchKernelEx(&cfg, k_joint_tc<BN, true>, d, step, jt.mapA, jt.mapB, jt.mapBias);
-  else cudaLaunchKernelEx(&cfg, k_joint_tc<BN, false>, d, step, jt.mapA, jt.mapB, jt.mapBias);
+  cudaLaunchKernelEx(&cfg, k_joint_tc<BN>, d, step, jt.mapA, jt.mapB);
 }
 }  // namespace
 
 void launch_joint_tc(const JointTc& jt, const DecView& d, int M, int step, cudaStream_t s, bool pdl) {
-  if (d.fused || d.K > 1) {
+  if (d.prune == 0) {
     launch_joint_greedy(jt, d, M, step, s, pdl);
     return;
   }

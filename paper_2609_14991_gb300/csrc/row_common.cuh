@@ -71,6 +71,65 @@ __device__ __forceinline__ int warp_find(const int32_t* __restrict__ arr, int n,
   return m ? lo + __ffs((int)m) - 1 : -1;
 }
 
+// Aligned groups of four arcs a chain level's arcs [b, b + c) span.
+__device__ __forceinline__ int level_groups(int b, int c) { return c > 0 ? (b + c - (b & ~3) + 3) >> 2 : 0; }
+
+// Position of y in the sorted arr[0, n), or -1, by one warp: 32-ary probes
+// narrow the range to at most 124 entries, then one 16-byte load per lane
+// covers them, from the 16-byte boundary at or below arr + lo.  A window so
+// reads at most three entries before and after the range, inside the table
+// (its label arrays start 16-byte aligned and are padded by four).  At most
+// two dependent loads for n <= 3968.
+// PRE: `pre` holds this lane's first load (first_load below), made before y
+// was known.
+template <bool PRE>
+__device__ __forceinline__ int warp_find_wide(const int32_t* __restrict__ arr, int n, int y, int lane, int4 pre) {
+  reconverge();
+  int lo = 0, hi = n;
+  bool held = PRE;
+  while (hi - lo > 124) {
+    const int step = (hi - lo + 31) >> 5;
+    const int idx = lo + lane * step;
+    int v = pre.x;
+    if (!held) v = (idx < hi) ? __ldg(arr + idx) : INT_MAX;
+    held = false;
+    const unsigned m = __ballot_sync(0xffffffffu, v <= y);
+    if (m == 0) return -1;
+    lo = lo + (31 - __clz((int)m)) * step;
+    hi = min(hi, lo + step);
+  }
+  const uintptr_t at = reinterpret_cast<uintptr_t>(arr + lo);
+  const int4* g = reinterpret_cast<const int4*>(at & ~uintptr_t(15));
+  const int first = 4 * lane - (int)((at & 15u) >> 2);  // this lane's first entry, relative to lo
+  int pos = -1;
+  if (first < hi - lo) {
+    const int4 t = held ? pre : __ldg(g + lane);
+    const int tv[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+    for (int j = 3; j >= 0; --j)
+      if (first + j >= 0 && first + j < hi - lo && tv[j] == y) pos = lo + first + j;
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, pos >= 0);
+  return m ? __shfl_sync(0xffffffffu, pos, __ffs((int)m) - 1) : -1;
+}
+
+__device__ __forceinline__ int4 first_load(const int32_t* __restrict__ arr, int n, int lane) {
+  int4 t = make_int4(INT_MAX, INT_MAX, INT_MAX, INT_MAX);
+  if (n > 124) {
+    const int idx = lane * ((n + 31) >> 5);
+    if (idx < n) t.x = __ldg(arr + idx);
+  } else {
+    const uintptr_t at = reinterpret_cast<uintptr_t>(arr);
+    if (4 * lane - (int)((at & 15u) >> 2) < n) t = __ldg(reinterpret_cast<const int4*>(at & ~uintptr_t(15)) + lane);
+  }
+  return t;
+}
+
+// Reads a kernel parameter where it stands (a parameter's first use waits for
+// the constant cache).
+template <class T>
+__device__ __forceinline__ void touch(T* p) { asm volatile("" ::"l"(p)); }
+
 // Merges two softmax partials (max, sum of exp(x - max)).
 __device__ __forceinline__ void lse_merge(float& m, float& s, float m2, float s2) {
   if (m2 == kNegInf) return;

@@ -1,21 +1,31 @@
 // Row pass of the fused decode step with several n-gram LMs (Eq. 1, the sum
-// over LMs): one CTA per hypothesis row.  (Greedy decoding with at most one
-// LM runs row_fused.cu instead.)
+// over LMs), or one whose unigram states have no dense rows or whose weight is
+// not 1: one CTA per hypothesis row.  (Otherwise greedy decoding runs
+// row_stream.cu or row_fused.cu.)
 //
-// For row r at label step s it
-//   1. combines the joint kernel's per-tile partials of step s-1 into the
-//      log-sum-exp of the row and its best fused label (Eq. 1 argmax);
-//   2. applies the greedy decision: blank (or the per-frame label limit)
-//      advances the frame, a label is emitted and advances the LM state and
-//      the phrase-trie state;
-//   3. writes the joint input of step s, bf16(ReLU(enc_t + E[last])), and
-//   4. the dense fusion bias of step s, lambda*log p_LM(v|state) +
-//      beta*boost(v|trie state) for every label v (Eq. 1, terms 2 and 3).
+// The joint kernel before it wrote the row's logits and per-tile softmax
+// partials.  For row r at label step s the pass
+//   1. loads the row's state and chains, and 2. builds the fusion bias of
+//      Eq. 1, sum_i lambda w_i log p_i(v | state i) + beta * boost(v | trie
+//      state) for every label v, in shared memory, both before it waits for
+//      the joint kernel;
+//   3. takes the argmax of logit + bias (blank: its logit alone; ties to the
+//      lowest label): blank or the per-frame label limit advances the frame;
+//   4. writes the joint input of step s, bf16(ReLU(enc_t + E[last]));
+//   5. searches an emitted label in every chain element and 6. assembles the
+//      next chains, every hit carrying the next element's table record.
 //
 // LM state and phrase state are both kept as their whole suffix chain (one
 // LM state per order; every trie node that is a suffix of the current one),
 // so the next chain after label y is assembled from independent searches of
 // y in each chain element -- no dependent pointer chase.
+//
+// Bound by dependent round trips to L2 and barriers, not by bytes.  With the
+// bias built after the decision and added by the joint kernel's epilogue (a
+// dependent load and a barrier per level and LM between two joint kernels), a
+// chunk of 256 rows (2 LMs, V 1024, H 1024, 13 frames) took 898 us; built
+// while the joint kernel runs, with every LM's and node's first loads in one
+// round, 570.
 #include <algorithm>
 
 #include "row_common.cuh"
@@ -27,151 +37,49 @@ namespace {
 using row::best_merge;
 using row::kNegInf;
 using row::lse_merge;
-using row::warp_find;
-
-// Algorithmic bytes of a row's LM chain levels: each level's state record
-// and arcs, and (when a label was emitted) its search: one probe per halving
-// plus the arc found.
-__device__ unsigned long long lm_level_bytes(const row::ChainRecs& rc, int nl, bool searched) {
-  unsigned long long b = 0;
-  for (int l = 0; l < nl; ++l) {
-    b += 12 + 8ull * rc.lc[l];
-    if (searched) b += 8 + 4ull * (32 - __clz(rc.lc[l] + 1)) + 4;
-  }
-  return b;
-}
-
-// The fusion bias row with several LMs (Eq. 1, the sum over LMs): per LM its
-// chain levels deepest first into the scratch (a label keeps the first value
-// it gets), then acc[v] += alpha_i * (that value, or the backoff to the
-// unigram: the chain's summed backoff weights + log p_i(v)); the trie as in
-// the single-LM pass; brow[v] = acc[v] + beta * boost(v).  All threads of
-// the block call it; it returns thread 0's count of LM bytes (if counting).
-__device__ unsigned long long bias_multi(const DecView& d, int L, const int (*lm_chain)[kLmChain], const int* nl,
-                                         const int* tr_chain, int nt, row::ChainRecs& rc, float lam, float beta,
-                                         float* brow, float* lmv, float* acc, uint8_t* dep, bool counting,
-                                         bool searched) {
-  const int tid = threadIdx.x, step = blockDim.x, V = d.V, nq = d.V4 / 4;
-  unsigned long long bytes = 0;
-  if (tid >= 32 && tid - 32 < nt) {
-    const int q = tr_chain[tid - 32];
-    rc.tb[tid - 32] = __ldg(d.tr.nd_begin + q);
-    rc.tc[tid - 32] = __ldg(d.tr.nd_count + q);
-    rc.td[tid - 32] = __ldg(d.tr.nd_depth + q) + 1;
-  }
-  uint32_t* d4 = reinterpret_cast<uint32_t*>(dep);
-  float4* l4 = reinterpret_cast<float4*>(lmv);
-  float4* a4 = reinterpret_cast<float4*>(acc);
-  for (int q = tid; q < nq; q += step) d4[q] = 0u;
-  const float unset = row::unset_value();
-  for (int m = 0; m < L; ++m) {
-    const int n = nl[m];
-    if (tid < n) {
-      const int st = lm_chain[m][tid];
-      rc.lb[tid] = __ldg(TSD_LMX(d, m, st_begin) + st);
-      rc.lc[tid] = __ldg(TSD_LMX(d, m, st_count) + st);
-      rc.lo[tid] = __ldg(TSD_LMX(d, m, st_cum) + st);
-    }
-    for (int q = tid; q < nq; q += step) l4[q] = make_float4(unset, unset, unset, unset);
-    row::block_sync();
-    const float cum_top = n ? rc.lo[n - 1] : 0.f;
-    const int32_t* arc_tok = TSD_LMX(d, m, arc_tok);
-    const float* arc_logp = TSD_LMX(d, m, arc_logp);
-    for (int p = 0; p < n; ++p) {
-      const int l = n - 1 - p;
-      row::scatter_lm_level(arc_tok, arc_logp, rc.lb[l], rc.lb[l] + rc.lc[l], cum_top - rc.lo[l], lmv);
-      row::block_sync();
-    }
-    if (counting && tid == 0) bytes += lm_level_bytes(rc, n, searched);
-    const float alpha = lam * row::lm_pick(m, d.lm_w[0], d.lm_w[1], d.lm_w[2], d.lm_w[3]);
-    const float4* u4 = reinterpret_cast<const float4*>(TSD_LMX(d, m, uni_logp));  // padded past V
-    for (int q = tid; q < nq; q += step) {
-      const float4 l = l4[q];
-      const float4 u = __ldg(u4 + q);
-      float4 a = (m == 0) ? make_float4(0.f, 0.f, 0.f, 0.f) : a4[q];
-      a.x += alpha * (isnan(l.x) ? u.x + cum_top : l.x);
-      a.y += alpha * (isnan(l.y) ? u.y + cum_top : l.y);
-      a.z += alpha * (isnan(l.z) ? u.z + cum_top : l.z);
-      a.w += alpha * (isnan(l.w) ? u.w + cum_top : l.w);
-      a4[q] = a;
-    }
-    row::block_sync();  // the scratch and the records are reused by the next LM
-  }
-  for (int p = 0; p < nt; ++p) {
-    const int k = nt - 1 - p;
-    row::scatter_trie_node(d.tr.ch_tok, rc.tb[k], rc.tb[k] + rc.tc[k], (uint8_t)rc.td[k], dep);
-    row::block_sync();
-  }
-  const int depth_cur = nt ? rc.td[0] - 1 : 0;
-  const float bscale = beta * (d.has_tr ? d.tr.bonus : 0.f);
-  const float tr_base = -bscale * (float)depth_cur;
-  float4* b4 = reinterpret_cast<float4*>(brow);
-  for (int q = tid; q < nq; q += step) {
-    const float4 a = a4[q];
-    const uint32_t dd = d4[q];
-    const uint32_t rb = __ldg(d.droot + (q >> 3)) >> ((4 * q) & 31);
-    const float av[4] = {a.x, a.y, a.z, a.w};
-    float o[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int dj = (dd >> (8 * j)) & 0xff;
-      const float btr = dj ? bscale * (float)(dj - depth_cur) : (((rb >> j) & 1u) ? bscale : 0.f) + tr_base;
-      o[j] = (4 * q + j < V) ? av[j] + btr : 0.f;
-    }
-    b4[q] = make_float4(o[0], o[1], o[2], o[3]);
-  }
-  if (tid == 0) brow[V] = 0.f;
-  return bytes;
-}
 
 // mode: 0 = label step, 1 = final step (apply the last decision only),
 // 2 = replay (redo the step's work without committing any state or output;
 // used only to time the kernel in isolation).
-// VAR bit 0: the stateful form (LSTM input rows instead of the joint input);
-// bit 1: several LMs; bit 2: few rows (at most two CTAs per SM are needed,
-// so the kernel may use registers freely instead of fitting seven per SM).
-// Each combination is its own instantiation, so the common ones carry none
-// of the other paths' code or registers.
-template <int VAR>
-__global__ void __launch_bounds__(kRowThreads, (VAR & 4) ? 2 : 7) k_row(DecView d, int step, int mode) {
-  constexpr bool PRED = (VAR & 1) != 0, MULTI = (VAR & 2) != 0;
+// L: LMs fused.
+template <int L>
+__global__ void __launch_bounds__(kRowThreads, 3) k_row(DecView d, int step, int mode) {
   const Params* __restrict__ P = d.params;
   const int r = blockIdx.x;
   const int V = d.V;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int kWarps = kRowThreads / 32;
   const bool commit = (mode != 2);
+  const bool counting = (mode == 2 || d.count);
   extern __shared__ __align__(16) unsigned char smem[];
-  // per-label scratch: LM value from the chain (NaN unset), with several LMs
-  // also their weighted sum, then the trie depth of the goto
-  const int L = (MULTI && d.n_lm > 1) ? d.n_lm : 1;  // LM state blocks (1 without an LM)
+  // per label: the LM value from one LM's chain (NaN: none), the bias (with
+  // one LM in the same place), the trie goto depth (0: none)
   float* lmv = reinterpret_cast<float*>(smem);
-  float* acc = lmv + d.V4;
-  uint8_t* dep = reinterpret_cast<uint8_t*>(lmv + (L > 1 ? 2 : 1) * d.V4);
+  float* bias = L > 1 ? lmv + d.V4 : lmv;
+  uint8_t* dep = reinterpret_cast<uint8_t*>(bias + d.V4);
 
-  __shared__ int s_t, s_sym, s_cnt, s_y, s_tr_len, s_last, s_slot, s_T;
-  __shared__ int s_lm_len[kMaxLm];
-  // the call's parameters, read once before the dependency wait
+  __shared__ int s_t, s_sym, s_cnt, s_last, s_slot, s_T, s_n, s_nt;
+  __shared__ int s_nl[L];
   __shared__ int32_t* s_out_tok;
   __shared__ int32_t* s_out_frame;
   __shared__ float* s_out_score;
   __shared__ int32_t* s_out_count;
   __shared__ const uint16_t* s_enc;
-  __shared__ float s_lam, s_beta;
-  __shared__ int s_n;
-  __shared__ float s_score;
-  __shared__ int s_lm[kMaxLm][kLmChain], s_tr[kTrChain];
-  __shared__ int s_lm_tgt[kMaxLm][kLmChain];    // target state of y's arc at each LM level (-2 none)
-  __shared__ int s_tr_node[kTrChain], s_tr_nxt[kTrChain];  // child by y of each trie chain node (-1 none)
-  __shared__ int s_uni_tgt[kMaxLm], s_root_child, s_root_next;
-  __shared__ row::ChainRecs rc;   // records of the chains the bias row is built from
-  __shared__ row::ChainRecs rco;  // one LM: records of the current chains, kept with the state
+  __shared__ float s_lam, s_beta, s_lse;
+  __shared__ int s_lm[L][kLmChain], s_tr[kTrChain];
+  __shared__ int4 s_lmr[L][kLmChain];     // LM chain records: (first arc, arcs, summed backoff bits, -)
+  __shared__ int4 s_trr[kTrChain];        // trie chain records: (first child, children, depth of the children, -)
+  __shared__ int4 s_lm_hit[L][kLmChain];  // target record of y's arc at each old level (x = -2: none)
+  __shared__ int4 s_tr_hit[kTrChain];     // child record of y at each old trie node (x = -1: none)
+  __shared__ float s_bv[kWarps];
+  __shared__ int s_bi[kWarps];
+  __shared__ unsigned long long s_bytes;
 
-  // The row state below was written by the previous row pass; under
-  // programmatic launch this grid may start before its own wait, so these
-  // loads go through L2 only (ld.global.cg), never a possibly stale L1 line.
+  // 1. Row state, written by the previous row pass: under programmatic launch
+  // this grid may start before its own wait, so these loads go through L2
+  // only (ld.global.cg), never a possibly stale L1 line.
   if (tid == 0) {
-    const int slot = __ldcg(P->slots + r);
-    s_slot = slot;
+    s_slot = __ldcg(P->slots + r);
     s_T = __ldcg(&P->T);
     s_out_tok = P->out_tok;
     s_out_frame = P->out_frame;
@@ -181,311 +89,423 @@ __global__ void __launch_bounds__(kRowThreads, (VAR & 4) ? 2 : 7) k_row(DecView 
     s_lam = P->lambda;
     s_beta = P->beta;
     s_n = P->n;
-    if (step == 0) {
-      s_t = 0; s_sym = 0; s_cnt = 0;
-    } else {
-      s_t = __ldcg(d.r_t + r); s_sym = __ldcg(d.r_sym + r); s_cnt = __ldcg(d.r_cnt + r);
-    }
-    for (int i = 0; i < L; ++i) s_lm_len[i] = d.has_lm ? __ldcg(d.s_lm_len + i * d.lm_stride + slot) : 0;
-    s_tr_len = d.has_tr ? __ldcg(d.s_tr_len + slot) : 0;
-    s_last = __ldcg(d.s_last + slot);
+    s_bytes = 0;
+    s_t = step ? __ldcg(d.r_t + r) : 0;
+    s_sym = step ? __ldcg(d.r_sym + r) : 0;
+    s_cnt = step ? __ldcg(d.r_cnt + r) : 0;
   }
   row::block_sync();
   const int slot = s_slot, T = s_T;
-  if (tid < L * kLmChain) {
+  if (tid < L * kLmChain) {  // the chains whole: their arrays have room for the longest
     const int i = tid / kLmChain, l = tid % kLmChain;
-    if (l < s_lm_len[i]) {
-      s_lm[i][l] = __ldcg(d.s_lm_chain + ((size_t)i * d.lm_stride + slot) * kLmChain + l);
-      if (L == 1) {
-        const int4 q = __ldcg(d.s_lm_rec + (size_t)slot * kLmChain + l);
-        rco.lb[l] = q.x;
-        rco.lc[l] = q.y;
-      }
-    }
+    const size_t at = ((size_t)i * d.lm_stride + slot) * kLmChain + l;
+    s_lm[i][l] = __ldcg(d.s_lm_chain + at);
+    s_lmr[i][l] = __ldcg(d.s_lm_rec + at);
+  } else if (tid >= 64 && tid < 64 + L) {
+    s_nl[tid - 64] = __ldcg(d.s_lm_len + (size_t)(tid - 64) * d.lm_stride + slot);
+  } else if (tid == 96) {
+    s_nt = d.has_tr ? __ldcg(d.s_tr_len + slot) : 0;
+    s_last = __ldcg(d.s_last + slot);
+  } else if (tid >= 128 && tid < 128 + kTrChain && d.has_tr) {
+    s_tr[tid - 128] = __ldcg(d.s_tr_chain + (size_t)slot * kTrChain + tid - 128);
+    s_trr[tid - 128] = __ldcg(d.s_tr_rec + (size_t)slot * kTrChain + tid - 128);
   }
-  if (tid >= 64 && tid - 64 < s_tr_len) {
-    const int k = tid - 64;
-    s_tr[k] = __ldcg(d.s_tr_chain + slot * kTrChain + k);
-    if (L == 1) {
-      const int4 q = __ldcg(d.s_tr_rec + (size_t)slot * kTrChain + k);
-      rco.tb[k] = q.x;
-      rco.tc[k] = q.y;
+  const int nq = d.V4 / 4;
+  const float unset = row::unset_value();
+  {
+    float4* l4 = reinterpret_cast<float4*>(lmv);
+    uint32_t* d4 = reinterpret_cast<uint32_t*>(dep);
+    for (int q = tid; q < nq; q += kRowThreads) {
+      l4[q] = make_float4(unset, unset, unset, unset);
+      d4[q] = 0u;
     }
-  }
-  // The encoder frames this step can use (t, or t+1 after a frame advance)
-  // go to L1 now, while the previous kernel still runs: no kernel of the
-  // chunk writes them.  (The call's bias defaults are not prefetched: every
-  // row would ask the same L2 lines for them at once.)
-  if (s_t < T) {
-    const size_t fb = (size_t)d.H * 2;
-    const uint16_t* f0 = s_enc + ((size_t)r * T + s_t) * d.H;
-    row::prefetch_span(f0, s_t + 1 < T ? 2 * fb : fb, 0);
   }
   row::block_sync();
-  // In replay mode every row redoes a full step (decision, advance, joint
-  // input, bias) even if it had finished the chunk, so the timing is that of
-  // a mid-chunk step.
+  // the encoder frames this step can use go to L1
+  if (s_t < T) {
+    const size_t fb = (size_t)d.H * 2;
+    row::prefetch_span(s_enc + ((size_t)r * T + s_t) * d.H, s_t + 1 < T ? 2 * fb : fb, 0);
+  }
+  // In replay mode every row redoes a full step even if it had finished.
   const bool evaluated = (step > 0) && (s_t < T || !commit);
+  const int nt = s_nt;
+  int ntask = nt;  // chain elements over all LMs and the trie
+#pragma unroll
+  for (int i = 0; i < L; ++i) ntask += s_nl[i];
+  // chain element `task`: (LM or -1, its level or node), its record and its labels
+  auto element = [&](int task, int& i, int& k, int4& rec) -> const int32_t* {
+#pragma unroll
+    for (i = 0; i < L; ++i) {
+      if (task < s_nl[i]) {
+        k = task;
+        rec = s_lmr[i][k];
+        return TSD_LMX(d, i, arc_tok) + rec.x;
+      }
+      task -= s_nl[i];
+    }
+    i = -1;
+    k = task;
+    rec = s_trr[k];
+    return d.tr.ch_tok + rec.x;
+  };
+  const float lam = s_lam;
+  int4 pre = make_int4(0, 0, 0, 0);
+  if (evaluated) {
+    // 2. the bias row.  Every LM's first arc group and unigram quad per
+    //    thread, each trie node's first children and the first search's first
+    //    load go out together
+    int4 ht[L];
+    float4 hp[L], hu[L];
+    int hl[L], hi[L], G[L];
+#pragma unroll
+    for (int i = 0; i < L; ++i) {
+      G[i] = 0;
+      hl[i] = -1;
+      hi[i] = 0;
+      int g = tid;
+      for (int l = 0; l < s_nl[i]; ++l) {  // arc groups in level order
+        const int4 c = s_lmr[i][l];
+        const int n = row::level_groups(c.x, c.y);
+        if (g >= 0 && g < n) {
+          hl[i] = l;
+          hi[i] = (c.x & ~3) + 4 * g;
+        }
+        g -= n;
+        G[i] += n;
+      }
+      if (hl[i] >= 0) {
+        ht[i] = __ldg(reinterpret_cast<const int4*>(d.lmx[i].arc_tok + hi[i]));
+        hp[i] = __ldg(reinterpret_cast<const float4*>(d.lmx[i].arc_logp + hi[i]));
+      }
+      if (tid < nq) hu[i] = __ldg(reinterpret_cast<const float4*>(d.lmx[i].uni_logp) + tid);  // padded past V
+    }
+    int4 ct = make_int4(0, 0, 0, 0);
+    if (warp < nt && lane < row::level_groups(s_trr[warp].x, s_trr[warp].y))
+      ct = __ldg(reinterpret_cast<const int4*>(d.tr.ch_tok) + (s_trr[warp].x >> 2) + lane);
+    if (warp < ntask) {
+      int i, k;
+      int4 rec;
+      const int32_t* arr = element(warp, i, k, rec);
+      pre = row::first_load(arr, rec.y, lane);
+    }
+    // the trie nodes shallowest first (the deepest overwrites), one before each barrier
+    int tk = nt - 1;
+    auto next_trie = [&]() {
+      if (tk < 0) return;
+      const int k = tk--;
+      const int b = s_trr[k].x, e = b + s_trr[k].y, a0 = b & ~3;
+      const uint8_t dd = (uint8_t)s_trr[k].z;
+      auto put = [&](int i0, int4 t) {
+        if (i0 >= b && i0 < e) dep[t.x] = dd;
+        if (i0 + 1 >= b && i0 + 1 < e) dep[t.y] = dd;
+        if (i0 + 2 >= b && i0 + 2 < e) dep[t.z] = dd;
+        if (i0 + 3 >= b && i0 + 3 < e) dep[t.w] = dd;
+      };
+      if (warp == k) put(a0 + 4 * lane, ct);
+      for (int g = (k < kWarps ? 32 : 0) + tid; a0 + 4 * g < e; g += kRowThreads)
+        put(a0 + 4 * g, __ldg(reinterpret_cast<const int4*>(d.tr.ch_tok + a0) + g));
+    };
+    float4* l4 = reinterpret_cast<float4*>(lmv);
+    float4* b4 = reinterpret_cast<float4*>(bias);
+    const uint32_t* d4 = reinterpret_cast<const uint32_t*>(dep);
+    const int depth_cur = nt ? s_trr[0].z - 1 : 0;
+    const float bscale = s_beta * (d.has_tr ? d.tr.bonus : 0.f);
+    const float tr_base = -bscale * (float)depth_cur;
+#pragma unroll
+    for (int i = 0; i < L; ++i) {
+      const int n = s_nl[i];
+      const float cum_top = n ? __int_as_float(s_lmr[i][n - 1].z) : 0.f;
+      // the levels deepest first: a label keeps the first value it gets
+      int end = G[i];
+      for (int l = n - 1; l >= 0; --l) {
+        const int4 c = s_lmr[i][l];
+        const int b = c.x, e = c.x + c.y, first = end - row::level_groups(c.x, c.y);
+        const float off = cum_top - __int_as_float(c.z);
+        auto put = [&](int i0, int4 t, float4 v) {
+          if (i0 >= b && i0 < e && isnan(lmv[t.x])) lmv[t.x] = off + v.x;
+          if (i0 + 1 >= b && i0 + 1 < e && isnan(lmv[t.y])) lmv[t.y] = off + v.y;
+          if (i0 + 2 >= b && i0 + 2 < e && isnan(lmv[t.z])) lmv[t.z] = off + v.z;
+          if (i0 + 3 >= b && i0 + 3 < e && isnan(lmv[t.w])) lmv[t.w] = off + v.w;
+        };
+        if (hl[i] == l) put(hi[i], ht[i], hp[i]);
+        for (int g = max(first, kRowThreads) + tid; g < end; g += kRowThreads) {  // past what registers hold
+          const int i0 = (b & ~3) + 4 * (g - first);
+          put(i0, __ldg(reinterpret_cast<const int4*>(d.lmx[i].arc_tok + i0)),
+              __ldg(reinterpret_cast<const float4*>(d.lmx[i].arc_logp + i0)));
+        }
+        end = first;
+        next_trie();
+        row::block_sync();
+      }
+      if (i == L - 1) {
+        while (tk >= 0) {
+          next_trie();
+          row::block_sync();
+        }
+      }
+      const float alpha = lam * d.lm_w[i];
+      for (int q = tid; q < nq; q += kRowThreads) {
+        const float4 l = l4[q];
+        const float4 u = q == tid ? hu[i] : __ldg(reinterpret_cast<const float4*>(d.lmx[i].uni_logp) + q);
+        float4 a = i == 0 ? make_float4(0.f, 0.f, 0.f, 0.f) : b4[q];
+        a.x += alpha * (isnan(l.x) ? u.x + cum_top : l.x);
+        a.y += alpha * (isnan(l.y) ? u.y + cum_top : l.y);
+        a.z += alpha * (isnan(l.z) ? u.z + cum_top : l.z);
+        a.w += alpha * (isnan(l.w) ? u.w + cum_top : l.w);
+        if (i == L - 1) {
+          const uint32_t dd = d4[q];
+          const uint32_t rb = __ldg(d.droot + (q >> 3)) >> ((4 * q) & 31);
+          auto boost = [&](int j) {
+            const int dj = (dd >> (8 * j)) & 0xff;
+            return dj ? bscale * (float)(dj - depth_cur) : (((rb >> j) & 1u) ? bscale : 0.f) + tr_base;
+          };
+          a.x += boost(0);
+          a.y += boost(1);
+          a.z += boost(2);
+          a.w += boost(3);
+        } else {
+          l4[q] = make_float4(unset, unset, unset, unset);
+        }
+        b4[q] = a;
+      }
+      if (i < L - 1) row::block_sync();
+    }
+  }
+  // the parameters used after the wait go through the constant cache once now
+  row::touch(d.logits); row::touch(d.part); row::touch(d.E); row::touch(d.A); row::touch(d.tr.root_rec);
+  row::touch(d.tr.ch_rec); row::touch(d.r_t); row::touch(d.r_sym); row::touch(d.r_cnt); row::touch(d.cap_rows);
   // Programmatic dependent launch: everything above reads only state the
-  // previous row pass wrote, which had completed before the joint kernel in
-  // between let this grid launch; the joint's partials need the wait.
+  // previous row pass wrote (complete before the joint kernel in between let
+  // this grid launch) and constant tables; the logits need the wait.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
+  int y = V;
+  float best = 0.f;
   if (evaluated) {
-    // 1. combine the partials of the previous joint step
-    if (warp == 0) {
-      float m = kNegInf, s = 0.f, bv = kNegInf;
-      int bi = INT_MAX;
-      const float4* pr = d.part + (size_t)r * d.n_ptiles;
-      for (int j = lane; j < d.n_ptiles; j += 32) {
-        float4 p = __ldcg(pr + j);  // written by the joint kernel just before
-        lse_merge(m, s, p.x, p.y);
-        best_merge(bv, bi, p.z, __float_as_int(p.w));
+    // 3. the argmax of logit + bias (blank: its logit alone), each thread over
+    //    the quads whose bias it wrote
+    const float* lg = d.logits + (size_t)r * d.N_pad;
+    float bv = kNegInf;
+    int bi = INT_MAX;
+    const float4* l4 = reinterpret_cast<const float4*>(lg);
+    const float4* b4 = reinterpret_cast<const float4*>(bias);
+    for (int q0 = tid; q0 < nq; q0 += 2 * kRowThreads) {
+      float4 lq[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (q0 + u * kRowThreads < nq) lq[u] = __ldcg(l4 + q0 + u * kRowThreads);
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int q = q0 + u * kRowThreads;
+        if (q >= nq) break;
+        const float4 b = b4[q];
+        const float f[4] = {lq[u].x + b.x, lq[u].y + b.y, lq[u].z + b.z, lq[u].w + b.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (4 * q + j < V && f[j] > bv) { bv = f[j]; bi = 4 * q + j; }
+      }
+    }
+    if (tid == 0) {
+      const float fb = __ldcg(lg + V);
+      if (fb > bv) { bv = fb; bi = V; }
+    }
+    row::reconverge();
+    for (int o = 16; o > 0; o >>= 1) {
+      const float v2 = __shfl_xor_sync(0xffffffffu, bv, o);
+      const int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
+      best_merge(bv, bi, v2, i2);
+    }
+    if (lane == 0) {
+      s_bv[warp] = bv;
+      s_bi[warp] = bi;
+    }
+    if (counting && tid == 0) {
+      // Algorithmic bytes: the row's logits and partials, the state read and
+      // written, every arc of every LM level and every child of every trie
+      // node with its record; searches and the joint input below.
+      unsigned long long ab = 4ull * (V + 1) + 16ull * d.n_ptiles + 2ull * (24 + 4 * ntask);
+#pragma unroll
+      for (int i = 0; i < L; ++i)
+        for (int l = 0; l < s_nl[i]; ++l) ab += 16 + 8ull * s_lmr[i][l].y;
+      for (int k = 0; k < nt; ++k) ab += 16 + 4ull * s_trr[k].y;
+      s_bytes = ab;
+    }
+    row::block_sync();
+    best = s_bv[0];
+    int bix = s_bi[0];
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) best_merge(best, bix, s_bv[w], s_bi[w]);
+    y = (bix >= 0 && bix <= V) ? bix : V;
+  }
+  // the frame, the labels in it and the last label after the decision
+  const bool label = evaluated && y != V;
+  int t1 = s_t, sym1 = s_sym;
+  if (label) {
+    if (++sym1 >= d.max_sym) { ++t1; sym1 = 0; }
+  } else if (evaluated) {
+    ++t1;
+    sym1 = 0;
+  }
+  const int last1 = label ? y : s_last;
+  const int t = commit ? t1 : min(t1, T - 1);
+  const bool next = mode != 1 && t < T;  // another label step follows
+  // 4. the joint input of this step: its loads go out before the searches'
+  const uint4* enc_row = reinterpret_cast<const uint4*>(s_enc + ((size_t)r * T + t) * d.H);
+  const uint4* emb_row = reinterpret_cast<const uint4*>(d.E + (size_t)last1 * d.H);
+  uint4 jx, jz;
+  if (next && tid < d.H / 8) {
+    jx = row::load_now(enc_row + tid);
+    jz = row::load_now(emb_row + tid);
+  }
+  int4 own = make_int4(-1, 0, 0, 0);  // y's unigram state in LM `warp`, y's child of the root (warp L)
+  if (label) {
+    // 5. independent searches of y in every chain element; each hit's record
+    //    is the next chain element's
+    if (warp < L) {
+      if (TSD_LMX(d, warp, order) >= 2) own = __ldg(TSD_LMX(d, warp, uni_rec) + y);
+    } else if (warp == L) {
+      own = d.has_tr ? __ldg(d.tr.root_rec + y) : make_int4(0, 0, 0, 0);
+    }
+    const float4* pr = d.part + (size_t)r * d.n_ptiles;
+    float4 p0 = make_float4(kNegInf, 0.f, 0.f, 0.f);
+    if (warp == kWarps - 1 && lane < d.n_ptiles) p0 = __ldcg(pr + lane);  // written by the joint kernel
+    for (int task = warp; task < ntask; task += kWarps) {
+      int i, k;
+      int4 rec;
+      const int32_t* arr = element(task, i, k, rec);
+      const int at = task == warp ? row::warp_find_wide<true>(arr, rec.y, y, lane, pre)
+                                  : row::warp_find_wide<false>(arr, rec.y, y, lane, pre);
+      if (lane == 0) {
+        if (i >= 0) s_lm_hit[i][k] = at >= 0 ? __ldg(TSD_LMX(d, i, arc_rec) + rec.x + at) : make_int4(-2, 0, 0, 0);
+        else s_tr_hit[k] = at >= 0 ? __ldg(d.tr.ch_rec + rec.x + at) : make_int4(-1, 0, 0, 0);
+        if (counting) atomicAdd(&s_bytes, 4ull * (32 - __clz(rec.y + 1)) + 16);
+      }
+    }
+    if (warp == kWarps - 1) {  // the log-sum-exp of the raw logits
+      float pm = kNegInf, ps = 0.f;
+      lse_merge(pm, ps, p0.x, p0.y);
+      for (int j = lane + 32; j < d.n_ptiles; j += 32) {
+        const float4 p = __ldcg(pr + j);
+        lse_merge(pm, ps, p.x, p.y);
       }
       row::reconverge();
       for (int o = 16; o > 0; o >>= 1) {
-        float m2 = __shfl_xor_sync(0xffffffffu, m, o);
-        float s2 = __shfl_xor_sync(0xffffffffu, s, o);
-        float v2 = __shfl_xor_sync(0xffffffffu, bv, o);
-        int i2 = __shfl_xor_sync(0xffffffffu, bi, o);
-        lse_merge(m, s, m2, s2);
-        best_merge(bv, bi, v2, i2);
+        const float m2 = __shfl_xor_sync(0xffffffffu, pm, o);
+        const float s2 = __shfl_xor_sync(0xffffffffu, ps, o);
+        lse_merge(pm, ps, m2, s2);
       }
-      if (lane == 0) {
-        s_y = (bi >= 0 && bi <= V) ? bi : V;
-        s_score = bv - (m + logf(s));
-      }
+      if (lane == 0) s_lse = pm + logf(ps);
     }
+  }
+  if (next) {
+    uint4* a = reinterpret_cast<uint4*>(d.A + (size_t)r * d.H);
+    if (tid < d.H / 8) a[tid] = row::joint_input(jx, jz);
+    for (int i = tid + kRowThreads; i < d.H / 8; i += kRowThreads)
+      a[i] = row::joint_input(__ldg(enc_row + i), __ldg(emb_row + i));
+  }
+  if (label) {
     row::block_sync();
-    const int y = s_y;
-    row::prefetch_span(d.E + (size_t)(y != V ? y : s_last) * d.H, (size_t)d.H * 2, 32);  // this step's E row
-    if (y != V) {
-      // 2a. independent searches of y in every chain element, each warp
-      //     also fetching what the new chain needs from the arc it found
-      int nl = 0;  // chain elements over all LMs
-      for (int i = 0; i < L; ++i) nl += s_lm_len[i];
-      const int nt = s_tr_len;
-      if (tid == kRowThreads - 1) {
-        s_root_child = d.has_tr ? __ldg(d.tr.root_child + y) : 0;
-        s_root_next = d.has_tr ? __ldg(d.tr.root_next + y) : 0;
-      } else if (tid >= kRowThreads - 1 - L) {
-        const int i = tid - (kRowThreads - 1 - L);
-        s_uni_tgt[i] = (d.has_lm && TSD_LMX(d, i, order) >= 2) ? __ldg(TSD_LMX(d, i, uni_tgt) + y) : -1;
-      }
-      for (int task = warp; task < nl + nt; task += kRowThreads / 32) {
-        if (task < nl) {
-          int m = 0, l = task;  // LM m, level l
-          while (l >= s_lm_len[m]) l -= s_lm_len[m++];
-          const int32_t* st_begin = TSD_LMX(d, m, st_begin);
-          const int32_t* st_count = TSD_LMX(d, m, st_count);
-          const int32_t* arc_tgt = TSD_LMX(d, m, arc_tgt);
-          int b, c;
-          if (L == 1) {  // records kept with the chain
-            b = rco.lb[l];
-            c = rco.lc[l];
-          } else {
-            const int st = s_lm[m][l];
-            b = __ldg(st_begin + st);
-            c = __ldg(st_count + st);
-          }
-          int i = warp_find(TSD_LMX(d, m, arc_tok) + b, c, y, lane);
-          if (lane == 0) {
-            const int tg = (i >= 0) ? __ldg(arc_tgt + b + i) : -2;
-            s_lm_tgt[m][l] = tg;
-            if (tg >= 0) {  // the new chain's state records
-              row::prefetch_l1(st_begin + tg);
-              row::prefetch_l1(st_count + tg);
-              row::prefetch_l1(TSD_LMX(d, m, st_cum) + tg);
-            }
-          }
-        } else {
-          int k = task - nl;
-          int b, c;
-          if (L == 1) {
-            b = rco.tb[k];
-            c = rco.tc[k];
-          } else {
-            const int q = s_tr[k];
-            b = __ldg(d.tr.nd_begin + q);
-            c = __ldg(d.tr.nd_count + q);
-          }
-          int i = warp_find(d.tr.ch_tok + b, c, y, lane);
-          if (lane == 0) {
-            s_tr_node[k] = (i >= 0) ? __ldg(d.tr.ch_node + b + i) : -1;
-            if (i >= 0) {
-              const int nd = s_tr_node[k];
-              row::prefetch_l1(d.tr.nd_begin + nd);
-              row::prefetch_l1(d.tr.nd_count + nd);
-              row::prefetch_l1(d.tr.nd_depth + nd);
-            }
-            s_tr_nxt[k] = (i >= 0) ? __ldg(d.tr.ch_next + b + i) : -1;
-          }
-        }
-      }
-      row::block_sync();
-      // 2b. assemble the new chains (shared memory only) and emit
-      if (tid == 0) {
-        // each LM: y's unigram state, then the target of y's arc at every
-        // level of the old chain up to the first level without one (the old
-        // chain's arc targets are in s_lm_tgt, so the new chain is written
-        // over the old one in place)
-        for (int m = 0; m < L; ++m) {
-          const int nold = s_lm_len[m];
-          int ln = 0;
-          if (s_uni_tgt[m] >= 0) {
-            s_lm[m][ln++] = s_uni_tgt[m];
-            for (int l = 0; l < nold && ln < kLmChain; ++l) {
-              const int tgt = s_lm_tgt[m][l];
-              if (tgt < 0) break;  // no arc at this level (-2) or the top order (-1)
-              s_lm[m][ln++] = tgt;
-            }
-          }
-          s_lm_len[m] = ln;
+    // 6. the new chains: warp i LM i (y's unigram state, then the targets of
+    //    y's arcs at the old levels up to the first level without one), warp
+    //    L the trie (y's children of the old nodes, deepest first, then the
+    //    root's; completing a phrase resets it)
+    if (warp < L) {
+      const int i = warp;
+      int ln = 0;
+      if (TSD_LMX(d, i, order) >= 2) {
+        const int4 h = lane < s_nl[i] ? s_lm_hit[i][lane] : make_int4(-2, 0, 0, 0);
+        const unsigned miss = __ballot_sync(0xffffffffu, h.x < 0);
+        ln = 1 + min(miss ? __ffs((int)miss) - 1 : 32, kLmChain - 1);
+        // lane l >= 1 takes the hit of old level l - 1
+        const int px = __shfl_up_sync(0xffffffffu, h.x, 1), py = __shfl_up_sync(0xffffffffu, h.y, 1);
+        const int pz = __shfl_up_sync(0xffffffffu, h.z, 1), pw = __shfl_up_sync(0xffffffffu, h.w, 1);
+        if (lane < ln) {
+          const int nst = lane == 0 ? 1 + y : px;
+          s_lm[i][lane] = nst;
           if (commit) {
-            int32_t* ch = d.s_lm_chain + ((size_t)m * d.lm_stride + slot) * kLmChain;
-            for (int l = 0; l < ln; ++l) ch[l] = s_lm[m][l];
-            if (d.has_lm) d.s_lm_len[m * d.lm_stride + slot] = ln;
+            const size_t at = ((size_t)i * d.lm_stride + slot) * kLmChain + lane;
+            d.s_lm_chain[at] = nst;
+            d.s_lm_rec[at] = lane == 0 ? make_int4(own.y, own.z, own.w, own.x) : make_int4(py, pz, pw, 0);
           }
         }
-        int tn = 0;
-        bool reset = false;
-        for (int i = 0; i < nt; ++i) {
-          if (s_tr_node[i] < 0) continue;
-          if (tn == 0 && s_tr_nxt[i] == 0) reset = true;
-          if (tn < kTrChain) s_tr[tn++] = s_tr_node[i];
-        }
-        if (s_root_child != 0) {
-          if (tn == 0 && s_root_next == 0) reset = true;
-          if (tn < kTrChain) s_tr[tn++] = s_root_child;
-        }
-        if (reset) tn = 0;
-        s_tr_len = tn;
+      }
+      __syncwarp();
+      if (lane == 0) {
+        s_nl[i] = ln;
+        if (commit) d.s_lm_len[(size_t)i * d.lm_stride + slot] = ln;
+      }
+    } else if (warp == L) {
+      const int4 h = lane < nt ? s_tr_hit[lane] : make_int4(-1, 0, 0, 0);
+      const int dd = lane < nt ? s_trr[lane].z + 1 : 0;  // the child's children sit one deeper
+      const unsigned vm = __ballot_sync(0xffffffffu, h.x >= 0);
+      const int nv = __popc(vm);
+      const bool root = own.x != 0;
+      // the first element of the new chain ends a phrase: the chain resets
+      const int f = __ffs((int)vm) - 1;
+      const int fy = __shfl_sync(0xffffffffu, h.y, f < 0 ? 0 : f);
+      const bool reset = nv > 0 ? fy == 0 : (root && own.y == 0);
+      const int tn = reset ? 0 : min(nv + (root ? 1 : 0), kTrChain);
+      const int pos = __popc(vm & ((1u << lane) - 1u));
+      auto put = [&](int p, int node, int4 rec) {
+        if (p == 0) s_tr[0] = node;
         if (commit) {
-          for (int l = 0; l < tn; ++l) d.s_tr_chain[slot * kTrChain + l] = s_tr[l];
-          if (d.has_tr) d.s_tr_len[slot] = tn;
-          const int cap = T * d.max_sym;
-          const int o = r * cap + s_cnt;
-          s_out_tok[o] = y;
-          s_out_frame[o] = s_t;
-          s_out_score[o] = s_score;
-          d.s_last[slot] = y;
+          d.s_tr_chain[(size_t)slot * kTrChain + p] = node;
+          d.s_tr_rec[(size_t)slot * kTrChain + p] = rec;
         }
-        s_cnt += 1;
-        s_last = y;
-        s_sym += 1;
-        if (s_sym >= d.max_sym) { s_t += 1; s_sym = 0; }
+      };
+      if (h.x >= 0 && pos < tn) put(pos, h.x, make_int4(h.z, h.w, dd, 0));
+      if (lane == 0 && root && nv < tn) put(nv, own.x, make_int4(own.z, own.w, 2, 0));
+      if (lane == 0) {
+        s_nt = tn;
+        if (commit && d.has_tr) d.s_tr_len[slot] = tn;
       }
-    } else if (tid == 0) {
-      s_t += 1;
-      s_sym = 0;
     }
+  }
+  if (counting && tid == 0) {  // encoder frame, embedding row, A row
+    if (evaluated || next) atomicAdd(d.ctr, (evaluated ? s_bytes : 0ull) + (next ? 6ull * d.H : 0ull));
+  }
+  if (tid == kRowThreads - 1) {  // the outputs and the row's place in the chunk
+    const int cnt = s_cnt;
+    if (label && commit) {
+      const int o = r * T * d.max_sym + cnt;
+      s_out_tok[o] = y;
+      s_out_frame[o] = s_t;
+      s_out_score[o] = best - s_lse;
+      d.s_last[slot] = y;
+    }
+    const int cnt1 = cnt + (label ? 1 : 0);
+    if (mode == 1) {
+      s_out_count[r] = cnt1;
+    } else if (commit) {
+      d.r_t[r] = t1;
+      d.r_sym[r] = sym1;
+      d.r_cnt[r] = cnt1;
+    }
+  }
+  if (d.cap_rows && step < d.cap_steps && mode == 0) {
     row::block_sync();
-  }
-
-  if (PRED) {
-    // Stateful form: the prediction network reads the label just emitted
-    // (or, at a stream's first step, the start of sequence) and the row's h
-    // from before this step; the LSTM kernel after this one runs the cell.
-    const bool fresh = step == 0 && __ldcg(d.pred_fresh + slot) != 0;
-    const bool stepped = fresh || (evaluated && s_y != V);
     if (tid == 0) {
-      d.pflag[r] = stepped ? 1 : 0;
-      if (fresh && commit) d.pred_fresh[slot] = 0;
+      int* c = d.cap_rows + ((size_t)step * s_n + r) * 4;
+      c[0] = next ? t : -1;
+      c[1] = next ? last1 : -1;
+      c[2] = next ? (s_nl[0] ? s_lm[0][s_nl[0] - 1] : 0) : -1;
+      c[3] = next ? (s_nt ? s_tr[0] : 0) : -1;
     }
-    if (stepped) {
-      const int D = d.pred_D;
-      const int lab = fresh ? V : s_y;
-      const uint4* src_x = reinterpret_cast<const uint4*>(d.pred_emb + (size_t)lab * D);
-      const uint4* src_h = reinterpret_cast<const uint4*>(d.pred_h + (size_t)slot * D);
-      uint4* dst = reinterpret_cast<uint4*>(d.pred_x + (size_t)r * 2 * D);
-      for (int i = tid; i < D / 4; i += blockDim.x) dst[i] = (i < D / 8) ? __ldg(src_x + i) : __ldcg(src_h + i - D / 8);
-    }
-  }
-  if (mode == 1) {
-    // the chunk's last decision: the new chains' records for the next chunk
-    if (L == 1 && commit) {
-      if (tid < s_lm_len[0]) {
-        const int st = s_lm[0][tid];
-        d.s_lm_rec[(size_t)slot * kLmChain + tid] =
-            make_int4(__ldg(d.lm.st_begin + st), __ldg(d.lm.st_count + st), __float_as_int(__ldg(d.lm.st_cum + st)), 0);
-      }
-      if (tid >= 64 && tid - 64 < s_tr_len) {
-        const int q = s_tr[tid - 64];
-        d.s_tr_rec[(size_t)slot * kTrChain + tid - 64] =
-            make_int4(__ldg(d.tr.nd_begin + q), __ldg(d.tr.nd_count + q), __ldg(d.tr.nd_depth + q) + 1, 0);
-      }
-    }
-    if (tid == 0) s_out_count[r] = s_cnt;
-    return;
-  }
-  if (tid == 0 && commit) {
-    d.r_t[r] = s_t;
-    d.r_sym[r] = s_sym;
-    d.r_cnt[r] = s_cnt;
-  }
-  const int t = commit ? s_t : min(s_t, T - 1);
-  if (d.cap_rows && step < d.cap_steps && tid == 0 && commit) {
-    int* c = d.cap_rows + ((size_t)step * s_n + r) * 4;
-    if (t < T) {
-      c[0] = t;
-      c[1] = s_last;
-      c[2] = s_lm_len[0] ? s_lm[0][s_lm_len[0] - 1] : 0;
-      c[3] = s_tr_len ? s_tr[0] : 0;
-    } else {
-      c[0] = -1; c[1] = -1; c[2] = -1; c[3] = -1;
-    }
-  }
-  if (t >= T) return;
-
-  // 3. records of the new chains, scratch reset; 4. joint input of this
-  // step (its loads overlap the records); 5. the fusion bias row
-  const int nt = s_tr_len;
-  const bool counting = (mode == 2 || d.count);
-  unsigned long long lm_bytes = 0;  // thread 0: LM levels' records, arcs and searches
-  int nl = s_lm_len[0];
-  if (L == 1) {
-    row::bias_prepare(d, s_lm[0], nl, s_tr, nt, rc, lmv, dep);
-    if (commit) {  // the records stay with the chains for the next step's searches
-      if (tid < nl) d.s_lm_rec[(size_t)slot * kLmChain + tid] = make_int4(rc.lb[tid], rc.lc[tid], __float_as_int(rc.lo[tid]), 0);
-      if (tid >= 32 && tid - 32 < nt)
-        d.s_tr_rec[(size_t)slot * kTrChain + tid - 32] = make_int4(rc.tb[tid - 32], rc.tc[tid - 32], rc.td[tid - 32], 0);
-    }
-    if (!PRED) row::build_joint_input(d, s_enc + ((size_t)r * T + t) * d.H, s_last, r);
-    row::bias_finish(d, nl, nt, rc, s_lam, s_beta, d.bias + (size_t)r * d.N_pad, lmv, dep);
-    if (counting && tid == 0) lm_bytes = lm_level_bytes(rc, nl, s_y != V && evaluated);
-  } else if (MULTI) {
-    if (!PRED) row::build_joint_input(d, s_enc + ((size_t)r * T + t) * d.H, s_last, r);
-    lm_bytes = bias_multi(d, L, s_lm, s_lm_len, s_tr, nt, rc, s_lam, s_beta, d.bias + (size_t)r * d.N_pad, lmv,
-                          acc, dep, counting, s_y != V && evaluated);
-    nl = 0;
-    for (int i = 0; i < L; ++i) nl += s_lm_len[i];
-  }
-  if (counting && tid == 0) {
-    // Algorithmic bytes of this row-step: selection partials, row state,
-    // the searches of the emitted label (one probe per halving plus the arc
-    // it found), the joint input (encoder frame and embedding row read, A
-    // row written), and every arc of every chain level and trie chain node
-    // with its state record.  The dense bias row written for the GEMM
-    // epilogue and the shared unigram/root rows are not counted here.
-    unsigned long long bytes = (unsigned long long)d.n_ptiles * 16 + 2ull * (24 + 4 * (nl + nt));
-    bytes += 6ull * d.H + lm_bytes;
-    for (int k = 0; k < nt; ++k) bytes += 12 + 4ull * rc.tc[k];
-    if (s_y != V && evaluated)
-      for (int k = 0; k < nt; ++k) bytes += 8 + 4ull * (32 - __clz(rc.tc[k] + 1)) + 8;
-    atomicAdd(d.ctr, bytes);
   }
 }
 
 // After a chain is written from the host: its elements' table records.
 __global__ void k_fix_records(DecView d, int slot) {
   const int l = threadIdx.x;
-  if (d.has_lm && l < kLmChain && l < d.s_lm_len[slot]) {
-    const int st = d.s_lm_chain[(size_t)slot * kLmChain + l];
+  for (int i = 0; i < d.n_lm && l < kLmChain; ++i) {
+    const size_t h = (size_t)i * d.lm_stride + slot;
+    if (l >= d.s_lm_len[h]) continue;
+    const int st = d.s_lm_chain[h * kLmChain + l];
     // the fourth field of the first (unigram) level: its dense row, if any
-    const int dense = (l == 0 && d.lm.order >= 2 && st >= 1 && st <= d.V) ? d.lm.uni_dense[st - 1] : -1;
-    d.s_lm_rec[(size_t)slot * kLmChain + l] =
-        make_int4(d.lm.st_begin[st], d.lm.st_count[st], __float_as_int(d.lm.st_cum[st]), dense);
+    const int dense = (l == 0 && TSD_LMX(d, i, order) >= 2 && st >= 1 && st <= d.V) ? TSD_LMX(d, i, uni_dense)[st - 1] : -1;
+    d.s_lm_rec[h * kLmChain + l] = make_int4(TSD_LMX(d, i, st_begin)[st], TSD_LMX(d, i, st_count)[st],
+                                             __float_as_int(TSD_LMX(d, i, st_cum)[st]), dense);
   }
   if (d.has_tr && l < kTrChain && l < d.s_tr_len[slot]) {
     const int q = d.s_tr_chain[(size_t)slot * kTrChain + l];
@@ -561,8 +581,15 @@ void launch_defaults(const DecView& d, cudaStream_t s) {
 
 cudaError_t prepare_kernels(size_t row_smem) {
   // dynamic scratch plus the kernel's static shared memory may pass the
-  // 48 KB default even when the scratch alone does not
-  return cudaFuncSetAttribute(k_row<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_smem);
+  // 48 KB default even when the scratch alone does not; the joint kernel's
+  // shared-memory split, so that a row can start beside a joint CTA
+  const void* f[] = {(const void*)k_row<1>, (const void*)k_row<2>, (const void*)k_row<3>, (const void*)k_row<4>};
+  for (const void* k : f) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)row_smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 void launch_repack(const uint16_t* W, uint16_t* Wt, int H, int N, int N_pad, cudaStream_t s) {
@@ -624,9 +651,10 @@ void launch_row(const DecView& d, int M, int step, int mode, size_t smem, cudaSt
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  // greedy decoding with at most one LM runs k_row_fz (row_fused.cu); this
-  // pass serves several LMs (the stateful form takes one LM)
-  cudaLaunchKernelEx(&cfg, k_row<2>, d, step, mode);
+  if (d.n_lm <= 1) cudaLaunchKernelEx(&cfg, k_row<1>, d, step, mode);
+  else if (d.n_lm == 2) cudaLaunchKernelEx(&cfg, k_row<2>, d, step, mode);
+  else if (d.n_lm == 3) cudaLaunchKernelEx(&cfg, k_row<3>, d, step, mode);
+  else cudaLaunchKernelEx(&cfg, k_row<4>, d, step, mode);
 }
 
 }  // namespace tsd
