@@ -261,6 +261,36 @@ __global__ void __launch_bounds__((DSmem<BN, BM>::kThreads), 1)
           for (int i = 0; i < kCW; ++i)
             if (c0 + i >= N) l[i] = kNegInf;
         }
+        if constexpr (!DENSE) {
+          // the warp's boxes of logit + D go out first, by TMA stores from
+          // staging buffers in the drained stages (two sets per warp,
+          // alternating by block; the 128-byte swizzle keeps the
+          // row-per-thread writes conflict-free); the softmax pass runs while
+          // they are written
+          const float4* dv4 = reinterpret_cast<const float4*>(sD + b * kCW);
+          unsigned char* stg = smem + S::kStageOff + (warp - 2) * S::kStageWarp + (k & 1) * kWB * S::kBoxBytes;
+          if (k >= 2) {
+            if (lane == 0) tma_store_wait_read<kWB>();  // the stores of two blocks ago have read this set
+            __syncwarp();
+          }
+          if (lane < S::kQRows) {
+#pragma unroll
+            for (int e = 0; e < kCW / 4; ++e) {
+              const float4 dq = dv4[e];
+              *reinterpret_cast<float4*>(stg + (e / 8) * S::kBoxBytes + lane * 128 + (((e & 7) ^ (lane & 7)) << 4)) =
+                  make_float4(l[4 * e] + dq.x, l[4 * e + 1] + dq.y, l[4 * e + 2] + dq.z, l[4 * e + 3] + dq.w);
+            }
+          }
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+#pragma unroll
+            for (int j = 0; j < kWB; ++j) {
+              tma_store_2d(&tmLogits, stg + j * S::kBoxBytes, c0 + 32 * j, m0 + q * S::kQRows);
+              tma_store_commit();
+            }
+          }
+        }
         const float cm = block_max<kCW>(l);
         if (cm != kNegInf) {
           const float m2 = fmaxf(mx, cm);
@@ -285,35 +315,6 @@ __global__ void __launch_bounds__((DSmem<BN, BM>::kThreads), 1)
 #pragma unroll
               for (int i = 0; i < 32; ++i)
                 if ((mk >> i) & 1u) lo[i] = l[32 * j + i];
-            }
-          }
-        } else {
-          // the warp's 32-row boxes of logit + D by TMA stores from staging
-          // buffers in the drained stages (two sets per warp, alternating by
-          // block; the 128-byte swizzle keeps the row-per-thread writes
-          // conflict-free)
-          const float4* dv4 = reinterpret_cast<const float4*>(sD + b * kCW);
-#pragma unroll
-          for (int j = 0; j < kCW / 4; ++j) {
-            const float4 dq = dv4[j];
-            l[4 * j] += dq.x; l[4 * j + 1] += dq.y; l[4 * j + 2] += dq.z; l[4 * j + 3] += dq.w;
-          }
-          unsigned char* stg = smem + S::kStageOff + (warp - 2) * S::kStageWarp + (k & 1) * kWB * S::kBoxBytes;
-          if (lane == 0) tma_store_wait_read<kWB>();  // the stores of two blocks ago have read this set
-          __syncwarp();
-#pragma unroll
-          for (int j = 0; j < kWB; ++j)
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-              if (lane < S::kQRows) *reinterpret_cast<float4*>(stg + j * S::kBoxBytes + lane * 128 + ((e ^ (lane & 7)) << 4)) =
-                  make_float4(l[32 * j + 4 * e], l[32 * j + 4 * e + 1], l[32 * j + 4 * e + 2], l[32 * j + 4 * e + 3]);
-          fence_async_smem();
-          __syncwarp();
-          if (lane == 0) {
-#pragma unroll
-            for (int j = 0; j < kWB; ++j) {
-              tma_store_2d(&tmLogits, stg + j * S::kBoxBytes, c0 + 32 * j, m0 + q * S::kQRows);
-              tma_store_commit();
             }
           }
         }
