@@ -11,6 +11,11 @@
 
 namespace tsd {
 struct JointTc;
+// gemm_tc.cu: TMA maps of a GEMM's K-major bf16 operands for its two tile
+// shapes (B's rows are padded to a multiple of 128; a box past them reads zeros)
+struct GemmMaps {
+  CUtensorMap a, b, a64, b64;
+};
 struct ChunkShape;
 
 // Per-call parameters, copied to the device before each chunk so that one
@@ -198,7 +203,7 @@ struct tsd_decoder {
     int D = 0, Henc = 0, G_pad = 0, H_pad = 0, MT_pad = 0;
     uint16_t *Wg = nullptr, *Wp = nullptr, *We = nullptr;
     float *bg = nullptr, *bp = nullptr, *be = nullptr;
-    CUtensorMap encA, encB, lstmA, lstmB, projA, projB;
+    tsd::GemmMaps enc, lstm, proj;
   } pred;
   int joint_kind = 0;           // 0 tensor cores, 1 CUDA cores
   int pdl = 1;                  // programmatic dependent launch between kernels

@@ -18,12 +18,8 @@ struct GemmArgs {
   float* out;         // kEncProj: [M][ld]
 };
 
-// TMA maps of a K-major bf16 operand: A (128-row boxes) and B (boxes of the
-// epilogue's output-tile width; B's rows are padded to a multiple of 128).
-bool gemm_tc_map_a(CUtensorMap* m, const uint16_t* A, int rows, int K);
-bool gemm_tc_map_b(CUtensorMap* m, int epi, const uint16_t* B, int rows, int K);
+bool gemm_tc_maps(GemmMaps* m, int epi, const uint16_t* A, int a_rows, const uint16_t* B, int b_rows, int K);
 cudaError_t gemm_tc_prepare();
-void launch_gemm_tc(int epi, const DecView& d, const GemmArgs& g, const CUtensorMap& a, const CUtensorMap& b,
-                    cudaStream_t s, bool pdl);
+void launch_gemm_tc(int epi, const DecView& d, const GemmArgs& g, const GemmMaps& m, cudaStream_t s, bool pdl);
 
 }  // namespace tsd
