@@ -326,6 +326,39 @@ __device__ __forceinline__ void tile_block(const unsigned char* W, int wstride, 
     }
 }
 
+// Row n's logits of labels 4 lane .. of the block: the warps' partials in a fixed order.
+template <int NB>
+__device__ __forceinline__ float4 sum_parts(const float* part, int n, int ps, int lane) {
+  float4 s[8];
+#pragma unroll
+  for (int w = 0; w < 8; ++w) s[w] = *reinterpret_cast<const float4*>(part + (w * 8 * NB + n) * ps + 4 * lane);
+#pragma unroll
+  for (int h = 1; h < 8; h *= 2)
+#pragma unroll
+    for (int w = 0; w < 8; w += 2 * h) {
+      s[w].x += s[w + h].x;
+      s[w].y += s[w + h].y;
+      s[w].z += s[w + h].z;
+      s[w].w += s[w + h].w;
+    }
+  return s[0];
+}
+
+// The block's softmax partial (max, sum of exp(x - max)), by a warp whose
+// lanes hold four logits each, nv of them labels.
+__device__ __forceinline__ float2 block_softmax(float4 v, int nv) {
+  const float l[4] = {nv > 0 ? v.x : kNegInf, nv > 1 ? v.y : kNegInf, nv > 2 ? v.z : kNegInf, nv > 3 ? v.w : kNegInf};
+  const float m = key_value(__reduce_max_sync(0xffffffffu, order_key(fmaxf(fmaxf(l[0], l[1]), fmaxf(l[2], l[3])))));
+  const float m2 = m * tc::kLog2e;
+  float z = 0.f;
+  if (m != kNegInf)
+    z = (tc::ex2_approx(fmaf(l[0], tc::kLog2e, -m2)) + tc::ex2_approx(fmaf(l[1], tc::kLog2e, -m2))) +
+        (tc::ex2_approx(fmaf(l[2], tc::kLog2e, -m2)) + tc::ex2_approx(fmaf(l[3], tc::kLog2e, -m2)));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+  return make_float2(m, z);
+}
+
 // Whether the product may take its rows in several passes of 8 NB.
 __host__ __device__ constexpr bool several_passes(int NB, int RG) { return RG == 3 || (RG == 1 && NB == 1); }
 
@@ -394,13 +427,8 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
       const float2* sp = reinterpret_cast<const float2*>(c.sm + c.L.rows + warp * c.L.row_bytes + c.L.lse) + slot * c.CS * nb;
       float m = kNegInf, z = 0.f;
       for (int x = lane; x < c.CS * nb; x += 32) lse_merge(m, z, sp[x].x, sp[x].y);
-      __syncwarp();
-      const float top = key_value(__reduce_max_sync(0xffffffffu, order_key(m)));
-      z = z > 0.f ? z * expf(m - top) : 0.f;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-      if (lane == 0)
-        P.out_score[(size_t)(c.row0 + own) * (P.T * d.max_sym) + said.w] = __int_as_float(said.z) - (top + logf(z));
+      const float lse = row::warp_lse(m, z);
+      if (lane == 0) P.out_score[(size_t)(c.row0 + own) * (P.T * d.max_sym) + said.w] = __int_as_float(said.z) - lse;
     };
     if (active == 0) {
       if (score) write_score();
@@ -445,21 +473,9 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
           const int n = 8 * j + warp, i = i0 + n;
           if (!on[j] || lane >= nq) continue;
           const int grp = i / c.CS, owner = i - grp * c.CS;
-          float4 s[8];
-#pragma unroll
-          for (int w = 0; w < 8; ++w) s[w] = *reinterpret_cast<const float4*>(part + (w * 8 * NB + n) * ps + 4 * lane);
-#pragma unroll
-          for (int h = 1; h < 8; h *= 2)
-#pragma unroll
-            for (int w = 0; w < 8; w += 2 * h) {
-              s[w].x += s[w + h].x;
-              s[w].y += s[w + h].y;
-              s[w].z += s[w + h].z;
-              s[w].w += s[w + h].w;
-            }
+          sum[j] = sum_parts<NB>(part, n, ps, lane);
           const uint32_t dst = sm0 + c.L.rows + grp * c.L.row_bytes + c.L.logits + 4 * (c.rank * c.nl + m0 + 4 * lane);
-          send16(map_rank(dst, owner), s[0], map_rank(tc::smem_u32(c.lbar + grp), owner));
-          sum[j] = s[0];
+          send16(map_rank(dst, owner), sum[j], map_rank(tc::smem_u32(c.lbar + grp), owner));
         }
         // the block's softmax partials (max, sum of exp) follow: an emitted
         // label's score needs them, one step later
@@ -470,20 +486,11 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
           if (!on[j]) continue;  // the same for the warp's lanes
           const int grp = i / c.CS, owner = i - grp * c.CS;
           const int v0 = c.rank * c.nl + m0 + 4 * lane, nv = lane < nq ? d.N - v0 : 0;
-          const float l[4] = {nv > 0 ? sum[j].x : kNegInf, nv > 1 ? sum[j].y : kNegInf, nv > 2 ? sum[j].z : kNegInf,
-                              nv > 3 ? sum[j].w : kNegInf};
-          const float m = key_value(__reduce_max_sync(0xffffffffu, order_key(fmaxf(fmaxf(l[0], l[1]), fmaxf(l[2], l[3])))));
-          const float m2 = m * tc::kLog2e;
-          float z = 0.f;
-          if (m != kNegInf)
-            z = (tc::ex2_approx(fmaf(l[0], tc::kLog2e, -m2)) + tc::ex2_approx(fmaf(l[1], tc::kLog2e, -m2))) +
-                (tc::ex2_approx(fmaf(l[2], tc::kLog2e, -m2)) + tc::ex2_approx(fmaf(l[3], tc::kLog2e, -m2)));
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+          const float2 p = block_softmax(sum[j], nv);
           if (lane == 0) {
             const int buf = slot == 2 ? 0 : slot + 1;
             const uint32_t dst = sm0 + c.L.rows + grp * c.L.row_bytes + c.L.lse + 8 * ((buf * c.CS + c.rank) * nb + m0 / kMB);
-            send8(map_rank(dst, owner), __float_as_int(m), __float_as_int(z), map_rank(tc::smem_u32(c.sbar + grp), owner));
+            send8(map_rank(dst, owner), __float_as_int(p.x), __float_as_int(p.y), map_rank(tc::smem_u32(c.sbar + grp), owner));
           }
         }
         __syncwarp();
@@ -681,24 +688,21 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
       if (k) sync();
     }
     sync();
-    const float cr = lam * (nl ? __int_as_float(s.lmr[nl - 1].z) : 0.f) - bscale * (float)(nt ? s.trr[0].z - 1 : 0);
+    const float cr = row::row_constant(lam, nl ? __int_as_float(s.lmr[nl - 1].z) : 0.f, bscale, nt ? s.trr[0].z - 1 : 0);
     for (int q = tid; q < Q; q += GT) {
       const float4 kq = reinterpret_cast<const float4*>(term)[q];
-      float o[4] = {lam * kq.x, lam * kq.y, lam * kq.z, lam * kq.w};
+      uint32_t mv[4] = {0u, 0u, 0u, 0u}, rb = 0u;
       if (nt) {
         const uint4 mq = reinterpret_cast<const uint4*>(mark)[q];
-        const uint32_t mv[4] = {mq.x >> 16, mq.y >> 16, mq.z >> 16, mq.w >> 16};
-        if (mv[0] | mv[1] | mv[2] | mv[3]) {
-          const uint32_t rb = root[q >> 3] >> ((4 * q) & 31);
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (mv[j]) o[j] += bscale * (float)mv[j] - (((rb >> j) & 1u) ? bscale : 0.f);
-        }
+        mv[0] = mq.x >> 16, mv[1] = mq.y >> 16, mv[2] = mq.z >> 16, mv[3] = mq.w >> 16;
+        if (mv[0] | mv[1] | mv[2] | mv[3]) rb = root[q >> 3] >> ((4 * q) & 31);
       }
-      // (labels past V never win)
-      const int v = 4 * q;
-      reinterpret_cast<float4*>(term)[q] = make_float4(v < V ? cr + o[0] : kNegInf, v + 1 < V ? cr + o[1] : kNegInf,
-                                                       v + 2 < V ? cr + o[2] : kNegInf, v + 3 < V ? cr + o[3] : kNegInf);
+      const float x[4] = {kq.x, kq.y, kq.z, kq.w};
+      float o[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)  // (labels past V never win)
+        o[j] = 4 * q + j < V ? row::row_term(cr, lam, x[j], mv[j], (rb >> j) & 1u, bscale) : kNegInf;
+      reinterpret_cast<float4*>(term)[q] = make_float4(o[0], o[1], o[2], o[3]);
     }
     // (a thread reads back only what it wrote here: no barrier)
   };
@@ -973,9 +977,7 @@ __global__ void __launch_bounds__(kGemm + RG * group_threads(RG), 1)
   for (int v = tid; v < (d.V4 + 31) / 32 * 32; v += blockDim.x) {
     const bool rc = d.has_tr && v < d.V && __ldg(d.tr.root_child + v) != 0;
     const float u = d.has_lm && v < d.V ? __ldg(d.lm.uni_logp + v) : 0.f;
-    float x = d.has_lm ? P.lambda * u : 0.f;
-    if (rc) x += P.beta * d.tr.bonus;
-    if (v < d.V4) dflt[v] = x, uni[v] = u;
+    if (v < d.V4) dflt[v] = row::default_term(P.lambda, u, rc, P.beta, d.tr.bonus), uni[v] = u;
     const unsigned m = __ballot_sync(0xffffffffu, rc);  // whole warps: the bound is a multiple of 32
     if ((tid & 31) == 0) root[v / 32] = m;
   }
@@ -997,6 +999,99 @@ __global__ void __launch_bounds__(kGemm + RG * group_threads(RG), 1)
   }
   __syncthreads();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The joint kernel of the stateful form with few rows (its label step cannot
+// stay in one launch: the prediction network runs between two joint products):
+// the same product, sums and softmax partials as the loop above, so that both
+// forms give the same bits.  CTA (c, b): labels [c nl, (c+1) nl) of rows
+// 8 NB b .., its slice of W_out requested before the wait for the joint
+// input (further rows follow in steps of the grid); the row pass
+// (row_stream.cu) finishes Eq. 1 from the stored logits.
+template <int NB>
+__global__ void __launch_bounds__(kGemm, 1) k_joint_rows(const __grid_constant__ DecView d, int step, int nl) {
+  extern __shared__ __align__(128) unsigned char raw[];
+  unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(raw) + 127) & ~uintptr_t(127));
+  uint64_t* wbar = reinterpret_cast<uint64_t*>(sm);
+  const int H = d.H, U = H / 32, wstride = 2 * H + kWPad;
+  const unsigned char* W = sm + 128;
+  const int ps = ((nl < kMB ? nl : kMB) + 11) / 16 * 16 + 4;  // as in layout()
+  float* part = reinterpret_cast<float*>(sm + 128 + (nl * wstride + 127) / 128 * 128);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, k4 = lane & 3;
+  const int rank = blockIdx.x, n = d.params->n;
+  if (tid == 0) {
+    tc::mbar_init(wbar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    tc::mbar_expect_tx(wbar, (uint32_t)(nl * 2 * H));
+    for (int j = 0; j < nl; ++j)
+      tc::bulk_g2s(sm + 128 + j * wstride, d.Wt + (size_t)(rank * nl + j) * H, 2u * (uint32_t)H, wbar);
+  }
+  __syncthreads();
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int nb = (nl + kMB - 1) / kMB;
+  bool first = true;
+#pragma unroll 1
+  for (int i0 = blockIdx.y * 8 * NB; i0 < n; i0 += gridDim.y * 8 * NB) {
+    uint4 b[kUnits][NB];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+      const int i = i0 + 8 * j + g;
+      const uint4* a = reinterpret_cast<const uint4*>(d.A + (size_t)min(i, n - 1) * H) + k4;
+#pragma unroll
+      for (int u = 0; u < kUnits; ++u) {
+        const int un = warp + 8 * u;
+        b[u][j] = un < U && i < n ? __ldcg(a + 4 * un) : make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
+    if (first) {
+      first = false;
+      const bool ok = __syncthreads_and(tc::mbar_wait(wbar, 0, d.wait_ns) ? 1 : 0);
+      if (!ok) {
+        if (tid == 0) atomicOr(d.err, 1);
+        tc::mbar_wait(wbar, 0);  // the copies land before the CTA's shared memory goes (the long limit)
+        return;
+      }
+    }
+    for (int m0 = 0; m0 < nl; m0 += kMB) {
+      const int left = nl - m0;
+      if (left > 64) tile_block<10, NB, -1>(W, wstride, nl, m0, U, warp, g, k4, b, part, ps);
+      else if (left > 32) tile_block<8, NB, -1>(W, wstride, nl, m0, U, warp, g, k4, b, part, ps);
+      else tile_block<4, NB, -1>(W, wstride, nl, m0, U, warp, g, k4, b, part, ps);
+      __syncthreads();
+      const int nq = min(kMB, nl - m0) / 4;
+#pragma unroll
+      for (int j = 0; j < NB; ++j) {
+        const int i = i0 + 8 * j + warp;
+        __syncwarp();
+        if (i >= n) continue;  // the same for the warp's lanes
+        const int v0 = rank * nl + m0 + 4 * lane;
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (lane < nq) {
+          s = sum_parts<NB>(part, 8 * j + warp, ps, lane);
+          const float4 dv = __ldcg(reinterpret_cast<const float4*>(d.dvec + v0));
+          *reinterpret_cast<float4*>(d.logits + (size_t)i * d.N_pad + v0) =
+              make_float4(s.x + dv.x, s.y + dv.y, s.z + dv.z, s.w + dv.w);
+          if (d.cap_logits && step < d.cap_steps) {
+            float* cl = d.cap_logits + ((size_t)step * n + i) * d.N + v0;
+            const float l[4] = {s.x, s.y, s.z, s.w};
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+              if (v0 + x < d.N) cl[x] = l[x];
+          }
+        }
+        const float2 p = block_softmax(s, lane < nq ? d.N - v0 : 0);
+        if (lane == 0)
+          d.part[(size_t)i * d.n_ptiles + rank * nb + m0 / kMB] = make_float4(p.x, p.y, kNegInf, __int_as_float(INT_MAX));
+      }
+      __syncthreads();
+    }
+  }
+}
+
+int joint_rows_smem(int H, int nl, int NB) {
+  const int ps = ((nl < kMB ? nl : kMB) + 11) / 16 * 16 + 4;
+  return 128 + 128 + (nl * (2 * H + kWPad) + 127) / 128 * 128 + 8 * 8 * NB * ps * 4;
 }
 
 typedef void (*ChunkFn)(DecView, ChunkArgs);
@@ -1075,6 +1170,47 @@ const ChunkShape* chunk_cluster_pick(const std::vector<ChunkShape>& shapes, int 
     if (!best || c < cost) best = &s, cost = c;
   }
   return best;
+}
+
+int joint_rows_tiles(const ChunkShape& s) { return s.CS * ((s.nl + kMB - 1) / kMB); }
+
+int joint_rows_max_tiles(int N) {
+  int most = 0;
+  for (int CS = 8; CS <= 16; CS *= 2) {
+    ChunkShape s;
+    s.CS = CS, s.nl = ((N + CS - 1) / CS + 3) / 4 * 4;
+    most = std::max(most, joint_rows_tiles(s));
+  }
+  return most;
+}
+
+cudaError_t joint_rows_prepare() {
+  int dev = 0, lim = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_joint_rows<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_joint_rows<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  return e;
+}
+
+void launch_joint_rows(const ChunkShape& s, const DecView& d, int n, int step, cudaStream_t st, bool pdl) {
+  // 16 rows per CTA where their partials fit, and no more CTAs than SMs: most
+  // of W_out is then read before the wait.  A chunk of 5 frames (V 1024, H 1024,
+  // LSTM 640) in us, against the tensor-core joint kernel: 1 row 387 / 416, 16
+  // rows 426 / 441, 64 rows 449 / 454 (8 per CTA: 490), 112 rows 504 / 461.
+  const int NB = n > 8 && joint_rows_smem(d.H, s.nl, 2) <= 227 * 1024 ? 2 : 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)s.CS, (unsigned)std::min((n + 8 * NB - 1) / (8 * NB), std::max(1, d.sms / s.CS)));
+  cfg.blockDim = dim3(kGemm);
+  cfg.dynamicSmemBytes = (size_t)joint_rows_smem(d.H, s.nl, NB);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  if (NB == 1) cudaLaunchKernelEx(&cfg, k_joint_rows<1>, d, step, s.nl);
+  else cudaLaunchKernelEx(&cfg, k_joint_rows<2>, d, step, s.nl);
 }
 
 cudaError_t launch_chunk_cluster(const ChunkShape& s, const DecView& d, ChunkArgs& a, cudaStream_t st) {

@@ -36,6 +36,13 @@ struct ChunkShape {
 cudaError_t chunk_cluster_shapes(const DecView& d, std::vector<ChunkShape>& out);
 // The shape for n rows, or nullptr if none holds them in one wave.
 const ChunkShape* chunk_cluster_pick(const std::vector<ChunkShape>& shapes, int n, int H);
+// The stateful form's joint product with the same sums, for rows that a shape
+// holds: softmax partials per row (of a shape, and the most of any for N
+// labels), launch.
+int joint_rows_tiles(const ChunkShape& s);
+int joint_rows_max_tiles(int N);
+cudaError_t joint_rows_prepare();
+void launch_joint_rows(const ChunkShape& s, const DecView& d, int n, int step, cudaStream_t st, bool pdl);
 cudaError_t launch_chunk_cluster(const ChunkShape& s, const DecView& d, ChunkArgs& a, cudaStream_t st);
 
 }  // namespace tsd

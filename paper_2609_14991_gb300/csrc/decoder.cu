@@ -44,6 +44,14 @@ const ChunkShape* one_launch_shape(const tsd_decoder* d, int n) {
   return chunk_cluster_pick(d->chunk_shapes, n, d->cfg.H);
 }
 
+// The stateful form: the shape whose sums its joint product takes, with as
+// many rows as the stateless form decodes in one launch (the same bits), or
+// nullptr where the tensor-core kernel runs.
+const ChunkShape* joint_rows_shape(const tsd_decoder* d, int n) {
+  if (!d->one_launch || !d->pred.D || !d->view.fused || d->view.fz_dense || d->joint_kind != 0) return nullptr;
+  return chunk_cluster_pick(d->chunk_shapes, n, d->cfg.H);
+}
+
 // Events enqueue_chunk records with timing on: a mark before every row pass
 // and joint launch (and, for the stateful form, before the chunk's encoder
 // projection and each step's prediction-network GEMMs), and one at the end.
@@ -68,6 +76,8 @@ void enqueue_chunk(tsd_decoder* d, int M, int T, cudaStream_t s, const std::vect
     ++e;
   };
   const tsd_decoder::Pred& pr = d->pred;
+  const ChunkShape* rows = joint_rows_shape(d, M);
+  if (rows) v.n_ptiles = joint_rows_tiles(*rows);
   launch_defaults(v, s);
   if (pr.D) {
     // the chunk's encoder frames to a fixed buffer, then their projection
@@ -98,7 +108,8 @@ void enqueue_chunk(tsd_decoder* d, int M, int T, cudaStream_t s, const std::vect
     }
     if (step < S) {
       mark(1);
-      if (d->joint_kind == 0) launch_joint_tc(*d->jtc, v, M, step, s, d->pdl && !ev);
+      if (rows) launch_joint_rows(*rows, v, M, step, s, d->pdl && !ev);
+      else if (d->joint_kind == 0) launch_joint_tc(*d->jtc, v, M, step, s, d->pdl && !ev);
       else launch_joint(v, M, step, s);
     }
   }
@@ -219,7 +230,7 @@ tsd_status create_impl(const tsd_decoder_cfg* cfg, const void* W_out_bf16, const
   tsd_status st;
   if ((st = A.alloc(&Wt, (size_t)d->N_pad * c.H)) || (st = A.alloc(&E, (size_t)d->N * c.H)) ||
       (st = A.alloc(&Abuf, (size_t)d->M_pad * c.H)) ||
-      (st = A.alloc(&part, (size_t)d->M_pad * (d->N_pad / 64))) || (st = A.alloc(&err, 1)) || (st = A.alloc(&ctr, 2)) || (st = A.alloc(&dflt, (size_t)d->V4)) || (st = A.alloc(&droot, (size_t)(d->V4 + 31) / 32)) || (st = A.alloc(&rt, (size_t)d->M_pad)) ||
+      (st = A.alloc(&part, (size_t)d->M_pad * std::max(d->N_pad / 64, pw ? joint_rows_max_tiles(d->N) : 0))) || (st = A.alloc(&err, 1)) || (st = A.alloc(&ctr, 2)) || (st = A.alloc(&dflt, (size_t)d->V4)) || (st = A.alloc(&droot, (size_t)(d->V4 + 31) / 32)) || (st = A.alloc(&rt, (size_t)d->M_pad)) ||
       (st = A.alloc(&rs, (size_t)d->M_pad)) || (st = A.alloc(&rc, (size_t)d->M_pad)) ||
       (st = A.alloc(&sl, SK)) || (st = A.alloc(&sll, SK * NL)) || (st = A.alloc(&slc, SK * NL * kLmChain)) ||
       (st = A.alloc(&stl, SK)) || (st = A.alloc(&stc, SK * kTrChain)) || (st = A.alloc(&pdev, d->params_bytes)) ||
@@ -462,7 +473,9 @@ tsd_status create_impl(const tsd_decoder_cfg* cfg, const void* W_out_bf16, const
   v.pool_tok = ptok;
   v.pool_n = pn;
   v.pool_cap = kPoolCap;
-  if (fused && !pw && (ce = chunk_cluster_shapes(v, d->chunk_shapes)) != cudaSuccess)
+  if (fused && pw && (ce = joint_rows_prepare()) != cudaSuccess)
+    return cleanup(cuda_fail(ce, "tsd_decoder_create_pred: kernel attributes"));
+  if (fused && (ce = chunk_cluster_shapes(v, d->chunk_shapes)) != cudaSuccess)
     return cleanup(cuda_fail(ce, "tsd_decoder_create: cluster launch shapes"));
   d->slot_open.assign((size_t)c.max_streams, 0);
   d->last_stream = s;
@@ -1092,7 +1105,7 @@ extern "C" tsd_status tsd_decoder_set_option(tsd_decoder* d, const char* name, i
     // 1: a chunk that fits runs in one launch; 0: every label step is a row pass and a joint launch
     if (value != 0 && value != 1) return fail(TSD_EINVAL, "tsd_decoder_set_option: one_launch must be 0 or 1");
     d->one_launch = (int)value;
-    return TSD_OK;
+    return d->pred.D ? drop_graphs(d) : TSD_OK;  // the stateful form's graphs hold its joint kernel
   }
   if (n == "joint_bn") {
     if (value != 64 && value != 128 && value != 256) return fail(TSD_EINVAL, "tsd_decoder_set_option: joint_bn must be 64, 128 or 256");

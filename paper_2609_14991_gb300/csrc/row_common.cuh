@@ -151,6 +151,35 @@ __device__ __forceinline__ void best_merge(float& v, int& i, float v2, int i2) {
   if (v2 > v || (v2 == v && i2 < i)) { v = v2; i = i2; }
 }
 
+// The log-sum-exp of softmax partials (max, sum of exp(x - max)) by one warp,
+// whose lanes have merged every 32nd one.
+__device__ __forceinline__ float warp_lse(float m, float z) {
+  reconverge();
+  const float top = key_value(__reduce_max_sync(0xffffffffu, order_key(m)));
+  z = z > 0.f ? z * expf(m - top) : 0.f;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+  return top + logf(z);
+}
+
+// Terms of Eq. 1 in the streaming form, each operation rounded by itself (not
+// fused), so that every kernel that forms them gets the same bits: the call's
+// default D of a label, the row's constant c_r, and c_r + delta of a label,
+// from x = log p(v | s_l) - cum_l - log p(v), the depth e of its trie goto node
+// (0: none) and whether the root has a child for it.
+__device__ __forceinline__ float default_term(float lam, float logp, bool root, float beta, float bonus) {
+  const float x = __fmul_rn(lam, logp);
+  return root ? __fadd_rn(x, __fmul_rn(beta, bonus)) : x;
+}
+__device__ __forceinline__ float row_constant(float lam, float cum, float bscale, int depth) {
+  return __fsub_rn(__fmul_rn(lam, cum), __fmul_rn(bscale, (float)depth));
+}
+__device__ __forceinline__ float row_term(float cr, float lam, float x, uint32_t e, bool root, float bscale) {
+  float o = __fmul_rn(lam, x);
+  if (e) o = __fadd_rn(o, __fsub_rn(__fmul_rn(bscale, (float)e), root ? bscale : 0.f));
+  return __fadd_rn(cr, o);
+}
+
 // Eight values of the joint input, bf16(ReLU(x + z)).
 __device__ __forceinline__ uint4 joint_input(uint4 x, uint4 z) {
   const __nv_bfloat162* xa = reinterpret_cast<const __nv_bfloat162*>(&x);

@@ -555,12 +555,9 @@ __global__ void k_defaults(DecView d) {
   if (i < d.V4) d.dflt[i] = (d.has_lm && i < d.V) ? lam * __ldg(d.lm.uni_logp + i) : 0.f;
   if (d.fused && i < d.N_pad) {
     // the defaults the joint kernel adds to its logits (0 from blank on)
-    float x = 0.f;
-    if (i < d.V) {
-      if (d.has_lm) x = lam * __ldg(d.lm.uni_logp + i);
-      if (d.has_tr && __ldg(d.tr.root_child + i) != 0) x += P->beta * d.tr.bonus;
-    }
-    d.dvec[i] = x;
+    const bool label = i < d.V;
+    d.dvec[i] = row::default_term(lam, label && d.has_lm ? __ldg(d.lm.uni_logp + i) : 0.f,
+                                  label && d.has_tr && __ldg(d.tr.root_child + i) != 0, P->beta, d.tr.bonus);
   }
 
   if (i < (d.V4 + 31) / 32) {

@@ -256,7 +256,7 @@ __global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
       return (s_lmr[l].x & ~3) + 4 * g;
     };
     auto delta_of = [&](int l, float lp, int v) {
-      return lam * (lp - __int_as_float(s_lmr[l].z)) - lam * __ldg(d.lm.uni_logp + v);
+      return (lp - __int_as_float(s_lmr[l].z)) - __ldg(d.lm.uni_logp + v);
     };
     // 1a. the levels above 0 (few arcs: they continue longer contexts): each
     //     thread loads its first arc groups, labels and log-probabilities,
@@ -296,10 +296,12 @@ __global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
       for (int g = (held ? 32 : 0) + tid; a0 + 4 * g < e; g += kFzThreads)
         put(a0 + 4 * g, __ldg(reinterpret_cast<const int4*>(d.tr.ch_tok + a0) + g));
     };
+    // (dlm holds x = log p(v | s_l) - cum_l - log p(v), delta's LM term over lambda)
     // 1b. level 0 (the previous label's continuations, up to all V labels),
     //     streamed once: every label's level-0 delta (0 for no arc), which
     //     the deepest level above overwrites below
-    if (nl_old > 0 && s_lmr[0].w >= 0 && s_lmr[0].y >= max(32, V / 8)) {  // many continuations
+    if (nl_old > 0 && s_lmr[0].w >= 0 && (PRED || s_lmr[0].y >= max(32, V / 8))) {
+      // many continuations (the stateful form: any, as in the one-launch form, whose bits it gives)
       // the state's dense row: per label log p(v | u) - log p(v) - cum_0, 0
       // for no arc (whose delta is 0 as well), contiguous
       const float4* R = reinterpret_cast<const float4*>(d.lm.dense0 + (size_t)s_lmr[0].w * d.lm.V4);
@@ -315,7 +317,7 @@ __global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
 #pragma unroll
         for (int u = 0; u < kDense; ++u) {
           const int q = q0 + u * kFzThreads;
-          if (q < nq4) k4[q] = make_float4(lam * rq[u].x, lam * rq[u].y, lam * rq[u].z, lam * rq[u].w);
+          if (q < nq4) k4[q] = rq[u];
         }
       }
     } else {
@@ -324,7 +326,7 @@ __global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
       for (int q = tid; q < d.V4 / 4; q += blockDim.x) k4[q] = make_float4(0.f, 0.f, 0.f, 0.f);
       row::block_sync();
     }
-    if (nl_old > 0 && !(s_lmr[0].w >= 0 && s_lmr[0].y >= max(32, V / 8))) {
+    if (nl_old > 0 && !(s_lmr[0].w >= 0 && (PRED || s_lmr[0].y >= max(32, V / 8)))) {
       const int b0 = s_lmr[0].x, c0 = s_lmr[0].y;
       const int a0 = b0 & ~3, G0 = level_groups(b0, c0);
       for (int gb = 0; gb < G0; gb += kStream * kFzThreads) {
@@ -401,7 +403,7 @@ __global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
         for (int j = 0; j < 4; ++j) {
           const int i = hi[u] + j;
           if (i >= b && i < b + c && checked(tv[j] >= 0 && tv[j] < V, d.err, 9) && deepest(tv[j]) == l)
-            dlm[tv[j]] = lam * (pv[j] - __int_as_float(s_lmr[l].z)) - lam * hu[u][j];
+            dlm[tv[j]] = (pv[j] - __int_as_float(s_lmr[l].z)) - hu[u][j];
         }
       }
     }
@@ -461,7 +463,7 @@ __global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
       // c_r = lambda*(summed backoff of the state) - beta*bonus*depth
       const float cum_top = nl_old ? __int_as_float(s_lmr[nl_old - 1].z) : 0.f;
       const int depth_cur = nt_old ? s_trr[0].z - 1 : 0;
-      const float cr = lam * cum_top - bscale * (float)depth_cur;
+      const float cr = row::row_constant(lam, cum_top, bscale, depth_cur);
       const int nq = (V + 3) >> 2;  // quads holding labels < V
       const float4* l4 = reinterpret_cast<const float4*>(lg);
       const float4* k4 = reinterpret_cast<const float4*>(dlm);
@@ -480,18 +482,12 @@ __global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
             const float4 kq = k4[q];
             const uint32_t eq = e4[q];
             const float lv[4] = {lq[u].x, lq[u].y, lq[u].z, lq[u].w};
-            float dl[4] = {kq.x, kq.y, kq.z, kq.w};
-            if (eq) {  // a label of this quad has a trie goto node
-              const uint32_t rb = __ldg(d.droot + (q >> 3)) >> ((4 * q) & 31);
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const uint32_t e = (eq >> (8 * j)) & 0xffu;
-                if (e) dl[j] += bscale * (float)e - (((rb >> j) & 1u) ? bscale : 0.f);
-              }
-            }
+            const float dl[4] = {kq.x, kq.y, kq.z, kq.w};
+            // (a label of this quad has a trie goto node)
+            const uint32_t rb = eq ? __ldg(d.droot + (q >> 3)) >> ((4 * q) & 31) : 0u;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              const float fv = lv[j] + (cr + dl[j]);
+              const float fv = lv[j] + row::row_term(cr, lam, dl[j], (eq >> (8 * j)) & 0xffu, (rb >> j) & 1u, bscale);
               if (4 * q + j < V && fv > bv) { bv = fv; bi = 4 * q + j; }
             }
           }
@@ -589,13 +585,8 @@ __global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
         const float4 p = __ldcg(pr + j);
         lse_merge(pm, ps, p.x, p.y);
       }
-      row::reconverge();
-      for (int o = 16; o > 0; o >>= 1) {
-        const float m2 = __shfl_xor_sync(0xffffffffu, pm, o);
-        const float s2 = __shfl_xor_sync(0xffffffffu, ps, o);
-        lse_merge(pm, ps, m2, s2);
-      }
-      if (lane == 0) s_lse = pm + logf(ps);
+      const float lse = row::warp_lse(pm, ps);
+      if (lane == 0) s_lse = lse;
     }
   }
   if (joint) {
