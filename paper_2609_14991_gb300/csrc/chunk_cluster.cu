@@ -700,8 +700,11 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
       const float x[4] = {kq.x, kq.y, kq.z, kq.w};
       float o[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j)  // (labels past V never win)
-        o[j] = 4 * q + j < V ? row::row_term(cr, lam, x[j], mv[j], (rb >> j) & 1u, bscale) : kNegInf;
+      for (int j = 0; j < 4; ++j) {  // (labels past V never win)
+        o[j] = __fmul_rn(lam, x[j]);
+        if (mv[j]) o[j] = row::trie_delta(o[j], mv[j], (rb >> j) & 1u, bscale);
+        o[j] = 4 * q + j < V ? __fadd_rn(cr, o[j]) : kNegInf;
+      }
       reinterpret_cast<float4*>(term)[q] = make_float4(o[0], o[1], o[2], o[3]);
     }
     // (a thread reads back only what it wrote here: no barrier)

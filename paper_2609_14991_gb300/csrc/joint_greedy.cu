@@ -73,10 +73,17 @@ struct DSmem {
 // Sum over a block of 2^(l[i] * log2 e - s2) in four independent accumulators.
 template <int W>
 __device__ __forceinline__ float sum_exp2_block(const float* l, float s2) {
-  float a[4] = {0.f, 0.f, 0.f, 0.f};
+  uint64_t a[2] = {0u, 0u};
 #pragma unroll
-  for (int i = 0; i < W; ++i) a[i & 3] += ex2_approx(fmaf(l[i], kLog2e, -s2));
-  return (a[0] + a[1]) + (a[2] + a[3]);
+  for (int i = 0; i < W; i += 2) {
+    float x, y;
+    unpair(fma2(pair_of(l[i], l[i + 1]), pair_of(kLog2e, kLog2e), pair_of(-s2, -s2)), x, y);
+    a[(i >> 1) & 1] = add2(a[(i >> 1) & 1], pair_of(ex2_approx(x), ex2_approx(y)));
+  }
+  float b[4];
+  unpair(a[0], b[0], b[1]);
+  unpair(a[1], b[2], b[3]);
+  return (b[0] + b[1]) + (b[2] + b[3]);
 }
 
 // The maximum of a block by a tree (the block is left unchanged).
@@ -277,8 +284,10 @@ __global__ void __launch_bounds__((DSmem<BN, BM>::kThreads), 1)
 #pragma unroll
             for (int e = 0; e < kCW / 4; ++e) {
               const float4 dq = dv4[e];
-              *reinterpret_cast<float4*>(stg + (e / 8) * S::kBoxBytes + lane * 128 + (((e & 7) ^ (lane & 7)) << 4)) =
-                  make_float4(l[4 * e] + dq.x, l[4 * e + 1] + dq.y, l[4 * e + 2] + dq.z, l[4 * e + 3] + dq.w);
+              float4 o;
+              unpair(add2(pair_of(l[4 * e], l[4 * e + 1]), pair_of(dq.x, dq.y)), o.x, o.y);
+              unpair(add2(pair_of(l[4 * e + 2], l[4 * e + 3]), pair_of(dq.z, dq.w)), o.z, o.w);
+              *reinterpret_cast<float4*>(stg + (e / 8) * S::kBoxBytes + lane * 128 + (((e & 7) ^ (lane & 7)) << 4)) = o;
             }
           }
           fence_async_smem();
@@ -383,12 +392,11 @@ __global__ void __launch_bounds__((DSmem<BN, BM>::kThreads), 1)
     float* xbase = reinterpret_cast<float*>(smem);
     int* xok = reinterpret_cast<int*>(xbase + BM * 4 * (kEW - 1));  // [quadrant][warp 1..]
     if (ehalf > 0 && lane < S::kQRows) {
-      float* xch = xbase + (row * (kEW - 1) + ehalf - 1) * 4;
       if (ok) {
-        xch[0] = mx;
-        xch[1] = se;
-        xch[2] = bv;
-        xch[3] = __int_as_float(bi);
+        if constexpr (DENSE)
+          reinterpret_cast<float4*>(xbase)[(ehalf - 1) * BM + row] = make_float4(mx, se, bv, __int_as_float(bi));
+        else
+          reinterpret_cast<float2*>(xbase)[(ehalf - 1) * BM + row] = make_float2(mx, se);
       }
       if (lane == 0) xok[q * (kEW - 1) + ehalf - 1] = ok ? 1 : 0;
     }
@@ -401,8 +409,14 @@ __global__ void __launch_bounds__((DSmem<BN, BM>::kThreads), 1)
           all = false;
           continue;
         }
-        const float* xch = xbase + (row * (kEW - 1) + e - 1) * 4;
-        const float m1 = xch[0], s1 = xch[1];
+        float4 xch;
+        if constexpr (DENSE) {
+          xch = reinterpret_cast<const float4*>(xbase)[(e - 1) * BM + row];
+        } else {
+          const float2 x2 = reinterpret_cast<const float2*>(xbase)[(e - 1) * BM + row];
+          xch = make_float4(x2.x, x2.y, kNegInf, __int_as_float(INT_MAX));
+        }
+        const float m1 = xch.x, s1 = xch.y;
         if (m1 != kNegInf) {
           if (mx == kNegInf) {
             mx = m1;
@@ -413,8 +427,8 @@ __global__ void __launch_bounds__((DSmem<BN, BM>::kThreads), 1)
             mx = m2;
           }
         }
-        const float v1 = xch[2];
-        const int i1 = __float_as_int(xch[3]);
+        const float v1 = xch.z;
+        const int i1 = __float_as_int(xch.w);
         if (v1 > bv || (v1 == bv && i1 < bi)) { bv = v1; bi = i1; }
       }
       if (all) d.part[(size_t)gr * d.n_ptiles + blockIdx.x] = make_float4(mx, se, bv, __int_as_float(bi));

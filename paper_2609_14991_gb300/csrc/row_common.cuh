@@ -164,9 +164,9 @@ __device__ __forceinline__ float warp_lse(float m, float z) {
 
 // Terms of Eq. 1 in the streaming form, each operation rounded by itself (not
 // fused), so that every kernel that forms them gets the same bits: the call's
-// default D of a label, the row's constant c_r, and c_r + delta of a label,
-// from x = log p(v | s_l) - cum_l - log p(v), the depth e of its trie goto node
-// (0: none) and whether the root has a child for it.
+// default D of a label, the row's constant c_r, and delta of a label that has a
+// trie goto node, from delta's LM term o = lambda*(log p(v | s_l) - cum_l -
+// log p(v)), the node's depth e and whether the root has a child for it.
 __device__ __forceinline__ float default_term(float lam, float logp, bool root, float beta, float bonus) {
   const float x = __fmul_rn(lam, logp);
   return root ? __fadd_rn(x, __fmul_rn(beta, bonus)) : x;
@@ -174,10 +174,8 @@ __device__ __forceinline__ float default_term(float lam, float logp, bool root, 
 __device__ __forceinline__ float row_constant(float lam, float cum, float bscale, int depth) {
   return __fsub_rn(__fmul_rn(lam, cum), __fmul_rn(bscale, (float)depth));
 }
-__device__ __forceinline__ float row_term(float cr, float lam, float x, uint32_t e, bool root, float bscale) {
-  float o = __fmul_rn(lam, x);
-  if (e) o = __fadd_rn(o, __fsub_rn(__fmul_rn(bscale, (float)e), root ? bscale : 0.f));
-  return __fadd_rn(cr, o);
+__device__ __forceinline__ float trie_delta(float o, uint32_t e, bool root, float bscale) {
+  return __fadd_rn(o, __fsub_rn(__fmul_rn(bscale, (float)e), root ? bscale : 0.f));
 }
 
 // Eight values of the joint input, bf16(ReLU(x + z)).

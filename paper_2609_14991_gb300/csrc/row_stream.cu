@@ -256,7 +256,7 @@ __global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
       return (s_lmr[l].x & ~3) + 4 * g;
     };
     auto delta_of = [&](int l, float lp, int v) {
-      return (lp - __int_as_float(s_lmr[l].z)) - __ldg(d.lm.uni_logp + v);
+      return __fmul_rn(lam, (lp - __int_as_float(s_lmr[l].z)) - __ldg(d.lm.uni_logp + v));
     };
     // 1a. the levels above 0 (few arcs: they continue longer contexts): each
     //     thread loads its first arc groups, labels and log-probabilities,
@@ -296,7 +296,6 @@ __global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
       for (int g = (held ? 32 : 0) + tid; a0 + 4 * g < e; g += kFzThreads)
         put(a0 + 4 * g, __ldg(reinterpret_cast<const int4*>(d.tr.ch_tok + a0) + g));
     };
-    // (dlm holds x = log p(v | s_l) - cum_l - log p(v), delta's LM term over lambda)
     // 1b. level 0 (the previous label's continuations, up to all V labels),
     //     streamed once: every label's level-0 delta (0 for no arc), which
     //     the deepest level above overwrites below
@@ -317,7 +316,8 @@ __global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
 #pragma unroll
         for (int u = 0; u < kDense; ++u) {
           const int q = q0 + u * kFzThreads;
-          if (q < nq4) k4[q] = rq[u];
+          if (q < nq4)
+            k4[q] = make_float4(__fmul_rn(lam, rq[u].x), __fmul_rn(lam, rq[u].y), __fmul_rn(lam, rq[u].z), __fmul_rn(lam, rq[u].w));
         }
       }
     } else {
@@ -403,7 +403,7 @@ __global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
         for (int j = 0; j < 4; ++j) {
           const int i = hi[u] + j;
           if (i >= b && i < b + c && checked(tv[j] >= 0 && tv[j] < V, d.err, 9) && deepest(tv[j]) == l)
-            dlm[tv[j]] = (pv[j] - __int_as_float(s_lmr[l].z)) - hu[u][j];
+            dlm[tv[j]] = __fmul_rn(lam, (pv[j] - __int_as_float(s_lmr[l].z)) - hu[u][j]);
         }
       }
     }
@@ -482,12 +482,18 @@ __global__ void __maxnreg__(72) k_row_fz(DecView d, int step, int mode) {
             const float4 kq = k4[q];
             const uint32_t eq = e4[q];
             const float lv[4] = {lq[u].x, lq[u].y, lq[u].z, lq[u].w};
-            const float dl[4] = {kq.x, kq.y, kq.z, kq.w};
-            // (a label of this quad has a trie goto node)
-            const uint32_t rb = eq ? __ldg(d.droot + (q >> 3)) >> ((4 * q) & 31) : 0u;
+            float dl[4] = {kq.x, kq.y, kq.z, kq.w};
+            if (eq) {  // a label of this quad has a trie goto node
+              const uint32_t rb = __ldg(d.droot + (q >> 3)) >> ((4 * q) & 31);
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const uint32_t e = (eq >> (8 * j)) & 0xffu;
+                if (e) dl[j] = row::trie_delta(dl[j], e, (rb >> j) & 1u, bscale);
+              }
+            }
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-              const float fv = lv[j] + row::row_term(cr, lam, dl[j], (eq >> (8 * j)) & 0xffu, (rb >> j) & 1u, bscale);
+              const float fv = lv[j] + __fadd_rn(cr, dl[j]);
               if (4 * q + j < V && fv > bv) { bv = fv; bi = 4 * q + j; }
             }
           }
