@@ -365,7 +365,8 @@ TSD_API tsd_status tsd_decoder_check(tsd_decoder* dec);
  *              calls, and calls with set_timing(1), joint kernel 1, a chosen
  *              joint_bn or fusion_path 1 run a row pass and a joint kernel per
  *              label step.  Both take the same decisions; their fp32 sums
- *              differ in order;
+ *              differ in order.  The stateful form takes the one launch's
+ *              sums for as many rows, in a joint kernel of its own;
  *   "pdl"      1 (default) / 0: programmatic dependent launch between the
  *              row pass and the joint kernel, so each kernel's set-up
  *              overlaps the tail of the one before;
@@ -554,7 +555,7 @@ TSD_API tsd_status tsd_encoder_timing(tsd_encoder* enc, double* ms, int64_t* lau
 TSD_API tsd_status tsd_encoder_gemm_flops(const tsd_encoder* enc, int32_t n, int32_t C, double* flops);
 /* Kernel launches of one encode_chunk(n, C) with timing off (for launch
  * accounting): the call's streams run as up to two parallel graph branches
- * of at least 256 frame rows each, each branch the subsampling GEMM, the
+ * of at least 256 frame rows each (one where its GEMMs fill the SMs), each branch the subsampling GEMM, the
  * first block's first layer norm and 14 kernels per block (a block's
  * closing layer norm also computes the next block's first one), then one
  * kernel that advances the frame counts.  TSD_EINVAL on n, C outside

@@ -260,17 +260,20 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else if (warp == 1) {
     if (rank == 0 && elect()) {
       const uint32_t idesc = idesc_bf16(kTM, BN);
-      int it = 0, tl = 0;
-      bool ok = true;
+      int tl = 0, s = 0;
+      uint32_t ph = 0;
+      bool ok = true, ready = mbar_test(full, 0);
       for (int t = first; t < tiles && ok; t += stride, ++tl) {
         const int buf = tl & 1, use = tl >> 1;
         if (tl >= 2 && !mbar_wait(acce + buf, (uint32_t)(use - 1) & 1u)) { ok = false; break; }
         fence_after();
         const uint32_t acc = tmem + (uint32_t)(buf * BN);
-        for (int kb = 0; kb < KB; ++kb, ++it) {
-          const int s = it % kStages;
-          const uint32_t ph = (uint32_t)(it / kStages) & 1u;
-          if (!mbar_wait(full + s, ph)) { ok = false; break; }
+        for (int kb = 0; kb < KB; ++kb) {
+          if (!ready && !mbar_wait(full + s, ph)) { ok = false; break; }
+          // the next stage's barrier is read while this stage's MMAs are issued
+          const int s1 = s + 1 == kStages ? 0 : s + 1;
+          const uint32_t ph1 = s1 == 0 ? ph ^ 1u : ph;
+          ready = mbar_test(full + s1, ph1);
           fence_after();
           const uint32_t sa = smem_u32(smem + s * S::kStageBytes);
           const uint64_t ad = sw128_desc(sa), bd = sw128_desc(sa + kABytes);
@@ -278,6 +281,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int k = 0; k < kBK / 16; ++k)
             mma<PAIR>(acc, ad + (uint64_t)(2 * k), bd + (uint64_t)(2 * k), idesc, (kb | k) ? 1u : 0u);
           commit<PAIR>(empty + s);
+          s = s1;
+          ph = ph1;
         }
         commit<PAIR>(accf + buf);  // also after a timeout: nothing is left in flight
       }
