@@ -7,8 +7,8 @@
 // few rows is not work but the chain of launches and round trips to L2: 9.4 us
 // a step for one stream (V = 1024, H = 640), 10.4 us for 64, against well
 // under 1 us of arithmetic.  Here a step has no launch, no grid-wide
-// dependency and no logits in memory (13 frames of one stream: 616 -> 192 us,
-// of 64 streams: 670 -> 295 us; 16 streams x 1 frame, H = 1024: 70 -> 31 us):
+// dependency and no logits in memory (13 frames of one stream: 650 -> 204 us,
+// of 64 streams: 665 -> 255 us; 16 streams x 1 frame, H = 1024: 71 -> 30 us):
 //   * CTA c of the cluster keeps labels [c nl, (c+1) nl) of W_out in shared
 //     memory for the whole chunk (read once per chunk, not once per step);
 //   * warps 0-7 (GEMM) compute the slice's logits of all R rows: bf16

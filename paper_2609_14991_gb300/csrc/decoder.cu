@@ -1,9 +1,10 @@
 // Decoder host driver: creation, stream slots and the per-chunk label loop.
 //
 // One decode_chunk(n, T) is T*max_sym label steps (the most any stream can
-// need); each step is a row pass (decide, advance, joint input, fusion bias)
-// followed by the joint GEMM with its fused selection epilogue, and a final
-// row pass applies the last decision.  Every launch reads the call's
+// need); each step is a row pass (decide, advance, joint input) followed by
+// the joint GEMM with its softmax partials, and a final row pass applies the
+// last decision; few rows take the whole chunk in one launch
+// (chunk_cluster.cu).  Every launch reads the call's
 // arguments from a small device block written just before, so the whole
 // chunk is captured once per (n, T) as a CUDA graph and replayed.
 #include <algorithm>
