@@ -73,7 +73,7 @@ constexpr int kStream = 4;  // level-0 arc groups of four per thread whose loads
 // 2 = replay (redo the step's work without committing any state or output;
 // used only to time the kernel in isolation).
 // VAR bit 0: the stateful form (LSTM input rows instead of the joint input);
-// bit 2: few rows (at most two per SM): eight warps, so that every chain
+// bit 2: few rows (two or three per SM): eight warps, so that every chain
 // element's search is one warp's and its first load precedes the wait.
 // Otherwise four warps: seven CTAs per SM at 72 registers.  72 also let two
 // rows of eight warps start beside a joint CTA (80 registers and 192 threads:
@@ -740,7 +740,14 @@ cudaError_t prepare_stream_kernels(size_t smem) {
 void launch_row_stream(const DecView& d, int M, int step, int mode, size_t smem, cudaStream_t s, bool pdl) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(M);
-  const bool few = M <= 2 * d.sms;
+  // Eight warps a row up to two rows per SM: 304 rows, V 1024: 732 us a chunk of
+  // 13 frames against 733 with four, 208 rows: 588 / 711.  A third row leaves no
+  // room for a joint CTA beside the rows (400 rows: 804 / 769; V 512, 450 rows:
+  // 712 / 628), which costs nothing where the joint kernel's tiles fill the SMs
+  // by themselves (not its 64-row tiles): 400 rows, V 2048: 803 / 974, V 4096:
+  // 895 / 1054.
+  const bool tiles64 = d.n_ptiles * 64 >= d.N && (M + 63) / 64 * d.n_ptiles <= d.sms;
+  const bool few = M <= (tiles64 || d.pred_D ? 2 : 3) * d.sms;
   cfg.blockDim = dim3(few ? kThreadsOf<4> : kThreadsOf<0>);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
