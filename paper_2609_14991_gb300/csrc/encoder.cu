@@ -389,7 +389,9 @@ __global__ void __launch_bounds__(128) k_dwconv(ConvArgs a) {
 // thread's window slides through registers, every load is 8 bytes and the
 // cached frames, taps and affine map load before the wait for the GLU outputs.
 // With a channel per thread and 2-byte loads the 0.6B shape's 256 streams took
-// 18 us (its 22 MB need 4); with four 10.3, of which the launch is two.
+// 18 us (its 22 MB need 4); with four 10.3, of which the launch is two.  Swish
+// with one range check for the four (tc::swish2): the 0.6B chunk 5785 us, 5863
+// with a division each.
 constexpr int kConvThreads = 64;
 __global__ void __launch_bounds__(kConvThreads) k_dwconv9(ConvArgs a) {
   constexpr int K = 9, K1 = K - 1;
@@ -448,9 +450,12 @@ __global__ void __launch_bounds__(kConvThreads) k_dwconv9(ConvArgs a) {
           float acc = 0.f;
 #pragma unroll
           for (int k = 0; k < K; ++k) acc = fmaf(wk[k][j], win[k][j], acc);
-          const float yv = (acc + bi[j]) * s1[j] + s0[j];
-          o[j] = yv * tc::sigmoid(yv);
+          o[j] = (acc + bi[j]) * s1[j] + s0[j];
         }
+        uint64_t y[2] = {tc::pair_of(o[0], o[1]), tc::pair_of(o[2], o[3])};
+        tc::swish2(y, y);
+        tc::unpair(y[0], o[0], o[1]);
+        tc::unpair(y[1], o[2], o[3]);
         z[(t0 + u) * row] = make_uint2((uint32_t)f2bf(o[0]) | ((uint32_t)f2bf(o[1]) << 16),
                                        (uint32_t)f2bf(o[2]) | ((uint32_t)f2bf(o[3]) << 16));
       }

@@ -24,11 +24,12 @@
 // What bounds them (0.6B shape, 3328 x 4096 x 1024 with Swish, 20.5 us in the
 // kernel): 1.5 us to the first operands, 5.2 us per tile and pair of which the
 // MMAs are 4.2 (the operands' way from L2 is the rest), 2.4 us of epilogue
-// after the last tile.  With 128 x 128 tiles for everything, libm's expf and an
-// IEEE division and row-per-thread stores the same rows took two launches of
-// 26.7 us, 18.5 us of each without the epilogue.  Swish and GLU use the
-// hardware's 2^x and reciprocal (tc::sigmoid, relative error below 4e-7,
-// rounded to bf16 after) on pairs of values, and blocks of 32 rows leave through
+// after the last tile.  With 128 x 128 tiles for everything, a division's range
+// check per value and row-per-thread stores the same rows took two launches of
+// 26.7 us, 18.5 us of each without the epilogue.  Swish and GLU give the bits of
+// 1 / (1 + expf(-x)), checked for range once per block of 32 values and reckoned
+// in pairs (tc::sigmoid2); the hardware's 2^x and reciprocal alone were 3 to 5%
+// of a chunk faster, with twice the error.  Blocks of 32 rows leave through
 // shared memory by TMA: bf16 stores, and for the residual update an fp32
 // add in L2 (one writer per element), so x is not read at all.
 //
@@ -72,22 +73,6 @@ struct Shape {
   static_assert((2 * kStages + 4) * 8 + 4 <= 512, "barrier area");
   static_assert(kSmem <= 227 * 1024 && kStages >= 4, "shared memory per CTA");
 };
-
-// tc::sigmoid of two values
-__device__ __forceinline__ uint64_t sigmoid2(uint64_t x) {
-  const uint64_t c = pair_of(-kLog2e, -kLog2e);
-  const uint64_t hi = mul2(x, c);
-  float h0, h1;
-  unpair(hi, h0, h1);
-  const uint64_t lo = fma2(x, c, pair_of(-h0, -h1));
-  const uint64_t e = pair_of(ex2_approx(h0), ex2_approx(h1));
-  const uint64_t e1 = add2(fma2(e, mul2(lo, pair_of(0.6931471805599453f, 0.6931471805599453f)), e), pair_of(1.f, 1.f));
-  float a, b;
-  unpair(e1, a, b);
-  asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(a));
-  asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(b));
-  return pair_of(a, b);
-}
 
 __device__ __forceinline__ uint32_t pack_bf16(uint64_t x) {
   float a, b;
@@ -340,8 +325,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             __syncwarp();
             uint64_t a[16], b[16];
             load_cols(tc0 + 32, g.bias + c0 + 32, b);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) b[i] = sigmoid2(b[i]);
+            sigmoid2(b, b);
             load_cols(tc0, g.bias + c0, a);
             uint32_t w[16];
 #pragma unroll
@@ -383,8 +367,10 @@ __global__ void __launch_bounds__(kThreads, 1)
                 if (whole) ship(st, c0 + 32 * h, r0, EPI == kEResid);
               } else {
                 if (EPI == kESwish) {
+                  uint64_t g16[16];
+                  sigmoid2(v, g16);
 #pragma unroll
-                  for (int i = 0; i < 16; ++i) v[i] = mul2(v[i], sigmoid2(v[i]));
+                  for (int i = 0; i < 16; ++i) v[i] = mul2(v[i], g16[i]);
                 }
                 uint32_t w[16];
 #pragma unroll

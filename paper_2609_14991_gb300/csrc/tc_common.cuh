@@ -20,17 +20,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-// 1 / (1 + e^-x): the exponent's product with log2 e in two parts, so that
-// the approximations of 2^x and 1/x (relative errors of 2^-22 and 2^-23) are
-// what remains at any x.
-__device__ __forceinline__ float sigmoid(float x) {
-  const float hi = x * -kLog2e, lo = fmaf(x, -kLog2e, -hi);
-  const float e = ex2_approx(hi);
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + fmaf(e, lo * 0.6931471805599453f, e)));
-  return r;
-}
-
 // Pairs of fp32 values in one instruction (each rounded as the scalar ones).
 __device__ __forceinline__ uint64_t pair_of(float a, float b) {
   uint64_t r;
@@ -52,6 +41,84 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
+}
+
+// 1 / x for x in [1, 2^125], correctly rounded: the hardware's approximation
+// and one Newton step with fused multiply-adds (P. Markstein, IBM J. Res. Dev.
+// 34, 1990).
+constexpr float kRecipMax = 0x1p125f;
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ uint64_t recip2(uint64_t x) {
+  float a, b;
+  unpair(x, a, b);
+  a = rcp_approx(a), b = rcp_approx(b);
+  const uint64_t r = pair_of(a, b);
+  return fma2(r, fma2(x, pair_of(-a, -b), pair_of(1.f, 1.f)), r);
+}
+
+// y = 1 / (1 + e^-x), the bits of 1.f / (1.f + expf(-x)) at every x (0 where e^-x
+// overflows).  One range check for the whole block: a division's own, per
+// value, keeps the values apart.
+template <int N>
+__device__ __forceinline__ void sigmoid2(const uint64_t (&x)[N], uint64_t (&y)[N]) {
+  float top = 0.f;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    float a, b;
+    unpair(x[i], a, b);
+    a = expf(-a), b = expf(-b);
+    top = fmaxf(top, fmaxf(a, b));
+    y[i] = add2(pair_of(a, b), pair_of(1.f, 1.f));
+  }
+  if (top < kRecipMax) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) y[i] = recip2(y[i]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      float a, b;
+      unpair(y[i], a, b);
+      y[i] = pair_of(1.f / a, 1.f / b);
+    }
+  }
+}
+
+// y = x / (1 + e^-x), the bits of x / (1.f + expf(-x)) at every x: a quotient from
+// the correctly rounded reciprocal and one remainder (as above) is correctly
+// rounded while it and its remainder are normal numbers.
+template <int N>
+__device__ __forceinline__ void swish2(const uint64_t (&x)[N], uint64_t (&y)[N]) {
+  uint64_t d[N];
+  bool plain = true;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    float a, b;
+    unpair(x[i], a, b);
+    const float e = expf(-a), f = expf(-b);
+    plain = plain && fmaxf(e, f) < 0x1p40f && fminf(fabsf(a), fabsf(b)) > 0x1p-80f && fmaxf(fabsf(a), fabsf(b)) < 0x1p100f;
+    d[i] = add2(pair_of(e, f), pair_of(1.f, 1.f));
+  }
+  if (plain) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const uint64_t r = recip2(d[i]), q = mul2(x[i], r);
+      float a, b;
+      unpair(d[i], a, b);
+      y[i] = fma2(fma2(pair_of(-a, -b), q, x[i]), r, q);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      float a, b, u, v;
+      unpair(x[i], a, b);
+      unpair(d[i], u, v);
+      y[i] = pair_of(a / u, b / v);
+    }
+  }
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
