@@ -27,8 +27,9 @@
 // Clusters never wait for one another.  Messages inside a cluster complete
 // bytes on the receiver's mbarriers: `ybar` (every CTA: the R rows' labels of
 // a step) and `lbar` (per owned row: its logits), one phase per step each.
-// `sbar` (per owned row) does the same for the softmax partials that a score
-// needs: GEMM warp q finishes row q's scores one step late, while it would wait.
+// `sbar` (two per owned row, in turn: chunk_partials.h) does the same for the
+// softmax partials that a score needs: GEMM warp q finishes row q's scores one
+// step late, while it would wait.
 // What is left of a step, in clocks, one stream: argmax 710, publishing 350,
 // the label's records 1700, chains 770, deltas 1930 (three of these five wait
 // for L2 once), beside labels to operands 1460, product 1430, sums and sending
@@ -47,6 +48,7 @@
 
 #include "row_common.cuh"
 #include "chunk_cluster.h"
+#include "chunk_partials.h"
 #include "tc_common.cuh"
 
 namespace tsd {
@@ -187,7 +189,7 @@ __host__ __device__ inline Layout layout(int H, int V4, int nl, int CS, int NB, 
   Layout L;
   auto up = [](int x) { return (x + 127) & ~127; };
   int o = 0;
-  L.bars = o, o += 128;                      // ybar, wbar, lbar[RG], sbar[RG], fail flag
+  L.bars = o, o += 128;                      // ybar, wbar, lbar[RG], sbar[RG][kPartBars], fail flag
   L.y = o, o = up(o + 16 * CS * RG);         // every row's (previous label, frame or -1, fused value, output place or -1)
   L.w = o, o = up(o + nl * (2 * H + kWPad));
   // row stride of the partials, 4 mod 16: lanes (n = 2c, m = g) fall in different banks
@@ -199,7 +201,7 @@ __host__ __device__ inline Layout layout(int H, int V4, int nl, int CS, int NB, 
   L.rows = o;
   int r = (int)((sizeof(RowSm) + 127) & ~size_t(127));
   L.logits = r, r = up(r + 4 * CS * nl);
-  L.lse = r, r = up(r + 3 * 8 * CS * ((nl + kMB - 1) / kMB));  // softmax partials of three steps
+  L.lse = r, r = up(r + kPartBufs * 8 * CS * ((nl + kMB - 1) / kMB));  // softmax partials
   L.term = r, r = up(r + 4 * V4);
   L.mark = r, r = up(r + 4 * V4);
   L.list = RG < 3 ? r : -1;                  // level 0's labels
@@ -374,8 +376,8 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
   const uint32_t sm0 = tc::smem_u32(c.sm);
   const int nb = (c.nl + kMB - 1) / kMB;  // softmax partials per CTA
   // Warp q < RG also finishes the scores of the CTA's row q: a step's softmax
-  // partials (three buffers in turn) are consumed one step later, while the
-  // warp would wait for the next labels.
+  // partials are consumed one step later, while the warp would wait for the
+  // next labels.
   const int own = warp * c.CS + c.rank;
   const bool mine = warp < RG && own < c.R;
   bool armed = false, ok = true;
@@ -394,7 +396,7 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
       }
     }
   };
-  for (int step = 0, slot = 2; ; ++step) {  // slot: the buffer of the step before (step - 1 mod 3)
+  for (int step = 0; ; ++step) {
     // the rows' labels (at first, W_out's slice as well)
     ok = wait_cluster(c.ybar, step & 1, d.wait_ns, c.fail) && ok;
     if (step == 0) ok = ok && wait_cluster(c.wbar, 0, d.wait_ns, c.fail);
@@ -416,15 +418,18 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
     bool score = false;
     if (mine) {
       said = c.y[own];
-      if (armed) {  // the step before's partials are all in; before any of this step's can be sent
-        ok = __all_sync(0xffffffffu, wait_cluster(c.sbar + warp, (step - 1) & 1, d.wait_ns, c.fail));
+      if (armed) {  // the step before's partials are all in; before this CTA sends any logits of this step
+        ok = __all_sync(0xffffffffu, wait_cluster(c.sbar + kPartBars * warp + part_bar(step - 1), part_parity(step - 1),
+                                                  d.wait_ns, c.fail));
         score = ok && said.w >= 0;
       }
       armed = ok && said.y >= 0;
-      if (armed && lane == 0) tc::mbar_expect_tx(c.sbar + warp, 8u * (uint32_t)(c.CS * nb));
+      if (armed && lane == 0)
+        tc::mbar_expect_tx(c.sbar + kPartBars * warp + part_bar(step), 8u * (uint32_t)(c.CS * nb));
     }
     auto write_score = [&]() {
-      const float2* sp = reinterpret_cast<const float2*>(c.sm + c.L.rows + warp * c.L.row_bytes + c.L.lse) + slot * c.CS * nb;
+      const float2* sp = reinterpret_cast<const float2*>(c.sm + c.L.rows + warp * c.L.row_bytes + c.L.lse) +
+                         part_buf(step - 1) * c.CS * nb;
       float m = kNegInf, z = 0.f;
       for (int x = lane; x < c.CS * nb; x += 32) lse_merge(m, z, sp[x].x, sp[x].y);
       const float lse = row::warp_lse(m, z);
@@ -488,9 +493,10 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
           const int v0 = c.rank * c.nl + m0 + 4 * lane, nv = lane < nq ? d.N - v0 : 0;
           const float2 p = block_softmax(sum[j], nv);
           if (lane == 0) {
-            const int buf = slot == 2 ? 0 : slot + 1;
-            const uint32_t dst = sm0 + c.L.rows + grp * c.L.row_bytes + c.L.lse + 8 * ((buf * c.CS + c.rank) * nb + m0 / kMB);
-            send8(map_rank(dst, owner), __float_as_int(p.x), __float_as_int(p.y), map_rank(tc::smem_u32(c.sbar + grp), owner));
+            const uint32_t dst =
+                sm0 + c.L.rows + grp * c.L.row_bytes + c.L.lse + 8 * ((part_buf(step) * c.CS + c.rank) * nb + m0 / kMB);
+            send8(map_rank(dst, owner), __float_as_int(p.x), __float_as_int(p.y),
+                  map_rank(tc::smem_u32(c.sbar + kPartBars * grp + part_bar(step)), owner));
           }
         }
         __syncwarp();
@@ -498,7 +504,6 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
       }
     }
     if (score) write_score();
-    slot = slot == 2 ? 0 : slot + 1;
   }
 }
 
@@ -957,14 +962,15 @@ __global__ void __launch_bounds__(kGemm + RG * group_threads(RG), 1)
   c.wbar = c.ybar + 1;
   c.lbar = c.ybar + 2;
   c.sbar = c.lbar + RG;
-  int* fail = reinterpret_cast<int*>(c.sbar + RG);
+  static_assert((2 + (1 + kPartBars) * RG) * 8 + 4 <= 128, "barrier area");
+  int* fail = reinterpret_cast<int*>(c.sbar + kPartBars * RG);
   c.fail = fail;
   c.y = reinterpret_cast<int4*>(c.sm + c.L.y);
   const int tid = threadIdx.x;
   if (tid == 0) {
     tc::mbar_init(c.ybar, 1);
     tc::mbar_init(c.wbar, 1);
-    for (int g = 0; g < 2 * RG; ++g) tc::mbar_init(c.lbar + g, 1);  // lbar, then sbar
+    for (int g = 0; g < (1 + kPartBars) * RG; ++g) tc::mbar_init(c.lbar + g, 1);  // lbar, then sbar
     *fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     tc::mbar_expect_tx(c.ybar, 16u * (uint32_t)c.R);  // the rows' first labels
