@@ -203,7 +203,7 @@ __host__ __device__ inline Layout layout(int H, int V4, int nl, int CS, int NB, 
   L.logits = r, r = up(r + 4 * CS * nl);
   L.lse = r, r = up(r + kPartBufs * 8 * CS * ((nl + kMB - 1) / kMB));  // softmax partials
   L.term = r, r = up(r + 4 * V4);
-  L.mark = r, r = up(r + 4 * V4);
+  L.mark = r, r = up(r + 4 * V4);                               // levels and trie depths, 16 bits each
   L.list = RG < 3 ? r : -1;                  // level 0's labels
   if (RG < 3) r = up(r + 4 * V4 + 32);
   L.row_bytes = r;
@@ -522,8 +522,10 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
   RowSm& s = *reinterpret_cast<RowSm*>(rs);
   const float* lg = reinterpret_cast<const float*>(rs + c.L.logits);
   float* term = reinterpret_cast<float*>(rs + c.L.term);          // every label's c_r + delta (while built: its LM delta / lambda)
-  // per label: bits 0-15 the LM chain levels above 0 with an arc for it, byte 2 its trie goto depth (0: none)
-  uint32_t* mark = reinterpret_cast<uint32_t*>(rs + c.L.mark);
+  // per label: the LM chain levels above 0 with an arc for it (bit l), and its trie goto depth (0: none); apart,
+  // because the first is set by 32-bit atomics (two labels each) while the second is stored
+  uint16_t* lev = reinterpret_cast<uint16_t*>(rs + c.L.mark);
+  uint16_t* dep = lev + d.V4;
   int* list = c.L.list >= 0 ? reinterpret_cast<int*>(rs + c.L.list) : nullptr;  // level 0's labels from its aligned first arc
   const float* dflt = reinterpret_cast<const float*>(c.sm + c.L.dflt);
   const float* uni = reinterpret_cast<const float*>(c.sm + c.L.uni);
@@ -584,13 +586,13 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
   };
   // level 0 of the deltas: label u's dense row by asynchronous copies (u < 0:
-  // no LM state, every delta 0), and the marks cleared
+  // no LM state, every delta 0), and levels and depths cleared
   auto begin_deltas = [&](int u) {
     const float* R = d.lm.dense0 + (size_t)max(u, 0) * d.lm.V4;
     for (int q = tid; q < Q; q += GT) {
       if (u >= 0) copy16(term + 4 * q, R + 4 * q);
       else reinterpret_cast<float4*>(term)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-      reinterpret_cast<uint4*>(mark)[q] = make_uint4(0u, 0u, 0u, 0u);
+      reinterpret_cast<uint2*>(lev)[q] = reinterpret_cast<uint2*>(dep)[q] = make_uint2(0u, 0u);
     }
   };
   // A thread's group of four arcs of the levels above 0 (level hl, first arc
@@ -638,7 +640,7 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
       const int tv[4] = {tk.x, tk.y, tk.z, tk.w};
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        if (i0 + j >= q.x && i0 + j < q.x + q.y) reinterpret_cast<uint8_t*>(mark + tv[j])[2] = (uint8_t)q.z;
+        if (i0 + j >= q.x && i0 + j < q.x + q.y) dep[tv[j]] = (uint16_t)q.z;
     };
     auto scatter = [&](int k) {
       const int4 q = s.trr[k];
@@ -659,8 +661,8 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
 #pragma unroll
       for (int j = 0; j < 4; ++j)
         if (i0 + j >= q.x && i0 + j < q.x + q.y && checked(tv[j] >= 0 && tv[j] < V, d.err, 9)) {
-          if (!settle) atomicOr(mark + tv[j], 1u << l);
-          else if (nl == 2 || ((mark[tv[j]] & 0xffffu) >> l) == 1u) term[tv[j]] = (pv[j] - cum) - uni[tv[j]];
+          if (!settle) atomicOr(reinterpret_cast<uint32_t*>(lev) + (tv[j] >> 1), 1u << (l + 16 * (tv[j] & 1)));
+          else if (nl == 2 || (lev[tv[j]] >> l) == 1) term[tv[j]] = (pv[j] - cum) - uni[tv[j]];
         }
     };
     // past what a thread holds (rare: more than four times GT arcs above level 0)
@@ -698,8 +700,8 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
       const float4 kq = reinterpret_cast<const float4*>(term)[q];
       uint32_t mv[4] = {0u, 0u, 0u, 0u}, rb = 0u;
       if (nt) {
-        const uint4 mq = reinterpret_cast<const uint4*>(mark)[q];
-        mv[0] = mq.x >> 16, mv[1] = mq.y >> 16, mv[2] = mq.z >> 16, mv[3] = mq.w >> 16;
+        const uint2 mq = reinterpret_cast<const uint2*>(dep)[q];
+        mv[0] = mq.x & 0xffffu, mv[1] = mq.x >> 16, mv[2] = mq.y & 0xffffu, mv[3] = mq.y >> 16;
         if (mv[0] | mv[1] | mv[2] | mv[3]) rb = root[q >> 3] >> ((4 * q) & 31);
       }
       const float x[4] = {kq.x, kq.y, kq.z, kq.w};
@@ -734,7 +736,7 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
   const uint32_t row_bytes = 4u * (uint32_t)(c.CS * c.nl);
   bool ok = true, moved = true;
   begin_deltas(s.nl > 0 ? s.lmr[0].w : -1);
-  sync();  // the marks are cleared before anyone sets one
+  sync();  // levels and depths are cleared before anyone sets one
   while (t < T) {
     if (tid == 0) tc::mbar_expect_tx(c.lbar + grp, row_bytes);
     if (moved) finish_deltas();
