@@ -364,9 +364,13 @@ TSD_API tsd_status tsd_decoder_check(tsd_decoder* dec);
  *              smaller W_out); 0, other
  *              calls, and calls with set_timing(1), joint kernel 1, a chosen
  *              joint_bn or fusion_path 1 run a row pass and a joint kernel per
- *              label step.  Both take the same decisions; their fp32 sums
- *              differ in order.  The stateful form takes the one launch's
- *              sums for as many rows, in a joint kernel of its own;
+ *              label step.  A stream's results are the same bits in all calls
+ *              of a decoder that run in one launch, whatever else they hold,
+ *              and in all that do not.  Between the two the fp32 sums differ
+ *              in order: scores in their last bits, and of two labels that
+ *              close either may be taken.  0 gives the same bits at any row
+ *              count.  The stateful form takes the one launch's sums for as
+ *              many rows, in a joint kernel of its own;
  *   "pdl"      1 (default) / 0: programmatic dependent launch between the
  *              row pass and the joint kernel, so each kernel's set-up
  *              overlaps the tail of the one before;

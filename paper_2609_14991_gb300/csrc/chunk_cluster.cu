@@ -9,8 +9,8 @@
 // under 1 us of arithmetic.  Here a step has no launch, no grid-wide
 // dependency and no logits in memory (13 frames of one stream: 650 -> 204 us,
 // of 64 streams: 665 -> 255 us; 16 streams x 1 frame, H = 1024: 71 -> 30 us):
-//   * CTA c of the cluster keeps labels [c nl, (c+1) nl) of W_out in shared
-//     memory for the whole chunk (read once per chunk, not once per step);
+//   * CTA c of the cluster keeps its slice of W_out's labels in shared memory for
+//     the whole chunk (read once per chunk, not once per step);
 //   * warps 0-7 (GEMM) compute the slice's logits of all R rows: bf16
 //     mma.sync 16 x 8 x 16 with labels as the 16-row operand and rows as the
 //     8-column one, so one row costs one eighth of what a 128-row tcgen05 tile
@@ -42,8 +42,9 @@
 // lambda * delta), see row_stream.cu.  Level 0 of the LM chain comes from the
 // unigram state's dense row (copied by cp.async while the label is searched),
 // the levels above overwrite their labels' deltas.  The order of every sum
-// depends on V and H only, so a row's result does not depend on the other
-// rows, on R or on CS.
+// depends on V and H only (the softmax partials are of units of labels that are
+// the same for clusters of 8 and of 16), so a row's result does not depend
+// on the other rows of the call, on R or on CS, as long as the call runs here.
 #include <algorithm>
 
 #include "row_common.cuh"
@@ -181,15 +182,56 @@ struct RowSm {
   int nl, nt;
 };
 
+// The labels of a CTA, and the softmax partials they make.  The labels are cut
+// into eight slices and each slice into two units (u0 labels and the rest; of
+// N = 1025: 132 = 68 + 64); a cluster of 8 gives a CTA a slice, a cluster of
+// 16 a unit.  A unit makes a partial per kMB of its labels.
+struct Slice {
+  int start;           // its labels
+  uint16_t len, first; // how many, and of those its first unit
+  int part0, parts;    // its first partial among a row's, and a row's partials
+};
+__host__ __device__ inline int slice_labels(int N) { return (N + 31) / 32 * 4; }
+__host__ __device__ inline Slice slice_of(int N, int CS, int rank) {
+  const int nl = slice_labels(N), u0 = (nl + 7) / 8 * 4, u1 = nl - u0;
+  const int p0 = (u0 + kMB - 1) / kMB, p1 = (u1 + kMB - 1) / kMB;
+  Slice s;
+  s.parts = 8 * (p0 + p1);
+  if (CS == 8) {
+    s.start = rank * nl, s.len = (uint16_t)nl, s.first = (uint16_t)u0, s.part0 = rank * (p0 + p1);
+  } else {
+    const int h = rank & 1;
+    s.start = (rank >> 1) * nl + h * u0, s.len = s.first = (uint16_t)(h ? u1 : u0), s.part0 = (rank >> 1) * (p0 + p1) + h * p0;
+  }
+  return s;
+}
+
+// A block of a slice that the product takes at once: its end, and a lane's four
+// labels in it (from its start; -1: none).  A slice of at most kMB labels is one
+// block, its units on half a warp each; otherwise blocks end with their unit.
+struct Block {
+  int end;
+  bool halves;
+};
+__device__ __forceinline__ Block block_at(const Slice& s, int m0) {
+  if (s.len <= kMB) return {s.len, s.first < s.len};
+  return {min(m0 + kMB, m0 < s.first ? s.first : s.len), false};
+}
+__device__ __forceinline__ int lane_labels(const Slice& s, const Block& b, int m0, int lane) {
+  if (!b.halves) return 4 * lane < b.end - m0 ? 4 * lane : -1;
+  const int o = (lane >> 4) * s.first + 4 * (lane & 15);
+  return o < (lane < 16 ? s.first : s.len) ? o : -1;
+}
+
 // Shared-memory layout of a CTA (bytes from the 128-byte-aligned base).
 struct Layout {
   int w, part, ps, dflt, uni, root, y, bars, rows, row_bytes, logits, lse, term, mark, list, total;
 };
-__host__ __device__ inline Layout layout(int H, int V4, int nl, int CS, int NB, int RG) {
+__host__ __device__ inline Layout layout(int N, int H, int V4, int nl, int CS, int NB, int RG) {
   Layout L;
-  auto up = [](int x) { return (x + 127) & ~127; };
+  auto up = [](int x) { return (x + 15) & ~15; };
   int o = 0;
-  L.bars = o, o += 128;                      // ybar, wbar, lbar[RG], sbar[RG][kPartBars], fail flag
+  L.bars = o, o += 128;                      // ybar, wbar, lbar[RG], sbar[RG][kPartBars], fail flag, slice
   L.y = o, o = up(o + 16 * CS * RG);         // every row's (previous label, frame or -1, fused value, output place or -1)
   L.w = o, o = up(o + nl * (2 * H + kWPad));
   // row stride of the partials, 4 mod 16: lanes (n = 2c, m = g) fall in different banks
@@ -199,9 +241,9 @@ __host__ __device__ inline Layout layout(int H, int V4, int nl, int CS, int NB, 
   L.uni = o, o = up(o + 4 * V4);             // log p(v)
   L.root = o, o = up(o + (V4 + 31) / 32 * 4);
   L.rows = o;
-  int r = (int)((sizeof(RowSm) + 127) & ~size_t(127));
+  int r = up((int)sizeof(RowSm));
   L.logits = r, r = up(r + 4 * CS * nl);
-  L.lse = r, r = up(r + kPartBufs * 8 * CS * ((nl + kMB - 1) / kMB));  // softmax partials
+  L.lse = r, r = up(r + kPartBufs * 8 * slice_of(N, CS, 0).parts);  // softmax partials
   L.term = r, r = up(r + 4 * V4);
   L.mark = r, r = up(r + 4 * V4);                               // levels and trie depths, 16 bits each
   L.list = RG < 3 ? r : -1;                  // level 0's labels
@@ -267,7 +309,8 @@ struct Ctx {
   uint64_t *ybar, *wbar, *lbar, *sbar;
   volatile int* fail;
   int4* y;
-  int CS, rank, nl, R, row0;
+  const Slice* sl;  // in shared memory: the product's warps have few registers to spare
+  int CS, rank, R, row0;
 };
 
 // ---------------------------------------------------------------- GEMM warps
@@ -328,12 +371,12 @@ __device__ __forceinline__ void tile_block(const unsigned char* W, int wstride, 
     }
 }
 
-// Row n's logits of labels 4 lane .. of the block: the warps' partials in a fixed order.
+// Row n's logits of four labels of the block from o: the warps' partials in a fixed order.
 template <int NB>
-__device__ __forceinline__ float4 sum_parts(const float* part, int n, int ps, int lane) {
+__device__ __forceinline__ float4 sum_parts(const float* part, int n, int ps, int o) {
   float4 s[8];
 #pragma unroll
-  for (int w = 0; w < 8; ++w) s[w] = *reinterpret_cast<const float4*>(part + (w * 8 * NB + n) * ps + 4 * lane);
+  for (int w = 0; w < 8; ++w) s[w] = *reinterpret_cast<const float4*>(part + (w * 8 * NB + n) * ps + o);
 #pragma unroll
   for (int h = 1; h < 8; h *= 2)
 #pragma unroll
@@ -346,18 +389,25 @@ __device__ __forceinline__ float4 sum_parts(const float* part, int n, int ps, in
   return s[0];
 }
 
-// The block's softmax partial (max, sum of exp(x - max)), by a warp whose
-// lanes hold four logits each, nv of them labels.
-__device__ __forceinline__ float2 block_softmax(float4 v, int nv) {
+// A unit's softmax partial (max, sum of exp(x - max)), by a warp whose lanes hold
+// four logits each, nv of them labels.  halves: two units, of 16 lanes each
+// (every lane gets its own unit's; the sums' order is that of a unit alone).
+__device__ __forceinline__ float2 unit_softmax(float4 v, int nv, bool halves, int lane) {
   const float l[4] = {nv > 0 ? v.x : kNegInf, nv > 1 ? v.y : kNegInf, nv > 2 ? v.z : kNegInf, nv > 3 ? v.w : kNegInf};
-  const float m = key_value(__reduce_max_sync(0xffffffffu, order_key(fmaxf(fmaxf(l[0], l[1]), fmaxf(l[2], l[3])))));
+  const int key = order_key(fmaxf(fmaxf(l[0], l[1]), fmaxf(l[2], l[3])));
+  const int low = __reduce_max_sync(0xffffffffu, halves && lane >= 16 ? INT_MIN : key);
+  const int high = __reduce_max_sync(0xffffffffu, halves && lane < 16 ? INT_MIN : key);
+  const int top = lane < 16 ? low : high;
+  const float m = key_value(top);
   const float m2 = m * tc::kLog2e;
   float z = 0.f;
   if (m != kNegInf)
     z = (tc::ex2_approx(fmaf(l[0], tc::kLog2e, -m2)) + tc::ex2_approx(fmaf(l[1], tc::kLog2e, -m2))) +
         (tc::ex2_approx(fmaf(l[2], tc::kLog2e, -m2)) + tc::ex2_approx(fmaf(l[3], tc::kLog2e, -m2)));
+  const float other = __shfl_xor_sync(0xffffffffu, z, 16);
+  z = halves ? z : z + other;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+  for (int o = 8; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
   return make_float2(m, z);
 }
 
@@ -374,12 +424,13 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
   const unsigned char* W = c.sm + c.L.w;
   float* part = reinterpret_cast<float*>(c.sm + c.L.part);
   const uint32_t sm0 = tc::smem_u32(c.sm);
-  const int nb = (c.nl + kMB - 1) / kMB;  // softmax partials per CTA
   // Warp q < RG also finishes the scores of the CTA's row q: a step's softmax
   // partials are consumed one step later, while the warp would wait for the
   // next labels.
   const int own = warp * c.CS + c.rank;
   const bool mine = warp < RG && own < c.R;
+  Slice sl;  // what the product needs of the slice stays in registers
+  sl.start = c.sl->start, sl.len = c.sl->len, sl.first = c.sl->first;
   bool armed = false, ok = true;
   // this warp's operands of row i (zero for a finished row or none)
   auto load = [&](int i, Piece& q) {
@@ -425,13 +476,13 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
       }
       armed = ok && said.y >= 0;
       if (armed && lane == 0)
-        tc::mbar_expect_tx(c.sbar + kPartBars * warp + part_bar(step), 8u * (uint32_t)(c.CS * nb));
+        tc::mbar_expect_tx(c.sbar + kPartBars * warp + part_bar(step), 8u * (uint32_t)c.sl->parts);
     }
     auto write_score = [&]() {
       const float2* sp = reinterpret_cast<const float2*>(c.sm + c.L.rows + warp * c.L.row_bytes + c.L.lse) +
-                         part_buf(step - 1) * c.CS * nb;
+                         part_buf(step - 1) * c.sl->parts;
       float m = kNegInf, z = 0.f;
-      for (int x = lane; x < c.CS * nb; x += 32) lse_merge(m, z, sp[x].x, sp[x].y);
+      for (int x = lane; x < c.sl->parts; x += 32) lse_merge(m, z, sp[x].x, sp[x].y);
       const float lse = row::warp_lse(m, z);
       if (lane == 0) P.out_score[(size_t)(c.row0 + own) * (P.T * d.max_sym) + said.w] = __int_as_float(said.z) - lse;
     };
@@ -457,17 +508,19 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
 #pragma unroll
         for (int j = 0; j < NB; ++j) b[u][j] = joint8(q[j].x[u], q[j].z[u]);
       __syncwarp();
-      for (int m0 = 0; m0 < c.nl; m0 += kMB) {
-        const int left = c.nl - m0;
-        if (left > 72) tile_block<10, NB, FU>(W, wstride, c.nl, m0, U, warp, g, k4, b, part, ps);
-        else if (left > 64) tile_block<9, NB, FU>(W, wstride, c.nl, m0, U, warp, g, k4, b, part, ps);
-        else if (left > 48) tile_block<8, NB, FU>(W, wstride, c.nl, m0, U, warp, g, k4, b, part, ps);
-        else if (left > 32) tile_block<6, NB, FU>(W, wstride, c.nl, m0, U, warp, g, k4, b, part, ps);
-        else if (left > 16) tile_block<4, NB, FU>(W, wstride, c.nl, m0, U, warp, g, k4, b, part, ps);
-        else tile_block<2, NB, FU>(W, wstride, c.nl, m0, U, warp, g, k4, b, part, ps);
+      int p0 = 0;
+      for (int m0 = 0; m0 < sl.len;) {
+        const Block bl = block_at(sl, m0);
+        const int left = bl.end - m0;
+        if (left > 72) tile_block<10, NB, FU>(W, wstride, sl.len, m0, U, warp, g, k4, b, part, ps);
+        else if (left > 64) tile_block<9, NB, FU>(W, wstride, sl.len, m0, U, warp, g, k4, b, part, ps);
+        else if (left > 48) tile_block<8, NB, FU>(W, wstride, sl.len, m0, U, warp, g, k4, b, part, ps);
+        else if (left > 32) tile_block<6, NB, FU>(W, wstride, sl.len, m0, U, warp, g, k4, b, part, ps);
+        else if (left > 16) tile_block<4, NB, FU>(W, wstride, sl.len, m0, U, warp, g, k4, b, part, ps);
+        else tile_block<2, NB, FU>(W, wstride, sl.len, m0, U, warp, g, k4, b, part, ps);
+        const int lo = lane_labels(sl, bl, m0, lane), v0 = sl.start + m0 + lo;
         // the warps' partials summed in a fixed order and sent to the rows' owners
         group_sync(1, kGemm);
-        const int nq = min(kMB, c.nl - m0) / 4;
         float4 sum[NB];
         bool on[NB];  // read before the sends: a row's next label may follow its logits at once
 #pragma unroll
@@ -476,13 +529,13 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
 #pragma unroll
         for (int j = 0; j < NB; ++j) {
           const int n = 8 * j + warp, i = i0 + n;
-          if (!on[j] || lane >= nq) continue;
+          if (!on[j] || lo < 0) continue;
           const int grp = i / c.CS, owner = i - grp * c.CS;
-          sum[j] = sum_parts<NB>(part, n, ps, lane);
-          const uint32_t dst = sm0 + c.L.rows + grp * c.L.row_bytes + c.L.logits + 4 * (c.rank * c.nl + m0 + 4 * lane);
+          sum[j] = sum_parts<NB>(part, n, ps, lo);
+          const uint32_t dst = sm0 + c.L.rows + grp * c.L.row_bytes + c.L.logits + 4 * v0;
           send16(map_rank(dst, owner), sum[j], map_rank(tc::smem_u32(c.lbar + grp), owner));
         }
-        // the block's softmax partials (max, sum of exp) follow: an emitted
+        // the units' softmax partials (max, sum of exp) follow: an emitted
         // label's score needs them, one step later
 #pragma unroll
         for (int j = 0; j < NB; ++j) {
@@ -490,17 +543,18 @@ __device__ void gemm_loop(const DecView& d, const ChunkArgs& P, const Ctx& c) {
           __syncwarp();
           if (!on[j]) continue;  // the same for the warp's lanes
           const int grp = i / c.CS, owner = i - grp * c.CS;
-          const int v0 = c.rank * c.nl + m0 + 4 * lane, nv = lane < nq ? d.N - v0 : 0;
-          const float2 p = block_softmax(sum[j], nv);
-          if (lane == 0) {
-            const uint32_t dst =
-                sm0 + c.L.rows + grp * c.L.row_bytes + c.L.lse + 8 * ((part_buf(step) * c.CS + c.rank) * nb + m0 / kMB);
+          const float2 p = unit_softmax(sum[j], lo >= 0 ? d.N - v0 : 0, bl.halves, lane);
+          if (lane == 0 || (bl.halves && lane == 16)) {
+            const uint32_t dst = sm0 + c.L.rows + grp * c.L.row_bytes + c.L.lse +
+                                 8 * (part_buf(step) * c.sl->parts + c.sl->part0 + p0 + (lane >> 4));
             send8(map_rank(dst, owner), __float_as_int(p.x), __float_as_int(p.y),
                   map_rank(tc::smem_u32(c.sbar + kPartBars * grp + part_bar(step)), owner));
           }
         }
         __syncwarp();
         group_sync(1, kGemm);
+        m0 = bl.end;
+        p0 += 1;
       }
     }
     if (score) write_score();
@@ -733,7 +787,7 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
   };
 
   int t = 0, sym = 0, cnt = 0, step = 0;
-  const uint32_t row_bytes = 4u * (uint32_t)(c.CS * c.nl);
+  const uint32_t row_bytes = 32u * (uint32_t)slice_labels(d.N);
   bool ok = true, moved = true;
   begin_deltas(s.nl > 0 ? s.lmr[0].w : -1);
   sync();  // levels and depths are cleared before anyone sets one
@@ -955,8 +1009,7 @@ __global__ void __launch_bounds__(kGemm + RG * group_threads(RG), 1)
   Ctx c;
   c.sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(raw) + 127) & ~uintptr_t(127));
   c.CS = P.CS;
-  c.nl = P.nl;
-  c.L = layout(d.H, d.V4, c.nl, c.CS, NB, RG);
+  c.L = layout(d.N, d.H, d.V4, P.nl, c.CS, NB, RG);
   c.rank = (int)(blockIdx.x % (unsigned)c.CS);
   c.row0 = (int)(blockIdx.x / (unsigned)c.CS) * P.R;
   c.R = min(P.R, P.n - c.row0);
@@ -964,12 +1017,16 @@ __global__ void __launch_bounds__(kGemm + RG * group_threads(RG), 1)
   c.wbar = c.ybar + 1;
   c.lbar = c.ybar + 2;
   c.sbar = c.lbar + RG;
-  static_assert((2 + (1 + kPartBars) * RG) * 8 + 4 <= 128, "barrier area");
   int* fail = reinterpret_cast<int*>(c.sbar + kPartBars * RG);
   c.fail = fail;
   c.y = reinterpret_cast<int4*>(c.sm + c.L.y);
+  static_assert((2 + (1 + kPartBars) * RG) * 8 + 4 + sizeof(Slice) <= 128, "barrier area");
+  Slice* sl = reinterpret_cast<Slice*>(fail + 1);
+  c.sl = sl;
   const int tid = threadIdx.x;
   if (tid == 0) {
+    const Slice own = slice_of(d.N, c.CS, c.rank);
+    *sl = own;
     tc::mbar_init(c.ybar, 1);
     tc::mbar_init(c.wbar, 1);
     for (int g = 0; g < (1 + kPartBars) * RG; ++g) tc::mbar_init(c.lbar + g, 1);  // lbar, then sbar
@@ -977,9 +1034,9 @@ __global__ void __launch_bounds__(kGemm + RG * group_threads(RG), 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     tc::mbar_expect_tx(c.ybar, 16u * (uint32_t)c.R);  // the rows' first labels
     // this CTA's labels of W_out, row by row
-    tc::mbar_expect_tx(c.wbar, (uint32_t)(c.nl * 2 * d.H));
-    for (int j = 0; j < c.nl; ++j)
-      tc::bulk_g2s(c.sm + c.L.w + j * (2 * d.H + kWPad), d.Wt + (size_t)(c.rank * c.nl + j) * d.H, 2u * (uint32_t)d.H, c.wbar);
+    tc::mbar_expect_tx(c.wbar, (uint32_t)(own.len * 2 * d.H));
+    for (int j = 0; j < own.len; ++j)
+      tc::bulk_g2s(c.sm + c.L.w + j * (2 * d.H + kWPad), d.Wt + (size_t)(own.start + j) * d.H, 2u * (uint32_t)d.H, c.wbar);
   }
   // the call's shared rows: the defaults D, log p(v), and the labels that start a phrase
   float* dflt = reinterpret_cast<float*>(c.sm + c.L.dflt);
@@ -1015,7 +1072,7 @@ __global__ void __launch_bounds__(kGemm + RG * group_threads(RG), 1)
 // The joint kernel of the stateful form with few rows (its label step cannot
 // stay in one launch: the prediction network runs between two joint products):
 // the same product, sums and softmax partials as the loop above, so that both
-// forms give the same bits.  CTA (c, b): labels [c nl, (c+1) nl) of rows
+// forms give the same bits.  CTA (c, b): slice c of the labels, of rows
 // 8 NB b .., its slice of W_out requested before the wait for the joint
 // input (further rows follow in steps of the grid); the row pass
 // (row_stream.cu) finishes Eq. 1 from the stored logits.
@@ -1029,18 +1086,18 @@ __global__ void __launch_bounds__(kGemm, 1) k_joint_rows(const __grid_constant__
   const int ps = ((nl < kMB ? nl : kMB) + 11) / 16 * 16 + 4;  // as in layout()
   float* part = reinterpret_cast<float*>(sm + 128 + (nl * wstride + 127) / 128 * 128);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, k4 = lane & 3;
-  const int rank = blockIdx.x, n = d.params->n;
+  const Slice sl = slice_of(d.N, gridDim.x, blockIdx.x);
+  const int n = d.params->n;
   if (tid == 0) {
     tc::mbar_init(wbar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    tc::mbar_expect_tx(wbar, (uint32_t)(nl * 2 * H));
-    for (int j = 0; j < nl; ++j)
-      tc::bulk_g2s(sm + 128 + j * wstride, d.Wt + (size_t)(rank * nl + j) * H, 2u * (uint32_t)H, wbar);
+    tc::mbar_expect_tx(wbar, (uint32_t)(sl.len * 2 * H));
+    for (int j = 0; j < sl.len; ++j)
+      tc::bulk_g2s(sm + 128 + j * wstride, d.Wt + (size_t)(sl.start + j) * H, 2u * (uint32_t)H, wbar);
   }
   __syncthreads();
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int nb = (nl + kMB - 1) / kMB;
   bool first = true;
 #pragma unroll 1
   for (int i0 = blockIdx.y * 8 * NB; i0 < n; i0 += gridDim.y * 8 * NB) {
@@ -1064,22 +1121,23 @@ __global__ void __launch_bounds__(kGemm, 1) k_joint_rows(const __grid_constant__
         return;
       }
     }
-    for (int m0 = 0; m0 < nl; m0 += kMB) {
-      const int left = nl - m0;
-      if (left > 64) tile_block<10, NB, -1>(W, wstride, nl, m0, U, warp, g, k4, b, part, ps);
-      else if (left > 32) tile_block<8, NB, -1>(W, wstride, nl, m0, U, warp, g, k4, b, part, ps);
-      else tile_block<4, NB, -1>(W, wstride, nl, m0, U, warp, g, k4, b, part, ps);
+    int p0 = sl.part0;
+    for (int m0 = 0; m0 < sl.len;) {
+      const Block bl = block_at(sl, m0);
+      const int left = bl.end - m0;
+      if (left > 64) tile_block<10, NB, -1>(W, wstride, sl.len, m0, U, warp, g, k4, b, part, ps);
+      else if (left > 32) tile_block<8, NB, -1>(W, wstride, sl.len, m0, U, warp, g, k4, b, part, ps);
+      else tile_block<4, NB, -1>(W, wstride, sl.len, m0, U, warp, g, k4, b, part, ps);
       __syncthreads();
-      const int nq = min(kMB, nl - m0) / 4;
+      const int lo = lane_labels(sl, bl, m0, lane), v0 = sl.start + m0 + lo;
 #pragma unroll
       for (int j = 0; j < NB; ++j) {
         const int i = i0 + 8 * j + warp;
         __syncwarp();
         if (i >= n) continue;  // the same for the warp's lanes
-        const int v0 = rank * nl + m0 + 4 * lane;
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (lane < nq) {
-          s = sum_parts<NB>(part, 8 * j + warp, ps, lane);
+        if (lo >= 0) {
+          s = sum_parts<NB>(part, 8 * j + warp, ps, lo);
           const float4 dv = __ldcg(reinterpret_cast<const float4*>(d.dvec + v0));
           *reinterpret_cast<float4*>(d.logits + (size_t)i * d.N_pad + v0) =
               make_float4(s.x + dv.x, s.y + dv.y, s.z + dv.z, s.w + dv.w);
@@ -1091,11 +1149,13 @@ __global__ void __launch_bounds__(kGemm, 1) k_joint_rows(const __grid_constant__
               if (v0 + x < d.N) cl[x] = l[x];
           }
         }
-        const float2 p = block_softmax(s, lane < nq ? d.N - v0 : 0);
-        if (lane == 0)
-          d.part[(size_t)i * d.n_ptiles + rank * nb + m0 / kMB] = make_float4(p.x, p.y, kNegInf, __int_as_float(INT_MAX));
+        const float2 p = unit_softmax(s, lo >= 0 ? d.N - v0 : 0, bl.halves, lane);
+        if (lane == 0 || (bl.halves && lane == 16))
+          d.part[(size_t)i * d.n_ptiles + p0 + (lane >> 4)] = make_float4(p.x, p.y, kNegInf, __int_as_float(INT_MAX));
       }
       __syncthreads();
+      m0 = bl.end;
+      p0 += 1;
     }
   }
 }
@@ -1148,8 +1208,8 @@ cudaError_t chunk_cluster_shapes(const DecView& d, std::vector<ChunkShape>& out)
       for (int CS = 8; CS <= 16; CS *= 2) {
         ChunkShape s;
         s.CS = CS, s.RG = RG, s.NB = NB;
-        s.nl = ((d.N + CS - 1) / CS + 3) / 4 * 4;
-        const Layout L = layout(d.H, d.V4, s.nl, CS, NB, RG);
+        s.nl = slice_of(d.N, CS, 0).len;  // (the largest)
+        const Layout L = layout(d.N, d.H, d.V4, s.nl, CS, NB, RG);
         if (L.total > lim) continue;
         s.smem = L.total;
         cudaLaunchAttribute a[1];
@@ -1183,17 +1243,7 @@ const ChunkShape* chunk_cluster_pick(const std::vector<ChunkShape>& shapes, int 
   return best;
 }
 
-int joint_rows_tiles(const ChunkShape& s) { return s.CS * ((s.nl + kMB - 1) / kMB); }
-
-int joint_rows_max_tiles(int N) {
-  int most = 0;
-  for (int CS = 8; CS <= 16; CS *= 2) {
-    ChunkShape s;
-    s.CS = CS, s.nl = ((N + CS - 1) / CS + 3) / 4 * 4;
-    most = std::max(most, joint_rows_tiles(s));
-  }
-  return most;
-}
+int joint_rows_tiles(int N) { return slice_of(N, 8, 0).parts; }
 
 cudaError_t joint_rows_prepare() {
   int dev = 0, lim = 0;

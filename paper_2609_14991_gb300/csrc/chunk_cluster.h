@@ -18,7 +18,7 @@ struct ChunkArgs {
   int32_t* out_count;
   int32_t n, T;
   float lambda, beta;
-  int32_t CS, nl, R;  // CTAs per cluster, labels per CTA, rows per cluster
+  int32_t CS, nl, R;  // CTAs per cluster, most labels of a CTA, rows per cluster
   int32_t slots[kChunkMaxRows];
 };
 
@@ -26,7 +26,7 @@ struct ChunkShape {
   int CS = 0;        // CTAs per cluster
   int RG = 0;        // row groups per CTA
   int NB = 0;        // 8-row blocks of the product
-  int nl = 0;        // labels per CTA
+  int nl = 0;        // most labels of a CTA
   int smem = 0;      // bytes per CTA
   int clusters = 0;  // clusters the device runs at once
 };
@@ -37,10 +37,8 @@ cudaError_t chunk_cluster_shapes(const DecView& d, std::vector<ChunkShape>& out)
 // The shape for n rows, or nullptr if none holds them in one wave.
 const ChunkShape* chunk_cluster_pick(const std::vector<ChunkShape>& shapes, int n, int H);
 // The stateful form's joint product with the same sums, for rows that a shape
-// holds: softmax partials per row (of a shape, and the most of any for N
-// labels), launch.
-int joint_rows_tiles(const ChunkShape& s);
-int joint_rows_max_tiles(int N);
+// holds: softmax partials per row of N labels, launch.
+int joint_rows_tiles(int N);
 cudaError_t joint_rows_prepare();
 void launch_joint_rows(const ChunkShape& s, const DecView& d, int n, int step, cudaStream_t st, bool pdl);
 cudaError_t launch_chunk_cluster(const ChunkShape& s, const DecView& d, ChunkArgs& a, cudaStream_t st);

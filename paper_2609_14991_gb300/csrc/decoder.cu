@@ -78,7 +78,7 @@ void enqueue_chunk(tsd_decoder* d, int M, int T, cudaStream_t s, const std::vect
   };
   const tsd_decoder::Pred& pr = d->pred;
   const ChunkShape* rows = joint_rows_shape(d, M);
-  if (rows) v.n_ptiles = joint_rows_tiles(*rows);
+  if (rows) v.n_ptiles = joint_rows_tiles(d->N);
   launch_defaults(v, s);
   if (pr.D) {
     // the chunk's encoder frames to a fixed buffer, then their projection
@@ -231,7 +231,7 @@ tsd_status create_impl(const tsd_decoder_cfg* cfg, const void* W_out_bf16, const
   tsd_status st;
   if ((st = A.alloc(&Wt, (size_t)d->N_pad * c.H)) || (st = A.alloc(&E, (size_t)d->N * c.H)) ||
       (st = A.alloc(&Abuf, (size_t)d->M_pad * c.H)) ||
-      (st = A.alloc(&part, (size_t)d->M_pad * std::max(d->N_pad / 64, pw ? joint_rows_max_tiles(d->N) : 0))) || (st = A.alloc(&err, 1)) || (st = A.alloc(&ctr, 2)) || (st = A.alloc(&dflt, (size_t)d->V4)) || (st = A.alloc(&droot, (size_t)(d->V4 + 31) / 32)) || (st = A.alloc(&rt, (size_t)d->M_pad)) ||
+      (st = A.alloc(&part, (size_t)d->M_pad * std::max(d->N_pad / 64, pw ? joint_rows_tiles(d->N) : 0))) || (st = A.alloc(&err, 1)) || (st = A.alloc(&ctr, 2)) || (st = A.alloc(&dflt, (size_t)d->V4)) || (st = A.alloc(&droot, (size_t)(d->V4 + 31) / 32)) || (st = A.alloc(&rt, (size_t)d->M_pad)) ||
       (st = A.alloc(&rs, (size_t)d->M_pad)) || (st = A.alloc(&rc, (size_t)d->M_pad)) ||
       (st = A.alloc(&sl, SK)) || (st = A.alloc(&sll, SK * NL)) || (st = A.alloc(&slc, SK * NL * kLmChain)) ||
       (st = A.alloc(&stl, SK)) || (st = A.alloc(&stc, SK * kTrChain)) || (st = A.alloc(&pdev, d->params_bytes)) ||
