@@ -406,13 +406,15 @@ TSD_API tsd_status tsd_debug_fail_alloc(int32_t n);
  * label step reps times back to back on cuda_stream -- kernel 0 the row
  * pass (in a mode that redoes the step's work but commits no state or
  * output), kernel 1 the joint GEMM (idempotent) -- so a caller can time it
- * with CUDA events in isolation.  Later decode_chunk calls are unaffected.
+ * with CUDA events in isolation.  After a chunk that ran in one launch, the
+ * two kernels that would have taken its last step.  Later decode_chunk calls
+ * are unaffected.
  * If algo_bytes is non-NULL the call waits for the stream and stores the
  * algorithmic bytes of one launch: for the row pass, counted by the kernel
  * (partials, row state, label searches, joint input, every LM arc and trie
  * child of the chains, plus the shared unigram/root rows once; not the
- * dense bias it writes); for the joint kernel, its operands, bias rows and
- * partials.  TSD_ESTATE before the first decode_chunk. */
+ * dense bias a beam's writes); for the joint kernel, its operands and what it
+ * writes, logits and partials.  TSD_ESTATE before the first decode_chunk. */
 TSD_API tsd_status tsd_decoder_replay(tsd_decoder* dec, int32_t kernel, int32_t reps, void* cuda_stream,
                                       int64_t* algo_bytes);
 

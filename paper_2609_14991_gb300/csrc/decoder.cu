@@ -1143,14 +1143,19 @@ extern "C" tsd_status tsd_decoder_replay(tsd_decoder* d, int32_t kernel, int32_t
     launch_defaults(d->view, s);
   }
   if (algo_bytes) TSD_CUDA(cudaMemsetAsync(d->view.ctr, 0, sizeof(unsigned long long), s));
+  // the stateful form with few rows has its own joint kernel and partials, as in enqueue_chunk
+  DecView v = d->view;
+  const ChunkShape* rows = joint_rows_shape(d, M);
+  if (rows) v.n_ptiles = joint_rows_tiles(d->N);
   for (int i = 0; i < reps; ++i) {
-    if (kernel == 0 && d->cfg.beam_k > 1) launch_row_beam(d->view, d->last_n, S - 1, 2, d->row_smem, s, false);
-    else if (kernel == 0 && d->cfg.prune_k > 0) launch_row_pruned(d->view, M, S - 1, 2, s, false);
-    else if (kernel == 0 && d->view.fused && d->view.fz_dense) launch_row_fused(d->view, M, S - 1, 2, row_fused_smem_bytes(d->V4, d->N_pad), s, false);
-    else if (kernel == 0 && d->view.fused) launch_row_stream(d->view, M, S - 1, 2, row_stream_smem_bytes(d->V4), s, false);
-    else if (kernel == 0) launch_row(d->view, M, S - 1, 2, d->row_smem, s, false);
-    else if (d->joint_kind == 0) launch_joint_tc(*d->jtc, d->view, M, 1 << 30, s, false);
-    else launch_joint(d->view, M, 1 << 30, s);
+    if (kernel == 0 && d->cfg.beam_k > 1) launch_row_beam(v, d->last_n, S - 1, 2, d->row_smem, s, false);
+    else if (kernel == 0 && d->cfg.prune_k > 0) launch_row_pruned(v, M, S - 1, 2, s, false);
+    else if (kernel == 0 && v.fused && v.fz_dense) launch_row_fused(v, M, S - 1, 2, row_fused_smem_bytes(d->V4, d->N_pad), s, false);
+    else if (kernel == 0 && v.fused) launch_row_stream(v, M, S - 1, 2, row_stream_smem_bytes(d->V4), s, false);
+    else if (kernel == 0) launch_row(v, M, S - 1, 2, d->row_smem, s, false);
+    else if (rows) launch_joint_rows(*rows, v, M, 1 << 30, s, false);
+    else if (d->joint_kind == 0) launch_joint_tc(*d->jtc, v, M, 1 << 30, s, false);
+    else launch_joint(v, M, 1 << 30, s);
   }
   TSD_CUDA(cudaGetLastError());
   if (algo_bytes) {
@@ -1165,7 +1170,7 @@ extern "C" tsd_status tsd_decoder_replay(tsd_decoder* d, int32_t kernel, int32_t
       // joint, streaming epilogue: the operands once (A rows, W_out), the
       // logits written and the softmax partials
       *algo_bytes = (int64_t)M * d->cfg.H * 2 + (int64_t)d->N * d->cfg.H * 2 + (int64_t)M * d->N * 4 +
-                    (int64_t)M * d->n_ptiles * 8;
+                    (int64_t)M * v.n_ptiles * 8;
     } else if (d->view.fused) {
       // joint, dense epilogue: the operands once (A rows, W_out), each row's
       // dense LM row and mask, the defaults, the partials written (the
