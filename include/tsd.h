@@ -414,7 +414,7 @@ TSD_API tsd_status tsd_debug_fail_alloc(int32_t n);
  * (partials, row state, label searches, joint input, every LM arc and trie
  * child of the chains, plus the shared unigram/root rows once; not the
  * dense bias a beam's writes); for the joint kernel, its operands and what it
- * writes, logits and partials.  TSD_ESTATE before the first decode_chunk. */
+ * writes: logits (or, pruned, the tiles' best labels) and partials.  TSD_ESTATE before the first decode_chunk. */
 TSD_API tsd_status tsd_decoder_replay(tsd_decoder* dec, int32_t kernel, int32_t reps, void* cuda_stream,
                                       int64_t* algo_bytes);
 

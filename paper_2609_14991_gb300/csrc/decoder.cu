@@ -1178,9 +1178,10 @@ extern "C" tsd_status tsd_decoder_replay(tsd_decoder* d, int32_t kernel, int32_t
       *algo_bytes = (int64_t)M * d->cfg.H * 2 + (int64_t)d->N * d->cfg.H * 2 + (int64_t)M * d->V4 * 4 +
                     (int64_t)M * d->view.mask_words * 4 + (int64_t)d->N_pad * 4 + (int64_t)M * d->n_ptiles * 16;
     } else {
-      // joint: the operands once (A rows, W_out) and the bias rows read by the epilogue
-      *algo_bytes = (int64_t)M * d->cfg.H * 2 + (int64_t)d->N * d->cfg.H * 2 + (int64_t)M * d->N * 4 +
-                    (int64_t)M * d->n_ptiles * 16;
+      // joint, pruned fusion: the operands once (A rows, W_out), each tile's
+      // softmax partial and best labels written
+      *algo_bytes = (int64_t)M * d->cfg.H * 2 + (int64_t)d->N * d->cfg.H * 2 +
+                    (int64_t)M * d->n_ptiles * 8 * (1 + d->cfg.prune_k);
     }
   }
   return TSD_OK;
