@@ -58,10 +58,14 @@ namespace {
 
 using row::best_merge;
 using row::checked;
+using row::first_load;
 using row::key_value;
 using row::kNegInf;
+using row::level_groups;
 using row::lse_merge;
 using row::order_key;
+using row::warp_find_wide;
+using tc::map_rank;
 
 constexpr int kGemm = 256;     // GEMM threads (8 warps, each an eighth of H)
 constexpr int kTiles = 5;      // 16-label tiles per accumulator block
@@ -69,12 +73,6 @@ constexpr int kMB = 16 * kTiles;
 constexpr int kUnits = 4;      // 32-wide pieces of H per warp: H <= 1024
 constexpr int kTrHeld = 3;     // trie chain nodes whose first children a thread requests together
 constexpr int kWPad = 64;      // bytes after a W_out row: neighbouring rows start 16 banks apart
-
-__device__ __forceinline__ uint32_t map_rank(uint32_t addr, int rank) {
-  uint32_t r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
 
 // Remote stores that complete their bytes on a barrier of the receiving CTA.
 __device__ __forceinline__ void send16(uint32_t dst, float4 v, uint32_t bar) {
@@ -251,56 +249,6 @@ __host__ __device__ inline Layout layout(int N, int H, int V4, int nl, int CS, i
   L.row_bytes = r;
   L.total = o + RG * r + 128;                // and the alignment of the base
   return L;
-}
-
-// Aligned groups of four arcs a chain level's arcs [b, b + c) span.
-__device__ __forceinline__ int level_groups(int b, int c) { return c > 0 ? (b + c - (b & ~3) + 3) >> 2 : 0; }
-
-// Position of y in the sorted arr[0, n), or -1, by one warp (row_stream.cu
-// describes the search).  pre: this lane's probe of the whole range (n > 124)
-// or its four entries (n <= 124), loaded before y was known.
-__device__ __forceinline__ int find_from(const int32_t* __restrict__ arr, int n, int y, int lane, int4 pre) {
-  row::reconverge();
-  int lo = 0, hi = n;
-  bool whole = n <= 124;
-  if (!whole) {
-    int v = pre.x;
-    for (;;) {
-      const int step = (hi - lo + 31) >> 5;
-      const unsigned m = __ballot_sync(0xffffffffu, v <= y);
-      if (m == 0) return -1;
-      lo = lo + (31 - __clz((int)m)) * step;
-      hi = min(hi, lo + step);
-      if (hi - lo <= 124) break;
-      const int idx = lo + lane * ((hi - lo + 31) >> 5);
-      v = (idx < hi) ? __ldg(arr + idx) : INT_MAX;
-    }
-  }
-  const uintptr_t at = reinterpret_cast<uintptr_t>(arr + lo);
-  const int first = 4 * lane - (int)((at & 15u) >> 2);
-  int pos = -1;
-  if (first < hi - lo) {
-    const int4 t = whole ? pre : __ldg(reinterpret_cast<const int4*>(at & ~uintptr_t(15)) + lane);
-    const int tv[4] = {t.x, t.y, t.z, t.w};
-#pragma unroll
-    for (int j = 3; j >= 0; --j)
-      if (first + j >= 0 && first + j < hi - lo && tv[j] == y) pos = lo + first + j;
-  }
-  const unsigned m = __ballot_sync(0xffffffffu, pos >= 0);
-  return m ? __shfl_sync(0xffffffffu, pos, __ffs((int)m) - 1) : -1;
-}
-
-// What find_from wants in `pre` for the range arr[0, n).
-__device__ __forceinline__ int4 first_probe(const int32_t* __restrict__ arr, int n, int lane) {
-  int4 pre = make_int4(INT_MAX, INT_MAX, INT_MAX, INT_MAX);
-  if (n > 124) {
-    const int at = lane * ((n + 31) >> 5);
-    if (at < n) pre.x = __ldg(arr + at);
-  } else {
-    const uintptr_t a = reinterpret_cast<uintptr_t>(arr);
-    if (4 * lane - (int)((a & 15u) >> 2) < n) pre = __ldg(reinterpret_cast<const int4*>(a & ~uintptr_t(15)) + lane);
-  }
-  return pre;
 }
 
 struct Ctx {
@@ -893,7 +841,7 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
       int4 r0;
       if (warp == 0 && nl > 0) {
         const int4 q = s.lmr[0];
-        a0 = list ? find_list(y) : find_from(d.lm.arc_tok + q.x, q.y, y, lane, first_probe(d.lm.arc_tok + q.x, q.y, lane));
+        a0 = list ? find_list(y) : warp_find_wide<true>(d.lm.arc_tok + q.x, q.y, y, lane, first_load(d.lm.arc_tok + q.x, q.y, lane));
         if (lane == 0 && a0 >= 0) r0 = __ldg(d.lm.arc_rec + q.x + a0);
       }
       if (t < T) begin_deltas(lm2 ? y : -1);
@@ -915,7 +863,7 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
           const bool is_lm = task < nl;
           const int4 q = is_lm ? s.lmr[task] : s.trr[task - nl];
           const int32_t* arr = (is_lm ? d.lm.arc_tok : d.tr.ch_tok) + q.x;
-          const int at = find_from(arr, q.y, y, lane, first_probe(arr, q.y, lane));
+          const int at = warp_find_wide<true>(arr, q.y, y, lane, first_load(arr, q.y, lane));
           if (lane == 0 && at >= 0) {
             if (is_lm) s.lm_hit[task] = __ldg(d.lm.arc_rec + q.x + at);
             else s.tr_hit[task - nl] = __ldg(d.tr.ch_rec + q.x + at), s.dd[task - nl] = q.z + 1;
@@ -923,7 +871,7 @@ __device__ void row_loop(const DecView& d, const ChunkArgs& P, const Ctx& c, int
         }
         if (nl == 0 && warp == 0 && nt > 0) {  // (no LM chain: the first task is the deepest trie node)
           const int4 q = s.trr[0];
-          const int at = find_from(d.tr.ch_tok + q.x, q.y, y, lane, first_probe(d.tr.ch_tok + q.x, q.y, lane));
+          const int at = warp_find_wide<true>(d.tr.ch_tok + q.x, q.y, y, lane, first_load(d.tr.ch_tok + q.x, q.y, lane));
           if (lane == 0 && at >= 0) s.tr_hit[0] = __ldg(d.tr.ch_rec + q.x + at), s.dd[0] = q.z + 1;
         }
       }

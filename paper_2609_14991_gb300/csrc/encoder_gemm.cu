@@ -81,12 +81,6 @@ __device__ __forceinline__ uint32_t pack_bf16(uint64_t x) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-__device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-
 // TMA load whose bytes complete on a barrier of this CTA or its pair's leader.
 template <bool PAIR>
 __device__ __forceinline__ void load_2d(void* dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
@@ -178,8 +172,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int Mt = (g.M + kTM - 1) / kTM, Nt = (g.N + BN - 1) / BN;
   const int tiles = Mt * Nt;
 
-  // the kernel after this one may start its own set-up (it waits for this
-  // grid's end before it touches anything the chunk writes)
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(full + s, 1);

@@ -262,7 +262,7 @@ __global__ void __launch_bounds__((DSmem<BN, BM>::kThreads), 1)
         __syncwarp();
         const int c0 = n0 + b * kCW;
         float l[kCW];
-        tmem_ld<kCW>(tbase + (uint32_t)(b * kCW), l);
+        tmem_ld32(tbase + (uint32_t)(b * kCW), l);
         if (c0 + kCW > N) {
 #pragma unroll
           for (int i = 0; i < kCW; ++i)
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__((DSmem<BN, BM>::kThreads), 1)
         __syncwarp();
         const int c0 = n0 + b * kCW;
         float l[kCW];
-        tmem_ld<kCW>(tbase + (uint32_t)(b * kCW), l);
+        tmem_ld32(tbase + (uint32_t)(b * kCW), l);
         if (c0 + kCW > N) {
 #pragma unroll
           for (int i = 0; i < kCW; ++i)

@@ -245,12 +245,8 @@ __global__ void __launch_bounds__(kRowThreads) k_row_beam(DecView d, int step, i
         const float4 p = __ldcg(d.part + (size_t)rk * d.n_ptiles + j);
         lse_merge(m, z, p.x, p.y);
       }
-      row::reconverge();
-      const float top = row::key_value(__reduce_max_sync(0xffffffffu, row::order_key(m)));
-      z = z > 0.f ? z * expf(m - top) : 0.f;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-      if (lane == 0) s_lse = top + logf(z);
+      const float lse = row::warp_lse(m, z);
+      if (lane == 0) s_lse = lse;
     }
     // each warp's K best of its labels, then the first warp's K best of those
     // (a thread reads only the labels it wrote: no barrier before)
