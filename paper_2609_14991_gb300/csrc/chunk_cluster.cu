@@ -273,8 +273,7 @@ struct Piece {
 // warp's part of H for 8 NB rows, written to the partials [warp][row][label].
 // Labels past the slice read its last row again, and the upper half of an odd
 // last tile its lower half: their sums are never sent.
-// FU >= 0: every warp has FU pieces of H and some one more (their products
-// are scheduled together); -1: any number.
+// FU >= 0: every warp has FU pieces of H (H / 256) and some one more; -1: any number.
 template <int HT, int NB, int FU>
 __device__ __forceinline__ void tile_block(const unsigned char* W, int wstride, int nl, int m0, int U, int warp, int g, int k4,
                                            const uint4 (&b)[kUnits][NB], float* part, int ps) {
@@ -1114,13 +1113,31 @@ int joint_rows_smem(int H, int nl, int NB) {
 }
 
 typedef void (*ChunkFn)(DecView, ChunkArgs);
-// The kernel of a shape (nullptr: there is none), for hidden size H.
+// The kernel of a shape (nullptr: there is none), for hidden size H.  Fixed trip
+// counts let the product's loads of W_out be scheduled ahead of its MMAs, where
+// there are registers for it.  A chunk of 13 frames without and with them, us:
+//   one group, 16 rows a pass: 64 streams, V 1024: H 320 244 / 229, 640 248 / 235,
+//     832 267 / 260, 1024 348 / 328;
+//   one group, 8 rows: one stream, H 320 181.7 / 180.5, 640 172.7 / 171.9, 832
+//     186.4 / 186.5, 1024 164.5 / 166.6; 100 streams, V 2048, H 512, 564 / 548;
+//   two groups: 128 streams, V 700, H 320 435 / 368; V 512, H 640 314 / 298, 1024
+//     467 / 472; 224 streams, H 832 429 / 420;
+//   three groups: V 512, 300 streams, H 320 501 / 451, 336, 640 562 / 512; 128, V 1024,
+//     H 640 588 / 520; 224, H 1024 499 / 499.
+template <int NB, int RG, int MAX>
+ChunkFn fixed_trips(int H) {
+  switch (H / 256) {
+    case 1: return k_chunk<NB, RG, 1>;
+    case 2: return k_chunk<NB, RG, 2>;
+    case 3: if constexpr (MAX >= 3) return k_chunk<NB, RG, 3>; break;
+    case 4: if constexpr (MAX >= 4) return k_chunk<NB, RG, 4>; break;
+  }
+  return k_chunk<NB, RG, -1>;
+}
 ChunkFn kernel_of(int NB, int RG, int H) {
-  const int fu = H == 1024 ? 4 : (H >= 512 && H < 768 ? 2 : -1);
-  if (RG == 1 && NB == 1) return fu == 4 ? k_chunk<1, 1, 4> : fu == 2 ? k_chunk<1, 1, 2> : k_chunk<1, 1, -1>;
-  if (RG == 1) return fu == 4 ? k_chunk<2, 1, 4> : fu == 2 ? k_chunk<2, 1, 2> : k_chunk<2, 1, -1>;
-  if (RG == 2) return NB == 1 ? k_chunk<1, 2, -1> : k_chunk<2, 2, -1>;
-  return NB == 1 ? nullptr : fu == 4 ? k_chunk<2, 3, 4> : k_chunk<2, 3, -1>;
+  if (RG == 1) return NB == 1 ? fixed_trips<1, 1, 2>(H) : fixed_trips<2, 1, 4>(H);
+  if (RG == 2) return NB == 1 ? k_chunk<1, 2, -1> : fixed_trips<2, 2, 3>(H);
+  return NB == 1 ? nullptr : fixed_trips<2, 3, 4>(H);
 }
 
 cudaLaunchConfig_t config(const ChunkShape& s, int clusters, cudaLaunchAttribute* a, cudaStream_t st) {

@@ -87,7 +87,8 @@ def test_tables(case):
     pu.assert_reports(pu.replay(inp, one, range(w.B)))
 
 
-@pytest.mark.parametrize("V,H", [(15, 64), (255, 320), (511, 320), (639, 640), (700, 448), (1023, 640), (1300, 512)])
+@pytest.mark.parametrize("V,H", [(15, 64), (255, 320), (511, 320), (639, 640), (700, 448), (1023, 640), (1300, 512),
+                                 (600, 832), (500, 1024), (300, 192)])
 def test_results_do_not_depend_on_the_other_rows(V, H):
     """The same bits alone and in calls whose rows take clusters of 8 and of
     16, one to three row groups and one or two passes of the product."""
