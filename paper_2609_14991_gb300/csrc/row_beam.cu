@@ -73,6 +73,10 @@ __device__ __forceinline__ double log_add(double a, double b) {
   return m + log(1.0 + exp(fmin(a, b) - m));  // (the larger one's exponential is 1)
 }
 
+// A score as the ranks compare it: NaN (from a logit that is NaN or infinite)
+// counts as the lowest, so that ranks are distinct and every place is taken.
+__device__ __forceinline__ double ranked(double s) { return s == s ? s : -(double)__builtin_huge_val(); }
+
 // candidate order: score desc, hypothesis asc, label asc
 __device__ __forceinline__ bool cand_before(double s1, int h1, int t1, double s2, int h2, int t2) {
   if (s1 != s2) return s1 > s2;
@@ -315,7 +319,7 @@ __global__ void __launch_bounds__(kRowThreads) k_row_beam(DecView d, int step, i
     for (int e = tid; e < CC * CC; e += kRowThreads) {
       const int c = e / CC, x = e - c * CC, hc = c / K, hx = x / K;
       const bool cin = c_tok[c] >= 0 && o_live[hc], xin = c_tok[x] >= 0 && o_live[hx];
-      const double sc = o_score[hc] + (double)c_inc[c], sx = o_score[hx] + (double)c_inc[x];
+      const double sc = ranked(o_score[hc] + (double)c_inc[c]), sx = ranked(o_score[hx] + (double)c_inc[x]);
       if (cin && xin && cand_before(sx, hx, c_tok[x], sc, hc, c_tok[c])) atomicAdd(s_rank + c, 1);
     }
     row::block_sync();
@@ -517,7 +521,7 @@ __global__ void __launch_bounds__(kRowThreads) k_row_beam(DecView d, int step, i
         for (int x = 0; x < nf; ++x) {
           int rank = 0;
           for (int y = 0; y < nf; ++y)
-            if (q_score[y] > q_score[x] || (q_score[y] == q_score[x] && y < x)) ++rank;
+            if (ranked(q_score[y]) > ranked(q_score[x]) || (ranked(q_score[y]) == ranked(q_score[x]) && y < x)) ++rank;
           if (rank < K) f_src[fc++] = q_src[x];
         }
       }
