@@ -152,11 +152,11 @@ __device__ __forceinline__ void best_merge(float& v, int& i, float v2, int i2) {
 }
 
 // The log-sum-exp of softmax partials (max, sum of exp(x - max)) by one warp,
-// whose lanes have merged every 32nd one.
+// whose lanes have merged every 32nd one.  A NaN sum gives NaN.
 __device__ __forceinline__ float warp_lse(float m, float z) {
   reconverge();
   const float top = key_value(__reduce_max_sync(0xffffffffu, order_key(m)));
-  z = z > 0.f ? z * expf(m - top) : 0.f;
+  z = z == 0.f ? 0.f : z * expf(m - top);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
   return top + logf(z);

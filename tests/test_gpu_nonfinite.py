@@ -1,5 +1,6 @@
 """Infinite and NaN encoder frames in one stream of a call: the other streams'
-results keep their bits, every label stays in range and the decoder goes on."""
+results keep their bits, every label stays in range and the decoder goes on.
+A NaN logit makes its row's scores NaN."""
 import numpy as np
 import pytest
 
@@ -55,3 +56,28 @@ def test_beam(K, S):
             assert 0 <= n <= 3 * w.T * S
     for h in got_h:
         assert len(h) <= K and all(0 <= t < w.V for toks, _ in h for t in toks)
+
+
+@pytest.mark.parametrize("form", ["one launch", "row pass, few rows", "row pass, many rows", "several lms"])
+def test_a_nan_logit_reaches_the_scores(form):
+    import paper_2609_14991_gb300 as tsd
+
+    w = synth.scaled(synth.WORKLOADS[0], V=300, H=128, B=480 if form == "row pass, many rows" else 4, T=4, lm_total=6000)
+    lmA, ph = synth.ngram_lm(7, w.V, 3, 6000, 1.1), synth.phrases(7, w.V, 6, 1, 3, 0.0)
+    E, W = synth.joint_weights(w)
+    W = W.copy()
+    W[5, 250] = 0x7FC0
+    dev = torch.device("cuda", 0)
+    lm = tsd.NGram.from_arrays(lmA)
+    how = dict(lms=[(lm, 1.0), (lm, 0.5)]) if form == "several lms" else dict(lm=lm)
+    dec = tsd.Decoder(w.V, w.H, torch.from_numpy(W.view(np.int16)).to(dev), torch.from_numpy(E.view(np.int16)).to(dev),
+                      boost=tsd.Boost.from_phrases(w.V, ph, w.bonus), max_symbols=w.max_sym, max_streams=w.B, max_T=w.T, **how)
+    dec.set_option("one_launch", 1 if form == "one launch" else 0)
+    slots = [dec.open() for _ in range(w.B)]
+    o = dec.decode_chunk(slots, torch.from_numpy(synth.enc_chunk(w, range(w.B), 0).view(np.int16)).to(dev), w.lam, w.beta)
+    torch.cuda.synchronize()
+    tok, sc, n = (x.cpu().numpy() for x in (o.tokens, o.scores, o.counts))
+    dec.check()
+    assert n.sum() > 0
+    for i in range(w.B):
+        assert (tok[i, :n[i]] != 250).all() and np.isnan(sc[i, :n[i]]).all(), (i, sc[i, :n[i]])
