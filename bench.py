@@ -646,7 +646,8 @@ def run_ours(args, w):
     joint_roof = {"kernel": ("k_joint_greedy<dense>: joint GEMM (tcgen05) + epilogue applying Eq. 1 with the dense "
                              "LM row, log-softmax and selection partials") if ep else
                             ("k_joint_greedy<streaming>: joint GEMM (tcgen05) + epilogue writing logit + defaults "
-                             "(TMA stores) and log-softmax partials") if not args.prune_k else
+                             "(TMA stores) and log-softmax partials"
+                             + ("; with few rows k_joint_rows (mma.sync)" if args.pred else "")) if not args.prune_k else
                             "k_joint_tc: joint GEMM (tcgen05) + log-softmax/top-K epilogue",
                   "bound": "tensor", "unit": "TFLOP/s",
                   "achieved": flop_per_launch / (joint_ms / 1000.0) / 1e12,

@@ -73,12 +73,17 @@ __device__ __forceinline__ double log_add(double a, double b) {
   return m + log(1.0 + exp(fmin(a, b) - m));  // (the larger one's exponential is 1)
 }
 
-// A score as the ranks compare it: NaN (from a logit that is NaN or infinite)
-// counts as the lowest, so that ranks are distinct and every place is taken.
-__device__ __forceinline__ double ranked(double s) { return s == s ? s : -(double)__builtin_huge_val(); }
+// A score as an integer of the same order, for the ranks.  NaN (from a logit
+// that is NaN or infinite) counts as the lowest, so that ranks are distinct and
+// every place is taken.
+__device__ __forceinline__ long long rank_key(double s) {
+  const long long i = __double_as_longlong(s), low = 0x7fffffffffffffffll;
+  if ((i & low) > 0x7ff0000000000000ll) return -low - 1;
+  return (i & low) == 0 ? 0 : i ^ ((i >> 63) & low);  // (-0 is 0)
+}
 
 // candidate order: score desc, hypothesis asc, label asc
-__device__ __forceinline__ bool cand_before(double s1, int h1, int t1, double s2, int h2, int t2) {
+__device__ __forceinline__ bool cand_before(long long s1, int h1, int t1, long long s2, int h2, int t2) {
   if (s1 != s2) return s1 > s2;
   if (h1 != h2) return h1 < h2;
   return t1 < t2;
@@ -319,7 +324,7 @@ __global__ void __launch_bounds__(kRowThreads) k_row_beam(DecView d, int step, i
     for (int e = tid; e < CC * CC; e += kRowThreads) {
       const int c = e / CC, x = e - c * CC, hc = c / K, hx = x / K;
       const bool cin = c_tok[c] >= 0 && o_live[hc], xin = c_tok[x] >= 0 && o_live[hx];
-      const double sc = ranked(o_score[hc] + (double)c_inc[c]), sx = ranked(o_score[hx] + (double)c_inc[x]);
+      const long long sc = rank_key(o_score[hc] + (double)c_inc[c]), sx = rank_key(o_score[hx] + (double)c_inc[x]);
       if (cin && xin && cand_before(sx, hx, c_tok[x], sc, hc, c_tok[c])) atomicAdd(s_rank + c, 1);
     }
     row::block_sync();
@@ -521,7 +526,7 @@ __global__ void __launch_bounds__(kRowThreads) k_row_beam(DecView d, int step, i
         for (int x = 0; x < nf; ++x) {
           int rank = 0;
           for (int y = 0; y < nf; ++y)
-            if (ranked(q_score[y]) > ranked(q_score[x]) || (ranked(q_score[y]) == ranked(q_score[x]) && y < x)) ++rank;
+            if (rank_key(q_score[y]) > rank_key(q_score[x]) || (rank_key(q_score[y]) == rank_key(q_score[x]) && y < x)) ++rank;
           if (rank < K) f_src[fc++] = q_src[x];
         }
       }
