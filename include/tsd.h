@@ -359,9 +359,9 @@ TSD_API tsd_status tsd_decoder_check(tsd_decoder* dec);
 /* Tuning knobs, by name (drops captured graphs):
  *   "one_launch" 1 (default) / 0: greedy decoding with at most one LM runs a
  *              whole chunk in one launch where W_out fits a thread-block
- *              cluster's shared memory and the call's rows fit one wave of
- *              clusters (112 rows at V = 1024, H = 1024; up to 336 with a
- *              smaller W_out); 0, other
+ *              cluster's shared memory, the call's rows fit one wave of
+ *              clusters and that is no slower (112 rows at V = 1024, H = 1024;
+ *              up to 336 with a smaller W_out); 0, other
  *              calls, and calls with set_timing(1), joint kernel 1, a chosen
  *              joint_bn or fusion_path 1 run a row pass and a joint kernel per
  *              label step.  A stream's results are the same bits in all calls

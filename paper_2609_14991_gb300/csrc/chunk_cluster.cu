@@ -1186,12 +1186,22 @@ cudaError_t chunk_cluster_shapes(const DecView& d, std::vector<ChunkShape>& out)
   return cudaSuccess;
 }
 
-// Every shape measured was faster than the two-kernel step, 40 label steps
-// each (n rows, V x H): 112, 1024 x 1024: 233 against 498 us; 100, 2048 x 512 in two
-// passes: 312 / 438; three groups of 64 threads 200, 512 x 640: 208 / 417; 336: 358 /
-// 415; 128, 1024 x 640: 377 / 437 -- but where three groups read more than 192
-// KB of W_out per step (passes x slice): 256, 1024 x 512 (210 KB): 487 / 405;
-// 256, 1024 x 640 (261 KB): 571 / 440.
+// Where the one launch is no slower than the two-kernel step (7 to 8 us a label
+// step at these sizes).  A chunk of 13 frames, one launch / two kernels, us:
+//   one group, one pass, always: 112 rows, V 1024, H 1024: 388 / 517; 120, H 640: 346 /
+//     478; 112, V 1500, H 512: 305 / 462; V 2048, H 320: 370 / 504;
+//   in two passes of 8 rows up to 10 rows a cluster: V 1300, H 896: 70 rows 460 / 481,
+//     112: 482 / 481; V 2048, H 512: 57 rows 527 / 491, 112: 578 / 504;
+//   two groups, where a slice is one block of the product or H < 512: 200 rows, V 512,
+//     H 640: 314 / 482; H 1024: 491 / 528; V 600, H 832: 494 / 491; V 1024, H 320: 342 /
+//     467; H 448: 456 / 480; V 1200, H 320: 522 / 515; not V 700, H 512: 506 / 486; H 640:
+//     534 / 478;
+//   three groups of 64 threads, in clusters of 8, a slice one block, H < 768 and up to
+//     170 KB of W_out a step: 300 rows, V 512, H 320 (85 KB): 409 / 480; V 620, H 448
+//     (140): 440 / 494; V 639, H 512 (160): 490 / 500; 336, V 512, H 640 (170): 508 / 496;
+//     not 260 rows, V 600, H 640 (190): 542 / 494; V 512, H 768: 638 / 514; V 1024, H 320:
+//     560 / 486; nor clusters of 16: 200, V 1024, H 640: 665 / 492; 160, V 1500, H 512:
+//     741 / 460.
 const ChunkShape* chunk_cluster_pick(const std::vector<ChunkShape>& shapes, int n, int H) {
   const ChunkShape* best = nullptr;
   double cost = 0;
@@ -1200,7 +1210,9 @@ const ChunkShape* chunk_cluster_pick(const std::vector<ChunkShape>& shapes, int 
     const int R = (n + s.clusters - 1) / s.clusters;
     const int passes = (R + 8 * s.NB - 1) / (8 * s.NB);
     if (R > s.CS * s.RG || (passes > 1 && !several_passes(s.NB, s.RG))) continue;
-    if (s.RG == 3 && (double)passes * s.nl * H * 2 > 192.0 * 1024) continue;
+    if (s.RG == 1 && passes > 1 && R > 10) continue;
+    if (s.RG == 2 && s.nl > kMB && H >= 512) continue;
+    if (s.RG == 3 && (s.CS != 8 || s.nl > kMB || H >= 768 || passes * s.nl * H * 2 > 170 * 1024)) continue;
     // bytes of W_out a CTA reads per step, a pass's overhead, another row group
     const double c = passes * ((double)s.nl * H * 2 + 32768.0 + 16384.0 * s.NB) + 20000.0 * ((R + s.CS - 1) / s.CS);
     if (!best || c < cost) best = &s, cost = c;

@@ -34,7 +34,8 @@ struct ChunkShape {
 // The shapes whose shared memory holds W_out and the rows' scratch (none:
 // the decoder takes the two-kernel step).
 cudaError_t chunk_cluster_shapes(const DecView& d, std::vector<ChunkShape>& out);
-// The shape for n rows, or nullptr if none holds them in one wave.
+// The shape for n rows, or nullptr if none holds them in one wave or the
+// two-kernel step is faster.
 const ChunkShape* chunk_cluster_pick(const std::vector<ChunkShape>& shapes, int n, int H);
 // The stateful form's joint product with the same sums, for rows that a shape
 // holds: softmax partials per row of N labels, launch.
