@@ -67,9 +67,10 @@ KERNEL_SOURCES = {
 }
 # keyed by (config, streams, kernel, fusion_path)
 TRAFFIC = {
-    (4, 1024, "row", 1): (10575616, "cadf021270fce30e"),
-    (4, 1024, "joint", 0): (11052032, "b67360efb4e1a0ff"),
-    (4, 1024, "row", 0): (29132544, "c491ab3e394847c6"),
+    (4, 1024, "row", 1): (10605312, "b27f1c3eed447754"),
+    (4, 1024, "joint", 0): (11049728, "cd23afe6f21f83fb"),
+    (4, 1024, "joint", 1): (17991168, "cd23afe6f21f83fb"),
+    (4, 1024, "row", 0): (29455616, "61f87a3dc638f818"),
 }
 
 
@@ -91,7 +92,7 @@ def kernel_source_hash(kernel: str) -> str:
 
 # The encoder GEMMs' DRAM traffic per chunk (every k_egemm launch of one
 # chunk step, summed), keyed by (encoder shape, streams, frames per chunk).
-ENC_TRAFFIC = {}  # none recorded for the current encoder GEMM build
+ENC_TRAFFIC = {("0.6b", 256, 13): (4769841408, "bd01849aed58a729")}
 
 
 def recorded_traffic(w: synth.Workload, kernel: str, key=None, path=None):
