@@ -7,8 +7,8 @@
 // few rows is not work but the chain of launches and round trips to L2: 9.4 us
 // a step for one stream (V = 1024, H = 640), 10.4 us for 64, against well
 // under 1 us of arithmetic.  Here a step has no launch, no grid-wide
-// dependency and no logits in memory (13 frames of one stream: 650 -> 204 us,
-// of 64 streams: 665 -> 255 us; 16 streams x 1 frame, H = 1024: 71 -> 30 us):
+// dependency and no logits in memory (13 frames of one stream: 614 -> 169 us,
+// of 64 streams: 665 -> 243 us; 16 streams x 1 frame, H = 1024: 71 -> 29 us):
 //   * CTA c of the cluster keeps its slice of W_out's labels in shared memory for
 //     the whole chunk (read once per chunk, not once per step);
 //   * warps 0-7 (GEMM) compute the slice's logits of all R rows: bf16
@@ -1171,6 +1171,7 @@ cudaError_t chunk_cluster_shapes(const DecView& d, std::vector<ChunkShape>& out)
       if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess) return e;
       if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess) return e;
       for (int CS = 8; CS <= 16; CS *= 2) {
+        if (slice_of(d.N, CS, CS - 1).len == 0) continue;  // every CTA sends logits (chunk_partials.h)
         ChunkShape s;
         s.CS = CS, s.RG = RG, s.NB = NB;
         s.nl = slice_of(d.N, CS, 0).len;  // (the largest)

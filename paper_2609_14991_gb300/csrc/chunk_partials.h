@@ -6,7 +6,8 @@
 // CTA's partial of step s may arrive after another one's of step s + 1: two
 // barriers in turn, so that neither step counts the other's bytes.  Step s + 2
 // cannot overtake: its partials follow every CTA's logits of step s + 1, and
-// the owner sends its own after it has waited for step s's partials.  It reads
+// the owner sends its own (every CTA has labels) after it has waited for step
+// s's partials.  It reads
 // them only at the end of step s + 1, when those of s + 2 may arrive: three
 // buffers.
 #pragma once
